@@ -3,24 +3,44 @@
 // Each problem of a launch is the forward pass of Sec. 3 / Algorithm 1 for one layer (3x3, or the 1x1
 // extension of the appendix) on its own input: decoded +1/-1 weights as 4-bit e2m1 operands (binary
 // activations) or fp16 operands (fp16 activations), implicit GEMM over a padded, flattened position space
-// in which the nine taps are the same staged activations read from shifted start addresses.  One CTA per
+// in which the taps are the same staged activations read from shifted start addresses.  One CTA per
 // SM walks through all problems without any grid-wide step in between: while the MMAs of one problem's
 // last tile run, the expander warps already stage the next problem's first activations, the weight
-// producer streams its first stages, and the epilogue warps still drain the tile before.  Start-up, first
-// loads and last drain, which cost a single-layer launch about as much as its MMAs at batch 64, are paid
-// once per launch.  A single layer is a launch of one problem.
+// producer streams its first stages, and the epilogue warps still drain the tile before.  A single layer is a
+// launch of one problem.
+//
+// Orientation.  The weights are the M operand (128 rows of output channels), the positions the N operand (up to
+// 240, or 256 with fp16), so an accumulator has channels along its lanes and positions along its columns:
+//   * an MMA reads 32 + N/4 shared-memory lines of 128 bytes and takes max(N/2, 32 + N/4) cycles (measured for
+//     N = 16..256, any operand type, any start shift): at N = 240 it leaves a quarter of the shared-memory
+//     bandwidth to the other roles, at N = 128 none;
+//   * a stage of weights serves 240 positions;
+//   * the 32 lanes of an epilogue warp are 32 consecutive channels of one pixel, so that a store instruction
+//     writes one whole 128-byte line straight from registers, with no transposition through shared memory, and any
+//     channel count and row alignment takes the same path.
+// Positions along M and channels along N (at most 128 to 160 of them beside the scale columns) is what this replaced:
+// there the shared memory was the bound (operands at N = 128 take all of its 128 bytes per cycle, the transposition
+// another 8 lines per output row, weights were streamed once per 128 positions).  ResNet-18 layers at batch 64, both on
+// one GPU: group 119 -> 111 us, with fp16 activations 307 -> 254 us, the ResNet-34 stack at batch 128 506 -> 450 us,
+// ResNet-20 group at batch 128 58 -> 46 us, the 1x1 layers 432 -> 397 us.
+//
+// Few output channels (binary activations only).  With at most 64, 32 or 16 channels a lane set holds G = 2, 4 or 8
+// neighbouring output pixels of a row: rows g*(128/G)..  of the weight operand are the channels of pixel G*j + g,
+// and position j of the operand stands for that group of pixels.  The taps of a group are the kernel rows times the
+// columns the group's windows span (stride*(G-1) + 3 instead of G times 3); a row of weights holds zeros where a
+// column is outside its pixel's window.  0 * (+1 / -1 / 0) is exactly 0; with fp16 activations 0 * infinity would
+// not be, so those keep G = 1.
 //
 // Independent problems (a group) need nothing else.  A chain (a stack: problem i + 1 reads the packed signs
 // problem i writes) runs in the same launch on per-tile completion counters: the epilogue bumps the counter
-// of a tile's row block when its part is written, and the expanders of the successor wait (bounded) until the
-// row blocks under a tile's input window are complete.  The launch is cooperative then, so that all CTAs are
+// of a position tile when its part is written, and the expanders of the successor wait (bounded) until the
+// tiles under a tile's input window are complete.  The launch is cooperative then, so that all CTAs are
 // resident while some of them wait.
 //
-// What makes this possible is a ring geometry that is the same for every problem:
+// What makes one launch possible is a ring geometry that is the same for every problem:
 //   activation units  NA slots of a_slot_bytes   (a problem's unit uses a prefix)
 //   weight stages     NS slots of b_slot_bytes   (a stage = whole taps of one channel block)
-//   accumulators      two or three buffers of tensor-memory columns (by operand mode and output kind:
-//                     3 x 160 for word outputs on e2m1 operands, else 2 x 240; 2 x 256 with fp16 operands)
+//   accumulators      n_acc buffers of acc_cols tensor-memory columns
 // so slots, barriers and phases simply carry on from one problem to the next.
 // Tiles of a problem are dealt to the CTAs round-robin; which CTAs get a problem's odd
 // tiles is decided on the host from the time the CTAs have been given so far, so that the
@@ -28,18 +48,21 @@
 //
 //      warp 0        one thread streams weight stages (cp.async.bulk onto mbarriers)
 //      warp 1        issues tcgen05.mma and commits barriers (warp-uniform, one elected lane)
-//      warps 2-9     epilogue: TMEM -> registers -> shared-memory transposition -> alpha ->
-//                    128-byte row stores; or TMEM -> registers -> threshold -> packed sign words
-//      warps 10-19   expanders (13 and 17 idle): packed bits -> e2m1 nibbles (or fp16 copied)
+//      warps 2-9     epilogue: TMEM -> registers -> alpha -> 128-byte stores; or TMEM -> registers ->
+//                    threshold -> 32 x 32 bit transposition in the warp -> packed sign words
+//      warps 10-19   expanders (but 13 and 17): packed bits -> e2m1 nibbles (or fp16 copied)
 //                    into the activation ring
-// The kernel is compiled per operand mode and per output kind (words, the common case of words alone, packed
-// signs, chain), so that no variant carries another one's code in its loops; the plan (tile shapes, accumulator
-// buffers) is made per output kind as well.
+//      warp 13       writes the epilogue's tables (where the columns of a tile go) ahead of it
+// The kernel is compiled per operand mode and per output kind (words, packed signs, chain), so that no variant
+// carries another one's code in its loops; the plan (tile shapes, accumulator buffers) is made per output kind.
 // Every wait is bounded; one that runs out raises a status word the host reads, and
 // the CTA still frees its tensor memory and returns.
 #include <algorithm>
 #include <cstdio>
+#include <cstring>
 #include <vector>
+
+#include <cuda.h>   // tensor maps (types only; the encoder is looked up at run time)
 
 #include "snn_tc_common.cuh"
 
@@ -54,58 +77,69 @@ namespace {
 enum { M_F16 = 1, M_FP4 = 2 };
 constexpr int G_EW = 8;                       // epilogue warps = expander warps
 
-// Warps 13 and 17 stay idle: a warp's scheduler is warp % 4, and the MMA-issuing warp (1) then
-// shares its scheduler with two epilogue warps only instead of two epilogue and two expander warps.
+// Warps 13 and 17 do not expand: a warp's scheduler is warp % 4, and the MMA-issuing warp (1) then shares its
+// scheduler with two epilogue warps and the table warp (13, which has little to do) instead of two expander warps.
 constexpr int G_THREADS = 64 + 64 * G_EW + 64;
 constexpr int G_EXP_THREADS = 32 * G_EW;
-constexpr int G_XTEAMS = 2;                    // teams of expander warps in the pipelined form
-constexpr int G_EXP_ROWS = 3;                 // rows of a unit one expander thread loads together
-constexpr int G_EPI_PITCH = 128;
-constexpr int G_EPI_ALPHA = 1024;              // per epilogue warp: the scales of a tile's channels (at most 256)
-constexpr int G_EPI_WARP = 32 * G_EPI_PITCH + G_EPI_ALPHA;
-constexpr int G_EPI_BYTES = G_EW * G_EPI_WARP;
+constexpr int G_XTEAMS = 2;                    // teams of expander warps (4-bit operands)
+constexpr int G_EXP_ITEMS = 4;                 // loads one expander thread has in flight together
+constexpr int G_ROWS = 128;                    // rows of the weight operand: lanes of an accumulator
+constexpr int G_MAX_CHUNKS = 8;                // 32-column slices of an accumulator (at most 256 columns)
+// What the epilogue needs to know of a tile, written by the table warp (see there), four tiles deep.
+struct GTile {
+  int l, mg, co, n_slices;             // problem (-1: no more tiles), position tile, first channel, 32-column slices
+  int K, kp_log, Np, out_kind;         // channels; logarithm of the rows per pixel; positions; 0 fp32, 1 int32, 2 packed signs
+  uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
+  uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
+  float alpha[G_ROWS], shift[G_ROWS];
+};
+constexpr int G_TILES = 4;
+constexpr int G_EPI_BYTES = G_TILES * (int)sizeof(GTile);
 constexpr int G_NS_MAX = 8;
-constexpr uint32_t G_ACC_COLS = 256;          // tensor-memory columns of one accumulator buffer
-constexpr uint32_t G_ACC_COLS_FP4 = 240;      // 4-bit mode, two buffers: columns 480..511 hold the (unit) block scales
-constexpr uint32_t G_ACC_COLS_FP4_3 = 160;    // 4-bit mode, three buffers
-// Accumulator buffers.  Word outputs on 4-bit operands use three: the MMAs of the tile after next run while both
-// epilogue groups still drain, so a group never waits for them (the epilogue is what bounds that variant).  The
-// other variants are bound elsewhere and do better with two larger buffers (larger tiles).
-constexpr int G_NACC = 2, G_NACC_WORDS = 3;
+constexpr uint32_t G_TMEM_FP4 = 480;          // 4-bit mode: columns 480..511 hold the (unit) block scales
+constexpr uint32_t G_TMEM_F16 = 512;
 constexpr uint32_t G_SCALE_COL = 480;
 constexpr size_t kGTail = 512;
 constexpr size_t kGSmemBudget = 226 * 1024;
-constexpr uint32_t kGASlotMax = 40 * 1024 + 512;   // largest activation unit a problem may stage
-constexpr uint32_t kGBSlot = 32 * 1024;            // bytes of a weight-stage slot
+constexpr uint32_t kGASlotMax = 44 * 1024;         // largest activation unit a problem may stage
+constexpr uint32_t kGASlotMaxTma = 60 * 1024;      // ... when it is fetched by TMA (fp16; whole rows of positions)
+constexpr int kGRowsMax = 1600;                    // ... and its most rows (the pixel tables hold one word per row)
+constexpr uint32_t kGBSlot = 32 * 1024, kGBSlotF16 = 16 * 1024;   // bytes of a weight-stage slot
+constexpr int kGTapsMax = 52;                      // 3 kernel rows x at most 17 columns of a group of 8 pixels
 
-// One problem of a group, as the kernel reads it from global memory.
+// One problem of a launch, as the kernel reads it from shared memory.
 struct GLayer {
-  const uint8_t* wt;      // [layout tile][channel block][tap][chunk][NtL][16 B], owned by the group
+  const uint8_t* wt;      // [channel tile][channel block][step][chunk][128][16 B], owned by the group
   const float* alpha;
   const float* shift;     // per-channel constant added to alpha*S before the sign is taken (packed-sign output)
-  int N, H, W, C, K, Cw, stride, pad, Ho, Wo;
-  int NtL, Nt;            // channels per layout tile of the weight operand / per tile
-  int Hq, Wq;             // rows per image / row pitch of the flattened position space
-  FastDiv dWq, dHq, dNt;
-  int n_planes, halo, Rr; // 1 or 4 planes; largest tap shift; staged rows per plane = 128*MT + halo
-  int MT;                 // M sub-tiles of 128 positions per tile
+  int N, H, W, C, K, Cw, pad, Ho, Wo;
+  int rs, cm, cs;         // input pixel of position (i, j) in plane (pr, pc): row rs*i + pr - pad, column cm*j + cs*pc - pad
+  int G, lg;              // output pixels per position and its logarithm
+  int Hq, Wg;             // rows per image / positions per row of the flattened position space
+  FastDiv dWg, dHq, dCt, dRr;
+  int n_planes, cpl;      // planes of a unit, logarithm of the number of column planes
+  int Np, Rr;             // positions per tile; staged rows per plane = Np + largest tap shift
   int cb_chunks, n_cb, kpt;
-  int taps;               // 9 (3x3 layers) or 1 (the 1x1 extension)
-  int st_taps;            // taps per weight stage (the last stage of a channel block holds taps % st_taps, if not 0)
-  uint32_t tap_bytes;     // weights of one tap of one channel block and channel tile = kpt * 2 * Nt * 16
-  int n_ntiles, total_tiles;
-  const uint16_t* rank;   // [grid] CTA b takes this problem's tiles rank[b], rank[b] + grid, ...
-  long long Qtot;
+  int tma;                // fp16: units are fetched by TMA, rows of 64 channels in the 128-byte swizzle
+  int n_pu, pu_end[4];    // units per channel block (fetched by TMA, each plane is a unit of its own) and the last step of each
+  int steps;              // taps of a tile, or pairs of taps (one activation word per pixel: a K = 64 step covers two taps)
+  int st_steps;           // steps per weight stage (the last stage of a channel block holds steps % st_steps, if not 0)
+  uint32_t step_bytes;    // weights of one step of one channel block = kpt * 2 * 128 * 16
+  int n_ct, total_tiles;  // channel tiles of 128
+  int first;              // this CTA's first tile, filled in by the kernel (GParams::ranks)
+  uint32_t Qtot;
   // A chain (every member reads the packed signs its predecessor writes, all in one launch): a tile may be
   // staged once the predecessor's tiles that hold its input pixels are complete, and says so itself when done.
-  const uint2* deps;          // [M groups] first and last M group of the predecessor this M group reads (x > y: none)
+  const uint2* deps;          // [position tiles] first and last position tile of the predecessor this one reads (x > y: none)
   const uint32_t* prev_done;  // the predecessor's completion counters, and the count that means "complete"
   uint32_t prev_target;
-  uint32_t* done;             // [M groups] epilogue warps that have finished the group, over all its channel tiles
+  uint32_t* done;             // [position tiles] epilogue warps that have finished the tile, over all its channel tiles
+  uint32_t tap[kGTapsMax];    // per step: start of its rows in the unit (16-byte units) | distance of its two chunks << 16
 };
 
 struct GParams {
   const GLayer* layers;
+  const uint16_t* ranks;  // [n_layers][grid] CTA b takes a problem's tiles ranks[b], ranks[b] + grid, ...
   int n_layers;
   const void* act[SNN_GROUP_MAX];
   void* out[SNN_GROUP_MAX];
@@ -116,7 +150,6 @@ struct GParams {
   int NA, NS;
   uint32_t a_slot_bytes, b_slot_bytes;
   uint32_t off_b, off_epi, off_pix, off_lay, off_tail;
-  uint32_t pix_words;     // entries of one pixel table (the pipelined expanders keep one per team)
 };
 
 // Profiling aid (build with -DSNN_TRACE): every role's reporting lane adds up the cycles it spends in its
@@ -124,8 +157,6 @@ struct GParams {
 #ifdef SNN_TRACE
 __device__ long long g_trace[256 * 16];
 #define TR_WAIT(var, expr) ([&]() { const long long _t = clock64(); const bool _r = (expr); var += clock64() - _t; return _r; }())
-#define TR_BEGIN(t) const long long t = clock64()
-#define TR_END(var, t) var += clock64() - t
 #define TR_REPORT(role, total, w0, w1, w2)                         \
   do {                                                             \
     long long* _o = g_trace + (size_t)blockIdx.x * 16 + (role)*4;  \
@@ -133,31 +164,31 @@ __device__ long long g_trace[256 * 16];
   } while (0)
 #else
 #define TR_WAIT(var, expr) (expr)
-#define TR_BEGIN(t) do { } while (0)
-#define TR_END(var, t) do { } while (0)
 #define TR_REPORT(role, total, w0, w1, w2) do { } while (0)
 #endif
 
-__device__ __forceinline__ int g_position_to_pixel(const GLayer& L, uint32_t q, int pa, int pb) {
-  if ((long long)q >= L.Qtot) return -1;
-  const uint32_t rg = fdiv(q, L.dWq);
-  const int j = (int)(q - rg * (uint32_t)L.Wq);
-  const uint32_t n = fdiv(rg, L.dHq);
-  const int i = (int)(rg - n * (uint32_t)L.Hq);
-  if ((int)n >= L.N) return -1;
-  const int r = L.stride * i + pa - L.pad, c = L.stride * j + pb - L.pad;
+// input pixel of row q (a position, possibly past a tile's own) in plane pl, or -1: padding or past the batch
+__host__ __device__ __forceinline__ int g_pixel_of(const GLayer& L, uint32_t n, int i, int j, int pl) {
+  const int r = L.rs * i + (pl >> L.cpl) - L.pad, c = L.cm * j + L.cs * (pl & ((1 << L.cpl) - 1)) - L.pad;
   if (r < 0 || r >= L.H || c < 0 || c >= L.W) return -1;
   return ((int)n * L.H + r) * L.W + c;
+}
+__device__ __forceinline__ int g_position_to_pixel(const GLayer& L, uint32_t q, int pl) {
+  if (q >= L.Qtot) return -1;
+  const uint32_t rg = fdiv(q, L.dWg);
+  const int j = (int)(q - rg * (uint32_t)L.Wg);
+  const uint32_t n = fdiv(rg, L.dHq);
+  return g_pixel_of(L, n, (int)(rg - n * (uint32_t)L.Hq), j, pl);
 }
 
 // Bounded wait until a completion counter another CTA advances has reached `target` (acquire: what that CTA
 // wrote before is visible afterwards).  False when the limit ran out or the CTA is giving up.
-__device__ __forceinline__ bool g_wait_counter(const uint32_t* ctr, uint32_t target, volatile int* abort_flag) {
-  for (uint32_t it = 0; it < (1u << 21); ++it) {
+__device__ __forceinline__ bool g_wait_counter(const uint32_t* ctr, uint32_t target, volatile int* abort_flag, uint32_t limit) {
+  for (uint32_t it = 0; it < limit; ++it) {
     uint32_t v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
     if (v >= target) return true;
-    if (*abort_flag) return false;
+    if (limit == 1 || *abort_flag) return false;
     __nanosleep(100);
   }
   return false;
@@ -170,53 +201,52 @@ __device__ __forceinline__ uint2 g_ld2(const uint32_t* p, bool fresh) {
 __device__ __forceinline__ uint4 g_ld4(const uint32_t* p, bool fresh) {
   return fresh ? __ldcg(reinterpret_cast<const uint4*>(p)) : __ldg(reinterpret_cast<const uint4*>(p));
 }
-
-// first tile of problem L for this CTA (tiles then follow at a stride of the grid)
-__device__ __forceinline__ int g_first_tile(const GLayer& L) {
-  return (int)__ldg(L.rank + blockIdx.x);
+// Words of a row that are loaded together: activations are 16-byte aligned, so a row can be read four (two) words
+// at a time where the words per pixel and per channel block are multiples of four (two).
+__host__ __device__ __forceinline__ int g_word_step(int Cw, int cb_chunks) {
+  return (Cw & 3) == 0 && (cb_chunks & 3) == 0 ? 4 : (Cw & 1) == 0 && (cb_chunks & 1) == 0 ? 2 : 1;
 }
 
-// The MMAs of one channel block of one tile: 9 taps x KPT K steps x MT sub-tiles.  The body of
-// a tap is straight-line code; the taps are a loop, because the issuing thread runs alone on
-// its warp and nine unrolled taps no longer fit the instruction cache closest to it.
-// Weight stages are waited for and released as the K-step counter crosses their boundaries.
-template <int MODE, int MT, int KPT>
-__device__ __forceinline__ bool g_issue_block(uint64_t a_unit, uint32_t wq, uint32_t plane_units, bool s2, uint32_t a_step,
-                                              uint64_t b_desc0, uint32_t b_slot_units, uint32_t b_step, uint32_t d0,
-                                              uint32_t nt, uint32_t idesc, uint32_t& acc, int taps, int st_taps, int NS,
-                                              uint32_t bar_bfull, uint32_t bar_bempty, int& b_slot, uint32_t& b_phase,
-                                              bool leader, uint32_t sf, long long& tr_b) {
-  uint32_t ky = 0, kx = 0;
-  int t = 0;
+// Tensor maps of the fp16 activations, a kernel parameter of its own (the other variants have one unused entry).
+template <int MODE>
+struct GMaps {
+  CUtensorMap m[MODE == M_F16 ? SNN_GROUP_MAX : 1];
+};
+
+// The MMAs of one activation unit of one tile: steps t..t_last x KPT.  The body of a step is straight-line code.
+// Weight stages are waited for and released as the step counter crosses their boundaries.
+template <int MODE, int KPT>
+__device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last, uint64_t a_fixed, uint32_t k_step, uint32_t a_unit, uint32_t w_base, uint32_t b_slot_units,
+                                              uint32_t d0, uint32_t idesc, uint32_t& acc, int NS, uint32_t bar_bfull,
+                                              uint32_t bar_bempty, int& b_slot, uint32_t& b_phase, bool leader, uint32_t sf,
+                                              long long& tr_b) {
+  constexpr uint64_t fixed = ((uint64_t)1 << 46) | ((uint64_t)8 << 32);   // descriptor version; 8-row groups 128 bytes apart
+  constexpr uint64_t w_fixed = fixed | ((uint64_t)128 << 16);             // the weights' chunks are 128 rows apart
+  const int st_steps = L.st_steps;
+  uint32_t tap = L.tap[t];
 #pragma unroll 1
-  while (t < taps) {
-    // a weight stage holds whole taps: one wait, then nothing but MMAs until its last tap
+  while (t < t_last) {
+    // a weight stage holds whole steps: one wait, then nothing but MMAs until its last step
     if (!TR_WAIT(tr_b, mbar_wait(bar_bfull + 8 * b_slot, b_phase))) return false;
     tc_fence_after();
-    uint64_t bd = b_desc0 + (uint64_t)((uint32_t)b_slot * b_slot_units);
-    const int t_end = t + st_taps < taps ? t + st_taps : taps;
+    uint32_t wa = w_base + (uint32_t)b_slot * b_slot_units;
+    const int t_end = t + st_steps < t_last ? t + st_steps : t_last;
 #pragma unroll 1
     for (; t < t_end; ++t) {
-      // rows (16-byte units) from a unit's origin to tap (ky, kx): a shift inside the plane, plus, for stride 2,
-      // the offset of the tap's parity plane
-      const uint32_t tap = s2 ? ((ky & 1u) * 2u + (kx & 1u)) * plane_units + (ky >> 1) * wq + (kx >> 1) : ky * wq + kx;
-      if (++kx == 3) { kx = 0; ++ky; }
-      const uint64_t ad_t = a_unit + (uint64_t)tap;
+      const uint32_t cur = tap;
+      if (t + 1 < t_last) tap = L.tap[t + 1];
+      const uint64_t bd = a_fixed | ((uint64_t)(cur >> 16) << 16) | (uint64_t)(a_unit + (cur & 0xffffu));
+      const uint64_t wd = w_fixed | (uint64_t)wa;
       if (leader) {
 #pragma unroll
         for (int k = 0; k < KPT; ++k) {
-#pragma unroll
-          for (int mt = 0; mt < MT; ++mt) {
-            const uint64_t ad = ad_t + (uint64_t)((uint32_t)k * a_step + (uint32_t)(mt * 128));
-            const uint64_t bdk = bd + (uint64_t)((uint32_t)k * b_step);
-            const uint32_t accum = k == 0 ? acc : 1u;
-            if (MODE == M_FP4) mma_ss_fp4(d0 + (uint32_t)mt * nt, ad, bdk, idesc, accum, sf, sf + 16);
-            else mma_ss_f16(d0 + (uint32_t)mt * nt, ad, bdk, idesc, accum);
-          }
+          const uint32_t accum = k == 0 ? acc : 1u;
+          if (MODE == M_FP4) mma_ss_fp4(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum, sf, sf + 16);
+          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum);
         }
       }
       acc = 1;
-      bd += (uint64_t)((uint32_t)KPT * b_step);
+      wa += KPT * 256;
     }
     if (leader) tc_commit(bar_bempty + 8 * b_slot);  // the slot is free once these MMAs have read it
     if (++b_slot == NS) { b_slot = 0; b_phase ^= 1u; }
@@ -224,70 +254,70 @@ __device__ __forceinline__ bool g_issue_block(uint64_t a_unit, uint32_t wq, uint
   return true;
 }
 
+// Rows of a 32 x 32 bit matrix (lane r holds row r) to columns (lane c holds column c, bit r = row r).
+__device__ __forceinline__ uint32_t g_transpose32(uint32_t x, int lane) {
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    const uint32_t m = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u : 0x55555555u;
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
+    x = (lane & s) ? ((x & ~m) | ((y >> s) & m)) : ((x & m) | ((y << s) & ~m));
+  }
+  return x;
+}
+
 }  // namespace
 
 // OUTK: what the epilogue is compiled for.  0: fp32 or int32 words for every member; 1: packed signs for every
 // member; 2: a chain - packed signs between the members, any type for the last, and the dependency waits and
 // completion counters.  Keeping the variants apart keeps each one's registers and code to what it needs.
-// 3: the common case of 0 compiled alone - fp32 outputs, 4-bit operands, every member's channel count a multiple
-// of 4 and its channel tile a multiple of 32, rows readable two words at a time: the expanders run their
-// two-stage load pipeline instead of the plain loop, and the epilogue has its one fast path and no other.  The
-// roles share instruction caches; what a variant does not carry makes the rest faster.
-enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2, OUT_WORDS_PIPED = 3 };
+enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2 };
 
 template <int MODE, int OUTK>
-__global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p) {
+__global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p, const __grid_constant__ GMaps<MODE> maps) {
   constexpr bool F16 = MODE == M_F16;   // fp16 activations (copied, not expanded)
   constexpr bool FP4 = MODE == M_FP4;   // binary activations as e2m1 nibbles
   constexpr bool CHAIN = OUTK == OUT_CHAIN;
-  constexpr bool WORDS = OUTK == OUT_WORDS || OUTK == OUT_WORDS_PIPED;
-  constexpr bool PIPED = OUTK == OUT_WORDS_PIPED;
-  // Word outputs (fp32 / int32) are bound by the stores: there the epilogue warps form two groups of four (one
-  // warp per quarter of the accumulator's lanes) that take the tiles in turn, group g draining accumulator
-  // buffer g, so that one group's stores drain while the other reads tensor memory and transposes.  Packed
-  // signs are bound by the epilogue's instructions: all eight warps drain every tile together.
-  constexpr bool G_EPI_SPLIT = WORDS;
-  constexpr int G_EPI_ARRIVALS = G_EPI_SPLIT ? G_EW / 2 : G_EW;   // epilogue warps that drain one tile
-  extern __shared__ __align__(128) uint8_t smem[];
-  // carve-up: [NA activation slots][NS weight slots][epilogue tiles][pixel table][problem table][barriers, flags]
+  constexpr bool WORDS = OUTK == OUT_WORDS;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  // carve-up: [NA activation slots][NS weight slots][epilogue tables][pixel tables][problem table][barriers, flags]
   uint8_t* a_smem = smem;
   uint8_t* b_smem = smem + p.off_b;
   uint8_t* epi_smem = smem + p.off_epi;
   int* pix_tab = reinterpret_cast<int*>(smem + p.off_pix);
   // The problems' descriptions are read from shared memory where they are needed instead of
-  // being held in registers: the roles are at different problems at the same time, and the
-  // epilogue's registers are all taken by the slices it transposes.
-  const GLayer* lay = reinterpret_cast<const GLayer*>(smem + p.off_lay);
+  // being held in registers: the roles are at different problems at the same time.
+  GLayer* lay = reinterpret_cast<GLayer*>(smem + p.off_lay);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_tail);
-  // barriers: b_full[8] b_empty[8] a_full[4] a_empty[4] acc_full[4] acc_empty[3]
-  // acc_full is indexed by the tile's sequence number in the CTA (seq % 4), not by the buffer: an epilogue group
-  // that takes every other tile then sees every phase of the barriers it waits on (seq % 4 = g and g + 2), and a
-  // barrier's next phase cannot complete before its last one was consumed (tile seq + 3 needs the buffer tile seq
-  // releases).  acc_empty is per buffer.
+  // barriers: b_full[8] b_empty[8] a_full[4] a_empty[4] acc_full[4] acc_empty[4] tab_full[4] tab_empty[4]
+  // acc_full and the epilogue's tables are indexed by the tile's sequence number in the CTA (seq % 4), acc_empty by
+  // the accumulator buffer.
   const uint32_t bar_bfull = smem_u32(bars), bar_bempty = smem_u32(bars + 8);
   const uint32_t bar_afull = smem_u32(bars + 16), bar_aempty = smem_u32(bars + 20);
   const uint32_t bar_accfull = smem_u32(bars + 24), bar_accempty = smem_u32(bars + 28);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 31);
+  const uint32_t bar_tabfull = smem_u32(bars + 32), bar_tabempty = smem_u32(bars + 36);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 40);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = p.NS, NA = p.NA;
   const int G = (int)gridDim.x;
 
-  if (tid < 31) {
+  if (tid < 40) {
     uint32_t count = 1;
-    if (tid >= 28) count = G_EPI_ARRIVALS;             // acc_empty: one arrival per epilogue warp of the tile
-    if (tid >= 16 && tid < 20)   // a_full: every expander thread arrives, or one lane per expander warp (pipelined form)
-      count = PIPED ? G_EXP_THREADS / 32 / G_XTEAMS : G_EXP_THREADS;
+    if ((tid >= 28 && tid < 32) || tid >= 36) count = G_EW;               // acc_empty, tab_empty: one arrival per epilogue warp of the tile
+    if (tid >= 16 && tid < 20) count = FP4 ? G_EW / G_XTEAMS : G_EW;    // a_full: one arrival per expander warp of the unit
     mbar_init(smem_u32(bars + tid), count);
   }
-  if (tid == 32) *abort_flag = 0;
+  if (tid == 64) *abort_flag = 0;
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
     uint32_t* dst = reinterpret_cast<uint32_t*>(smem + p.off_lay);
     const int words = p.n_layers * (int)(sizeof(GLayer) / 4);
     for (int i = tid; i < words; i += G_THREADS) dst[i] = __ldg(src + i);
   }
+  // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
+  int first = 0;
+  if (tid < p.n_layers) first = (int)__ldg(p.ranks + (size_t)tid * G + blockIdx.x);
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(512)
@@ -300,14 +330,15 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   grid_dep_launch();
+  if (tid < p.n_layers) lay[tid].first = first;
   if (FP4) {
     // unit block scales: every byte of the scale columns is the ue8m0 code of 1.0, in all 128 lanes
     // (warps 2..5 cover the four lane quarters), whatever part of them an MMA reads
     if (warp >= 2 && warp < 6) tmem_fill32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + G_SCALE_COL, 0x7f7f7f7fu);
     tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
   }
+  __syncthreads();
+  if (FP4) tc_fence_after();
 
   if (warp == 0) {
     // ------------------------------------------------ weight producer (one lane)
@@ -320,40 +351,26 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
       (void)tr_w0; (void)tr_t0;
       for (int l = 0; l < p.n_layers && ok; ++l) {
         const GLayer& L = lay[l];
-        const int Nt = L.Nt, NtL = L.NtL, n_cb = L.n_cb, n_ntiles = L.n_ntiles, total = L.total_tiles;
-        const int taps = L.taps, st_taps = L.st_taps, stages_per_cb = (taps + st_taps - 1) / st_taps;
-        const int chunks_per_tap = 2 * L.kpt;
-        const uint32_t tap_bytes = L.tap_bytes;
+        const int n_cb = L.n_cb, n_ct = L.n_ct, total = L.total_tiles, steps = L.steps, st_steps = L.st_steps, n_pu = L.n_pu;
+        const uint32_t step_bytes = L.step_bytes;
         const uint8_t* wt = L.wt;
-        const size_t cb_bytes = (size_t)taps * L.cb_chunks * NtL * 16;   // one channel block of one layout tile
-        const FastDiv dNt = L.dNt;
-        for (int tile = g_first_tile(L); tile < total && ok; tile += G) {
+        const size_t ct_bytes = (size_t)n_cb * (size_t)steps * step_bytes;   // one channel tile
+        const FastDiv dCt = L.dCt;
+        for (int tile = L.first; tile < total && ok; tile += G) {
           if (*abort_flag) { ok = false; break; }
-          const int nti = tile - (int)fdiv((uint32_t)tile, dNt) * n_ntiles;
-          const int n0 = nti * Nt;
-          const int ltile = Nt == NtL ? nti : n0 / NtL;
-          const int n_in = n0 - ltile * NtL;
-          const uint8_t* src_tile = wt + (size_t)ltile * n_cb * cb_bytes + (size_t)n_in * 16;
-          for (int cb = 0; cb < n_cb && ok; ++cb) {
-            const uint8_t* src = src_tile + (size_t)cb * cb_bytes;
-            for (int sg = 0; sg < stages_per_cb; ++sg) {
-              const int ntaps = taps - sg * st_taps < st_taps ? taps - sg * st_taps : st_taps;
-              const uint32_t stage_bytes = (uint32_t)ntaps * tap_bytes;
-              const int chunks_per_stage = ntaps * chunks_per_tap;
+          const uint8_t* src = wt + (size_t)(tile - (int)fdiv((uint32_t)tile, dCt) * n_ct) * ct_bytes;
+          for (int u = 0, t = 0; u < n_cb * n_pu && ok; ++u) {
+            const int t_last = L.pu_end[u & (n_pu - 1)];
+            for (t = t >= steps ? 0 : t; t < t_last; t += st_steps) {
+              const uint32_t stage_bytes = (uint32_t)(t_last - t < st_steps ? t_last - t : st_steps) * step_bytes;
               if (b_issued >= NS && !TR_WAIT(tr_w0, mbar_wait_backoff(bar_bempty + 8 * b_slot, b_phase, 32))) { ok = false; break; }
-              const uint32_t dst = smem_u32(b_smem) + (uint32_t)b_slot * p.b_slot_bytes;
               mbar_expect_tx(bar_bfull + 8 * b_slot, stage_bytes);
-              if (Nt == NtL) {
-                bulk_g2s(dst, src, stage_bytes, bar_bfull + 8 * b_slot);  // the stage's chunks are contiguous
-              } else {
-                for (int c = 0; c < chunks_per_stage; ++c)
-                  bulk_g2s(dst + (uint32_t)c * Nt * 16, src + (size_t)c * NtL * 16, (uint32_t)Nt * 16,
-                           bar_bfull + 8 * b_slot);
-              }
-              src += (size_t)chunks_per_stage * NtL * 16;
+              bulk_g2s(smem_u32(b_smem) + (uint32_t)b_slot * p.b_slot_bytes, src, stage_bytes, bar_bfull + 8 * b_slot);
+              src += stage_bytes;
               ++b_issued;
               if (++b_slot == NS) { b_slot = 0; b_phase ^= 1u; }
             }
+            t = t_last;
           }
         }
       }
@@ -384,46 +401,48 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
       long long tr_w0 = 0, tr_w1 = 0, tr_w2 = 0, tr_t0 = clock64();
       (void)tr_w0; (void)tr_w1; (void)tr_w2; (void)tr_t0;
       const uint32_t a_slot_units = p.a_slot_bytes >> 4, b_slot_units = p.b_slot_bytes >> 4;
+      const uint32_t a_base = smem_u32(a_smem) >> 4, w_base = smem_u32(b_smem) >> 4, sf = tmem_base + G_SCALE_COL;
       for (int l = 0; l < p.n_layers && ok; ++l) {
         const GLayer& L = lay[l];
-        const int Nt = L.Nt, Rr = L.Rr, n_cb = L.n_cb, MT = L.MT, kpt = L.kpt, total = L.total_tiles;
-        const int st_taps = L.st_taps;
+        const int n_units = L.n_cb * L.n_pu, n_pu = L.n_pu, kpt = L.kpt, total = L.total_tiles;
+        // activation operand: rows of 16 bytes, 8-row groups 128 bytes apart, a K step two chunks on; or rows of 128 bytes
+        // in the 128-byte swizzle, 8-row groups 1024 bytes apart, a K step 32 bytes on.  (The swizzle permutes address
+        // bits, so a tap's start may be any row.)
+        const bool swz = F16 && L.tma;
+        const uint64_t a_fixed = ((uint64_t)1 << 46) | (swz ? ((uint64_t)2 << 61) | ((uint64_t)64 << 32) : (uint64_t)8 << 32);
+        const uint32_t k_step = swz ? 2u : 2u * (uint32_t)(L.n_planes * L.Rr);
         // instruction descriptor: D format, A/B formats, K-major both, N>>3, M>>4
         // (4-bit mode: A/B format e2m1, scale format ue8m0, scale ids 0)
         const uint32_t idesc =
-            F16 ? ((1u << 4) | ((uint32_t)(Nt >> 3) << 17) | ((128u >> 4) << 24))
-                : ((1u << 7) | (1u << 10) | ((uint32_t)(Nt >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24));
-        const uint64_t a_desc0 = make_desc(smem_u32(a_smem), (uint32_t)Rr * 16, 128);
-        const uint64_t b_desc0 = make_desc(smem_u32(b_smem), (uint32_t)Nt * 16, 128);
-        const uint32_t a_step = 2u * (uint32_t)Rr, b_step = 2u * (uint32_t)Nt;  // two chunks per MMA
-        for (int tile = g_first_tile(L); tile < total && ok; tile += G, ++tiles_done) {
+            F16 ? ((1u << 4) | ((uint32_t)(L.Np >> 3) << 17) | ((128u >> 4) << 24))
+                : ((1u << 7) | (1u << 10) | ((uint32_t)(L.Np >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24));
+        for (int tile = L.first; tile < total && ok; tile += G, ++tiles_done) {
           if (tiles_done >= n_acc) {
             if (!TR_WAIT(tr_w0, mbar_wait(bar_accempty + 8 * acc_slot, acc_phase))) { ok = false; break; }
             tc_fence_after();
           }
           const uint32_t d0 = tmem_base + (uint32_t)acc_slot * p.acc_cols;
-          uint32_t acc = 0;  // 0 only for the first MMA of every sub-tile
-          for (int cb = 0; cb < n_cb && ok; ++cb) {
+          uint32_t acc = 0;  // 0 only for the first MMA of the tile
+          uint32_t row0 = 0;   // a unit fetched by TMA starts at the beginning of a row of positions
+          if (swz) {
+            const uint32_t Q0 = fdiv((uint32_t)tile, L.dCt) * (uint32_t)L.Np;
+            row0 = 8u * (Q0 - fdiv(Q0, L.dWg) * (uint32_t)L.Wg);
+          }
+          for (int u = 0, t = 0; u < n_units && ok; ++u) {
             if (!TR_WAIT(tr_w1, mbar_wait(bar_afull + 8 * a_slot, a_phase))) { ok = false; break; }
             tc_fence_after();
-            const uint64_t a_unit = a_desc0 + (uint64_t)((uint32_t)a_slot * a_slot_units);
-#define G_ISSUE(M, KP)                                                                                       \
-  ok = g_issue_block<MODE, M, KP>(a_unit, (uint32_t)L.Wq, (uint32_t)(L.cb_chunks * Rr), L.stride != 1, a_step, b_desc0, b_slot_units, b_step, d0, (uint32_t)Nt, idesc, acc, \
-                                  L.taps, st_taps, NS, bar_bfull, bar_bempty, b_slot, b_phase, leader,                   \
-                                  tmem_base + G_SCALE_COL, tr_w2)
-#define G_ISSUE_K(M)                   \
-  do {                                 \
-    if (kpt == 4) G_ISSUE(M, 4);       \
-    else if (kpt == 2) G_ISSUE(M, 2);  \
-    else if (kpt == 3) G_ISSUE(M, 3);  \
-    else G_ISSUE(M, 1);                \
-  } while (0)
-            if (MT == 4) G_ISSUE_K(4);
-            else if (MT == 3) G_ISSUE_K(3);
-            else if (MT == 2) G_ISSUE_K(2);
-            else G_ISSUE_K(1);
-#undef G_ISSUE_K
+            const uint32_t a_unit = a_base + (uint32_t)a_slot * a_slot_units + row0;
+            const int pu = u & (n_pu - 1), t_last = L.pu_end[pu];
+            if (pu == 0) t = 0;
+#define G_ISSUE(KP)                                                                                                  \
+  ok = g_issue_block<MODE, KP>(L, t, t_last, a_fixed, k_step, a_unit, w_base, b_slot_units, d0, idesc, acc, NS, bar_bfull, bar_bempty, b_slot, \
+                               b_phase, leader, sf, tr_w2)
+            if (kpt == 4) G_ISSUE(4);
+            else if (kpt == 2) G_ISSUE(2);
+            else if (kpt == 3) G_ISSUE(3);
+            else G_ISSUE(1);
 #undef G_ISSUE
+            t = t_last;
             if (!ok) break;
             if (leader) tc_commit(bar_aempty + 8 * a_slot);  // the activation unit may be overwritten
             if (++a_slot == NA) { a_slot = 0; a_phase ^= 1u; }
@@ -444,372 +463,307 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
   } else if (warp < 2 + G_EW) {
     // ------------------------------------------------ epilogue warps
     grid_dep_wait();  // an earlier kernel in the stream may still read the output buffers
-    // Warp w reads TMEM lanes 32*(w%4).. (rows of the tile); the two warps of a lane quarter take
-    // the 32-column slices in turn.  A slice goes through a per-warp shared-memory tile so that
-    // each store instruction writes whole 128-byte rows.
+    // Warp w reads TMEM lanes 32*(w%4)..: 32 rows of the weight operand = 32 channels (or, with 8 pixels per
+    // position, 16 channels of two pixels).  32 columns = 32 positions are read at a time.
     const int ew = warp - 2;
     const int rq = warp & 3, half = ew >> 2;
-    const int cfirst = G_EPI_SPLIT ? 0 : 32 * half, cstep = G_EPI_SPLIT ? 32 : 64;   // this warp's 32-column slices
-    long long seq = 0;   // tiles of this CTA so far, over all problems (the MMA issuer alternates the buffers the same way)
-    uint8_t* stage = epi_smem + (size_t)ew * G_EPI_WARP;
-    const uint32_t a_stage = smem_u32(stage) + 32 * G_EPI_PITCH;   // this warp's copy of the tile's scales
-    const int srow = lane >> 3, scol = lane & 7;  // this lane's (row mod 4, 16-byte column) when storing
-    // Staging tile: row r, 16-byte chunk c sits at r*128 + ((c ^ (r & 7)) << 4).  A lane writes its own row
-    // (chunk e at st_lane ^ (e << 4)) and reads chunk scol of rows srow + 4i.
-    const uint32_t st_lane = smem_u32(stage) + (uint32_t)(lane * G_EPI_PITCH + ((lane & 7) << 4));
-    const uint32_t ld_even = smem_u32(stage) + (uint32_t)(srow * G_EPI_PITCH + ((scol ^ srow) << 4));
-    const uint32_t ld_odd = smem_u32(stage) + (uint32_t)((srow + 4) * G_EPI_PITCH + ((scol ^ (srow + 4)) << 4));
-    (void)st_lane; (void)ld_even; (void)ld_odd;
-    int acc_slot = 0;   // buffer of tile seq: seq % n_acc, kept in step with seq
+    const int row = rq * 32 + lane;
     const int n_acc = p.n_acc;
-    bool live = true;
-    long long tr_w0 = 0, tr_w1 = 0, tr_w2 = 0, tr_t0 = clock64();
-    (void)tr_w0; (void)tr_w1; (void)tr_w2; (void)tr_t0;
-    for (int l = 0; l < p.n_layers && live; ++l) {
-      const GLayer& L = lay[l];
-      const int Nt = L.Nt, MT = L.MT, K = L.K;
-      const float* alpha = L.alpha;
-      const float* shift = L.shift;
-      const int out_i32 = PIPED ? 0 : WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
-      uint32_t* out32 = reinterpret_cast<uint32_t*>(p.out[l]);  // int32 and fp32 outputs share the layout
-      const bool fast = PIPED || (((K & 3) == 0) && ((Nt & 31) == 0));   // (checked on the host for variant 3)
-      for (int tile = g_first_tile(L); tile < L.total_tiles; tile += G, ++seq, acc_slot = acc_slot + 1 == n_acc ? 0 : acc_slot + 1) {
-        if (G_EPI_SPLIT && (int)(seq & 1) != half) continue;   // the other group's tile
-        const uint32_t full_bar = bar_accfull + 8u * (uint32_t)(seq & 3), full_phase = (uint32_t)((seq >> 2) & 1);
-        const int mg = (int)fdiv((uint32_t)tile, L.dNt), nti = tile - mg * L.n_ntiles;
-        const uint32_t Q0 = (uint32_t)mg * (uint32_t)(128 * MT);
-        const int n0 = nti * Nt;
-        int okw = 1;
-        if (lane == 0) okw = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(full_bar, full_phase, 100))) ? 1 : 0;
+    uint32_t seq = 0;   // tile of this CTA, over all problems
+    int acc_slot = 0;   // its buffer: seq % n_acc
+    long long tr_w0 = 0, tr_t0 = clock64();
+    (void)tr_w0; (void)tr_t0;
+    for (;;) {
+      const GTile* const T = reinterpret_cast<const GTile*>(epi_smem) + (seq & 3u);
+      const uint32_t tile_phase = (seq >> 2) & 1u;   // (acc_full and the tables are indexed and flip alike)
+      int okw = 1;
+      if (lane == 0) okw = (!*abort_flag && mbar_wait_backoff(bar_tabfull + 8u * (seq & 3u), tile_phase, 100)) ? 1 : 0;
+      okw = __shfl_sync(0xffffffffu, okw, 0);
+      if (!okw) {
+        if (lane == 0 && !*abort_flag) {
+          *abort_flag = 1;
+          raise_status(p.status, 6);
+        }
+        break;
+      }
+      __syncwarp();
+      const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
+      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, Np = h1.z;
+      if (l < 0) break;   // no more tiles
+      const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : h1.w;
+      uint32_t* const out32 = reinterpret_cast<uint32_t*>(p.out[l]);  // int32 and fp32 outputs share the layout
+      // this lane's row of the weight operand: pixel g of a position's group, channel c of the channel tile
+      const int g_lane = row >> kp_log, c_lane = row & ((1 << kp_log) - 1);
+      const int g_warp = (rq * 32) >> kp_log, c_warp = (rq * 32) & ((1 << kp_log) - 1);   // of lane 0
+      const int co = h0.z + c_lane, co_warp = h0.z + c_warp;
+      const bool active = co_warp < K;   // does any of the warp's rows hold a channel?
+      const float al = T->alpha[c_lane], sh = WORDS ? 0.f : T->shift[c_lane];
+      {
+        if (lane == 0) okw = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_accfull + 8u * (seq & 3u), tile_phase, 100))) ? 1 : 0;
         okw = __shfl_sync(0xffffffffu, okw, 0);
         if (!okw) {
           if (lane == 0 && !*abort_flag) {
             *abort_flag = 1;
             raise_status(p.status, 4);
           }
-          live = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d0 = tmem_base + (uint32_t)acc_slot * p.acc_cols;
-        // output pixel (n*Ho + y)*Wo + x of the row of sub-tile mt this lane owns in TMEM, or -1
-        auto row_pixel = [&](int mt) -> int {
-          const uint32_t q = Q0 + (uint32_t)(mt * 128 + rq * 32 + lane);
-          const uint32_t rg = fdiv(q, L.dWq);
-          const int x = (int)(q - rg * (uint32_t)L.Wq);
-          const uint32_t n = fdiv(rg, L.dHq);
-          const int y = (int)(rg - n * (uint32_t)L.Hq);
-          const bool valid = ((long long)q < L.Qtot) && ((int)n < L.N) && (y < L.Ho) && (x < L.Wo);
-          return valid ? ((int)n * L.Ho + y) * L.Wo + x : -1;
+        const uint32_t d0 = tmem_base + (uint32_t)acc_slot * p.acc_cols + ((uint32_t)(rq * 32) << 16);
+        // this warp has read its part of the accumulator buffer: hand it back to the MMA issuer
+        auto release = [&]() {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_accempty + 8 * acc_slot);
         };
-        if (!WORDS && out_i32 == 2) {
-          // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): a thread
-          // owns one position and the 32 (or 16) consecutive channels of a slice, i.e. one word (or
-          // half-word) of the next layer's binary input.  No transposition, one small store per slice.
-          const int Kw = (K + 31) >> 5;
-          // the scale and threshold arrays can be read four at a time (their allocations are; a tile starts at a multiple of 16)
-          const bool sign_vec = ((reinterpret_cast<uintptr_t>(alpha) | reinterpret_cast<uintptr_t>(shift)) & 15) == 0;
-          if ((Nt & 31) == 0) {
-            const int per_mt = (Nt - cfirst + cstep - 1) / cstep;
-#pragma unroll 1
-            for (int mt = 0; mt < MT; ++mt) {
-              const int pix = row_pixel(mt);
-#pragma unroll 1
-              for (int ci = 0; ci < per_mt; ++ci) {
-                const int c0 = cfirst + cstep * ci, co0 = n0 + c0;
-                uint32_t v[32];
-                __syncwarp();  // the load is a warp-wide instruction: no lane may still be in the store below
-                tmem_ld32(d0 + ((uint32_t)(rq * 32) << 16) + (uint32_t)(mt * Nt + c0), v);
-                tmem_ld_wait();
-                if (pix >= 0 && co0 + 32 <= K && sign_vec) {
-                  // all 32 channels exist: scales and thresholds four at a time (the same addresses in every
-                  // lane), multiply and add as packed fp32 pairs - each half rounds as the scalar instruction does
-                  uint32_t word = 0;
-#pragma unroll
-                  for (int e = 0; e < 32; e += 4) {
-                    const float4 a = __ldg(reinterpret_cast<const float4*>(alpha + co0 + e));
-                    const float4 t = __ldg(reinterpret_cast<const float4*>(shift + co0 + e));
-                    unsigned long long x0, x1, m0, m1, t0, t1;
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(x0) : "r"(v[e]), "r"(v[e + 1]));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(x1) : "r"(v[e + 2]), "r"(v[e + 3]));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(m0) : "f"(a.x), "f"(a.y));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(m1) : "f"(a.z), "f"(a.w));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(t0) : "f"(t.x), "f"(t.y));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(t1) : "f"(t.z), "f"(t.w));
-                    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x0) : "l"(m0));
-                    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x1) : "l"(m1));
-                    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x0) : "l"(t0));
-                    asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x1) : "l"(t1));
-                    float y0, y1, y2, y3;
-                    asm("mov.b64 {%0, %1}, %2;" : "=f"(y0), "=f"(y1) : "l"(x0));
-                    asm("mov.b64 {%0, %1}, %2;" : "=f"(y2), "=f"(y3) : "l"(x1));
-                    word |= (y0 >= 0.f ? 1u : 0u) << e;
-                    word |= (y1 >= 0.f ? 1u : 0u) << (e + 1);
-                    word |= (y2 >= 0.f ? 1u : 0u) << (e + 2);
-                    word |= (y3 >= 0.f ? 1u : 0u) << (e + 3);
-                  }
-                  out32[wide_mul((uint32_t)pix, (uint32_t)Kw) + (uint32_t)(co0 >> 5)] = word;
-                } else if (pix >= 0 && co0 < K) {
-                  uint32_t word = 0;
-#pragma unroll
-                  for (int e = 0; e < 32; ++e) {
-                    const float a = co0 + e < K ? __ldg(alpha + co0 + e) : -1.f;  // a missing channel gives bit 0 ...
-                    const float s = co0 + e < K ? __uint_as_float(v[e]) : 1.f;     // ... through 1 * -1 + 0 < 0
-                    const float t = co0 + e < K ? __ldg(shift + co0 + e) : 0.f;
-                    word |= (__fadd_rn(__fmul_rn(s, a), t) >= 0.f ? 1u : 0u) << e;
-                  }
-                  out32[wide_mul((uint32_t)pix, (uint32_t)Kw) + (uint32_t)(co0 >> 5)] = word;
-                }
-              }
-            }
-          } else {
-            // one channel tile whose width is an odd multiple of 16: half-words; the slice that ends
-            // the tile also clears the half-word behind it, so that every word is written in full
-            uint16_t* out16 = reinterpret_cast<uint16_t*>(out32);
-#pragma unroll 1
-            for (int mt = 0; mt < MT; ++mt) {
-              const int pix = row_pixel(mt);
-              for (int c0 = G_EPI_SPLIT ? 0 : 16 * half; c0 < Nt; c0 += G_EPI_SPLIT ? 16 : 32) {
-                uint32_t v[16];
-                __syncwarp();
-                tmem_ld16(d0 + ((uint32_t)(rq * 32) << 16) + (uint32_t)(mt * Nt + c0), v);
-                tmem_ld_wait();
-                const int co0 = n0 + c0;
-                if (pix >= 0) {
-                  uint32_t hw = 0;
-#pragma unroll
-                  for (int e = 0; e < 16; ++e) {
-                    const float a = co0 + e < K ? __ldg(alpha + co0 + e) : -1.f;
-                    const float s = co0 + e < K ? __uint_as_float(v[e]) : 1.f;
-                    const float t = co0 + e < K ? __ldg(shift + co0 + e) : 0.f;
-                    hw |= (__fadd_rn(__fmul_rn(s, a), t) >= 0.f ? 1u : 0u) << e;
-                  }
-                  const size_t at = wide_mul((uint32_t)pix, (uint32_t)(2 * Kw)) + (uint32_t)(co0 >> 4);
-                  if ((co0 >> 4) < 2 * Kw) out16[at] = (uint16_t)hw;
-                  if (c0 + 16 >= Nt && (co0 >> 4) + 1 < 2 * Kw) out16[at + 1] = 0;
-                }
-              }
-            }
-          }
-        } else if (OUTK == OUT_SIGNS) {
-          // (packed signs only: nothing else is compiled into this variant)
-        } else if (fast) {
-          // The warp's slices (sub-tile mt, columns c0..c0+31) form one sequence; the TMEM load of slice s+1 is
-          // issued as soon as slice s sits in the staging tile.  The loop is written for few instructions (this
-          // role is bound by how many it issues): shared-memory addresses are fixed per lane, values travel as
-          // 64-bit pairs from the staging tile through the packed fp32 multiply to the 16-byte store, and a row's
-          // place in the output is one 32-bit element offset per sub-tile.
-          const int per_mt = (Nt - cfirst + cstep - 1) / cstep;
-          const int total_sl = MT * per_mt;
-          uint32_t v[32];
-          uint32_t roff[8];   // element offset of (row srow + 4i, this lane's four channels of a slice's first column), or none
-          if (total_sl > 0) tmem_ld32(d0 + ((uint32_t)(rq * 32) << 16) + (uint32_t)cfirst, v);
-          if (PIPED) {
-            // The tile's scales go to shared memory once: a global load issued between the slices' stores waits
-            // behind them in the load/store unit's queue, one per slice was a stall of hundreds of cycles each.
-            __syncwarp();   // the previous tile's last slice has read its scales
-            for (int c = lane * 4; c < Nt; c += 128) {
-              float4 al = make_float4(0.f, 0.f, 0.f, 0.f);
-              if (n0 + c < K) al = __ldg(reinterpret_cast<const float4*>(alpha + n0 + c));
-              asm volatile("st.shared.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(a_stage + (uint32_t)c * 4u), "f"(al.x), "f"(al.y),
-                           "f"(al.z), "f"(al.w)
-                           : "memory");
-            }
-            __syncwarp();
-          }
-          int mt = 0, ci = 0;
-#pragma unroll 1
-          for (int sl = 0; sl < total_sl; ++sl) {
-            const int c0 = cfirst + cstep * ci;
-            if (ci == 0) {
-              const int mine = row_pixel(mt);
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const int r = __shfl_sync(0xffffffffu, mine, srow + 4 * i);
-                roff[i] = r >= 0 ? (uint32_t)r * (uint32_t)K + (uint32_t)(n0 + scol * 4) : 0xffffffffu;
-              }
-            }
-            const int co = n0 + c0 + scol * 4;
-            unsigned long long alA = 0, alB = 0;   // (alpha[co], alpha[co+1]) and (alpha[co+2], alpha[co+3])
-            if (PIPED) {
-              asm volatile("ld.shared.v2.b64 {%0,%1}, [%2];" : "=l"(alA), "=l"(alB) : "r"(a_stage + (uint32_t)(c0 + scol * 4) * 4u) : "memory");
-            } else if (!out_i32 && co < K) {
-              const float4 al = __ldg(reinterpret_cast<const float4*>(alpha + co));
-              asm("mov.b64 %0, {%1, %2};" : "=l"(alA) : "f"(al.x), "f"(al.y));
-              asm("mov.b64 %0, {%1, %2};" : "=l"(alB) : "f"(al.z), "f"(al.w));
-            }
-            tmem_ld_wait();
-#pragma unroll
-            for (int e = 0; e < 8; ++e)
-              asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(st_lane ^ (uint32_t)(e << 4)), "r"(v[4 * e]),
-                           "r"(v[4 * e + 1]), "r"(v[4 * e + 2]), "r"(v[4 * e + 3])
-                           : "memory");
-            __syncwarp();
-            if (++ci == per_mt) { ci = 0; ++mt; }
-            if (sl + 1 < total_sl)
-              tmem_ld32(d0 + ((uint32_t)(rq * 32) << 16) + (uint32_t)(mt * Nt + cfirst + cstep * ci), v);
-            if (co < K) {  // K is a multiple of 4 here, so the four channels exist together
-              const uint32_t* obase = out32 + c0;
-#pragma unroll
-              for (int hh = 0; hh < 2; ++hh) {   // four rows at a time: 16 registers of values in flight
-                unsigned long long ua[4], ub[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {    // row srow + 4i, i = 4hh + j: even i from ld_even, odd i from ld_odd
-                  const int i = 4 * hh + j;
-                  asm volatile("ld.shared.v2.b64 {%0,%1}, [%2];"
-                               : "=l"(ua[j]), "=l"(ub[j])
-                               : "r"(((i & 1) ? ld_odd : ld_even) + (uint32_t)((i >> 1) * 1024))
-                               : "memory");
-                }
-                if (!out_i32) {
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(ua[j]) : "l"(alA));
-                    asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(ub[j]) : "l"(alB));
-                  }
-                } else {
-                  // int32 sums asked of fp32 accumulators: the sums are integers, the conversion is exact
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    uint32_t x, y, z, w;
-                    asm("mov.b64 {%0, %1}, %2;" : "=r"(x), "=r"(y) : "l"(ua[j]));
-                    asm("mov.b64 {%0, %1}, %2;" : "=r"(z), "=r"(w) : "l"(ub[j]));
-                    x = (uint32_t)__float2int_rn(__uint_as_float(x)); y = (uint32_t)__float2int_rn(__uint_as_float(y));
-                    z = (uint32_t)__float2int_rn(__uint_as_float(z)); w = (uint32_t)__float2int_rn(__uint_as_float(w));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(ua[j]) : "r"(x), "r"(y));
-                    asm("mov.b64 %0, {%1, %2};" : "=l"(ub[j]) : "r"(z), "r"(w));
-                  }
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  if (roff[4 * hh + j] != 0xffffffffu)
-                    asm volatile("st.global.v2.b64 [%0], {%1,%2};" ::"l"(obase + roff[4 * hh + j]), "l"(ua[j]), "l"(ub[j])
-                                 : "memory");
-              }
-            }
-            __syncwarp();
-          }
+        if (!active || half >= n_slices) {
+          release();
         } else {
-          // c_out not a multiple of 4 or a channel tile not a multiple of 32: 16-column slices
-          // straight from registers, element by element
+          uint32_t* const obase = out32 + (size_t)((uint32_t)(g_lane * K + co));
 #pragma unroll 1
-          for (int mt = 0; mt < MT; ++mt) {
-            const int pix = row_pixel(mt);
-            const uint32_t trow = d0 + ((uint32_t)(rq * 32) << 16) + (uint32_t)(mt * Nt);
-            for (int c0 = G_EPI_SPLIT ? 0 : 16 * half; c0 < Nt; c0 += G_EPI_SPLIT ? 16 : 32) {
-              uint32_t v[16];
-              tmem_ld16(trow + (uint32_t)c0, v);
+          for (int s = half; s < n_slices; s += 2) {   // the two warps of a lane quarter take the slices in turn
+            uint32_t v[32];
+            __syncwarp();
+            if (32 * s + 32 <= Np) {
+              tmem_ld32(d0 + (uint32_t)(32 * s), v);
               tmem_ld_wait();
-              const int co0 = n0 + c0;
-              if (pix < 0 || co0 >= K) continue;
-              uint32_t* o = out32 + wide_mul((uint32_t)pix, (uint32_t)K) + co0;
-              if ((K & 3) == 0 && co0 + 16 <= K) {
-                // all 16 channels exist and rows are 16-byte aligned: four channels per load, multiply and store
+            } else {   // the last 16 columns
+              uint32_t u[16];
+              tmem_ld16(d0 + (uint32_t)(32 * s), u);
+              tmem_ld_wait();
 #pragma unroll
-                for (int e = 0; e < 16; e += 4) {
-                  uint4 r;
-                  if (out_i32) {
-                    r.x = (uint32_t)__float2int_rn(__uint_as_float(v[e]));
-                    r.y = (uint32_t)__float2int_rn(__uint_as_float(v[e + 1]));
-                    r.z = (uint32_t)__float2int_rn(__uint_as_float(v[e + 2]));
-                    r.w = (uint32_t)__float2int_rn(__uint_as_float(v[e + 3]));
-                  } else {
-                    const float4 al = __ldg(reinterpret_cast<const float4*>(alpha + co0 + e));
-                    r.x = __float_as_uint(__fmul_rn(__uint_as_float(v[e]), al.x));
-                    r.y = __float_as_uint(__fmul_rn(__uint_as_float(v[e + 1]), al.y));
-                    r.z = __float_as_uint(__fmul_rn(__uint_as_float(v[e + 2]), al.z));
-                    r.w = __float_as_uint(__fmul_rn(__uint_as_float(v[e + 3]), al.w));
-                  }
-                  *reinterpret_cast<uint4*>(o + e) = r;
+              for (int e = 0; e < 16; ++e) { v[e] = u[e]; v[16 + e] = 0; }
+            }
+            if (s + 2 >= n_slices) release();
+            if (WORDS || out_kind != 2) {
+              const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
+              // One column = one pixel of 32 channels per step: a predicated store of a whole 128-byte line.
+              auto store = [&](auto value) {
+#pragma unroll
+                for (int e = 0; e < 32; e += 4) {
+                  const uint4 o4 = *reinterpret_cast<const uint4*>(&T->offset[32 * s + e]);
+                  const uint32_t o[4] = {o4.x, o4.y, o4.z, o4.w};
+#pragma unroll
+                  for (int j = 0; j < 4; ++j)
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(obase + o[j]),
+                                 "r"(value(v[e + j])), "r"(mask & (1u << (e + j)))
+                                 : "memory");
                 }
-                continue;
+              };
+              if (out_kind == 0) store([&](uint32_t x) { return __float_as_uint(__fmul_rn(__uint_as_float(x), al)); });
+              else store([&](uint32_t x) { return (uint32_t)__float2int_rn(__uint_as_float(x)); });   // integer sums: exact
+            } else {
+              // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): bit of a channel =
+              // fl(fl(alpha*S) + shift) >= 0 = sign bit clear (no sum is -0 or NaN: alpha and shift are finite and
+              // shift is not -0).  Multiply and add as packed fp32 pairs (each half rounds as the scalar instruction
+              // does), a lane gathers the bits of its channel over the 32 columns, and the transposition gives
+              // lane j the word of column j.
+              unsigned long long a2, t2;
+              asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(al));
+              asm("mov.b64 %0, {%1, %1};" : "=l"(t2) : "f"(sh));
+              uint32_t w = 0;
+#pragma unroll
+              for (int e = 30; e >= 0; e -= 2) {
+                unsigned long long x;
+                asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v[e]), "r"(v[e + 1]));
+                asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(a2));
+                asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(t2));
+                uint32_t y0, y1;
+                asm("mov.b64 {%0, %1}, %2;" : "=r"(y0), "=r"(y1) : "l"(x));
+                w = __funnelshift_l(y1, w, 1);
+                w = __funnelshift_l(y0, w, 1);
               }
-#pragma unroll
-              for (int e = 0; e < 16; ++e) {
-                if (co0 + e < K) {
-                  if (out_i32) o[e] = (uint32_t)__float2int_rn(__uint_as_float(v[e]));
-                  else o[e] = __float_as_uint(__fmul_rn(__uint_as_float(v[e]), __ldg(alpha + co0 + e)));
-                }
+              w = co < K ? ~w : 0u;   // bits of channels that do not exist are 0
+              w = g_transpose32(w, lane);
+              const uint32_t px = T->offset[32 * s + lane], here = 1u << lane;
+              const uint32_t Kw = (uint32_t)(K + 31) >> 5;
+              if (kp_log >= 5) {
+                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) out32[wide_mul(px + (uint32_t)g_warp, Kw) + (uint32_t)(co_warp >> 5)] = w;
+              } else {   // 16 rows per pixel: one word each for two pixels
+                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) out32[px + (uint32_t)g_warp] = w & 0xffffu;
+                if (T->mask[(g_warp + 1) * G_MAX_CHUNKS + s] & here) out32[px + (uint32_t)g_warp + 1] = w >> 16;
               }
             }
           }
         }
-        // this warp has read its part of the accumulator buffer: hand it back to the MMA issuer
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_accempty + 8 * acc_slot);
-        if (CHAIN && L.done) {
+        if (CHAIN) {
           // chain: this warp's part of the tile is written; the successor may read it
           __threadfence();
           __syncwarp();
-          if (lane == 0) atomicAdd(L.done + mg, 1u);
+          if (lane == 0) atomicAdd(lay[l].done + h0.y, 1u);
         }
       }
+      __syncwarp();   // the table has been read
+      if (lane == 0) mbar_arrive(bar_tabempty + 8u * (seq & 3u));
+      ++seq;
+      if (++acc_slot == n_acc) acc_slot = 0;
     }
-    if (warp == 2 && lane == 0) TR_REPORT(2, clock64() - tr_t0, tr_w0, tr_w1, tr_w2);
-  } else if (warp != 13 && warp != 17) {
+    if (warp == 2 && lane == 0) TR_REPORT(2, clock64() - tr_t0, tr_w0, 0, 0);
+  } else if (warp == 13) {
+    // ------------------------------------------------ table warp
+    // Writes down what the epilogue needs of every tile, up to four tiles ahead: where its columns' pixels go, which
+    // of them exist, the scales and thresholds.  Done by the epilogue warps themselves, each for itself, this took a
+    // fifth of their time (the geometry is a chain of divisions, and a global load behind a warp's own stores waits
+    // until those have drained).
+    bool ok = true;
+    uint32_t seq = 0;
+    auto take_slot = [&]() -> bool {
+      if (seq < G_TILES) return true;
+      int okw = 1;
+      if (lane == 0) okw = (!*abort_flag && mbar_wait_backoff(bar_tabempty + 8u * (seq & 3u), ((seq >> 2) & 1u) ^ 1u, 100)) ? 1 : 0;
+      okw = __shfl_sync(0xffffffffu, okw, 0);
+      if (!okw && lane == 0 && !*abort_flag) {
+        *abort_flag = 1;
+        raise_status(p.status, 7);
+      }
+      return okw != 0;
+    };
+    for (int l = 0; l < p.n_layers && ok; ++l) {
+      const GLayer& L = lay[l];
+      const FastDiv dWg = L.dWg, dHq = L.dHq, dCt = L.dCt;
+      const int Np = L.Np, K = L.K, Wg = L.Wg, Hq = L.Hq, Ho = L.Ho, Wo = L.Wo, lg = L.lg, n_ct = L.n_ct, total = L.total_tiles;
+      const uint32_t Qtot = L.Qtot;
+      const int n_slices = (Np + 31) >> 5;
+      const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
+      const uint32_t scale = out_kind == 2 ? 1u : (uint32_t)K;
+      for (int tile = L.first; tile < total; tile += G, ++seq) {
+        if (!take_slot()) { ok = false; break; }
+        GTile* const T = reinterpret_cast<GTile*>(epi_smem) + (seq & 3u);
+        const int mg = (int)fdiv((uint32_t)tile, dCt), co = (tile - mg * n_ct) * G_ROWS;
+        float al[4], sh[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int c = co + 32 * i + lane;
+          al[i] = c < K ? __ldg(L.alpha + c) : 0.f;
+          sh[i] = !WORDS && c < K ? __ldg(L.shift + c) : 0.f;
+        }
+        if (lane == 0) {
+          *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
+          *reinterpret_cast<int4*>(&T->K) = make_int4(K, 7 - lg, Np, out_kind);
+        }
+#pragma unroll 4
+        for (int s = 0; s < n_slices; ++s) {
+          const int c = 32 * s + lane;
+          const uint32_t q = (uint32_t)mg * (uint32_t)Np + (uint32_t)c;
+          const uint32_t rg = fdiv(q, dWg), n = fdiv(rg, dHq);
+          const int x = (int)(q - rg * (uint32_t)Wg) << lg, y = (int)(rg - n * (uint32_t)Hq);
+          T->offset[c] = ((n * (uint32_t)Ho + (uint32_t)y) * (uint32_t)Wo + (uint32_t)x) * scale;
+          const int rem = c < Np && q < Qtot && y < Ho ? Wo - x : 0;   // pixels from x to the end of the row
+          for (int g = 0; g < (1 << lg); ++g) {
+            const uint32_t m = __ballot_sync(0xffffffffu, g < rem);
+            if (lane == 0) T->mask[g * G_MAX_CHUNKS + s] = m;
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          T->alpha[32 * i + lane] = al[i];
+          if (!WORDS) T->shift[32 * i + lane] = __fadd_rn(sh[i], 0.f);   // -0 becomes +0: then no sum with it is -0
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_tabfull + 8u * (seq & 3u));
+      }
+    }
+    if (ok && take_slot()) {   // the end mark
+      if (lane == 0) {
+        (reinterpret_cast<GTile*>(epi_smem) + (seq & 3u))->l = -1;
+        mbar_arrive(bar_tabfull + 8u * (seq & 3u));
+      }
+      __syncwarp();
+    }
+  } else if (warp != 17) {
     // ------------------------------------------------ expanders (warps 10-12, 14-16, 18, 19)
     // Fill activation unit (problem, tile, channel block) of the ring: for every plane, row and
-    // 32-channel word, bits -> two 16-byte chunks of +1/-1 bytes (fp16: copy two 8-channel chunks).
+    // 32-channel word, bits -> one 16-byte chunk of nibbles (fp16: 8-channel chunks are copied).
     grid_dep_wait();  // the activations may come from the previous kernel in the stream
     const int et = (warp - 10 - (warp > 13) - (warp > 17)) * 32 + lane;  // rank among the expander threads
     int a_slot = 0;
     long long a_done = 0;
     uint32_t a_phase = 1;  // parity of the previous use of a slot (valid from the second lap)
-    volatile int* exp_flag = abort_flag + 1;
-    volatile int* dep_flag = abort_flag + 2;
     bool stop = false;
     long long tr_w0 = 0, tr_t0 = clock64();
-    (void)tr_w0; (void)tr_t0; (void)exp_flag; (void)dep_flag;
-    if (!CHAIN && FP4) {
+    (void)tr_w0; (void)tr_t0; (void)a_done;
+    // one lane per warp waits until the MMAs have read what slot a_slot held
+    auto wait_slot = [&]() -> bool {
+      int okf = 1;
+      if (lane == 0) okf = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_aempty + 8 * a_slot, a_phase, 64))) ? 1 : 0;
+      okf = __shfl_sync(0xffffffffu, okf, 0);
+      if (!okf && lane == 0 && !*abort_flag) {
+        *abort_flag = 1;
+        raise_status(p.status, 1);
+      }
+      return okf != 0;
+    };
+    // this warp's part of a unit is written: make it visible to the tensor core and say so
+    auto unit_done = [&](int slot) {
+      fence_proxy_async();  // generic-proxy writes -> visible to the tensor core's reads
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_afull + 8 * slot);
+    };
+    if (FP4 && !CHAIN) {
       // Independent problems: all inputs exist when the launch starts and are small beside the L2 (1/29 of the
-      // outputs; fp16 inputs are not: half of the outputs).  The CTAs pull them into L2 together, once, so that the staging loads below see L2 latency
-      // instead of DRAM latency: a unit is one round trip, and the round trip is what the expanders' rate is.
+      // outputs; fp16 inputs are not: half of the outputs).  The CTAs pull them into L2 together, once, so that the
+      // staging loads below see L2 latency instead of DRAM latency.
       for (int l = 0; l < p.n_layers; ++l) {
         const GLayer& L = lay[l];
-        const size_t bytes = (size_t)L.N * L.H * L.W * (F16 ? (size_t)L.C * 2 : (size_t)L.Cw * 4);
+        const size_t bytes = (size_t)L.N * L.H * L.W * ((size_t)L.Cw * 4);
         const char* base = reinterpret_cast<const char*>(p.act[l]);
         for (size_t off = ((size_t)blockIdx.x * G_EXP_THREADS + et) * 128; off < bytes; off += (size_t)G * G_EXP_THREADS * 128)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
       }
     }
-    // Independent problems on 4-bit operands whose rows can be read two words at a time run a two-stage software
-    // pipeline per thread: a "group" is up to three rows of one unit with one vector load each; the loads of
-    // group g + 1 are issued (into registers) before group g is expanded into shared memory, so that a unit no
-    // longer costs a full round trip to memory - with few words per row the round trip is nearly all of it.
-    constexpr bool piped = PIPED;   // (the host has checked the alignment of all inputs)
-    if constexpr (PIPED) {
+    if constexpr (FP4) {
+      // A two-stage software pipeline per thread: a "group" is up to four items of one unit - an item is the words of
+      // one position in one plane that one load brings - and the loads of group g + 1 are issued (into registers)
+      // before group g is expanded into shared memory, so that a unit does not cost a full round trip to memory.
+      // A thread keeps the geometry of its position while it walks through the planes and words: these eight warps
+      // are bound by how many instructions a unit takes one warp, not by the issue slots of the SM.
+      constexpr int XI = G_EXP_ITEMS;
       struct XGroup {
-        uint4 t[G_EXP_ROWS];        // the rows' words (two or four of them)
-        uint32_t da[G_EXP_ROWS];    // where a row's first chunk goes
-        uint32_t cstride;           // bytes from one chunk of a plane to the next
-        uint32_t flags;             // bit j: row j exists; bit 4 + j: its pixel is inside the image; 8: four words per
-                                    // row; 9: first group of its unit; 10: last group of its unit
+        uint4 t[XI];       // the items' words (one, two or four of them)
+        uint32_t da[XI];   // where an item's first chunk goes
+        uint32_t cstride;  // bytes from one chunk to the next
+        uint32_t flags;    // bit j: item j exists; bit 4 + j: its words exist (the pixel is inside the image); bits
+                           // 12..14: words per item; 9: first group of its unit; 10: last group of its unit
       };
       // The expander warps form XG teams that take the units in turn (the ring has a multiple of XG slots, so a
       // slot always belongs to the same team): with few rows per unit a unit is a chain of latencies, and two
       // chains in flight are what doubles the rate.
       constexpr int XG = G_XTEAMS, XT = G_EXP_THREADS / XG;
       const int gx = et / XT, etg = et % XT;
-      int* const pix = pix_tab + gx * (int)p.pix_words;
-      // issue side: the unit (il, itile, icb) with sequence number iu, and the next group to load in it
-      int il = 0, itile = 0, itotal = 0, icb = 0, irb = 0, ik0 = 0, i_slot = 0, iu = 0;
-      int Rr = 0, n_planes = 0, n_cb = 0, cbc = 0, Cw = 0, all_rows = 0, kstep = 2;
-      int pix_l = -1, pix_t = -1;   // the tile the pixel table holds
+      // issue side: the unit (il, itile, icb) with sequence number iu, and the next item to load in it
+      int il = 0, itile = 0, itotal = 0, icb = 0, i_slot = 0, iu = 0;
+      int pos0 = 0, ipl = 0, ik0 = 0;                 // first position of the thread's row of positions, plane, word
+      int Rr = 0, n_cb = 0, cbc = 0, Cw = 0, planes = 1, kstep = 2, cpl = 0, H = 0, W = 0, cs = 0;
+      uint32_t Q0 = 0;
+      int row = 0, col = 0, img_row = 0;              // of this thread's position: input row and column in plane 0, n*H
+      bool inside = false;                            // it lies in the batch
       const uint32_t* act = nullptr;
-      bool ivalid = false;
+      bool ivalid = false, ready = false;             // is there a unit; may its input be read (chain)
+      uint32_t dep_at = 1, dep_end = 0;               // chain: predecessor tiles still to be waited for
+      auto enter_tile = [&]() {
+        const GLayer& L = lay[il];
+        const uint32_t mg = fdiv((uint32_t)itile, L.dCt);
+        Q0 = mg * (uint32_t)L.Np;
+        ready = true;
+        if (CHAIN && L.deps) {
+          const uint2 d = __ldg(L.deps + mg);
+          dep_at = d.x;
+          dep_end = d.y;
+          ready = false;
+        }
+      };
       auto enter_layer = [&]() {   // first layer from il on in which this CTA has a tile
         for (; il < p.n_layers; ++il) {
           const GLayer& L = lay[il];
-          itile = g_first_tile(L);
+          itile = L.first;
           itotal = L.total_tiles;
           if (itile >= itotal) continue;
-          Rr = L.Rr; n_planes = L.n_planes; n_cb = L.n_cb; cbc = L.cb_chunks; Cw = L.Cw;
-          all_rows = n_planes * Rr;
+          Rr = L.Rr; n_cb = L.n_cb; cbc = L.cb_chunks; Cw = L.Cw; planes = L.n_planes; cpl = L.cpl; H = L.H; W = L.W; cs = L.cs;
           act = reinterpret_cast<const uint32_t*>(p.act[il]);
-          kstep = ((reinterpret_cast<uintptr_t>(act) & 15) == 0 && (Cw & 3) == 0 && (cbc & 3) == 0) ? 4 : 2;
+          kstep = g_word_step(Cw, cbc);
           icb = 0;
           ivalid = true;
+          enter_tile();
           return;
         }
         ivalid = false;
@@ -823,59 +777,82 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
           if (itile >= itotal) {
             ++il;
             enter_layer();
+          } else {
+            enter_tile();
           }
         }
       };
-      auto seek_own = [&]() {      // on to this team's next unit; input pixel of each of this thread's rows of its tile
+      auto seek_own = [&]() {      // on to this team's next unit
         while (ivalid && (iu % XG) != gx) next_unit();
-        if (ivalid && (pix_l != il || pix_t != itile)) {
-          const GLayer& L = lay[il];
-          const int mg = (int)fdiv((uint32_t)itile, L.dNt);
-          const uint32_t Q0 = (uint32_t)mg * (uint32_t)(128 * L.MT);
-          for (int f = etg; f < all_rows; f += XT) {
-            const int pl = (f >= Rr) + (f >= 2 * Rr) + (f >= 3 * Rr);
-            pix[f] = g_position_to_pixel(L, Q0 + (uint32_t)(f - pl * Rr), pl >> 1, pl & 1);
-          }
-          pix_l = il;
-          pix_t = itile;
+      };
+      // chain: has the predecessor written every input pixel of the tile?  One lane per warp looks (blocking: waits,
+      // bounded); no barrier among the warps, so that one that gives up leaves none of the others waiting.
+      auto check_ready = [&](bool blocking) -> bool {
+        if (!CHAIN || ready) return true;
+        const GLayer& L = lay[il];
+        int okd = 1;
+        if (lane == 0) {
+          for (; dep_at <= dep_end; ++dep_at)
+            if (!g_wait_counter(L.prev_done + dep_at, L.prev_target, abort_flag, blocking ? 1u << 21 : 1u)) { okd = 0; break; }
         }
+        ready = __shfl_sync(0xffffffffu, okd, 0) != 0;
+        __syncwarp();   // what lane 0 acquired is visible to the whole warp
+        return ready;
       };
       auto issue = [&](XGroup& g) {   // loads of the group at the issue position; moves the position on
-        const uint32_t cs = (uint32_t)Rr * 16u;
-        uint32_t flags = (kstep == 4 ? 0x100u : 0u) | ((irb == 0 && ik0 == 0) ? 0x200u : 0u);
+        const GLayer& L = lay[il];
+        const bool fresh = CHAIN && L.deps != nullptr;   // written by other CTAs of this launch: read from L2
+        const uint32_t cstride = (uint32_t)(planes * Rr) * 16u;
+        uint32_t flags = ((uint32_t)kstep << 12) | ((pos0 | ipl | ik0) == 0 ? 0x200u : 0u);
         const uint32_t unit = smem_u32(a_smem) + (uint32_t)i_slot * p.a_slot_bytes;
+        bool ended = false;
 #pragma unroll
-        for (int j = 0; j < G_EXP_ROWS; ++j) {
-          const int f = irb + etg + j * XT;
-          const int px = f < all_rows ? pix[f] : -2;
-          const int pl = (f >= Rr) + (f >= 2 * Rr) + (f >= 3 * Rr);
-          g.da[j] = unit + (uint32_t)(pl * cbc * Rr + (f - pl * Rr)) * 16u + (uint32_t)ik0 * cs;
-          if (px != -2) flags |= 1u << j;
+        for (int j = 0; j < XI; ++j) {
+          if (ended) break;
+          const int pos = pos0 + etg;
+          if ((ipl | ik0) == 0) {
+            const uint32_t q = Q0 + (uint32_t)pos;
+            const uint32_t rg = fdiv(q, L.dWg), n = fdiv(rg, L.dHq);
+            row = L.rs * (int)(rg - n * (uint32_t)L.Hq) - L.pad;
+            col = L.cm * (int)(q - rg * (uint32_t)L.Wg) - L.pad;
+            img_row = (int)n * H;
+            inside = q < L.Qtot;
+          }
+          const int r = row + (ipl >> cpl), c = col + cs * (ipl & ((1 << cpl) - 1)), word = icb * cbc + ik0;
+          const bool on = inside && pos < Rr && (uint32_t)r < (uint32_t)H && (uint32_t)c < (uint32_t)W && word < Cw;
+          g.da[j] = unit + (uint32_t)ik0 * cstride + (uint32_t)(ipl * Rr + pos) * 16u;
           g.t[j] = make_uint4(0, 0, 0, 0);
-          if (px >= 0) {
+          if (pos < Rr) flags |= 1u << j;
+          if (on) {
             flags |= 0x10u << j;
-            const uint32_t* src = act + wide_mul((uint32_t)px, (uint32_t)Cw) + icb * cbc + ik0;
+            const uint32_t* src = act + wide_mul((uint32_t)((img_row + r) * W + c), (uint32_t)Cw) + word;
             if (kstep == 4) {
-              g.t[j] = __ldg(reinterpret_cast<const uint4*>(src));
-            } else {
-              const uint2 v = __ldg(reinterpret_cast<const uint2*>(src));
+              g.t[j] = g_ld4(src, fresh);
+            } else if (kstep == 2) {
+              const uint2 v = g_ld2(src, fresh);
               g.t[j].x = v.x;
               g.t[j].y = v.y;
+            } else {
+              g.t[j].x = g_ld1(src, fresh);
+            }
+          }
+          ik0 += kstep;
+          if (ik0 >= cbc) {
+            ik0 = 0;
+            if (++ipl == planes) {
+              ipl = 0;
+              pos0 += XT;
+              ended = pos0 >= Rr;
             }
           }
         }
-        g.cstride = cs;
-        ik0 += kstep;
-        if (ik0 >= cbc) {
-          ik0 = 0;
-          irb += G_EXP_ROWS * XT;
-          if (irb >= all_rows) {   // the unit ends with this group
-            irb = 0;
-            flags |= 0x400u;
-            next_unit();
-            seek_own();
-          }
+        if (ended) {   // the unit ends with this group
+          pos0 = 0;
+          flags |= 0x400u;
+          next_unit();
+          seek_own();
         }
+        g.cstride = cstride;
         g.flags = flags;
       };
       enter_layer();
@@ -883,249 +860,174 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
       // completion side: this team's slots gx, gx + XG, ... of the ring
       a_slot = gx;
       XGroup cur, nxt;
-      bool nvalid = ivalid;
-      if (nvalid) issue(nxt);
-      while (nvalid && !stop) {
-        cur = nxt;
-        nvalid = ivalid;
-        if (nvalid) issue(nxt);
-        if ((cur.flags & 0x200u) && a_done >= NA / XG) {
-          int okf = 1;
-          if (lane == 0) okf = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_aempty + 8 * a_slot, a_phase, 64))) ? 1 : 0;
-          okf = __shfl_sync(0xffffffffu, okf, 0);
-          if (!okf) {
+      bool nvalid = false;
+      while (ivalid || nvalid) {
+        if (!nvalid) {
+          if (!check_ready(true)) {
             if (lane == 0 && !*abort_flag) {
-              *abort_flag = 1;
-              raise_status(p.status, 1);
-            }
-            stop = true;
-            break;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < G_EXP_ROWS; ++j) {
-          if (cur.flags & (1u << j)) {
-            const bool on = (cur.flags & (0x10u << j)) != 0;
-            const uint32_t d = cur.da[j], cs = cur.cstride;
-            sts16(d, expand_word_fp4(cur.t[j].x, on));
-            sts16(d + cs, expand_word_fp4(cur.t[j].y, on));
-            if (cur.flags & 0x100u) {
-              sts16(d + 2 * cs, expand_word_fp4(cur.t[j].z, on));
-              sts16(d + 3 * cs, expand_word_fp4(cur.t[j].w, on));
-            }
-          }
-        }
-        if (cur.flags & 0x400u) {
-          fence_proxy_async();  // generic-proxy writes -> visible to the tensor core's reads
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_afull + 8 * a_slot);
-          ++a_done;
-          a_slot += XG;
-          if (a_slot >= NA) { a_slot -= NA; a_phase ^= 1u; }
-        }
-      }
-    }
-    for (int l = 0; l < (piped ? 0 : p.n_layers) && !stop; ++l) {
-      const GLayer& L = lay[l];
-      const int Rr = L.Rr, n_planes = L.n_planes, n_cb = L.n_cb, cb_chunks = L.cb_chunks, MT = L.MT;
-      const int C = L.C, Cw = L.Cw, total = L.total_tiles;
-      const FastDiv dNt = L.dNt;
-      const void* act = p.act[l];
-      const bool fresh = CHAIN && L.deps != nullptr;   // written by other CTAs of this launch: read from L2
-      // vector loads of a row's words need the base pointer and the row pitch aligned to the load
-      bool vec;
-      {
-        const uintptr_t addr = (uintptr_t)act;
-        if (F16) vec = (addr & 15) == 0 && (C & 7) == 0;
-        else if (FP4) vec = (addr & 7) == 0 && (Cw & 1) == 0;  // pairs of words (a block's first word is even)
-        else vec = false;
-      }
-      const bool vec4 = FP4 && vec && ((uintptr_t)act & 15) == 0 && (Cw & 3) == 0 && (cb_chunks & 3) == 0;
-      for (int tile = g_first_tile(L); tile < total && !stop; tile += G) {
-        const int mg = (int)fdiv((uint32_t)tile, dNt);
-        const uint32_t Q0 = (uint32_t)mg * (uint32_t)(128 * MT);
-        if (CHAIN && L.deps) {
-          // chain: wait until the predecessor has written every input pixel of this tile (one thread polls)
-          if (et == 0) {
-            const uint2 d = __ldg(L.deps + mg);
-            int okd = 1;
-            for (uint32_t m = d.x; m <= d.y && okd; ++m) okd = g_wait_counter(L.prev_done + m, L.prev_target, abort_flag) ? 1 : 0;
-            *dep_flag = okd;
-          }
-          asm volatile("bar.sync 3, %0;" ::"n"(G_EXP_THREADS) : "memory");
-          const int okd = *dep_flag;
-          if (!okd) {
-            if (et == 0 && !*abort_flag) {
               *abort_flag = 1;
               raise_status(p.status, 5);
             }
             stop = true;
             break;
           }
+          issue(nxt);
         }
-        // Input pixel of every staged row, once per tile.  The table is private to the expanders:
-        // the barrier keeps a fast thread from overwriting entries another still reads (and, in a chain,
-        // the polling thread from setting the next tile's flag before everyone has read this one).
-        asm volatile("bar.sync 3, %0;" ::"n"(G_EXP_THREADS) : "memory");
-        // (plane, row) pairs form one index space f = plane*Rr + row, dealt to the threads at a stride of
-        // the expander count, here and below: a thread reads back only entries it wrote itself
-        const int all_rows = n_planes * Rr;
-        for (int f = et; f < all_rows; f += G_EXP_THREADS) {
-          const int pl = (f >= Rr) + (f >= 2 * Rr) + (f >= 3 * Rr);
-          pix_tab[f] = g_position_to_pixel(L, Q0 + (uint32_t)(f - pl * Rr), pl >> 1, pl & 1);
+        cur = nxt;
+        // (a chain's next input may depend on the unit in hand: it is only looked at, never waited for, here)
+        nvalid = ivalid && check_ready(false);
+        if (nvalid) issue(nxt);
+        if ((cur.flags & 0x200u) && a_done >= NA / XG && !wait_slot()) {
+          stop = true;
+          break;
         }
-        for (int cb = 0; cb < n_cb; ++cb) {
-          if (a_done >= NA) {
-            // one elected thread polls; the rest wait on a hardware barrier instead of spinning
-            if (et == 0) *exp_flag = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_aempty + 8 * a_slot, a_phase, 64))) ? 1 : 0;
-            asm volatile("bar.sync 3, %0;" ::"n"(G_EXP_THREADS) : "memory");
-            const int okf = *exp_flag;
-            asm volatile("bar.sync 3, %0;" ::"n"(G_EXP_THREADS) : "memory");
-            if (!okf) {
-              if (et == 0 && !*abort_flag) {
-                *abort_flag = 1;
-                raise_status(p.status, 1);
+#pragma unroll
+        for (int j = 0; j < XI; ++j) {
+          if (cur.flags & (1u << j)) {
+            const bool on = (cur.flags & (0x10u << j)) != 0;
+            const uint32_t sign = on ? 0x88888888u : 0u, one = on ? 0x22222222u : 0u;
+            const uint32_t d = cur.da[j], cst = cur.cstride;
+            sts16(d, expand_word_fp4(cur.t[j].x, sign, one));
+            if (cur.flags & 0x6000u) {
+              sts16(d + cst, expand_word_fp4(cur.t[j].y, sign, one));
+              if (cur.flags & 0x4000u) {
+                sts16(d + 2 * cst, expand_word_fp4(cur.t[j].z, sign, one));
+                sts16(d + 3 * cst, expand_word_fp4(cur.t[j].w, sign, one));
               }
+            }
+          }
+        }
+        if (cur.flags & 0x400u) {
+          unit_done(a_slot);
+          ++a_done;
+          a_slot += XG;
+          if (a_slot >= NA) { a_slot -= NA; a_phase ^= 1u; }
+        }
+      }
+    } else {
+      int pending = 0, oldest = 0;   // units whose copies are still in flight, the slot of the oldest
+      auto complete = [&](int left) {   // say that all of them but the `left` newest are written
+        while (pending > left) {
+          if (pending == 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
+          else if (pending == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+          else asm volatile("cp.async.wait_group 0;" ::: "memory");
+          unit_done(oldest);
+          oldest = oldest + 1 == NA ? 0 : oldest + 1;
+          --pending;
+        }
+      };
+      for (int l = 0; l < p.n_layers && !stop; ++l) {
+        const GLayer& L = lay[l];
+        const int Rr = L.Rr, n_cb = L.n_cb, cb_chunks = L.cb_chunks, all_rows = L.n_planes * Rr;
+        const int C = L.C, total = L.total_tiles;
+        const FastDiv dCt = L.dCt, dRr = L.dRr;
+        const void* act = p.act[l];
+        const bool vec = (C & 7) == 0;                   // rows start at multiples of 16 bytes
+        if (L.tma) {
+          // The rows of positions a tile touches are fetched with one copy of 64 channels per row and plane, dealt to the
+          // warps (issuing them all from one thread took longer than the MMAs of a small map): padding columns, rows
+          // above and below the image and channels past the last are out of the tensor's bounds and read as zeros.
+          const uint32_t row_bytes = (uint32_t)L.Wg * 128u, ew = (uint32_t)(et >> 5), Hq = (uint32_t)L.Hq;
+          const FastDiv dHq = L.dHq, dWg = L.dWg;
+          const int n_pu = L.n_pu, rs = L.rs, pad = L.pad, cpl = L.cpl, Np = L.Np;
+          for (int tile = L.first; tile < total && !stop; tile += G) {
+            const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)Np;
+            const uint32_t r_first = fdiv(Q0, dWg), r_last = fdiv(Q0 + (uint32_t)Rr - 1u, dWg);
+            for (int u = 0; u < n_cb * n_pu; ++u) {
+              if (pending) complete(0);
+              if (a_done >= NA && !wait_slot()) {
+                stop = true;
+                break;
+              }
+              if (lane == 0) {
+                const uint32_t bar = bar_afull + 8u * (uint32_t)a_slot, unit = smem_u32(a_smem) + (uint32_t)a_slot * p.a_slot_bytes;
+                const int pl = u & (n_pu - 1), cb = n_pu == 1 ? u : u >> 2;
+                const int x = (pl & (rs - 1)) - pad, y0 = (pl >> cpl) - pad;
+                const uint32_t mine = r_last >= r_first + ew ? ((r_last - r_first - ew) >> 3) + 1u : 0u;   // this warp's rows
+                if (mine) mbar_expect_tx(bar, mine * row_bytes);
+                else mbar_arrive(bar);
+                for (uint32_t r = r_first + ew; r <= r_last; r += G_EW) {
+                  const uint32_t n = fdiv(r, dHq);
+                  tma_load_4d(unit + (r - r_first) * row_bytes, &maps.m[l], cb * 64, x, rs * (int)(r - n * Hq) + y0, (int)n, bar);
+                }
+              }
+              __syncwarp();
+              ++a_done;
+              if (++a_slot == NA) { a_slot = 0; a_phase ^= 1u; }
+            }
+          }
+          continue;
+        }
+        oldest = pending ? oldest : a_slot;
+        for (int tile = L.first; tile < total && !stop; tile += G) {
+          const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)L.Np;
+          // Input pixel of every staged row, once per tile; a thread reads back only entries it wrote itself.
+          // (plane, row) pairs form one index space f = plane*Rr + row, dealt to the threads at a stride of
+          // the expander count.
+          for (int f = et; f < all_rows; f += G_EXP_THREADS) {
+            const int pl = (int)fdiv((uint32_t)f, dRr);
+            pix_tab[f] = g_position_to_pixel(L, Q0 + (uint32_t)(f - pl * Rr), pl);
+          }
+          for (int cb = 0; cb < n_cb; ++cb) {
+            // the next slot is not free yet: finish the units in flight first, the MMAs may be waiting for them
+            if (pending && a_done >= NA &&
+                !__shfl_sync(0xffffffffu, lane == 0 ? (int)mbar_test(bar_aempty + 8 * a_slot, a_phase) : 0, 0))
+              complete(0);
+            if (a_done >= NA && !wait_slot()) {
               stop = true;
               break;
             }
-          }
-          uint8_t* unit = a_smem + (size_t)a_slot * p.a_slot_bytes;
-          // A thread has rows of several planes in flight together: a stride-2 unit (four short
-          // planes) costs one round trip to memory instead of four.
-          {
-            for (int rb = 0; rb < all_rows; rb += G_EXP_ROWS * G_EXP_THREADS) {
-              int pix[G_EXP_ROWS];  // input pixel of each of this thread's rows; -1 padding, -2 past the unit
-              uint8_t* dst[G_EXP_ROWS];  // where the row starts in its plane (chunk 0)
-#pragma unroll
-              for (int j = 0; j < G_EXP_ROWS; ++j) {
-                const int f = rb + et + j * G_EXP_THREADS;
-                pix[j] = f < all_rows ? pix_tab[f] : -2;
-                const int pl = (f >= Rr) + (f >= 2 * Rr) + (f >= 3 * Rr);
-                dst[j] = unit + ((size_t)pl * cb_chunks * Rr + (size_t)(f - pl * Rr)) * 16;
+            const uint32_t unit = smem_u32(a_smem) + (uint32_t)a_slot * p.a_slot_bytes;
+            const uint32_t cstride = (uint32_t)all_rows * 16u;   // bytes from one chunk to the next
+            if (vec) {
+              // Asynchronous 16-byte copies straight into the unit (zero-filled where the row is padding or the channels
+              // end), all in flight together.  A warp takes 32 rows at a time, its lanes run along a row's chunks
+              // first: an instruction reads whole lines.
+              const int per = 32 / cb_chunks, sub = lane / cb_chunks, chunk = lane - sub * cb_chunks;
+              const int ch = (cb * cb_chunks + chunk) * 8;  // first channel of this lane's chunk
+              for (int rb = et; rb - lane < all_rows; rb += G_EXP_THREADS) {
+                const int mine = rb < all_rows ? pix_tab[rb] : -2;
+                const uint32_t dst = unit + (uint32_t)(rb - lane) * 16u + (uint32_t)chunk * cstride;
+                for (int r0 = 0; r0 < 32; r0 += per) {
+                  const int px = __shfl_sync(0xffffffffu, mine, r0 + sub);
+                  if (sub >= per || r0 + sub >= 32 || px == -2) continue;
+                  const bool on = px >= 0 && ch < C;
+                  const __half* src = (const __half*)act + (on ? wide_mul((uint32_t)px, (uint32_t)C) + ch : 0);
+                  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + (uint32_t)(r0 + sub) * 16u), "l"(src),
+                               "r"(on ? 16 : 0)
+                               : "memory");
+                }
               }
-              if (F16 && vec) {
-                // fp16 activations are copied: asynchronous 16-byte copies straight into the unit (zero-filled where
-                // the row is padding or the channels end), all of a thread's chunks in flight together; the thread
-                // waits for its own copies before it makes them visible to the tensor core and arrives.
+            } else {
+              for (int f = et; f < all_rows; f += G_EXP_THREADS) {
+                const int px = pix_tab[f];
+                for (int c0 = 0; c0 < cb_chunks; ++c0) {
+                  const int ch = (cb * cb_chunks + c0) * 8;
+                  uint32_t w[4] = {0, 0, 0, 0};
+                  if (px >= 0) {
+                    const __half* src = (const __half*)act + wide_mul((uint32_t)px, (uint32_t)C) + ch;
 #pragma unroll
-                for (int j = 0; j < G_EXP_ROWS; ++j) {
-                  if (pix[j] == -2) continue;
-                  const __half* row = (const __half*)act + wide_mul((uint32_t)(pix[j] < 0 ? 0 : pix[j]), (uint32_t)C);
-                  const uint32_t d = smem_u32(dst[j]);
-                  for (int c0 = 0; c0 < cb_chunks; ++c0) {
-                    const int ch = (cb * cb_chunks + c0) * 8;  // first channel of the chunk
-                    const bool on = pix[j] >= 0 && ch < C;
-                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + (uint32_t)c0 * (uint32_t)Rr * 16u),
-                                 "l"(on ? (const void*)(row + ch) : act), "r"(on ? 16 : 0)
-                                 : "memory");
+                    for (int e = 0; e < 8; ++e)
+                      if (ch + e < C) w[e >> 1] |= (uint32_t)__half_as_ushort(src[e]) << (16 * (e & 1));
                   }
-                }
-              } else if (F16) {
-                for (int c0 = 0; c0 < cb_chunks; c0 += 2) {
-                  uint4 v[G_EXP_ROWS][2];
-#pragma unroll
-                  for (int j = 0; j < G_EXP_ROWS; ++j) {
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                      v[j][k] = make_uint4(0, 0, 0, 0);
-                      const int ch = (cb * cb_chunks + c0 + k) * 8;  // first channel of the chunk
-                      if (pix[j] >= 0 && ch < C) {
-                        const __half* src = (const __half*)act + wide_mul((uint32_t)pix[j], (uint32_t)C) + ch;
-                        if (vec) {
-                          v[j][k] = __ldg(reinterpret_cast<const uint4*>(src));
-                        } else {
-                          uint32_t w[4] = {0, 0, 0, 0};
-#pragma unroll
-                          for (int e = 0; e < 8; ++e)
-                            if (ch + e < C) w[e >> 1] |= (uint32_t)__half_as_ushort(src[e]) << (16 * (e & 1));
-                          v[j][k] = make_uint4(w[0], w[1], w[2], w[3]);
-                        }
-                      }
-                    }
-                  }
-#pragma unroll
-                  for (int j = 0; j < G_EXP_ROWS; ++j) {
-                    if (pix[j] != -2) {
-                      *reinterpret_cast<uint4*>(dst[j] + (size_t)c0 * Rr * 16) = v[j][0];
-                      *reinterpret_cast<uint4*>(dst[j] + (size_t)(c0 + 1) * Rr * 16) = v[j][1];
-                    }
-                  }
-                }
-              } else if (FP4) {
-                // A 32-channel word becomes one 16-byte chunk of nibbles.  The common case (an even number of
-                // words per pixel, so that a block's words are read two or four at a time) is kept free of
-                // per-word conditions: this role, too, is bound by the instructions it issues.
-                const int wb = cb * cb_chunks;
-                const uint32_t cstride = (uint32_t)Rr * 16u;   // bytes from one chunk of a plane to the next
-                uint32_t da[G_EXP_ROWS];
-#pragma unroll
-                for (int j = 0; j < G_EXP_ROWS; ++j) da[j] = smem_u32(dst[j]);
-                if (vec) {
-                  const uint32_t* src[G_EXP_ROWS];
-#pragma unroll
-                  for (int j = 0; j < G_EXP_ROWS; ++j)
-                    src[j] = (const uint32_t*)act + wide_mul((uint32_t)(pix[j] < 0 ? 0 : pix[j]), (uint32_t)Cw) + wb;
-                  if (vec4) {
-                    for (int k0 = 0; k0 < cb_chunks; k0 += 4) {
-                      uint4 t[G_EXP_ROWS];
-#pragma unroll
-                      for (int j = 0; j < G_EXP_ROWS; ++j) {
-                        t[j] = make_uint4(0, 0, 0, 0);
-                        if (pix[j] >= 0) t[j] = g_ld4(src[j] + k0, fresh);
-                      }
-#pragma unroll
-                      for (int j = 0; j < G_EXP_ROWS; ++j) {
-                        if (pix[j] != -2) {
-                          const bool on = pix[j] >= 0;
-                          const uint32_t d = da[j] + (uint32_t)k0 * cstride;
-                          sts16(d, expand_word_fp4(t[j].x, on));
-                          sts16(d + cstride, expand_word_fp4(t[j].y, on));
-                          sts16(d + 2 * cstride, expand_word_fp4(t[j].z, on));
-                          sts16(d + 3 * cstride, expand_word_fp4(t[j].w, on));
-                        }
-                      }
-                    }
-                  } else {
-                    for (int k0 = 0; k0 < cb_chunks; k0 += 2) {
-                      uint2 t[G_EXP_ROWS];
-#pragma unroll
-                      for (int j = 0; j < G_EXP_ROWS; ++j) {
-                        t[j] = make_uint2(0, 0);
-                        if (pix[j] >= 0) t[j] = g_ld2(src[j] + k0, fresh);
-                      }
-#pragma unroll
-                      for (int j = 0; j < G_EXP_ROWS; ++j) {
-                        if (pix[j] != -2) {
-                          const bool on = pix[j] >= 0;
-                          const uint32_t d = da[j] + (uint32_t)k0 * cstride;
-                          sts16(d, expand_word_fp4(t[j].x, on));
-                          sts16(d + cstride, expand_word_fp4(t[j].y, on));
-                        }
-                      }
-                    }
-                  }
-                } else {
-                  // an odd number of words per pixel, or a pointer that is not 8-byte aligned: word by word
-                  for (int k = 0; k < cb_chunks; ++k) {
-#pragma unroll
-                    for (int j = 0; j < G_EXP_ROWS; ++j) {
-                      if (pix[j] == -2) continue;
-                      const bool on = pix[j] >= 0 && wb + k < Cw;
-                      uint32_t w = 0;
-                      if (on) w = g_ld1((const uint32_t*)act + wide_mul((uint32_t)pix[j], (uint32_t)Cw) + wb + k, fresh);
-                      sts16(da[j] + (uint32_t)k * cstride, expand_word_fp4(w, on));
-                    }
-                  }
+                  sts16(unit + (uint32_t)f * 16u + (uint32_t)c0 * cstride, make_uint4(w[0], w[1], w[2], w[3]));
                 }
               }
             }
+            // the unit's copies stay in flight while the next two units' are issued
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            if (++pending == 3) complete(2);
+            ++a_done;
+            if (++a_slot == NA) { a_slot = 0; a_phase ^= 1u; }
           }
-          if (F16) asm volatile("cp.async.wait_all;" ::: "memory");
-          fence_proxy_async();  // generic-proxy writes -> visible to the tensor core's reads
-          mbar_arrive(bar_afull + 8 * a_slot);
-          ++a_done;
-          if (++a_slot == NA) { a_slot = 0; a_phase ^= 1u; }
+        }
+      }
+      if (!stop) complete(0);
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      if (stop && et == 0) {   // giving up: never leave with copies in flight (bounded)
+        for (int i = 0; i < NA && i < a_done; ++i) {
+          const long long last = a_done - 1 - i;
+          mbar_wait_backoff(bar_afull + 8u * (uint32_t)(last % NA), (uint32_t)((last / NA) & 1), 64);
         }
       }
     }
@@ -1144,46 +1046,73 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p)
 struct GroupDev {
   int count = 0, act_type = 0, mode = M_FP4;
   int kind = TCG_WORDS;           // what the tiles were planned for (word outputs, packed signs, chain)
-  bool hot = false;               // planned for the hot variant of the word-output kernel (see tcg_create)
   int chain = 0;                  // 1: member i + 1 reads the packed signs member i writes (one launch, dependency counters)
+  uint8_t* mem = nullptr;         // all device memory of the group; the pointers below lie in it
   uint8_t* chain_buf = nullptr;   // the packed signs between the members, one buffer per boundary
   size_t chain_off[SNN_GROUP_MAX] = {};
-  uint32_t* done = nullptr;       // completion counters of all members' M groups
+  uint32_t* done = nullptr;       // completion counters of all members' position tiles
   size_t done_words = 0;
-  uint2* deps = nullptr;
   GLayer* layers_dev = nullptr;   // [count]
-  uint8_t* weights = nullptr;     // the group's own weight operands, one after the other
   uint16_t* ranks = nullptr;      // [count][grid] tile assignment, see tcg_create
   GParams p{};                    // everything but the per-call pointers
   size_t smem = 0;
   int grid = 0;
+  struct Map { bool tma; int C, W, H, N, stride, box; } map[SNN_GROUP_MAX] = {};   // fp16 activations fetched by TMA
 };
 
 namespace {
 
-// Tile shape, channel blocks and weight stages of one problem under the group's fixed slot sizes.
-// Operand of the weights: wt[layout tile][channel block][tap][chunk][NtL][16 B]; a chunk is 16 bytes along the
-// input channels (16 int8, 8 fp16 or 32 e2m1 values), cb_chunks chunks per block, NtL output channels per
-// layout tile.  Channels that do not exist are zeros, so whatever the activation operand holds there adds 0.
+// The driver's tensor-map encoder, looked up once (the library does not link the driver).
+using MapEncoder = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                                const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+MapEncoder g_map_encoder() {
+  static const MapEncoder f = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    return reinterpret_cast<MapEncoder>(p);
+  }();
+  return f;
+}
+
+// Which tap each step of a layer applies, for the weight operand: per chunk of a step the kernel row and the column
+// s of the group's window (kernel column s - stride*g for pixel g), 255: none.  Steps of single taps name one tap twice.
+struct GTaps {
+  uint8_t row[kGTapsMax][2], col[kGTapsMax][2];
+};
+
+// Operand of the weights: wt[channel tile][channel block][step][chunk][128][16 B]; a chunk is 16 bytes along the
+// input channels (8 fp16 or 32 e2m1 values), cb_chunks chunks per block.  Row r of a tile is channel r % (128/G) of
+// pixel r / (128/G).  Channels that do not exist, and columns outside a pixel's window, are zeros, so whatever the
+// activation operand holds there adds 0.
 template <int MODE>
 __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, uint8_t* __restrict__ wt, int C, int K,
-                                        int Cw, long long total, int cb_chunks, int n_cb, int NtL, int taps) {
+                                        int Cw, long long total, int cb_chunks, int n_cb, int steps, int paired, int lg,
+                                        int win_step, int ksize, const GTaps taps) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= total) return;
-  int row = (int)(i % NtL);
-  long long r = i / NtL;
-  int c = (int)(r % cb_chunks);
-  r /= cb_chunks;
-  int t = (int)(r % taps);
-  r /= taps;
-  int cb = (int)(r % n_cb), tile = (int)(r / n_cb);
-  int co = tile * NtL + row;
+  const int row = (int)(i & (G_ROWS - 1));
+  long long r = i / G_ROWS;
+  const int chunks = paired ? 2 : cb_chunks;
+  const int c = (int)(r % chunks);
+  r /= chunks;
+  const int t = (int)(r % steps);
+  r /= steps;
+  const int cb = (int)(r % n_cb), tile = (int)(r / n_cb);
+  const int kp_log = 7 - lg;
+  const int g = row >> kp_log, co = tile * G_ROWS + (row & ((1 << kp_log) - 1));
+  const int which = paired ? c : 0;
+  const int ky = taps.row[t][which], kx = (int)taps.col[t][which] - win_step * g;
   constexpr int cpc = MODE == M_F16 ? 8 : 32;
   uint4 v = make_uint4(0, 0, 0, 0);
-  if (co < K) {
-    int ch0 = (cb * cb_chunks + c) * cpc;
-    int wd = ch0 >> 5, sh = ch0 & 31;
-    uint32_t bits = wd < Cw ? wplanes[((size_t)t * Cw + wd) * K + co] >> sh : 0u;
+  if (co < K && ky < ksize && kx >= 0 && kx < ksize) {
+    const int ch0 = paired ? 0 : (cb * cb_chunks + c) * cpc;
+    const int wd = ch0 >> 5, sh = ch0 & 31;
+    const uint32_t bits = wd < Cw ? wplanes[((size_t)(ky * ksize + kx) * Cw + wd) * K + co] >> sh : 0u;
     uint32_t w[4] = {0, 0, 0, 0};
     if (MODE == M_F16) {
 #pragma unroll
@@ -1192,114 +1121,242 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
     } else {
 #pragma unroll
       for (int e = 0; e < 32; ++e)
-        if (ch0 + e < C) w[e >> 3] |= (((bits >> e) & 1u) ? 0x2u : 0xau) << (4 * (e & 7));         // e2m1 +1.0 / -1.0
+        if (ch0 + e < C) w[e & 3] |= (((bits >> e) & 1u) ? 0x2u : 0xau) << (4 * (e >> 2));         // e2m1 +1.0 / -1.0
     }
     v = make_uint4(w[0], w[1], w[2], w[3]);
   }
   reinterpret_cast<uint4*>(wt)[i] = v;
 }
 
-cudaError_t g_expand_weights(int mode, const uint32_t* wplanes, void* dst, int C, int K, int Cw, int Kpad, int n_chunks,
-                             int cb_chunks, int NtL, int taps, cudaStream_t s) {
-  const long long total = (long long)taps * n_chunks * Kpad;
-  const unsigned blocks = (unsigned)((total + 255) / 256);
-  const int n_cb = n_chunks / cb_chunks;
-  if (mode == M_F16)
-    g_expand_weights_kernel<M_F16><<<blocks, 256, 0, s>>>(wplanes, (uint8_t*)dst, C, K, Cw, total, cb_chunks, n_cb, NtL, taps);
-  else
-    g_expand_weights_kernel<M_FP4><<<blocks, 256, 0, s>>>(wplanes, (uint8_t*)dst, C, K, Cw, total, cb_chunks, n_cb, NtL, taps);
-  return cudaGetLastError();
-}
-
 inline int g_mode_for(int act_type) { return act_type == SNN_ACT_F16 ? M_F16 : M_FP4; }
 
-// Cycles of one MMA of 128 positions x nt channels as measured on B200 (any operand type): half a cycle per
-// channel plus a constant that does not overlap the previous MMA.
-inline double g_mma_cycles(int nt) { return 0.5 * nt + 33.0; }
+// A planned layer and the planner's estimate of one tile, in SM cycles.
+struct GPlan {
+  GLayer L;
+  GTaps taps;
+  int paired = 0;
+  size_t w_bytes = 0, unit_bytes = 0;
+  double mma = 0, weights = 0, expand = 0, drain = 0;
+  double through() const {   // a tile among others: the slowest role
+    double t = mma;
+    if (weights > t) t = weights;
+    if (expand > t) t = expand;
+    if (drain > t) t = drain;
+    return t + 300.0;
+  }
+  double alone() const { return expand + (mma > weights ? mma : weights) + drain + 1500.0; }   // a tile by itself
+};
 
-// tensor-memory columns of one accumulator buffer when there are n_acc of them
-inline int g_acc_cols(int mode, int n_acc) {
-  return mode != M_FP4 ? (int)G_ACC_COLS : n_acc == G_NACC_WORDS ? (int)G_ACC_COLS_FP4_3 : (int)G_ACC_COLS_FP4;
-}
-
-bool g_plan_layer(const Geom& g, int mode, int n_acc, GLayer* L, int* n_chunks_out, int* Kpad_out) {
+// The plan of one layer with tiles of Np positions of 2^lg pixels; false where that does not fit.
+bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, GPlan* P) {
+  GLayer& o = P->L;
+  o = GLayer{};
   const int cpc = mode == M_F16 ? 8 : 32;
-  const int acc_cols = g_acc_cols(mode, n_acc);
-  const int raw = round_up(g.C, 2 * cpc) / cpc;  // 16-byte chunks along the channels, even
-  GLayer& o = *L;
+  const int S = g.stride, G = 1 << lg;
+  const bool one = g.ksize == 1;
   o.N = g.N; o.H = g.H; o.W = g.W; o.C = g.C; o.K = g.K; o.Cw = g.Cw;
-  o.stride = g.stride; o.pad = g.pad; o.Ho = g.Ho; o.Wo = g.Wo;
-  o.taps = g.ksize == 1 ? 1 : 9;
-  if (g.ksize == 1) {
-    // 1x1 layer: the positions are the output pixels themselves (input pixel = stride * output pixel), no halo
-    o.Hq = g.Ho; o.Wq = g.Wo; o.n_planes = 1; o.halo = 0;
-  } else if (g.stride == 1) {
-    o.Hq = g.H + g.pad; o.Wq = g.W + g.pad; o.n_planes = 1; o.halo = 2 * o.Wq + 2;
+  o.pad = g.pad; o.Ho = g.Ho; o.Wo = g.Wo; o.G = G; o.lg = lg; o.Np = Np;
+  if (lg && (mode != M_FP4 || g.K > G_ROWS >> lg)) return false;
+  o.rs = S;
+  o.cs = one ? S : 1;
+  o.cm = S * G;
+  int row_planes = 1, col_planes = G;
+  if (one) {
+    // 1x1 layer: the positions are (groups of) the output pixels themselves, no halo
+    o.Hq = g.Ho;
+    o.Wg = (g.Wo + G - 1) / G;
   } else {
-    o.Hq = g.Ho + 1; o.Wq = g.Wo + 1; o.n_planes = 4; o.halo = o.Wq + 1;
+    // one zero column per image row and one zero row per image are shared by neighbours; stride 2 splits the input
+    // into its row and column parity planes, in each of which the taps are plain shifts
+    row_planes = S;
+    col_planes = S * G;
+    o.Hq = S == 1 ? g.H + g.pad : g.Ho + 1;
+    o.Wg = ((S == 1 ? g.W + g.pad : g.Wo + 1) + G - 1) / G;
   }
-  o.dWq = make_fastdiv((uint32_t)o.Wq);
-  o.dHq = make_fastdiv((uint32_t)o.Hq);
-  o.Qtot = (long long)g.N * o.Hq * o.Wq;
-  if (g.N < 1) return false;
-  if (o.Qtot + 1024 + o.halo >= (1ll << 31)) return false;  // positions are 32-bit in the kernel
-  if (g.C > (1 << 20)) return false;                        // 9 * c_in stays far below 2^24: exact fp32 sums
-  if ((long long)g.N * g.H * g.W >= (1ll << 31) || (long long)g.N * g.Ho * g.Wo >= (1ll << 31)) return false;
-  if ((long long)g.N * g.Ho * g.Wo * g.K >= 0xffffffffLL) return false;   // output element offsets are 32-bit
-  // layout tile of the weight operand = channels per tile: all of them up to 256; beyond that 256
-  // when that pads little (fewer channel tiles re-expand the same activations), else 128
-  if (mode == M_FP4) o.NtL = g.K <= acc_cols ? round_up(g.K, 16) : 128;   // (columns 480..511 hold the scales)
-  else o.NtL = g.K <= 256 ? round_up(g.K, 16) : (round_up(g.K, 256) - g.K < 64 ? 256 : 128);
-  o.Nt = o.NtL;
-  const int Kpad = round_up(g.K, o.NtL);
-  o.n_ntiles = Kpad / o.Nt;
-  o.dNt = make_fastdiv((uint32_t)o.n_ntiles);
-  // channel block: the largest of 8/6/4/2 chunks that divides the channels and whose unit fits a slot
+  o.n_planes = row_planes * col_planes;
+  o.cpl = 0;
+  while ((1 << o.cpl) < col_planes) ++o.cpl;
+  const long long Q = (long long)g.N * o.Hq * o.Wg;
+  const int span = one ? S * (G - 1) + 1 : S * (G - 1) + 3;   // columns of a group's window, in input pixels
+  const int halo = one ? 0 : (2 / S) * o.Wg + (span - 1) / col_planes;
+  if (Q + 1024 + halo >= (1ll << 31)) return false;
+  o.Qtot = (uint32_t)Q;
+  o.Rr = Np + halo;
+  // fp16 units are fetched by TMA where the rows of the tensor are multiples of 16 bytes and a row of positions fits a box
+  o.tma = tma && mode == M_F16 && (g.C & 7) == 0 && o.Wg * S <= 256;
+  const int tma_rows = (2 * o.Wg + o.Rr - 2) / o.Wg;   // rows of positions a tile can touch
+  if (mode == M_F16 && !o.tma) o.Rr |= 1;   // odd: the chunks of a row are copied together, into different banks
+  if (!o.tma && (long long)o.n_planes * o.Rr > kGRowsMax) return false;
+  P->paired = mode == M_FP4 && g.Cw == 1;
   int d = 0;
-  for (int c = 8; c >= 2; c -= 2) {
-    if (raw % c) continue;
-    if ((size_t)o.n_planes * c * (128 + o.halo) * 16 <= kGASlotMax) { d = c; break; }
+  if (o.tma) {
+    // 64 channels (fewer where there are no more); every plane is a unit of its own
+    P->unit_bytes = (size_t)tma_rows * o.Wg * 128;
+    if (P->unit_bytes > kGASlotMaxTma) return false;
+    o.n_cb = (g.C + 63) / 64;
+    d = o.n_cb > 1 ? 8 : round_up(g.C, 16) / 8;
+    o.cb_chunks = d;
+    o.kpt = d / 2;
+    o.n_pu = o.n_planes;
+  } else {
+    // channel block: the largest of 8/6/4/2 chunks that divides the channels and whose unit fits a slot; one chunk where
+    // there is one activation word per pixel: a K = 64 step then covers two taps, one per chunk
+    const int raw = P->paired ? 1 : round_up(g.C, 2 * cpc) / cpc;  // 16-byte chunks along the channels, even
+    for (int c = P->paired ? 1 : 8; c >= 1; c -= 2) {
+      if (raw % c) continue;
+      if ((size_t)o.n_planes * c * o.Rr * 16 <= kGASlotMax) { d = c; break; }
+    }
+    if (!d) return false;
+    o.cb_chunks = d;
+    o.n_cb = raw / d;
+    o.kpt = P->paired ? 1 : d / 2;
+    o.n_pu = 1;
+    P->unit_bytes = (size_t)o.n_planes * d * o.Rr * 16;
   }
-  if (!d) return false;
-  o.cb_chunks = d;
-  o.n_cb = raw / d;
-  o.kpt = d / 2;
-  int MT = 1;
-  for (int m = 4; m >= 2; --m)
-    if ((size_t)o.n_planes * d * (128 * m + o.halo) * 16 <= kGASlotMax && m * o.Nt <= acc_cols) { MT = m; break; }
-  const long long mtiles = (o.Qtot + 127) / 128;
-  while (MT > 1 && mtiles < MT) --MT;  // a tiny problem does not need the larger tile
-  o.MT = MT;
-  o.Rr = 128 * MT + o.halo;
-  if ((uint32_t)o.Rr * 16 >= (1u << 18)) return false;  // leading-offset field of the descriptor
-  const long long mgroups = (mtiles + MT - 1) / MT;
-  if (mgroups * o.n_ntiles > 0x7fffffffLL || mgroups * o.Rr >= (1ll << 31)) return false;
-  o.total_tiles = (int)(mgroups * o.n_ntiles);
-  // weight stage: as many whole taps of a channel block as fit a slot
-  o.tap_bytes = (uint32_t)(o.kpt * 2 * o.Nt * 16);
-  int st = (int)(kGBSlot / o.tap_bytes);
-  if (st < 1) return false;
-  o.st_taps = st > o.taps ? o.taps : st;
-  *n_chunks_out = raw;
-  *Kpad_out = Kpad;
+  const int taps = one ? G : 3 * span;
+  o.steps = P->paired ? (taps + 1) / 2 : taps;
+  if (o.steps >= kGTapsMax) return false;
+  const uint32_t reach = o.tma ? 8u * (uint32_t)halo : (uint32_t)(o.n_planes * o.Rr);   // largest start of a tap, and chunk distance
+  if (reach > 0xffffu || (!o.tma && reach >= (1u << 14))) return false;                 // (the leading-offset field has 14 bits)
+  o.n_ct = lg ? 1 : (g.K + G_ROWS - 1) / G_ROWS;
+  const long long tiles = (Q + Np - 1) / Np * o.n_ct;
+  if (tiles > 0x7fffffffLL || (Q + Np - 1) / Np * o.Rr >= (1ll << 31)) return false;
+  o.total_tiles = (int)tiles;
+  // weight stage: as many whole steps of a channel block as fit a slot
+  o.step_bytes = (uint32_t)(o.kpt * 2 * G_ROWS * 16);
+  o.st_steps = (int)((mode == M_F16 ? kGBSlotF16 : kGBSlot) / o.step_bytes);
+  if (o.st_steps > o.steps) o.st_steps = o.steps;
+  P->w_bytes = (size_t)o.n_ct * o.n_cb * o.steps * o.step_bytes;
+  // One MMA reads 32 + Np/4 shared-memory lines and takes at least Np/2 cycles (measured).  The other figures are the
+  // rates the roles reach in the traces: bulk copies of weights 64 bytes per cycle, a 16-byte chunk of activations
+  // in 0.6 cycles (0.4 copied) plus the latency of the loads, stores 16 bytes per cycle.
+  const double mmas = (double)o.n_cb * o.steps * o.kpt;
+  const double lines = mmas * (32 + Np / 4) + (double)o.n_cb * (o.steps * o.step_bytes + (double)o.n_pu * P->unit_bytes) / 128.0;
+  P->mma = std::max(mmas * (Np / 2), 1.1 * lines);
+  P->weights = (double)o.n_cb * o.steps * o.step_bytes / 64.0;
+  P->expand = o.tma ? o.n_cb * o.n_pu * (P->unit_bytes / 40.0) + 1000.0 : o.n_cb * ((double)o.n_planes * o.Rr * d * (mode == M_F16 ? 3.0 : 0.6) + 500.0);
+  const int k_tile = g.K < G_ROWS ? g.K : G_ROWS;
+  P->drain = kind == TCG_WORDS ? (double)Np * G * k_tile * 4 / 16.0 : Np * 5.0;
   return true;
 }
 
-}  // namespace
-
-namespace {
-// host copy of the kernel's position -> input pixel map
-int h_position_to_pixel(const GLayer& L, long long q, int pa, int pb) {
-  if (q >= L.Qtot) return -1;
-  const long long rg = q / L.Wq;
-  const int j = (int)(q - rg * L.Wq);
-  const long long n = rg / L.Hq;
-  const int i = (int)(rg - n * L.Hq);
-  if (n >= L.N) return -1;
-  const int r = L.stride * i + pa - L.pad, c = L.stride * j + pb - L.pad;
-  if (r < 0 || r >= L.H || c < 0 || c >= L.W) return -1;
-  return (int)((n * L.H + r) * L.W + c);
+// The rest of a chosen plan: division constants, and where each step's rows start in the unit.
+void g_finish_plan(const Geom& g, GPlan* P) {
+  GLayer& o = P->L;
+  o.dWg = make_fastdiv((uint32_t)o.Wg);
+  o.dHq = make_fastdiv((uint32_t)o.Hq);
+  o.dCt = make_fastdiv((uint32_t)o.n_ct);
+  o.dRr = make_fastdiv((uint32_t)o.Rr);
+  const int S = g.stride, col_planes = 1 << o.cpl, span = S * (o.G - 1) + 3;
+  // taps in ascending order of where their rows start in the unit
+  struct Tap { int plane; uint32_t at; uint8_t row, col; } taps[64];
+  int n = 0;
+  if (g.ksize == 1) {
+    for (int q = 0; q < o.G; ++q) taps[n++] = {q, 0, 0, (uint8_t)(S * q)};
+  } else {
+    for (int ky = 0; ky < 3; ++ky)
+      for (int s = 0; s < span; ++s)
+        taps[n++] = {(ky % S) * col_planes + s % col_planes, (uint32_t)((ky / S) * o.Wg + s / col_planes), (uint8_t)ky, (uint8_t)s};
+  }
+  for (int t = 0; t < n; ++t) taps[t].at = o.tma ? taps[t].at * 8 : taps[t].at + (uint32_t)(taps[t].plane * o.Rr);
+  std::sort(taps, taps + n, [](const Tap& a, const Tap& b) { return a.plane != b.plane ? a.plane < b.plane : a.at < b.at; });
+  for (int t = 0; t < o.steps; ++t) {
+    const Tap& a = taps[P->paired ? 2 * t : t];
+    const bool second = P->paired && 2 * t + 1 < n;
+    const Tap& b = second ? taps[2 * t + 1] : a;
+    const uint32_t dist = P->paired ? b.at - a.at : o.tma ? 1u : (uint32_t)(o.n_planes * o.Rr);
+    o.tap[t] = a.at | (dist << 16);
+    P->taps.row[t][0] = a.row; P->taps.col[t][0] = a.col;
+    P->taps.row[t][1] = P->paired && !second ? 255 : b.row;
+    P->taps.col[t][1] = b.col;
+  }
+  for (int u = 0; u < 4; ++u) o.pu_end[u] = o.steps;
+  if (o.n_pu > 1)
+    for (int u = 0, t = 0; u < o.n_pu; ++u) {
+      while (t < n && taps[t].plane == u) ++t;
+      o.pu_end[u] = t;
+    }
 }
+
+// Does the tensor-core path take this layer?  The bound is that of a unit of 128 positions with its halo (row pitch of
+// the padded map) in a 40.5 KB slot, two of which fit beside the weight ring; shapes beyond it go to the other paths.
+// The tiles themselves are planned by g_plan_layer, which needs less.
+bool g_path_takes(const Geom& g, int mode) {
+  constexpr size_t slot_max = 40 * 1024 + 512, b_slot = 32 * 1024, epi = 40 * 1024, budget = 226 * 1024;
+  if (g.N < 1 || g.C > (1 << 20)) return false;            // 9 * c_in stays far below 2^24: exact fp32 sums
+  if ((long long)g.N * g.H * g.W >= (1ll << 31) || (long long)g.N * g.Ho * g.Wo >= (1ll << 31)) return false;
+  if ((long long)g.N * g.Ho * g.Wo * g.K >= 0xffffffffLL) return false;   // output element offsets are 32-bit
+  const int cpc = mode == M_F16 ? 8 : 32, raw = round_up(g.C, 2 * cpc) / cpc;
+  const bool one = g.ksize == 1;
+  const int Hq = one ? g.Ho : g.stride == 1 ? g.H + g.pad : g.Ho + 1;
+  const int Wq = one ? g.Wo : g.stride == 1 ? g.W + g.pad : g.Wo + 1;
+  const int planes = one || g.stride == 1 ? 1 : 4;
+  const int halo = one ? 0 : g.stride == 1 ? 2 * Wq + 2 : Wq + 1;
+  const long long Q = (long long)g.N * Hq * Wq;
+  if (Q + 1024 + halo >= (1ll << 31)) return false;
+  int d = 0;
+  for (int c = 8; c >= 2 && !d; c -= 2)
+    if (raw % c == 0 && (size_t)planes * c * (128 + halo) * 16 <= slot_max) d = c;
+  if (!d) return false;
+  for (int n_acc = 2; n_acc <= (mode == M_FP4 ? 3 : 2); ++n_acc) {
+    const int cols = mode == M_F16 ? 256 : n_acc == 3 ? 160 : 240;
+    const int nt = mode == M_FP4 ? (g.K <= cols ? round_up(g.K, 16) : 128)
+                                 : (g.K <= 256 ? round_up(g.K, 16) : (round_up(g.K, 256) - g.K < 64 ? 256 : 128));
+    const long long mtiles = (Q + 127) / 128;
+    int mt = 1;
+    for (int m = 4; m >= 2 && mt == 1; --m)
+      if ((size_t)planes * d * (128 * m + halo) * 16 <= slot_max && m * nt <= cols) mt = m;
+    while (mt > 1 && mtiles < mt) --mt;
+    const int rows = 128 * mt + halo;
+    const long long groups = (mtiles + mt - 1) / mt;
+    if ((uint32_t)rows * 16 >= (1u << 18)) return false;
+    if (groups * ((g.K + nt - 1) / nt) > 0x7fffffffLL || groups * rows >= (1ll << 31)) return false;
+    const size_t unit = (((size_t)planes * d * rows * 16) + 127) & ~(size_t)127;
+    const size_t pix = (((size_t)planes * rows * 4) + 127) & ~(size_t)127;
+    if (2 * unit + epi + 2 * pix + 256 + kGTail + 3 * b_slot > budget) return false;
+  }
+  return true;
+}
+
+// Tile sizes the planner chooses from (positions; multiples of 16).
+constexpr int kNpTable[] = {256, 240, 208, 192, 160, 144, 128, 112, 96, 80, 64, 48, 32, 16};
+
+// Best plan of one layer for tiles of at most `cap` positions: the group size 2^lg with the least time over all its tiles.
+bool g_best_group(const Geom& g, int mode, int kind, int cap, bool tma, GPlan* out) {
+  bool found = false;
+  double best = 0;
+  for (int lg = 0; lg <= 3; ++lg) {
+    for (int Np : kNpTable) {
+      if (Np > cap) continue;
+      GPlan P;
+      if (!g_plan_layer(g, mode, kind, lg, Np, tma, &P) && !g_plan_layer(g, mode, kind, lg, Np, false, &P)) continue;
+      const double t = P.L.total_tiles * P.through();
+      if (!found || t < best) { best = t; *out = P; found = true; }
+      break;   // the largest that fits
+    }
+  }
+  return found;
+}
+
+// Which CTAs take a problem's odd tiles.  Every CTA gets floor(tiles / grid) tiles of a problem
+// and the first (tiles % grid) CTAs in the problem's rank order get one more; the rank order is
+// by the time the CTAs have been given so far, least first, so that the CTAs end close
+// together although a tile of one problem may take six times as long as a tile of another.
+void g_assign(const std::vector<GPlan>& P, int grid, std::vector<uint16_t>* ranks) {
+  std::vector<double> busy(grid, 0.0);
+  std::vector<int> order(grid);
+  for (size_t i = 0; i < P.size(); ++i) {
+    const double cost = P[i].through();
+    for (int b = 0; b < grid; ++b) order[b] = b;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return busy[a] < busy[b]; });
+    const int base = P[i].L.total_tiles / grid, rem = P[i].L.total_tiles % grid;
+    for (int r = 0; r < grid; ++r) {
+      (*ranks)[i * grid + order[r]] = (uint16_t)r;
+      busy[order[r]] += cost * (base + (r < rem ? 1 : 0));
+    }
+  }
+}
+
 }  // namespace
 
 cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int act_type, int kind, cudaStream_t s,
@@ -1309,54 +1366,90 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   if (kind != TCG_WORDS && act_type != SNN_ACT_BIN) return cudaErrorInvalidConfiguration;
   const int chain = kind == TCG_CHAIN;
   const int mode = g_mode_for(act_type);
-  GLayer host[SNN_GROUP_MAX];
-  int n_chunks[SNN_GROUP_MAX], Kpad[SNN_GROUP_MAX];
-  size_t w_off[SNN_GROUP_MAX], w_total = 0;
-  size_t a_slot = 0, pix_bytes = 0;
-  long long tiles = 0;
-  // Word outputs on 4-bit operands get three accumulator buffers where the launch can run its hot variant (every
-  // member: c_out a multiple of 4, channel tile a multiple of 32, an even number of activation words per pixel);
-  // with the plain expanders two larger buffers measure faster, so everything else is planned with two.
-  int n_acc = (mode == M_FP4 && kind == TCG_WORDS) ? G_NACC_WORDS : G_NACC;
-  bool hot = n_acc == G_NACC_WORDS;
-  if (hot) {
-    for (int i = 0; i < count && hot; ++i) {
-      if (!g_plan_layer(gs[i], mode, n_acc, &host[i], &n_chunks[i], &Kpad[i])) return cudaErrorInvalidConfiguration;
-      if ((gs[i].Cw & 1) || (gs[i].K & 3) || (host[i].Nt & 31)) hot = false;
+  for (int i = 0; i < count; ++i)
+    if (!g_path_takes(gs[i], mode)) return cudaErrorInvalidConfiguration;
+  const int sms = sm_count();
+  const uint32_t tmem = mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16;
+  int cap_max = (int)tmem / 2;
+  const bool tma = mode == M_F16 && g_map_encoder() != nullptr;
+  // Tile sizes.  A chain's members run one after the other as far as their inputs go, so each takes the size that makes
+  // its own tiles end first; the members of a group share the machine, and one size limit for all of them is chosen by
+  // the time of the busiest CTA.
+  std::vector<GPlan> plan(count), trial(count);
+  double best = -1;
+  if (chain) {
+    for (int i = 0; i < count; ++i) {
+      best = -1;
+      for (int cap : kNpTable) {
+        if (cap > cap_max) continue;
+        for (int lg = 0; lg <= 3; ++lg) {
+          GPlan P;
+          if (!g_plan_layer(gs[i], mode, kind, lg, cap, false, &P)) continue;
+          const int waves = (P.L.total_tiles + sms - 1) / sms;
+          const double t = P.alone() + (waves - 1) * P.through();
+          if (best < 0 || t < best) { best = t; plan[i] = P; }
+        }
+      }
+      if (best < 0) return cudaErrorInvalidConfiguration;
     }
-    if (!hot) n_acc = G_NACC;
+  } else {
+    for (int cap : kNpTable) {
+      if (cap > cap_max) continue;
+      bool ok = true;
+      for (int i = 0; i < count && ok; ++i) ok = g_best_group(gs[i], mode, kind, cap, tma, &trial[i]);
+      if (!ok) continue;
+      // the machine's share of all tiles (whole tiles where there is one problem), and the last tile's way through the roles
+      double sum = 0, last = 0, slowest = 0;
+      for (const GPlan& P : trial) {
+        sum += count == 1 ? (double)((P.L.total_tiles + sms - 1) / sms) * sms * P.through() : P.L.total_tiles * P.through();
+        last = std::max(last, P.alone() - P.through());
+        slowest = std::max(slowest, P.through());
+      }
+      const double t = std::max(sum / sms, slowest) + last + (count > 1 ? slowest / 2 : 0);
+      if (best < 0 || t < best) { best = t; plan = trial; }
+    }
+    if (best < 0) return cudaErrorInvalidConfiguration;
   }
+  for (int i = 0; i < count; ++i) g_finish_plan(gs[i], &plan[i]);
+  size_t w_off[SNN_GROUP_MAX], w_total = 0, a_slot = 0, pix_bytes = 0;
+  long long tiles = 0, most = 0;
+  int widest = 16;
   for (int i = 0; i < count; ++i) {
-    if (!g_plan_layer(gs[i], mode, n_acc, &host[i], &n_chunks[i], &Kpad[i])) return cudaErrorInvalidConfiguration;
-    const size_t unit = (size_t)host[i].n_planes * host[i].cb_chunks * host[i].Rr * 16;
-    if (unit > a_slot) a_slot = unit;
-    const size_t pb = (size_t)host[i].n_planes * host[i].Rr * 4;
-    if (pb > pix_bytes) pix_bytes = pb;
+    const GLayer& o = plan[i].L;
+    a_slot = std::max(a_slot, plan[i].unit_bytes);
+    if (mode == M_F16 && !o.tma) pix_bytes = std::max(pix_bytes, (size_t)o.n_planes * o.Rr * 4);
+    widest = std::max(widest, o.Np);
     w_off[i] = w_total;
-    w_total += ((size_t)host[i].taps * n_chunks[i] * Kpad[i] * 16 + 255) & ~(size_t)255;
-    tiles += host[i].total_tiles;
+    w_total += (plan[i].w_bytes + 255) & ~(size_t)255;
+    tiles += o.total_tiles;
+    most = std::max(most, (long long)o.total_tiles);
   }
-  a_slot = (a_slot + 127) & ~(size_t)127;
+  // accumulator buffers: as many as fit, up to four
+  int n_acc = (int)tmem / widest;
+  if (n_acc > 4) n_acc = 4;
+  const uint32_t acc_cols = (tmem / (uint32_t)n_acc) & ~15u;
+  a_slot = (a_slot + 1023) & ~(size_t)1023;   // (the swizzle of the TMA units repeats every 1024 bytes)
+  const uint32_t b_slot = mode == M_F16 ? kGBSlotF16 : kGBSlot;
   pix_bytes = (pix_bytes + 127) & ~(size_t)127;
-  const size_t pix_one = pix_bytes;
-  if (hot) pix_bytes *= G_XTEAMS;   // one table per expander team
   const size_t lay_bytes = ((size_t)count * sizeof(GLayer) + 127) & ~(size_t)127;
   const size_t fixed = (size_t)G_EPI_BYTES + pix_bytes + lay_bytes + kGTail;
-  // ring depth: three slots if they fit, else two; the plan for word outputs on 4-bit operands takes two, a
-  // multiple of the number of expander teams (four slots never fit beside three weight slots of these sizes)
-  int na = hot ? 2 : 3, ns = 0;
-  static_assert(G_XTEAMS == 1 || G_XTEAMS == 2, "the ring depth below is a multiple of the team count");
+  // Ring depths: four activation slots if they fit beside four weight slots, else two (with the pipelined expanders a
+  // multiple of the number of teams) or three; the weights take what is left.
+  static_assert(G_XTEAMS == 1 || G_XTEAMS == 2, "the ring depths below are multiples of the team count");
+  int na = 4, ns = 0;
   for (; na >= 2; --na) {
-    if ((size_t)na * a_slot + fixed + 3 * (size_t)kGBSlot > kGSmemBudget) continue;
-    ns = (int)((kGSmemBudget - fixed - (size_t)na * a_slot) / kGBSlot);
+    if (mode == M_FP4 && na % G_XTEAMS) continue;
+    const int ns_min = mode == M_F16 ? 4 : na > 2 ? 4 : 3;
+    if ((size_t)na * a_slot + fixed + ns_min * (size_t)b_slot > kGSmemBudget) continue;
+    ns = (int)((kGSmemBudget - fixed - (size_t)na * a_slot) / b_slot);
     break;
   }
   if (na < 2 || ns < 3) return cudaErrorInvalidConfiguration;
   if (ns > G_NS_MAX) ns = G_NS_MAX;
-  const int sms = sm_count();
   int grid = tiles < sms ? (int)tiles : sms;
   // A chain's CTAs wait for one another, so all of them must be resident together (a cooperative launch
   // checks that); members with fewer tiles than CTAs simply leave some CTAs without work in that member.
+  if (chain && grid > most) grid = (int)most;
   std::vector<uint2> deps;
   std::vector<size_t> deps_off(count, 0), done_off(count, 0);
   size_t done_words = 0, chain_bytes = 0;
@@ -1365,7 +1458,8 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     for (int i = 0; i < count; ++i) {
       if (i > 0 && (gs[i].C != gs[i - 1].K || gs[i].H != gs[i - 1].Ho || gs[i].W != gs[i - 1].Wo || gs[i].N != gs[0].N))
         return cudaErrorInvalidConfiguration;
-      const int mgroups = host[i].total_tiles / host[i].n_ntiles;
+      const GLayer& L = plan[i].L;
+      const int mgroups = L.total_tiles / L.n_ct;
       done_off[i] = done_words;
       done_words += (size_t)mgroups;
       if (i + 1 < count) {
@@ -1373,29 +1467,31 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
         chain_bytes += (((size_t)gs[i].N * gs[i].Ho * gs[i].Wo * ((gs[i].K + 31) / 32) * 4) + 255) & ~(size_t)255;
       }
       if (i == 0) continue;
-      // which M groups of the predecessor hold the input pixels of each of this member's M groups
-      const GLayer& L = host[i];
-      const GLayer& P = host[i - 1];
+      // which position tiles of the predecessor hold the input pixels of each of this member's position tiles
+      const GLayer& P = plan[i - 1].L;
       deps_off[i] = deps.size();
       for (int mg = 0; mg < mgroups; ++mg) {
-        const long long Q0 = (long long)mg * 128 * L.MT;
+        const long long Q0 = (long long)mg * L.Np;
         long long lo = -1, hi = -1;
-        for (int pl = 0; pl < L.n_planes; ++pl)
-          for (int r = 0; r < L.Rr; ++r) {
-            const int px = h_position_to_pixel(L, Q0 + r, pl >> 1, pl & 1);
+        for (int r = 0; r < L.Rr; ++r) {
+          const long long q = Q0 + r;
+          if (q >= (long long)L.Qtot) break;
+          const long long rg = q / L.Wg, n = rg / L.Hq;
+          for (int pl = 0; pl < L.n_planes; ++pl) {
+            const int px = g_pixel_of(L, (uint32_t)n, (int)(rg - n * L.Hq), (int)(q - rg * L.Wg), pl);
             if (px < 0) continue;
             if (lo < 0 || px < lo) lo = px;
             if (px > hi) hi = px;
           }
+        }
         uint2 d = make_uint2(1u, 0u);
         if (lo >= 0) {
-          // output pixel of the predecessor -> its position -> its M group
+          // output pixel of the predecessor -> its position -> its position tile
           auto group_of = [&](long long px) {
             const long long n = px / ((long long)P.Ho * P.Wo);
             const long long rem = px - n * (long long)P.Ho * P.Wo;
             const long long y = rem / P.Wo, x = rem - y * P.Wo;
-            const long long q = (n * P.Hq + y) * P.Wq + x;
-            return (uint32_t)(q / (128 * P.MT));
+            return (uint32_t)(((n * P.Hq + y) * P.Wg + (x >> P.lg)) / P.Np);
           };
           d = make_uint2(group_of(lo), group_of(hi));
         }
@@ -1403,128 +1499,102 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
       }
     }
   }
-  // Which CTAs take a problem's odd tiles.  Every CTA gets floor(tiles / grid) tiles of a problem
-  // and the first (tiles % grid) CTAs in the problem's rank order get one more; the rank order is
-  // by the time the CTAs have been given so far, least first, so that the CTAs end close
-  // together although a tile of one problem may take six times as long as a tile of another.
-  // Time of a tile: the larger of its MMAs (73 cycles each up to 128 channels wide, 128 cycles at
-  // 256) and of its fp32 output at the write rate an SM gets (13 bytes per cycle).
   std::vector<uint16_t> ranks((size_t)count * grid);
-  {
-    std::vector<double> busy(grid, 0.0);
-    std::vector<int> order(grid);
-    for (int i = 0; i < count; ++i) {
-      const GLayer& o = host[i];
-      const double mma = (double)o.MT * o.n_cb * o.taps * o.kpt * g_mma_cycles(o.Nt);
-      const double wr = 128.0 * o.MT * (o.Nt < o.K ? o.Nt : o.K) * 4 / 13.0;
-      const double cost = (mma > wr ? mma : wr) + 300.0;
-      for (int b = 0; b < grid; ++b) order[b] = b;
-      std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return busy[a] < busy[b]; });
-      const int base = o.total_tiles / grid, rem = o.total_tiles % grid;
-      for (int r = 0; r < grid; ++r) {
-        ranks[(size_t)i * grid + order[r]] = (uint16_t)r;
-        busy[order[r]] += cost * (base + (r < rem ? 1 : 0));
-      }
-    }
+  g_assign(plan, grid, &ranks);
+  GroupDev* Gd = new GroupDev();
+  Gd->count = count;
+  Gd->act_type = act_type;
+  Gd->mode = mode;
+  Gd->grid = grid;
+  Gd->chain = chain;
+  Gd->kind = kind;
+  // One allocation and one copy for everything the group owns: [weight operands][descriptions][ranks][dependencies]
+  // [counters][packed signs between the members]; the middle three come from the host.
+  auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+  const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint16_t));
+  const size_t blob_bytes = deps_at + up(deps.size() * sizeof(uint2)), blob_at = up(w_total), done_at = blob_at + blob_bytes;
+  const size_t chain_at = done_at + up(done_words * sizeof(uint32_t));
+  cudaError_t e = cudaMalloc(&Gd->mem, chain_at + chain_bytes);
+  if (e == cudaSuccess) {
+    Gd->layers_dev = reinterpret_cast<GLayer*>(Gd->mem + blob_at);
+    Gd->ranks = reinterpret_cast<uint16_t*>(Gd->mem + blob_at + rank_at);
+    Gd->done = reinterpret_cast<uint32_t*>(Gd->mem + done_at);
+    Gd->chain_buf = Gd->mem + chain_at;
   }
-  GroupDev* G = new GroupDev();
-  G->count = count;
-  G->act_type = act_type;
-  G->mode = mode;
-  G->grid = grid;
-  G->chain = chain;
-  G->kind = kind;
-  G->hot = hot;
-  cudaError_t e = cudaMalloc(&G->weights, w_total);
-  if (chain) {
-    G->done_words = done_words;
-    for (int i = 0; i < count; ++i) G->chain_off[i] = chain_off[i];
-    if (e == cudaSuccess) e = cudaMalloc(&G->done, done_words * sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMalloc(&G->chain_buf, chain_bytes ? chain_bytes : 256);
-    if (e == cudaSuccess) e = cudaMalloc(&G->deps, (deps.size() ? deps.size() : 1) * sizeof(uint2));
-    if (e == cudaSuccess && !deps.empty())
-      e = cudaMemcpyAsync(G->deps, deps.data(), deps.size() * sizeof(uint2), cudaMemcpyHostToDevice, s);
-  }
-  if (e == cudaSuccess) e = cudaMalloc(&G->layers_dev, sizeof(GLayer) * count);
-  if (e == cudaSuccess) e = cudaMalloc(&G->ranks, ranks.size() * sizeof(uint16_t));
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(G->ranks, ranks.data(), ranks.size() * sizeof(uint16_t), cudaMemcpyHostToDevice, s);
+  Gd->done_words = done_words;
+  for (int i = 0; i < count; ++i) Gd->chain_off[i] = chain_off[i];
+  const uint2* const deps_dev = reinterpret_cast<const uint2*>(Gd->mem + blob_at + deps_at);
+  std::vector<uint8_t> blob(blob_bytes);
   for (int i = 0; i < count && e == cudaSuccess; ++i) {
-    host[i].rank = G->ranks + (size_t)i * grid;
-    host[i].wt = G->weights + w_off[i];
-    host[i].alpha = Ls[i]->alpha;
-    host[i].shift = Ls[i]->shift;
-    host[i].deps = nullptr; host[i].prev_done = nullptr; host[i].prev_target = 0; host[i].done = nullptr;
+    GLayer& L = plan[i].L;
+    L.wt = Gd->mem + w_off[i];
+    Gd->map[i] = {L.tma != 0, L.C, L.W, L.H, L.N, L.rs, L.Wg};
+    L.alpha = Ls[i]->alpha;
+    L.shift = Ls[i]->shift;
     if (chain) {
-      host[i].done = G->done + done_off[i];
+      L.done = Gd->done + done_off[i];
       if (i > 0) {
-        host[i].deps = G->deps + deps_off[i];
-        host[i].prev_done = G->done + done_off[i - 1];
-        host[i].prev_target = (uint32_t)(G_EW * host[i - 1].n_ntiles);   // (all eight warps drain a chain's tiles)
+        L.deps = deps_dev + deps_off[i];
+        L.prev_done = Gd->done + done_off[i - 1];
+        L.prev_target = (uint32_t)(G_EW * plan[i - 1].L.n_ct);   // (all eight warps drain a chain's tiles)
       }
     }
-    e = g_expand_weights(mode, Ls[i]->wplanes, G->weights + w_off[i], gs[i].C, gs[i].K, gs[i].Cw, Kpad[i],
-                         n_chunks[i], host[i].cb_chunks, host[i].NtL, host[i].taps, s);
+    const long long total = (long long)plan[i].w_bytes / 16;
+    const unsigned blocks = (unsigned)((total + 255) / 256);
+    const int win_step = gs[i].stride, ks = gs[i].ksize;
+    if (mode == M_F16)
+      g_expand_weights_kernel<M_F16><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
+                                                            total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, win_step,
+                                                            ks, plan[i].taps);
+    else
+      g_expand_weights_kernel<M_FP4><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
+                                                            total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, win_step,
+                                                            ks, plan[i].taps);
+    e = cudaGetLastError();
     if (e == cudaSuccess) *launched += 1;
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(G->layers_dev, host, sizeof(GLayer) * count, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // `host` and `ranks` live on this stack
+  for (int i = 0; i < count; ++i) memcpy(blob.data() + sizeof(GLayer) * (size_t)i, &plan[i].L, sizeof(GLayer));
+  memcpy(blob.data() + rank_at, ranks.data(), ranks.size() * sizeof(uint16_t));
+  if (!deps.empty()) memcpy(blob.data() + deps_at, deps.data(), deps.size() * sizeof(uint2));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(Gd->mem + blob_at, blob.data(), blob_bytes, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host arrays live on this stack
   if (e != cudaSuccess) {
-    tcg_destroy(G);
+    tcg_destroy(Gd);
     return e;
   }
-  GParams& p = G->p;
-  p.layers = G->layers_dev;
+  GParams& p = Gd->p;
+  p.layers = Gd->layers_dev;
+  p.ranks = Gd->ranks;
   p.n_layers = count;
   p.NA = na;
   p.NS = ns;
-  p.acc_cols = (uint32_t)g_acc_cols(mode, n_acc);
+  p.acc_cols = acc_cols;
   p.n_acc = n_acc;
   p.a_slot_bytes = (uint32_t)a_slot;
-  p.b_slot_bytes = kGBSlot;
+  p.b_slot_bytes = b_slot;
   p.off_b = (uint32_t)((size_t)na * a_slot);
-  p.off_epi = p.off_b + (uint32_t)ns * kGBSlot;
+  p.off_epi = p.off_b + (uint32_t)ns * b_slot;
   p.off_pix = p.off_epi + G_EPI_BYTES;
   p.off_lay = p.off_pix + (uint32_t)pix_bytes;
-  p.pix_words = (uint32_t)(pix_one / 4);
   p.off_tail = p.off_lay + (uint32_t)lay_bytes;
-  G->smem = (size_t)p.off_tail + kGTail;
-  if (G->smem > (size_t)kMaxDynSmem || G->smem >= (1u << 18)) {
-    tcg_destroy(G);
+  Gd->smem = (size_t)p.off_tail + kGTail;
+  if (Gd->smem > (size_t)kMaxDynSmem || Gd->smem >= (1u << 18)) {
+    tcg_destroy(Gd);
     return cudaErrorInvalidConfiguration;
   }
-  *out = G;
+  *out = Gd;
   return cudaSuccess;
 }
 
 void tcg_destroy(GroupDev* G) {
   if (!G) return;
-  cudaFree(G->weights);
-  cudaFree(G->layers_dev);
-  cudaFree(G->ranks);
-  cudaFree(G->done);
-  cudaFree(G->chain_buf);
-  cudaFree(G->deps);
+  cudaFree(G->mem);
   delete G;
 }
 
 int tcg_count(const GroupDev* G) { return G->count; }
 
-bool tcg_supported(const Geom& g, int act_type) {
-  // one problem alone, under every plan a launch may use: two activation slots, the fixed parts and three
-  // weight slots must fit
-  const int mode = g_mode_for(act_type);
-  for (int n_acc = G_NACC; n_acc <= (mode == M_FP4 ? G_NACC_WORDS : G_NACC); ++n_acc) {
-    GLayer L;
-    int n_chunks = 0, Kpad = 0;
-    if (!g_plan_layer(g, mode, n_acc, &L, &n_chunks, &Kpad)) return false;
-    const size_t unit = (((size_t)L.n_planes * L.cb_chunks * L.Rr * 16) + 127) & ~(size_t)127;
-    const size_t pix = (((size_t)L.n_planes * L.Rr * 4) + 127) & ~(size_t)127;
-    const size_t fixed = (size_t)G_EPI_BYTES + G_XTEAMS * pix + 256 + kGTail;
-    if (2 * unit + fixed + 3 * (size_t)kGBSlot > kGSmemBudget) return false;
-  }
-  return true;
-}
+bool tcg_supported(const Geom& g, int act_type) { return g_path_takes(g, g_mode_for(act_type)); }
 
 cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, int out_type, cudaStream_t s,
                         int* status_dev, int* launched) {
@@ -1562,25 +1632,34 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
   cfg.blockDim = dim3(G_THREADS);
   cfg.dynamicSmemBytes = G->smem;
   cudaError_t e;
+  GMaps<M_FP4> none{};
   const int outk = G->chain ? OUT_CHAIN : (out_type == 2 ? OUT_SIGNS : OUT_WORDS);
   if (!G->chain && (outk == OUT_SIGNS) != (G->kind == TCG_SIGNS)) return cudaErrorInvalidValue;  // planned for the other kind
-  bool piped = G->hot && outk == OUT_WORDS && out_type == 0;
-  // rows are read two or four words at a time by the pipelined expanders: every input 8-byte aligned
-  for (int i = 0; piped && i < G->count; ++i)
-    if (reinterpret_cast<uintptr_t>(act[i]) & 7) piped = false;
-#define G_LAUNCH(M, O)                                                      \
-  do {                                                                      \
-    static unsigned long long done = 0;                                     \
-    e = allow_max_smem(tcg_conv_kernel<M, O>, &done);                       \
-    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, tcg_conv_kernel<M, O>, p); \
+#define G_LAUNCH(M, O, MAPS)                                                    \
+  do {                                                                          \
+    static unsigned long long done = 0;                                         \
+    e = allow_max_smem(tcg_conv_kernel<M, O>, &done);                           \
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, tcg_conv_kernel<M, O>, p, MAPS); \
   } while (0)
   if (G->mode == M_F16) {
-    if (outk == OUT_WORDS) G_LAUNCH(M_F16, OUT_WORDS);
+    GMaps<M_F16> maps;
+    for (int i = 0; i < G->count; ++i) {
+      const GroupDev::Map& m = G->map[i];
+      if (!m.tma) continue;
+      // [N][H][W][C] halves; a box is 64 channels of one row of positions
+      const cuuint64_t dim[4] = {(cuuint64_t)m.C, (cuuint64_t)m.W, (cuuint64_t)m.H, (cuuint64_t)m.N};
+      const cuuint64_t pitch[3] = {(cuuint64_t)m.C * 2, (cuuint64_t)m.W * m.C * 2, (cuuint64_t)m.H * m.W * m.C * 2};
+      const cuuint32_t box[4] = {64, (cuuint32_t)((m.box - 1) * m.stride + 1), 1, 1}, step[4] = {1, (cuuint32_t)m.stride, 1, 1};
+      if (g_map_encoder()(&maps.m[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(act[i]), dim, pitch, box, step,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    }
+    if (outk == OUT_WORDS) G_LAUNCH(M_F16, OUT_WORDS, maps);
     else return cudaErrorInvalidValue;   // packed signs and chains need binary activations
-  } else if (outk == OUT_WORDS && piped) G_LAUNCH(M_FP4, OUT_WORDS_PIPED);
-  else if (outk == OUT_WORDS) G_LAUNCH(M_FP4, OUT_WORDS);
-  else if (outk == OUT_SIGNS) G_LAUNCH(M_FP4, OUT_SIGNS);
-  else G_LAUNCH(M_FP4, OUT_CHAIN);
+  } else if (outk == OUT_WORDS) G_LAUNCH(M_FP4, OUT_WORDS, none);
+  else if (outk == OUT_SIGNS) G_LAUNCH(M_FP4, OUT_SIGNS, none);
+  else G_LAUNCH(M_FP4, OUT_CHAIN, none);
 #undef G_LAUNCH
   if (e != cudaSuccess) return e;
   *launched += 1;

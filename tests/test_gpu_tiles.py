@@ -1,0 +1,115 @@
+"""Shapes at the edges of the tensor-core kernel's tiles: the channel counts at which a position starts to stand for
+2, 4 or 8 output pixels, maps whose width is no multiple of them, one activation word per pixel (two taps per K step),
+channel counts around a tile of 128, tiles of fewer than 32 positions, and fp16 units fetched by TMA or by copies.
+Sums and signs of binary layers are exact; fp16 outputs are checked at the tolerance of fp32 sums of exact products."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def snn():
+    import paper_2110_09195_b200 as snn
+    return snn
+
+
+@pytest.fixture(scope="module")
+def oracle_mod():
+    import oracle
+    oracle.build()
+    return oracle
+
+
+def _signs(y):
+    n, h, w, k = y.shape
+    bits = np.zeros((n, h, w, (k + 31) // 32 * 32), np.uint32)
+    bits[..., :k] = y >= 0
+    return (bits.reshape(n, h, w, -1, 32) << np.arange(32, dtype=np.uint32)).sum(axis=-1, dtype=np.uint32)
+
+
+@pytest.mark.parametrize("stride,pad", [(1, 1), (1, 0), (2, 1), (2, 0)])
+@pytest.mark.parametrize("c_in,c_out,h,w,n", [
+    (1, 1, 3, 3, 1), (16, 15, 7, 9, 2), (31, 16, 8, 16, 3), (32, 17, 9, 13, 2), (33, 32, 5, 31, 2), (64, 33, 11, 6, 2),
+    (20, 64, 6, 33, 3), (65, 65, 4, 40, 2), (96, 128, 10, 10, 2), (70, 129, 3, 57, 2), (160, 257, 6, 7, 3), (16, 16, 57, 3, 5),
+])
+def test_binary_tile_edges(snn, oracle_mod, c_in, c_out, h, w, n, stride, pad):
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, pad)
+    p = wl.draw_layer_params(shape, 6, 300 + c_in + c_out)
+    alpha = p.alpha.copy()
+    alpha[::3] *= -1.0
+    packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 301 + w))
+    s_ref, y_ref = oracle_mod.conv_bin(p.codebook, 6, p.idx_packed, alpha, c_in, c_out, stride, pad, packed)
+    shift = np.random.default_rng(7).normal(0, np.sqrt(9 * c_in), c_out).astype(np.float32)
+    shift[::5] = -0.0   # a negative zero sum counts as +1 like a positive one
+    layer = snn.SnnConv(c_in, c_out, 6, p.codebook, p.idx_packed, alpha, stride, pad, snn.ACT_BIN, shift=shift)
+    act = torch.from_numpy(packed.view(np.int32)).cuda()
+    assert layer.path_supported(snn.PATH_DECODED_TC, n, h, w)
+    sums = layer.forward(act, out_type=snn.OUT_I32, path=snn.PATH_DECODED_TC).cpu().numpy()
+    assert (sums == s_ref).all()
+    y = layer.forward(act, out_type=snn.OUT_F32, path=snn.PATH_DECODED_TC).cpu().numpy()
+    assert (y == s_ref.astype(np.float32) * alpha).all()
+    bits = layer.forward(act, out_type=snn.OUT_BITS).cpu().numpy().view(np.uint32)
+    assert (bits == _signs(s_ref.astype(np.float32) * alpha + shift)).all()
+    layer.destroy()
+
+
+def test_binary_tile_edges_in_one_launch(snn, oracle_mod):
+    """Members of every group size in one launch: one ring geometry for all of them."""
+    shapes = [(wl.LayerShape(16, 16, 32, 32, 1, 1), 9), (wl.LayerShape(40, 32, 9, 13, 2, 1), 2), (wl.LayerShape(64, 64, 20, 21, 1, 1), 6),
+              (wl.LayerShape(96, 200, 7, 7, 1, 1), 4), (wl.LayerShape(24, 16, 6, 5, 1, 0, 1), 3), (wl.LayerShape(512, 300, 5, 5, 1, 1), 2)]
+    layers, acts, refs = [], [], []
+    for i, (s, n) in enumerate(shapes):
+        p = wl.draw_layer_params(s, 5, 400 + i)
+        packed = wl.pack_activation_bits(wl.draw_activation_bits(s, n, 400 + i))
+        if s.ksize == 1:
+            refs.append(oracle_mod.conv1x1_bin(p.codebook, 5, p.idx_packed, p.alpha, s.c_in, s.c_out, s.stride, packed)[0])
+        else:
+            refs.append(oracle_mod.conv_bin(p.codebook, 5, p.idx_packed, p.alpha, s.c_in, s.c_out, s.stride, s.pad, packed)[0])
+        layers.append(snn.SnnConv(s.c_in, s.c_out, 5, p.codebook, p.idx_packed, p.alpha, s.stride, s.pad, ksize=s.ksize))
+        acts.append(torch.from_numpy(packed.view(np.int32)).cuda())
+    group = snn.SnnConvGroup(layers, [(n, s.h, s.w) for s, n in shapes])
+    for out, ref in zip(group.forward(acts, out_type=snn.OUT_I32), refs):
+        assert (out.cpu().numpy() == ref).all()
+    group.destroy()
+    for l in layers:
+        l.destroy()
+
+
+@pytest.mark.parametrize("c_in,c_out,h,w,stride,pad,n", [
+    (8, 16, 5, 4, 1, 1, 2),        # fewer channels than a box
+    (72, 40, 9, 11, 1, 0, 3),      # a second channel block that is mostly out of bounds
+    (128, 130, 30, 17, 2, 1, 2),   # parity planes as units of their own, two channel tiles
+    (64, 64, 3, 255, 1, 1, 1),     # the widest row of positions a box takes at stride 1 ...
+    (64, 64, 3, 256, 1, 1, 1),     # ... and one more: copied
+    (16, 24, 5, 250, 2, 1, 2),     # the same at stride 2
+    (16, 24, 5, 256, 2, 1, 2),
+    (20, 24, 6, 7, 1, 1, 2),       # rows that are no multiple of 16 bytes: copied element by element
+])
+def test_fp16_units(snn, oracle_mod, c_in, c_out, h, w, stride, pad, n):
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, pad)
+    p = wl.draw_layer_params(shape, 5, 500 + w)
+    act = wl.draw_activation_f16(shape, n, 501 + c_in)
+    ref = oracle_mod.conv_f16(p.codebook, 5, p.idx_packed, p.alpha, c_in, c_out, stride, pad, act).astype(np.float64)
+    layer = snn.SnnConv(c_in, c_out, 5, p.codebook, p.idx_packed, p.alpha, stride, pad, snn.ACT_F16)
+    assert layer.path_supported(snn.PATH_DECODED_TC, n, h, w)
+    y = layer.forward(torch.from_numpy(act).cuda(), path=snn.PATH_DECODED_TC).cpu().numpy().astype(np.float64)
+    # 9 * c_in exact products summed in fp32: each addition rounds by at most 2^-24 of the sum of magnitudes
+    mag = p.alpha.astype(np.float64) * 9 * c_in * np.abs(act.astype(np.float64)).max()
+    assert (np.abs(y - ref) <= 9 * c_in * 2.0 ** -24 * mag).all()
+    assert np.linalg.norm(y - ref) <= 1e-5 * np.linalg.norm(ref)
+    # an infinity reaches the outputs whose window holds it, and no other
+    at = (0, h // 2, w // 2, c_in // 2)
+    bad = act.copy()
+    bad[at] = np.inf
+    z = layer.forward(torch.from_numpy(bad).cuda(), path=snn.PATH_DECODED_TC).cpu().numpy()
+    hit = np.zeros(z.shape[1:3], bool)
+    for i in range(z.shape[1]):
+        for j in range(z.shape[2]):
+            hit[i, j] = abs(i * stride - pad + 1 - at[1]) <= 1 and abs(j * stride - pad + 1 - at[2]) <= 1
+    assert np.isinf(z[0][hit]).all()
+    assert (z[0][~hit] == y[0][~hit].astype(np.float32)).all() and (z[1:] == y[1:].astype(np.float32)).all()
+    layer.destroy()
