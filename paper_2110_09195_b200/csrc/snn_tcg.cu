@@ -133,7 +133,7 @@ struct GLayer {
   const uint2* deps;          // [position tiles] first and last position tile of the predecessor this one reads (x > y: none)
   const uint32_t* prev_done;  // the predecessor's completion counters, and the count that means "complete"
   uint32_t prev_target;
-  uint32_t* done;             // [position tiles] epilogue warps that have finished the tile, over all its channel tiles
+  uint32_t* done;             // [position tiles] epilogue warps that have written their part, over all its channel tiles
   uint32_t tap[kGTapsMax];    // per step: start of its rows in the unit (16-byte units) | distance of its two chunks << 16
 };
 
@@ -181,17 +181,25 @@ __device__ __forceinline__ int g_position_to_pixel(const GLayer& L, uint32_t q, 
   return g_pixel_of(L, n, (int)(rg - n * (uint32_t)L.Hq), j, pl);
 }
 
-// Bounded wait until a completion counter another CTA advances has reached `target` (acquire: what that CTA
-// wrote before is visible afterwards).  False when the limit ran out or the CTA is giving up.
-__device__ __forceinline__ bool g_wait_counter(const uint32_t* ctr, uint32_t target, volatile int* abort_flag, uint32_t limit) {
-  for (uint32_t it = 0; it < limit; ++it) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr) : "memory");
-    if (v >= target) return true;
-    if (limit == 1 || *abort_flag) return false;
-    __nanosleep(100);
+// Waits (bounded) until the completion counters first..last, advanced by other CTAs, have reached `target`.  Whole-warp
+// call: a lane looks at one counter, 32 at a time - one after the other, each look is a round trip to L2, and a tile's
+// window spans up to six tiles of the predecessor.  False when the limit ran out or the CTA is giving up.  What was
+// written before the counters were advanced is visible to the warp afterwards.
+__device__ __forceinline__ bool g_wait_counters(const uint32_t* ctr, uint32_t first, uint32_t last, uint32_t target, int lane,
+                                                volatile int* abort_flag) {
+  for (uint32_t it = 0; first <= last; ++it) {
+    uint32_t v = target;
+    if (first + (uint32_t)lane <= last)
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(ctr + first + (uint32_t)lane) : "memory");
+    if (__all_sync(0xffffffffu, v >= target)) {
+      first += 32u;
+    } else {
+      if (it >= (1u << 21) || __any_sync(0xffffffffu, *abort_flag != 0)) return false;
+      __nanosleep(20);
+    }
   }
-  return false;
+  __syncwarp();
+  return true;
 }
 // Activation words: through the read-only path, or - when another CTA of this launch wrote them - from L2.
 __device__ __forceinline__ uint32_t g_ld1(const uint32_t* p, bool fresh) { return fresh ? __ldcg(p) : __ldg(p); }
@@ -297,6 +305,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
   const uint32_t bar_tabfull = smem_u32(bars + 32), bar_tabempty = smem_u32(bars + 36);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 40);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  uint32_t* ready_tiles = tmem_slot + 2;   // chain: tiles of this CTA whose input has been written
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NS = p.NS, NA = p.NA;
@@ -308,7 +317,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
     if (tid >= 16 && tid < 20) count = FP4 ? G_EW / G_XTEAMS : G_EW;    // a_full: one arrival per expander warp of the unit
     mbar_init(smem_u32(bars + tid), count);
   }
-  if (tid == 64) *abort_flag = 0;
+  if (tid == 64) {
+    *abort_flag = 0;
+    *ready_tiles = 0;
+  }
   {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
     uint32_t* dst = reinterpret_cast<uint32_t*>(smem + p.off_lay);
@@ -588,9 +600,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
         }
         if (CHAIN) {
           // chain: this warp's part of the tile is written; the successor may read it
-          __threadfence();
-          __syncwarp();
-          if (lane == 0) atomicAdd(lay[l].done + h0.y, 1u);
+          if (active && half < n_slices) {
+            __syncwarp();
+            if (lane == 0) {
+              __threadfence();   // (cumulative: it covers what the other lanes wrote before the barrier)
+              asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(lay[l].done + h0.y) : "memory");
+            }
+          }
         }
       }
       __syncwarp();   // the table has been read
@@ -670,6 +686,36 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
       }
       __syncwarp();
     }
+  } else if (CHAIN && warp == 17) {
+    // ------------------------------------------------ dependency warp (chains)
+    // Waits, tile by tile, until the predecessor has written every input pixel of the tile, and counts the tiles whose
+    // input may be read.  One warp per CTA looks at the counters: when every expander warp did, the looks of all CTAs at
+    // the same few lines of L2 held up the counters themselves.
+    uint32_t done = 0;
+    for (int l = 0; l < p.n_layers; ++l) {
+      const GLayer& L = lay[l];
+      const uint2* const deps = L.deps;
+      const uint32_t* const ctr = L.prev_done;
+      const uint32_t target = L.prev_target;
+      const FastDiv dCt = L.dCt;
+      const int total = L.total_tiles;
+      bool ok = true;
+      for (int tile = L.first; tile < total && ok; tile += G) {
+        if (deps) {
+          const uint2 d = __ldg(deps + fdiv((uint32_t)tile, dCt));
+          ok = g_wait_counters(ctr, d.x, d.y, target, lane, abort_flag);
+        }
+        ++done;
+        if (ok && lane == 0) asm volatile("st.release.cta.shared.u32 [%0], %1;" ::"r"(smem_u32(ready_tiles)), "r"(done) : "memory");
+      }
+      if (!ok) {
+        if (lane == 0 && !*abort_flag) {
+          *abort_flag = 1;
+          raise_status(p.status, 5);
+        }
+        break;
+      }
+    }
   } else if (warp != 17) {
     // ------------------------------------------------ expanders (warps 10-12, 14-16, 18, 19)
     // Fill activation unit (problem, tile, channel block) of the ring: for every plane, row and
@@ -739,18 +785,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
       bool inside = false;                            // it lies in the batch
       const uint32_t* act = nullptr;
       bool ivalid = false, ready = false;             // is there a unit; may its input be read (chain)
-      uint32_t dep_at = 1, dep_end = 0;               // chain: predecessor tiles still to be waited for
+      uint32_t tile_seq = ~0u;                        // tile of the CTA, over all problems
       auto enter_tile = [&]() {
         const GLayer& L = lay[il];
         const uint32_t mg = fdiv((uint32_t)itile, L.dCt);
         Q0 = mg * (uint32_t)L.Np;
-        ready = true;
-        if (CHAIN && L.deps) {
-          const uint2 d = __ldg(L.deps + mg);
-          dep_at = d.x;
-          dep_end = d.y;
-          ready = false;
-        }
+        ready = !CHAIN;
+        ++tile_seq;
       };
       auto enter_layer = [&]() {   // first layer from il on in which this CTA has a tile
         for (; il < p.n_layers; ++il) {
@@ -785,18 +826,17 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
       auto seek_own = [&]() {      // on to this team's next unit
         while (ivalid && (iu % XG) != gx) next_unit();
       };
-      // chain: has the predecessor written every input pixel of the tile?  One lane per warp looks (blocking: waits,
-      // bounded); no barrier among the warps, so that one that gives up leaves none of the others waiting.
+      // chain: may the tile's input be read?  (blocking: waits, bounded.)
       auto check_ready = [&](bool blocking) -> bool {
         if (!CHAIN || ready) return true;
-        const GLayer& L = lay[il];
-        int okd = 1;
-        if (lane == 0) {
-          for (; dep_at <= dep_end; ++dep_at)
-            if (!g_wait_counter(L.prev_done + dep_at, L.prev_target, abort_flag, blocking ? 1u << 21 : 1u)) { okd = 0; break; }
+        for (uint32_t it = 0;; ++it) {
+          uint32_t v;
+          asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(ready_tiles)) : "memory");
+          ready = __all_sync(0xffffffffu, v > tile_seq);
+          if (ready || !blocking) break;
+          if (it >= (1u << 23) || __any_sync(0xffffffffu, *abort_flag != 0)) break;
+          __nanosleep(20);
         }
-        ready = __shfl_sync(0xffffffffu, okd, 0) != 0;
-        __syncwarp();   // what lane 0 acquired is visible to the whole warp
         return ready;
       };
       auto issue = [&](XGroup& g) {   // loads of the group at the issue position; moves the position on
@@ -1536,7 +1576,15 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
       if (i > 0) {
         L.deps = deps_dev + deps_off[i];
         L.prev_done = Gd->done + done_off[i - 1];
-        L.prev_target = (uint32_t)(G_EW * plan[i - 1].L.n_ct);   // (all eight warps drain a chain's tiles)
+        // the epilogue warps that have something to write of a position tile: one per 32 rows that hold a
+        // channel and, from two slices on, two per lane quarter
+        const GLayer& P = plan[i - 1].L;
+        int quarters = (gs[i - 1].K + 31) / 32;
+        if (P.lg) {
+          quarters = 0;
+          for (int r = 0; r < G_ROWS; r += 32) quarters += (r & ((G_ROWS >> P.lg) - 1)) < gs[i - 1].K ? 1 : 0;
+        }
+        L.prev_target = (uint32_t)(quarters * (P.Np > 32 ? 2 : 1));
       }
     }
     const long long total = (long long)plan[i].w_bytes / 16;
