@@ -549,21 +549,26 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
             if (s + 2 >= n_slices) release();
             if (WORDS || out_kind != 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
+              // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubled the code, and the
+              // roles share the instruction caches (ResNet-18 group 111 -> 103 us, 1x1 layers 402 -> 385, ResNet-34 stack 444 -> 417).
+              if (out_kind == 0) {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__fmul_rn(__uint_as_float(v[e]), al));
+              } else {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = (uint32_t)__float2int_rn(__uint_as_float(v[e]));   // integer sums: exact
+              }
               // One column = one pixel of 32 channels per step: a predicated store of a whole 128-byte line.
-              auto store = [&](auto value) {
 #pragma unroll
-                for (int e = 0; e < 32; e += 4) {
-                  const uint4 o4 = *reinterpret_cast<const uint4*>(&T->offset[32 * s + e]);
-                  const uint32_t o[4] = {o4.x, o4.y, o4.z, o4.w};
+              for (int e = 0; e < 32; e += 4) {
+                const uint4 o4 = *reinterpret_cast<const uint4*>(&T->offset[32 * s + e]);
+                const uint32_t o[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
-                  for (int j = 0; j < 4; ++j)
-                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(obase + o[j]),
-                                 "r"(value(v[e + j])), "r"(mask & (1u << (e + j)))
-                                 : "memory");
-                }
-              };
-              if (out_kind == 0) store([&](uint32_t x) { return __float_as_uint(__fmul_rn(__uint_as_float(x), al)); });
-              else store([&](uint32_t x) { return (uint32_t)__float2int_rn(__uint_as_float(x)); });   // integer sums: exact
+                for (int j = 0; j < 4; ++j)
+                  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(obase + o[j]),
+                               "r"(v[e + j]), "r"(mask & (1u << (e + j)))
+                               : "memory");
+              }
             } else {
               // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): bit of a channel =
               // fl(fl(alpha*S) + shift) >= 0 = sign bit clear (no sum is -0 or NaN: alpha and shift are finite and
