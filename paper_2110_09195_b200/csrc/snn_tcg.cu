@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
       // before group g is expanded into shared memory, so that a unit does not cost a full round trip to memory.
       // A thread keeps the geometry of its position while it walks through the planes and words: these eight warps
       // are bound by how many instructions a unit takes one warp, not by the issue slots of the SM.
-      constexpr int XI = G_EXP_ITEMS;
+      constexpr int XI = CHAIN ? G_EXP_ITEMS / 2 : G_EXP_ITEMS;   // (a chain's tiles are small: less code is worth more, 416 -> 407 us)
       struct XGroup {
         uint4 t[XI];       // the items' words (one, two or four of them)
         uint32_t da[XI];   // where an item's first chunk goes
