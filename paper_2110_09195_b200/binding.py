@@ -168,6 +168,16 @@ def forward_static(c_in, c_out, tau, codebook, idx_packed, alpha, act, out, stri
     return out
 
 
+def _raw_stream(device, stream):
+    """cudaStream_t of `stream`, by default torch's current stream on the device.  torch.cuda.current_stream builds a
+    Stream object for its handle, a quarter of the time of a small layer's call; the handle alone is one C call."""
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return raw(device) if raw is not None else torch.cuda.current_stream(device).cuda_stream
+
+
 class SnnConv:
     """One sub-bit 3x3 layer on one GPU (wraps a snn_conv_t handle)."""
 
@@ -235,24 +245,24 @@ class SnnConv:
     def forward(self, act, out=None, out_type=OUT_F32, path=PATH_AUTO, stream=None):
         """snn_conv_forward: act / out are CUDA tensors; asynchronous on `stream`
         (default: torch's current stream)."""
-        import torch
-        if not act.is_cuda or act.device.index != self.device:
+        if act.get_device() != self.device:
             raise SnnError(1, f"activations must live on cuda:{self.device}")
         self._check_act(act)
-        n, h, w = int(act.shape[0]), int(act.shape[1]), int(act.shape[2])
+        n, h, w, _ = act.shape
         if out is None:
             out = self.alloc_out(n, h, w, out_type)
         else:
+            import torch
             ho, wo = self.out_hw(h, w)
             want = torch.float32 if out_type == OUT_F32 else torch.int32
             last = (self.c_out + 31) // 32 if out_type == OUT_BITS else self.c_out
-            if (not out.is_cuda or out.device.index != self.device or out.dtype != want or not out.is_contiguous()
-                    or tuple(out.shape) != (n, ho, wo, last)):
+            if (out.get_device() != self.device or out.dtype != want or not out.is_contiguous()
+                    or out.shape != (n, ho, wo, last)):
                 raise SnnError(1, "output tensor has the wrong device, dtype, shape or layout")
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
-        _check(load_library().snn_conv_forward(self._h, act.data_ptr(), n, h, w, out.data_ptr(), int(out_type),
-                                               int(path), ctypes.c_void_p(stream.cuda_stream)))
+        st = (_lib or load_library()).snn_conv_forward(self._h, act.data_ptr(), n, h, w, out.data_ptr(), int(out_type),
+                                                       int(path), _raw_stream(self.device, stream))
+        if st:
+            _check(st)
         return out
 
     def forward_host(self, act, out=None, out_type=OUT_F32, path=PATH_AUTO):
@@ -321,6 +331,10 @@ class SnnConvGroup:
         _check(lib.snn_conv_group_create(hs, n, ns, hh, ww, ctypes.byref(g)))
         self._g = g
         self.device = self.layers[0].device
+        # what forward() expects of each member's tensors
+        self._act_shapes = [(*s, (l.c_in + 31) // 32 if l.act_type == ACT_BIN else l.c_in) for l, s in zip(self.layers, self.shapes)]
+        self._out_shapes = [(s[0], *l.out_hw(s[1], s[2]), l.c_out) for l, s in zip(self.layers, self.shapes)]
+        self._sign_shapes = [(*o[:3], (o[3] + 31) // 32) for o in self._out_shapes]
 
     def alloc_outs(self, out_type=OUT_F32):
         import torch
@@ -339,23 +353,21 @@ class SnnConvGroup:
         if outs is None:
             outs = self.alloc_outs(out_type)
         want = torch.float32 if out_type == OUT_F32 else torch.int32
-        for l, (nb, h, w), a, o in zip(self.layers, self.shapes, acts, outs):
-            last = (l.c_out + 31) // 32 if out_type == OUT_BITS else l.c_out
-            if not a.is_cuda or a.device.index != self.device:
-                raise SnnError(1, f"activations must live on cuda:{self.device}")
-            l._check_act(a)
-            ho, wo = l.out_hw(h, w)
-            if tuple(a.shape[:3]) != (nb, h, w):
+        dev = self.device
+        dtypes = (torch.int32, torch.uint32) if self.layers[0].act_type == ACT_BIN else (torch.float16,)
+        for l, a, o, ashape, oshape in zip(self.layers, acts, outs, self._act_shapes,
+                                           self._sign_shapes if out_type == OUT_BITS else self._out_shapes):
+            # one comparison of everything for the usual case; what is wrong is found out afterwards
+            if a.get_device() != dev or a.dtype not in dtypes or a.shape != ashape or not a.is_contiguous():
+                if a.get_device() != dev:
+                    raise SnnError(1, f"activations must live on cuda:{dev}")
+                l._check_act(a)
                 raise SnnError(1, "activation tensor does not have the shape the group was created for")
-            if (not o.is_cuda or o.device.index != self.device or o.dtype != want or not o.is_contiguous()
-                    or tuple(o.shape) != (nb, ho, wo, last)):
+            if o.get_device() != dev or o.dtype != want or o.shape != oshape or not o.is_contiguous():
                 raise SnnError(1, "output tensor has the wrong device, dtype, shape or layout")
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
         ap = (ctypes.c_void_p * n)(*[a.data_ptr() for a in acts])
         op = (ctypes.c_void_p * n)(*[o.data_ptr() for o in outs])
-        _check(load_library().snn_conv_group_forward(self._g, ap, op, int(out_type),
-                                                     ctypes.c_void_p(stream.cuda_stream)))
+        _check(load_library().snn_conv_group_forward(self._g, ap, op, int(out_type), _raw_stream(dev, stream)))
         return outs
 
     def destroy(self):
@@ -417,10 +429,8 @@ class SnnConvStack:
         if (not out.is_cuda or out.device.index != self.device or out.dtype != dt or not out.is_contiguous()
                 or tuple(out.shape) != (self.n, *self.out_hw, k)):
             raise SnnError(1, "output tensor has the wrong device, dtype, shape or layout")
-        if stream is None:
-            stream = torch.cuda.current_stream(self.device)
         _check(load_library().snn_conv_stack_forward(self._s, act.data_ptr(), out.data_ptr(), int(out_type),
-                                                     ctypes.c_void_p(stream.cuda_stream)))
+                                                     _raw_stream(self.device, stream)))
         return out
 
     def destroy(self):
