@@ -255,8 +255,8 @@ SNN_API snn_status_t snn_conv_stack_destroy(snn_conv_stack_t* s);
  * synchronisation an allocation may bring.  snn_conv_create allocates, so such
  * callers use this call instead: it takes the layer as the descriptor states it
  * (HOST arrays, as for snn_conv_create) together with the DEVICE activation and
- * output buffers, and does everything else - copy of the layer, decode, XOR +
- * popcount convolution - inside one fixed device array that is part of the
+ * output buffers, and does everything else - copy of the layer, decode,
+ * convolution - inside one fixed device array that is part of the
  * library image (SNN_STATIC_SCRATCH_BYTES on every GPU that loads the library,
  * held until the process exits).  It calls no cudaMalloc / cudaFree and no
  * allocating library routine.
@@ -275,6 +275,8 @@ SNN_API snn_status_t snn_conv_stack_destroy(snn_conv_stack_t* s);
  * contents: each call rewrites in full every region it reads, so results never
  * depend on an earlier call, but two calls whose GPU work overlaps (different
  * streams, or threads) race on it.  Serialise them.
+ * Errors beside those of snn_conv_forward: TIMEOUT (an earlier call's launch gave
+ * up a bounded wait).
  */
 #define SNN_STATIC_SCRATCH_BYTES (1536 * 1024)
 #define SNN_STATIC_MAX_CHANNELS 512

@@ -161,10 +161,8 @@ def forward_static(c_in, c_out, tau, codebook, idx_packed, alpha, act, out, stri
         raise SnnError(1, f"out must be {want} of shape {(n, ho, wo, int(c_out))}")
     d = _Desc(int(c_in), int(c_out), int(tau), int(stride), int(pad), ACT_BIN, int(device),
               cb.ctypes.data, ip.ctypes.data, al.ctypes.data, None, 3)
-    if stream is None:
-        stream = torch.cuda.current_stream(device)
     _check(load_library().snn_conv_forward_static(ctypes.byref(d), act.data_ptr(), n, h, w, out.data_ptr(),
-                                                  int(out_type), ctypes.c_void_p(stream.cuda_stream)))
+                                                  int(out_type), _raw_stream(int(device), stream)))
     return out
 
 

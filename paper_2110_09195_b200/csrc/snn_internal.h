@@ -69,6 +69,16 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
                         int* status_dev, int* launched);
 void tcg_destroy(GroupDev* G);
 int tcg_count(const GroupDev* G);
+// One launch from the stored form of a layer (index stream, codebook and scales in device memory), in memory of the
+// caller's: tcg_static_plan says how many bytes that takes (binary activations, fp32 / int32 outputs; false where the
+// tensor-core kernel cannot run the layer), tcg_static_forward writes the weight operand there and runs the layer.
+struct TcgStatic {
+  size_t bytes;
+  alignas(16) unsigned char opaque[3072];
+};
+bool tcg_static_plan(const Geom& g, TcgStatic* out);
+cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8_t* stream_dev, const uint16_t* codebook_dev,
+                               const float* alpha_dev, uint8_t* mem, const Launch& l, int* status_dev, int* launched);
 bool tcg_supported(const Geom& g, int act_type);   // can the tensor-core kernel run this layer at this shape?
 
 cudaError_t microbench(int kind, double* rate);

@@ -4,9 +4,11 @@
 // (the copied index stream, unpacked indices, codebook, scales, decoded weight
 // bit-planes, border corrections) lives here in ONE fixed device array that is
 // part of the library image.  Each call copies the layer description into that
-// array, decodes it there and runs the XOR + popcount kernel on it.
+// array, writes the tensor-core kernel's weight operand there and runs that kernel on it; a shape the tensor-core
+// kernel does not take is decoded to bit-planes and run by the XOR + popcount kernel.
 #include <cmath>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 
 #include "snn_internal.h"
@@ -26,15 +28,34 @@ constexpr int kMaxDevices = 64;
 std::mutex g_setup_mu;
 unsigned char* g_scratch_dev[kMaxDevices] = {nullptr};
 
-// Device address of the scratch on the current device, resolved once per device.
-cudaError_t scratch_address(int device, unsigned char** out) {
+// Where a tensor-core launch reports a bounded wait that gave up: one word per device in a page of the library image,
+// pinned and mapped at the first call (host memory; nothing is allocated on a device).
+struct alignas(4096) StatusPage {
+  volatile int word[4096 / sizeof(int)];
+};
+StatusPage g_status;
+int g_status_state = 0;   // 0: not pinned yet, 1: pinned, 2: cannot be (the popcount kernel, which does not wait, is used)
+int* g_status_dev[kMaxDevices] = {nullptr};
+
+// Device addresses of the scratch and of the status word on the current device, resolved once per device.
+cudaError_t scratch_address(int device, unsigned char** out, int** status) {
   std::lock_guard<std::mutex> lk(g_setup_mu);
   if (!g_scratch_dev[device]) {
     void* ptr = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_scratch);
     if (e != cudaSuccess) return e;
+    if (g_status_state == 0) {
+      g_status_state = cudaHostRegister(&g_status, sizeof(g_status), cudaHostRegisterMapped | cudaHostRegisterPortable) == cudaSuccess ? 1 : 2;
+      cudaGetLastError();
+    }
+    void* st = nullptr;
+    if (g_status_state == 1 && cudaHostGetDevicePointer(&st, const_cast<int*>(g_status.word), 0) == cudaSuccess)
+      g_status_dev[device] = static_cast<int*>(st) + device * 16;
+    else
+      cudaGetLastError();
     g_scratch_dev[device] = static_cast<unsigned char*>(ptr);
   }
+  *status = g_status_dev[device];
   *out = g_scratch_dev[device];
   return cudaSuccess;
 }
@@ -118,8 +139,56 @@ extern "C" SNN_API snn_status_t snn_conv_forward_static(const snn_conv_desc_t* d
 
   snn_status_t st = SNN_OK;
   unsigned char* base = nullptr;
-  cudaError_t e = scratch_address(d->device, &base);  // first call on a device resolves the symbol
+  int* status_dev = nullptr;
+  cudaError_t e = scratch_address(d->device, &base, &status_dev);  // first call on a device resolves the symbol
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  int launched = 0;
+  // The tensor-core kernel where it takes the shape (8 images of a 128-channel 28x28 layer: 19 us a call, by
+  // popcounts 48): [codebook][scales][index stream][weight operand, description].
+  const size_t t_alpha = 1024, t_stream = t_alpha + align256((size_t)g.K * 4), t_mem = align256(t_stream + stream_bytes);
+  TcgStatic plan;
+  g.ksize = 3;
+  if (e == cudaSuccess && status_dev && tcg_static_plan(g, &plan) && t_mem + plan.bytes <= kStaticScratchBytes) {
+    volatile int* const status = &g_status.word[d->device * 16];
+    if (*status) {
+      const int code = *status;
+      *status = 0;
+      if (prev >= 0 && prev != d->device) cudaSetDevice(prev);
+      return api_fail(SNN_ERR_TIMEOUT, "an earlier tensor-core launch gave up a bounded wait (code %d)", code);
+    }
+    // Pageable arrays are gathered into one copy (the runtime stages pageable memory before it returns).  Pinned or managed
+    // ones, which the stream may still be writing, and all of them under capture, where a replay reads them
+    // again, are copied from where they are.
+    auto pageable = [](const void* p) {
+      cudaPointerAttributes a;
+      return cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeUnregistered;
+    };
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(s, &capturing);
+    if (e == cudaSuccess && capturing == cudaStreamCaptureStatusNone && pageable(d->codebook) && pageable(d->alpha) &&
+        pageable(d->idx_packed)) {
+      alignas(16) unsigned char gather[32 * 1024];
+      const bool all = t_stream + stream_bytes <= sizeof(gather);   // a long stream goes by itself
+      memcpy(gather, d->codebook, (size_t)T * 2);
+      memcpy(gather + t_alpha, d->alpha, (size_t)g.K * 4);
+      if (all) memcpy(gather + t_stream, d->idx_packed, stream_bytes);
+      e = cudaMemcpyAsync(base, gather, all ? t_stream + stream_bytes : t_stream, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess && !all) e = cudaMemcpyAsync(base + t_stream, d->idx_packed, stream_bytes, cudaMemcpyHostToDevice, s);
+    } else {
+      if (e == cudaSuccess) e = cudaMemcpyAsync(base, d->codebook, (size_t)T * 2, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(base + t_alpha, d->alpha, (size_t)g.K * 4, cudaMemcpyHostToDevice, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(base + t_stream, d->idx_packed, stream_bytes, cudaMemcpyHostToDevice, s);
+    }
+    if (e == cudaSuccess) {
+      Launch l{act_dev, out_dev, out_type == SNN_OUT_I32, s};
+      e = tcg_static_forward(plan, g, base + t_stream, reinterpret_cast<const uint16_t*>(base), reinterpret_cast<const float*>(base + t_alpha),
+                             base + t_mem, l, status_dev, &launched);
+    }
+    api_count_launches(launched);
+    if (e != cudaSuccess) st = api_fail(SNN_ERR_CUDA, "snn_conv_forward_static: %s", cudaGetErrorString(e));
+    if (prev >= 0 && prev != d->device) cudaSetDevice(prev);
+    return st;
+  }
   LayerDev L;
   if (e == cudaSuccess) {
     L.idx = reinterpret_cast<uint16_t*>(base + o_idx);
@@ -132,7 +201,6 @@ extern "C" SNN_API snn_status_t snn_conv_forward_static(const snn_conv_desc_t* d
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(L.codebook, d->codebook, (size_t)T * 2, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(L.alpha, d->alpha, (size_t)g.K * 4, cudaMemcpyHostToDevice, s);
-  int launched = 0;
   // every region the kernels read is rewritten in full by this call, so nothing left
   // behind by the previous call can leak into the result and nothing needs clearing
   if (e == cudaSuccess) e = decode_layer(L, base + o_stream, g, SNN_ACT_BIN, s, &launched);

@@ -833,13 +833,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
       };
       // chain: may the tile's input be read?  (blocking: waits, bounded.)
       auto check_ready = [&](bool blocking) -> bool {
-        if (!CHAIN || ready) return true;
-        for (uint32_t it = 0;; ++it) {
+        for (uint32_t it = 0; CHAIN && !ready; ++it) {
           uint32_t v;
           asm volatile("ld.acquire.cta.shared.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(ready_tiles)) : "memory");
           ready = __all_sync(0xffffffffu, v > tile_seq);
-          if (ready || !blocking) break;
-          if (it >= (1u << 23) || __any_sync(0xffffffffu, *abort_flag != 0)) break;
+          if (ready || !blocking || it >= (1u << 23) || __any_sync(0xffffffffu, *abort_flag != 0)) break;
           __nanosleep(20);
         }
         return ready;
@@ -1195,7 +1193,8 @@ struct GPlan {
 // The plan of one layer with tiles of Np positions of 2^lg pixels; false where that does not fit.
 bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, GPlan* P) {
   GLayer& o = P->L;
-  o = GLayer{};
+  o.wt = nullptr; o.alpha = o.shift = nullptr; o.deps = nullptr; o.prev_done = nullptr; o.prev_target = 0; o.done = nullptr;
+  o.first = 0;
   const int cpc = mode == M_F16 ? 8 : 32;
   const int S = g.stride, G = 1 << lg;
   const bool one = g.ksize == 1;
@@ -1366,21 +1365,109 @@ bool g_path_takes(const Geom& g, int mode) {
 // Tile sizes the planner chooses from (positions; multiples of 16).
 constexpr int kNpTable[] = {256, 240, 208, 192, 160, 144, 128, 112, 96, 80, 64, 48, 32, 16};
 
-// Best plan of one layer for tiles of at most `cap` positions: the group size 2^lg with the least time over all its tiles.
-bool g_best_group(const Geom& g, int mode, int kind, int cap, bool tma, GPlan* out) {
+// A tile size under consideration: what has to be planned, and the estimates the choice is made by.
+struct GChoice {
+  int lg = 0, Np = 0, tiles = 0;
+  bool tma = false;
+  double through = 0, alone = 0;
+};
+
+// Best choice for one layer and tiles of at most `cap` positions: the group size 2^lg with the least time over all its tiles.
+bool g_best_group(const Geom& g, int mode, int kind, int cap, bool tma, GChoice* out) {
   bool found = false;
   double best = 0;
+  GPlan P;
   for (int lg = 0; lg <= 3; ++lg) {
+    if (lg && (mode != M_FP4 || g.K > G_ROWS >> lg)) break;
     for (int Np : kNpTable) {
       if (Np > cap) continue;
-      GPlan P;
-      if (!g_plan_layer(g, mode, kind, lg, Np, tma, &P) && !g_plan_layer(g, mode, kind, lg, Np, false, &P)) continue;
+      if (!g_plan_layer(g, mode, kind, lg, Np, tma, &P) && !(tma && g_plan_layer(g, mode, kind, lg, Np, false, &P))) continue;
       const double t = P.L.total_tiles * P.through();
-      if (!found || t < best) { best = t; *out = P; found = true; }
+      if (!found || t < best) {
+        best = t;
+        *out = {lg, Np, P.L.total_tiles, P.L.tma != 0, P.through(), P.alone()};
+        found = true;
+      }
       break;   // the largest that fits
     }
   }
   return found;
+}
+
+// The ring geometry of a launch of these problems and where its parts lie in shared memory; false where it does not fit.
+bool g_ring(const GPlan* plan, int count, int mode, GParams* p, size_t* smem) {
+  const uint32_t tmem = mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16;
+  size_t a_slot = 0, pix_bytes = 0;
+  int widest = 16;
+  for (int i = 0; i < count; ++i) {
+    const GLayer& o = plan[i].L;
+    a_slot = std::max(a_slot, plan[i].unit_bytes);
+    if (mode == M_F16 && !o.tma) pix_bytes = std::max(pix_bytes, (size_t)o.n_planes * o.Rr * 4);
+    widest = std::max(widest, o.Np);
+  }
+  // accumulator buffers: as many as fit, up to four
+  int n_acc = (int)tmem / widest;
+  if (n_acc > 4) n_acc = 4;
+  a_slot = (a_slot + 1023) & ~(size_t)1023;   // (the swizzle of the TMA units repeats every 1024 bytes)
+  const uint32_t b_slot = mode == M_F16 ? kGBSlotF16 : kGBSlot;
+  pix_bytes = (pix_bytes + 127) & ~(size_t)127;
+  const size_t lay_bytes = ((size_t)count * sizeof(GLayer) + 127) & ~(size_t)127;
+  const size_t fixed = (size_t)G_EPI_BYTES + pix_bytes + lay_bytes + kGTail;
+  // Ring depths: four activation slots if they fit beside four weight slots, else two (with the 4-bit expanders a
+  // multiple of the number of teams) or three; the weights take what is left.
+  static_assert(G_XTEAMS == 1 || G_XTEAMS == 2, "the ring depths below are multiples of the team count");
+  int na = 4, ns = 0;
+  for (; na >= 2; --na) {
+    if (mode == M_FP4 && na % G_XTEAMS) continue;
+    const int ns_min = mode == M_F16 ? 4 : na > 2 ? 4 : 3;
+    if ((size_t)na * a_slot + fixed + ns_min * (size_t)b_slot > kGSmemBudget) continue;
+    ns = (int)((kGSmemBudget - fixed - (size_t)na * a_slot) / b_slot);
+    break;
+  }
+  if (na < 2 || ns < 3) return false;
+  if (ns > G_NS_MAX) ns = G_NS_MAX;
+  p->n_layers = count;
+  p->NA = na;
+  p->NS = ns;
+  p->acc_cols = (tmem / (uint32_t)n_acc) & ~15u;
+  p->n_acc = n_acc;
+  p->a_slot_bytes = (uint32_t)a_slot;
+  p->b_slot_bytes = b_slot;
+  p->off_b = (uint32_t)((size_t)na * a_slot);
+  p->off_epi = p->off_b + (uint32_t)ns * b_slot;
+  p->off_pix = p->off_epi + G_EPI_BYTES;
+  p->off_lay = p->off_pix + (uint32_t)pix_bytes;
+  p->off_tail = p->off_lay + (uint32_t)lay_bytes;
+  *smem = (size_t)p->off_tail + kGTail;
+  return *smem <= (size_t)kMaxDynSmem && *smem < (1u << 18);
+}
+
+// Tiles of independent problems: one size limit for all of them, by the estimated time of the launch.
+bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma, int sms, GPlan* plan) {
+  GChoice trial[SNN_GROUP_MAX], chosen[SNN_GROUP_MAX];
+  double best = -1;
+  for (int cap : kNpTable) {
+    if (cap > (int)(mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16) / 2) continue;
+    bool ok = true;
+    for (int i = 0; i < count && ok; ++i) ok = g_best_group(gs[i], mode, kind, cap, tma, &trial[i]);
+    if (!ok) continue;
+    // the machine's share of all tiles (whole tiles where there is one problem), and the last tile's way through the roles
+    double sum = 0, last = 0, slowest = 0;
+    for (int i = 0; i < count; ++i) {
+      const GChoice& c = trial[i];
+      sum += count == 1 ? (double)((c.tiles + sms - 1) / sms) * sms * c.through : c.tiles * c.through;
+      last = std::max(last, c.alone - c.through);
+      slowest = std::max(slowest, c.through);
+    }
+    const double t = std::max(sum / sms, slowest) + last + (count > 1 ? slowest / 2 : 0);
+    if (best < 0 || t < best) {
+      best = t;
+      std::copy(trial, trial + count, chosen);
+    }
+  }
+  if (best < 0) return false;
+  for (int i = 0; i < count; ++i) g_plan_layer(gs[i], mode, kind, chosen[i].lg, chosen[i].Np, chosen[i].tma, &plan[i]);
+  return true;
 }
 
 // Which CTAs take a problem's odd tiles.  Every CTA gets floor(tiles / grid) tiles of a problem
@@ -1414,83 +1501,44 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   for (int i = 0; i < count; ++i)
     if (!g_path_takes(gs[i], mode)) return cudaErrorInvalidConfiguration;
   const int sms = sm_count();
-  const uint32_t tmem = mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16;
-  int cap_max = (int)tmem / 2;
+  const int cap_max = (int)G_TMEM_FP4 / 2;   // (a chain has binary activations)
   const bool tma = mode == M_F16 && g_map_encoder() != nullptr;
   // Tile sizes.  A chain's members run one after the other as far as their inputs go, so each takes the size that makes
   // its own tiles end first; the members of a group share the machine, and one size limit for all of them is chosen by
   // the time of the busiest CTA.
-  std::vector<GPlan> plan(count), trial(count);
-  double best = -1;
+  std::vector<GPlan> plan(count);
   if (chain) {
     for (int i = 0; i < count; ++i) {
-      best = -1;
-      for (int cap : kNpTable) {
-        if (cap > cap_max) continue;
+      double best = -1;
+      int best_lg = 0, best_np = 0;
+      GPlan P;
+      for (int Np : kNpTable) {
+        if (Np > cap_max) continue;
         for (int lg = 0; lg <= 3; ++lg) {
-          GPlan P;
-          if (!g_plan_layer(gs[i], mode, kind, lg, cap, false, &P)) continue;
+          if (!g_plan_layer(gs[i], mode, kind, lg, Np, false, &P)) continue;
           const int waves = (P.L.total_tiles + sms - 1) / sms;
           const double t = P.alone() + (waves - 1) * P.through();
-          if (best < 0 || t < best) { best = t; plan[i] = P; }
+          if (best < 0 || t < best) { best = t; best_lg = lg; best_np = Np; }
         }
       }
       if (best < 0) return cudaErrorInvalidConfiguration;
+      g_plan_layer(gs[i], mode, kind, best_lg, best_np, false, &plan[i]);
     }
-  } else {
-    for (int cap : kNpTable) {
-      if (cap > cap_max) continue;
-      bool ok = true;
-      for (int i = 0; i < count && ok; ++i) ok = g_best_group(gs[i], mode, kind, cap, tma, &trial[i]);
-      if (!ok) continue;
-      // the machine's share of all tiles (whole tiles where there is one problem), and the last tile's way through the roles
-      double sum = 0, last = 0, slowest = 0;
-      for (const GPlan& P : trial) {
-        sum += count == 1 ? (double)((P.L.total_tiles + sms - 1) / sms) * sms * P.through() : P.L.total_tiles * P.through();
-        last = std::max(last, P.alone() - P.through());
-        slowest = std::max(slowest, P.through());
-      }
-      const double t = std::max(sum / sms, slowest) + last + (count > 1 ? slowest / 2 : 0);
-      if (best < 0 || t < best) { best = t; plan = trial; }
-    }
-    if (best < 0) return cudaErrorInvalidConfiguration;
+  } else if (!g_plan_independent(gs, count, mode, kind, tma, sms, plan.data())) {
+    return cudaErrorInvalidConfiguration;
   }
   for (int i = 0; i < count; ++i) g_finish_plan(gs[i], &plan[i]);
-  size_t w_off[SNN_GROUP_MAX], w_total = 0, a_slot = 0, pix_bytes = 0;
+  GParams ring{};
+  size_t smem = 0;
+  if (!g_ring(plan.data(), count, mode, &ring, &smem)) return cudaErrorInvalidConfiguration;
+  size_t w_off[SNN_GROUP_MAX], w_total = 0;
   long long tiles = 0, most = 0;
-  int widest = 16;
   for (int i = 0; i < count; ++i) {
-    const GLayer& o = plan[i].L;
-    a_slot = std::max(a_slot, plan[i].unit_bytes);
-    if (mode == M_F16 && !o.tma) pix_bytes = std::max(pix_bytes, (size_t)o.n_planes * o.Rr * 4);
-    widest = std::max(widest, o.Np);
     w_off[i] = w_total;
     w_total += (plan[i].w_bytes + 255) & ~(size_t)255;
-    tiles += o.total_tiles;
-    most = std::max(most, (long long)o.total_tiles);
+    tiles += plan[i].L.total_tiles;
+    most = std::max(most, (long long)plan[i].L.total_tiles);
   }
-  // accumulator buffers: as many as fit, up to four
-  int n_acc = (int)tmem / widest;
-  if (n_acc > 4) n_acc = 4;
-  const uint32_t acc_cols = (tmem / (uint32_t)n_acc) & ~15u;
-  a_slot = (a_slot + 1023) & ~(size_t)1023;   // (the swizzle of the TMA units repeats every 1024 bytes)
-  const uint32_t b_slot = mode == M_F16 ? kGBSlotF16 : kGBSlot;
-  pix_bytes = (pix_bytes + 127) & ~(size_t)127;
-  const size_t lay_bytes = ((size_t)count * sizeof(GLayer) + 127) & ~(size_t)127;
-  const size_t fixed = (size_t)G_EPI_BYTES + pix_bytes + lay_bytes + kGTail;
-  // Ring depths: four activation slots if they fit beside four weight slots, else two (with the pipelined expanders a
-  // multiple of the number of teams) or three; the weights take what is left.
-  static_assert(G_XTEAMS == 1 || G_XTEAMS == 2, "the ring depths below are multiples of the team count");
-  int na = 4, ns = 0;
-  for (; na >= 2; --na) {
-    if (mode == M_FP4 && na % G_XTEAMS) continue;
-    const int ns_min = mode == M_F16 ? 4 : na > 2 ? 4 : 3;
-    if ((size_t)na * a_slot + fixed + ns_min * (size_t)b_slot > kGSmemBudget) continue;
-    ns = (int)((kGSmemBudget - fixed - (size_t)na * a_slot) / b_slot);
-    break;
-  }
-  if (na < 2 || ns < 3) return cudaErrorInvalidConfiguration;
-  if (ns > G_NS_MAX) ns = G_NS_MAX;
   int grid = tiles < sms ? (int)tiles : sms;
   // A chain's CTAs wait for one another, so all of them must be resident together (a cooperative launch
   // checks that); members with fewer tiles than CTAs simply leave some CTAs without work in that member.
@@ -1615,28 +1663,147 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     tcg_destroy(Gd);
     return e;
   }
-  GParams& p = Gd->p;
-  p.layers = Gd->layers_dev;
-  p.ranks = Gd->ranks;
-  p.n_layers = count;
-  p.NA = na;
-  p.NS = ns;
-  p.acc_cols = acc_cols;
-  p.n_acc = n_acc;
-  p.a_slot_bytes = (uint32_t)a_slot;
-  p.b_slot_bytes = b_slot;
-  p.off_b = (uint32_t)((size_t)na * a_slot);
-  p.off_epi = p.off_b + (uint32_t)ns * b_slot;
-  p.off_pix = p.off_epi + G_EPI_BYTES;
-  p.off_lay = p.off_pix + (uint32_t)pix_bytes;
-  p.off_tail = p.off_lay + (uint32_t)lay_bytes;
-  Gd->smem = (size_t)p.off_tail + kGTail;
-  if (Gd->smem > (size_t)kMaxDynSmem || Gd->smem >= (1u << 18)) {
-    tcg_destroy(Gd);
-    return cudaErrorInvalidConfiguration;
-  }
+  Gd->p = ring;
+  Gd->p.layers = Gd->layers_dev;
+  Gd->p.ranks = Gd->ranks;
+  Gd->smem = smem;
   *out = Gd;
   return cudaSuccess;
+}
+
+// ------------------------------------------------------------------ launches from the stored form of a layer
+namespace {
+
+struct StaticState {
+  GPlan plan;
+  GParams ring;
+  size_t smem;
+  int grid;
+};
+static_assert(sizeof(StaticState) <= sizeof(TcgStatic::opaque), "TcgStatic holds the plan of a launch");
+
+// Which step and chunk of the weight operand holds kernel row ky and window column s: step * 2 + chunk, 255: none.
+struct GStepOf {
+  uint8_t at[3][17];
+};
+
+// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook), and the description the launch
+// after it reads.  One thread per 32 input channels of one row of the operand: their 32 indices are consecutive bits of
+// the stream, looked up once for all taps.  Bound by latency, not by its work (16 K threads at most): all of a thread's
+// loads go out together.  With the launch after it, copies and host work included, a call on 8 images of a 128-channel
+// 28x28 layer takes 19 us; four decode kernels and the popcount kernel took 48.
+__global__ void __launch_bounds__(128) g_static_weights_kernel(const uint8_t* __restrict__ stream, long long n_bytes,
+                                                               const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
+                                                               const GLayer L, GLayer* __restrict__ layer_out,
+                                                               uint16_t* __restrict__ ranks_out, int grid, int tau, int paired,
+                                                               const GStepOf step_of) {
+  const int row = threadIdx.x, wd = blockIdx.x, ct = blockIdx.y;   // row of the operand, 32-channel word, channel tile
+  if (wd == 0 && ct == 0) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(&L);
+    for (int i = row; i < (int)(sizeof(GLayer) / 4); i += 128) reinterpret_cast<uint32_t*>(layer_out)[i] = src[i];
+    for (int i = row; i < grid; i += 128) ranks_out[i] = (uint16_t)i;
+  }
+  const int kp_log = 7 - L.lg, g = row >> kp_log, co = ct * G_ROWS + (row & ((1 << kp_log) - 1));
+  __shared__ uint16_t codes[512];
+  for (int i = row; i < (1 << tau); i += 128) codes[i] = codebook[i];
+  const int n_ch = co < L.K ? (L.C - 32 * wd < 32 ? L.C - 32 * wd : 32) : 0;   // channels of this word (none: all zeros)
+  const uint32_t exists = n_ch <= 0 ? 0u : 0xffffffffu >> (32 - n_ch);
+  // all loads first: one round trip to memory instead of one per index
+  uint32_t index[32];
+  {
+    long long bit = ((long long)co * L.C + 32 * wd) * tau;
+#pragma unroll
+    for (int b = 0; b < 32; ++b, bit += tau) {
+      const long long at = bit >> 3;   // an index spans at most two bytes (9 bits from any bit of a byte: 16 bits)
+      uint32_t v = 0;
+      if (b < n_ch) {
+        v = stream[at];
+        if (at + 1 < n_bytes) v |= (uint32_t)stream[at + 1] << 8;
+      }
+      index[b] = (v >> (bit & 7)) & ((1u << tau) - 1u);
+    }
+  }
+  __syncthreads();
+  uint32_t plane[9];   // bit b of plane t: tap t of channel 32*wd + b is +1
+#pragma unroll
+  for (int t = 0; t < 9; ++t) plane[t] = 0;
+#pragma unroll
+  for (int b = 0; b < 32; ++b) {
+    const uint32_t code = codes[index[b]];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) plane[t] |= ((code >> (8 - t)) & 1u) << b;
+  }
+  // nibbles in the expanders' order: channel 4n + k of the word in nibble n of word k
+  auto nibbles = [&](uint32_t bits, int k) {
+    const uint32_t e = ((exists >> k) & 0x11111111u) * 15u;
+    return ((~(bits << (3 - k)) & 0x88888888u) | 0x22222222u) & e;
+  };
+  const int chunks = paired ? 2 : L.cb_chunks, cb = paired ? 0 : wd / L.cb_chunks, c0 = paired ? 0 : wd - cb * L.cb_chunks;
+  uint4* const base = reinterpret_cast<uint4*>(wt) + (size_t)(ct * L.n_cb + cb) * L.steps * chunks * G_ROWS + row;
+  if (L.G > 1 || paired) {   // columns outside this pixel's window, and a last step's missing tap
+    for (int t = 0; t < L.steps; ++t)
+      for (int c = 0; c < (paired ? 2 : 1); ++c) base[(size_t)(t * chunks + c0 + c) * G_ROWS] = make_uint4(0, 0, 0, 0);
+  }
+#pragma unroll
+  for (int t = 0; t < 9; ++t) {
+    const int at = step_of.at[t / 3][t % 3 + L.rs * g];
+    base[(size_t)((at >> 1) * chunks + c0 + (at & 1)) * G_ROWS] =
+        make_uint4(nibbles(plane[t], 0), nibbles(plane[t], 1), nibbles(plane[t], 2), nibbles(plane[t], 3));
+  }
+}
+
+}  // namespace
+
+bool tcg_static_plan(const Geom& g, TcgStatic* out) {
+  if (g.ksize != 3 || !g_path_takes(g, M_FP4)) return false;
+  StaticState st;
+  const int sms = sm_count();
+  if (!g_plan_independent(&g, 1, M_FP4, TCG_WORDS, false, sms, &st.plan)) return false;
+  g_finish_plan(g, &st.plan);
+  st.ring = GParams{};
+  if (!g_ring(&st.plan, 1, M_FP4, &st.ring, &st.smem)) return false;
+  st.grid = st.plan.L.total_tiles < sms ? st.plan.L.total_tiles : sms;
+  out->bytes = ((st.plan.w_bytes + 255) & ~(size_t)255) + ((sizeof(GLayer) + 255) & ~(size_t)255) + (size_t)st.grid * sizeof(uint16_t);
+  memcpy(out->opaque, &st, sizeof(st));
+  return true;
+}
+
+cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8_t* stream_dev, const uint16_t* codebook_dev,
+                               const float* alpha_dev, uint8_t* mem, const Launch& l, int* status_dev, int* launched) {
+  StaticState st;
+  memcpy(&st, plan.opaque, sizeof(st));
+  GLayer& L = st.plan.L;
+  uint8_t* const layer_at = mem + ((st.plan.w_bytes + 255) & ~(size_t)255);
+  uint16_t* const ranks = reinterpret_cast<uint16_t*>(layer_at + ((sizeof(GLayer) + 255) & ~(size_t)255));
+  L.wt = mem;
+  L.alpha = alpha_dev;
+  GStepOf step_of;
+  memset(&step_of, 255, sizeof(step_of));
+  for (int t = 0; t < L.steps; ++t)
+    for (int c = 0; c < (st.plan.paired ? 2 : 1); ++c)
+      if (st.plan.taps.row[t][c] < 3) step_of.at[st.plan.taps.row[t][c]][st.plan.taps.col[t][c]] = (uint8_t)(2 * t + c);
+  const long long n_bytes = ((long long)g.K * g.C * g.tau + 7) / 8;
+  const dim3 blocks((unsigned)(st.plan.paired ? 1 : L.n_cb * L.cb_chunks), (unsigned)L.n_ct);
+  g_static_weights_kernel<<<blocks, G_ROWS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, reinterpret_cast<GLayer*>(layer_at),
+                                                           ranks, st.grid, g.tau, st.plan.paired, step_of);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  *launched += 1;
+  GParams p = st.ring;
+  p.layers = reinterpret_cast<const GLayer*>(layer_at);
+  p.ranks = ranks;
+  p.act[0] = l.act;
+  p.out[0] = l.out;
+  p.out_type[0] = (uint8_t)l.out_i32;
+  p.status = status_dev;
+  // An ordinary launch, not a programmatic dependent of the kernel above: the set-up reads what that one writes.
+  static unsigned long long done = 0;
+  e = allow_max_smem(tcg_conv_kernel<M_FP4, OUT_WORDS>, &done);
+  if (e != cudaSuccess) return e;
+  tcg_conv_kernel<M_FP4, OUT_WORDS><<<st.grid, G_THREADS, st.smem, l.stream>>>(p, GMaps<M_FP4>{});
+  e = cudaGetLastError();
+  if (e == cudaSuccess) *launched += 1;
+  return e;
 }
 
 void tcg_destroy(GroupDev* G) {

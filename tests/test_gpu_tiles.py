@@ -113,3 +113,51 @@ def test_fp16_units(snn, oracle_mod, c_in, c_out, h, w, stride, pad, n):
     assert np.isinf(z[0][hit]).all()
     assert (z[0][~hit] == y[0][~hit].astype(np.float32)).all() and (z[1:] == y[1:].astype(np.float32)).all()
     layer.destroy()
+
+
+@pytest.mark.parametrize("stride,pad", [(1, 1), (2, 0)])
+@pytest.mark.parametrize("c_in,c_out,h,w,n,tau", [
+    (1, 1, 3, 3, 1, 1), (16, 16, 9, 8, 2, 3), (31, 33, 6, 7, 2, 9), (64, 64, 5, 12, 2, 5), (70, 20, 8, 5, 3, 7), (129, 200, 4, 6, 2, 8),
+    (512, 128, 4, 4, 1, 9), (3, 512, 5, 6, 1, 2),
+])
+def test_operand_from_the_stored_form(snn, oracle_mod, c_in, c_out, h, w, n, tau, stride, pad):
+    """forward_static writes the weight operand from the index stream itself: indices of any width that straddle bytes and
+    end the stream, ragged words, groups of pixels, two taps per step."""
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, pad)
+    p = wl.draw_layer_params(shape, tau, 600 + c_in)
+    packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 601 + w))
+    s_ref, _ = oracle_mod.conv_bin(p.codebook, tau, p.idx_packed, p.alpha, c_in, c_out, stride, pad, packed)
+    act = torch.from_numpy(packed.view(np.int32)).cuda()
+    out = torch.full(s_ref.shape, -7, dtype=torch.int32, device="cuda")
+    snn.forward_static(c_in, c_out, tau, p.codebook, p.idx_packed, p.alpha, act, out, stride, pad, snn.OUT_I32)
+    assert (out.cpu().numpy() == s_ref).all()
+    # pinned arrays are copied from where they are, in stream order
+    pinned = torch.from_numpy(p.idx_packed).pin_memory()
+    out.fill_(-7)
+    snn.forward_static(c_in, c_out, tau, p.codebook, pinned.numpy(), p.alpha, act, out, stride, pad, snn.OUT_I32)
+    assert (out.cpu().numpy() == s_ref).all()
+
+
+def test_stored_form_under_capture(snn, oracle_mod):
+    """A captured call copies the layer's arrays at every replay, as it did before it was gathered into one copy."""
+    shape, n, tau = wl.LayerShape(64, 48, 8, 8, 1, 1), 2, 5
+    p, q = wl.draw_layer_params(shape, tau, 700), wl.draw_layer_params(shape, tau, 701)
+    packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 702))
+    refs = [oracle_mod.conv_bin(l.codebook, tau, l.idx_packed, l.alpha, 64, 48, 1, 1, packed)[0] for l in (p, q)]
+    act = torch.from_numpy(packed.view(np.int32)).cuda()
+    out = torch.zeros(refs[0].shape, dtype=torch.int32, device="cuda")
+    arrays = [torch.from_numpy(a.copy()).pin_memory() for a in (p.codebook.view(np.int16), p.idx_packed, p.alpha)]
+    args = (arrays[0].numpy().view(np.uint16), arrays[1].numpy(), arrays[2].numpy())
+    snn.forward_static(64, 48, tau, *args, act, out, out_type=snn.OUT_I32)   # the first call resolves the array
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        snn.forward_static(64, 48, tau, *args, act, out, out_type=snn.OUT_I32)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (out.cpu().numpy() == refs[0]).all()
+    for a, new in zip(arrays, (q.codebook.view(np.int16), q.idx_packed, q.alpha)):
+        a.copy_(torch.from_numpy(new.copy()))
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (out.cpu().numpy() == refs[1]).all()
