@@ -117,15 +117,18 @@ __global__ void __launch_bounds__(128, 1) mma_rate_kernel(int N, long long* cycl
     const uint64_t b0 = make_desc(smem_u32(smem + a_bytes), (uint32_t)N * 16, 128);
     const uint32_t idesc = FP4 ? ((1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24))
                                : ((1u << 4) | ((uint32_t)(N >> 3) << 17) | ((128u >> 4) << 24));
-    const int nacc = 2 * N <= (FP4 ? 480 : 512) ? 2 : 1;
+    // two accumulators (2 * N columns fit: 480 with the block scales, else 512), two MMAs per pass of the loop: with one, and
+    // the flag and addresses made anew for it, what was measured was the loop (33 cycles an MMA on top)
     const long long t0 = clock64();
-    for (int it = 0; it < MMA_ITERS; ++it) {
+    for (int it = 0; it < MMA_ITERS / 2; ++it) {
       if (leader) {
-        const uint32_t d = tb + (uint32_t)((it & (nacc - 1)) * N);
-        const uint64_t ad = a0 + (uint64_t)(((it >> 1) & 7) * 256);
-        const uint64_t bd = b0 + (uint64_t)(((it >> 1) & 7) * (N * 2));
-        if (FP4) mma_ss_fp4(d, ad, bd, idesc, it >= nacc ? 1u : 0u, tb + 480, tb + 496);
-        else mma_ss_f16(d, ad, bd, idesc, it >= nacc ? 1u : 0u);
+        const uint64_t ad = a0 + (uint64_t)((it & 7) * 256);
+        const uint64_t bd = b0 + (uint64_t)((it & 7) * (N * 2));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          if (FP4) mma_ss_fp4(tb + (uint32_t)(h * N), ad, bd, idesc, it ? 1u : 0u, tb + 480, tb + 496);
+          else mma_ss_f16(tb + (uint32_t)(h * N), ad, bd, idesc, it ? 1u : 0u);
+        }
       }
     }
     if (leader) tc_commit(smem_u32(&bar));
