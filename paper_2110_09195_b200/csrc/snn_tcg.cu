@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
       }
       __syncwarp();
       const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
-      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, Np = h1.z;
+      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y;
       if (l < 0) break;   // no more tiles
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : h1.w;
       uint32_t* const out32 = reinterpret_cast<uint32_t*>(p.out[l]);  // int32 and fp32 outputs share the layout
@@ -532,21 +532,15 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
           release();
         } else {
           uint32_t* const obase = out32 + (size_t)((uint32_t)(g_lane * K + co));
+          // (a last slice of 16 columns is read as 32: the others belong to the next buffer or the scales and go nowhere)
+          uint32_t v[32];
+          __syncwarp();
+          tmem_ld32(d0 + (uint32_t)(32 * half), v);
 #pragma unroll 1
           for (int s = half; s < n_slices; s += 2) {   // the two warps of a lane quarter take the slices in turn
-            uint32_t v[32];
-            __syncwarp();
-            if (32 * s + 32 <= Np) {
-              tmem_ld32(d0 + (uint32_t)(32 * s), v);
-              tmem_ld_wait();
-            } else {   // the last 16 columns
-              uint32_t u[16];
-              tmem_ld16(d0 + (uint32_t)(32 * s), u);
-              tmem_ld_wait();
-#pragma unroll
-              for (int e = 0; e < 16; ++e) { v[e] = u[e]; v[16 + e] = 0; }
-            }
-            if (s + 2 >= n_slices) release();
+            const bool last = s + 2 >= n_slices;
+            tmem_ld_wait();
+            if (last) release();
             if (WORDS || out_kind != 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
               // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubled the code, and the
@@ -569,6 +563,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
                                "r"(v[e + j]), "r"(mask & (1u << (e + j)))
                                : "memory");
               }
+              __syncwarp();   // the load is a warp-wide instruction
+              if (!last) tmem_ld32(d0 + (uint32_t)(32 * s + 64), v);
             } else {
               // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): bit of a channel =
               // fl(fl(alpha*S) + shift) >= 0 = sign bit clear (no sum is -0 or NaN: alpha and shift are finite and
@@ -578,18 +574,24 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
               unsigned long long a2, t2;
               asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(al));
               asm("mov.b64 %0, {%1, %1};" : "=l"(t2) : "f"(sh));
-              uint32_t w = 0;
+              uint32_t part[4] = {0, 0, 0, 0};   // four chains of eight bits: one of 32 waits for itself
 #pragma unroll
-              for (int e = 30; e >= 0; e -= 2) {
-                unsigned long long x;
-                asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v[e]), "r"(v[e + 1]));
-                asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(a2));
-                asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(t2));
-                uint32_t y0, y1;
-                asm("mov.b64 {%0, %1}, %2;" : "=r"(y0), "=r"(y1) : "l"(x));
-                w = __funnelshift_l(y1, w, 1);
-                w = __funnelshift_l(y0, w, 1);
+              for (int e = 6; e >= 0; e -= 2) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  unsigned long long x;
+                  asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v[8 * c + e]), "r"(v[8 * c + e + 1]));
+                  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(a2));
+                  asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(t2));
+                  uint32_t y0, y1;
+                  asm("mov.b64 {%0, %1}, %2;" : "=r"(y0), "=r"(y1) : "l"(x));
+                  part[c] = __funnelshift_l(y1, part[c], 1);
+                  part[c] = __funnelshift_l(y0, part[c], 1);
+                }
               }
+              __syncwarp();
+              if (!last) tmem_ld32(d0 + (uint32_t)(32 * s + 64), v);   // beside the transposition and the store
+              uint32_t w = part[0] | (part[1] << 8) | (part[2] << 16) | (part[3] << 24);
               w = co < K ? ~w : 0u;   // bits of channels that do not exist are 0
               w = g_transpose32(w, lane);
               const uint32_t px = T->offset[32 * s + lane], here = 1u << lane;
