@@ -150,6 +150,7 @@ struct GParams {
   int NA, NS;
   uint32_t a_slot_bytes, b_slot_bytes;
   uint32_t off_b, off_epi, off_pix, off_lay, off_tail;
+  GLayer one;             // n_layers == 1: the problem itself (layers and ranks are not read: its tiles go to the CTAs in order)
 };
 
 // Profiling aid (build with -DSNN_TRACE): every role's reporting lane adds up the cycles it spends in its
@@ -281,7 +282,7 @@ __device__ __forceinline__ uint32_t g_transpose32(uint32_t x, int lane) {
 enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2 };
 
 template <int MODE, int OUTK>
-__global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p, const __grid_constant__ GMaps<MODE> maps) {
+__global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_constant__ GParams p, const __grid_constant__ GMaps<MODE> maps) {
   constexpr bool F16 = MODE == M_F16;   // fp16 activations (copied, not expanded)
   constexpr bool FP4 = MODE == M_FP4;   // binary activations as e2m1 nibbles
   constexpr bool CHAIN = OUTK == OUT_CHAIN;
@@ -321,15 +322,21 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const GParams p,
     *abort_flag = 0;
     *ready_tiles = 0;
   }
+  int first = (int)blockIdx.x;
   {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
     uint32_t* dst = reinterpret_cast<uint32_t*>(smem + p.off_lay);
-    const int words = p.n_layers * (int)(sizeof(GLayer) / 4);
-    for (int i = tid; i < words; i += G_THREADS) dst[i] = __ldg(src + i);
+    if (p.n_layers == 1) {
+      // a launch of one problem is short: its description comes with the launch, not from memory
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(&p.one);
+      for (int i = tid; i < (int)(sizeof(GLayer) / 4); i += G_THREADS) dst[i] = src[i];
+    } else {
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
+      const int words = p.n_layers * (int)(sizeof(GLayer) / 4);
+      for (int i = tid; i < words; i += G_THREADS) dst[i] = __ldg(src + i);
+      // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
+      if (tid < p.n_layers) first = (int)__ldg(p.ranks + (size_t)tid * G + blockIdx.x);
+    }
   }
-  // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
-  int first = 0;
-  if (tid < p.n_layers) first = (int)__ldg(p.ranks + (size_t)tid * G + blockIdx.x);
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(512)
@@ -1668,6 +1675,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->p = ring;
   Gd->p.layers = Gd->layers_dev;
   Gd->p.ranks = Gd->ranks;
+  Gd->p.one = plan[0].L;
   Gd->smem = smem;
   *out = Gd;
   return cudaSuccess;
@@ -1689,22 +1697,15 @@ struct GStepOf {
   uint8_t at[3][17];
 };
 
-// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook), and the description the launch
-// after it reads.  One thread per 32 input channels of one row of the operand: their 32 indices are consecutive bits of
+// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook).  One thread per 32 input channels of one row of the operand: their 32 indices are consecutive bits of
 // the stream, looked up once for all taps.  Bound by latency, not by its work (16 K threads at most): all of a thread's
 // loads go out together.  With the launch after it, copies and host work included, a call on 8 images of a 128-channel
 // 28x28 layer takes 19 us; four decode kernels and the popcount kernel took 48.
 __global__ void __launch_bounds__(128) g_static_weights_kernel(const uint8_t* __restrict__ stream, long long n_bytes,
                                                                const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
-                                                               const GLayer L, GLayer* __restrict__ layer_out,
-                                                               uint16_t* __restrict__ ranks_out, int grid, int tau, int paired,
+                                                               const GLayer L, int tau, int paired,
                                                                const GStepOf step_of) {
   const int row = threadIdx.x, wd = blockIdx.x, ct = blockIdx.y;   // row of the operand, 32-channel word, channel tile
-  if (wd == 0 && ct == 0) {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(&L);
-    for (int i = row; i < (int)(sizeof(GLayer) / 4); i += 128) reinterpret_cast<uint32_t*>(layer_out)[i] = src[i];
-    for (int i = row; i < grid; i += 128) ranks_out[i] = (uint16_t)i;
-  }
   const int kp_log = 7 - L.lg, g = row >> kp_log, co = ct * G_ROWS + (row & ((1 << kp_log) - 1));
   __shared__ uint16_t codes[512];
   for (int i = row; i < (1 << tau); i += 128) codes[i] = codebook[i];
@@ -1765,7 +1766,7 @@ bool tcg_static_plan(const Geom& g, TcgStatic* out) {
   st.ring = GParams{};
   if (!g_ring(&st.plan, 1, M_FP4, &st.ring, &st.smem)) return false;
   st.grid = st.plan.L.total_tiles < sms ? st.plan.L.total_tiles : sms;
-  out->bytes = ((st.plan.w_bytes + 255) & ~(size_t)255) + ((sizeof(GLayer) + 255) & ~(size_t)255) + (size_t)st.grid * sizeof(uint16_t);
+  out->bytes = st.plan.w_bytes;
   memcpy(out->opaque, &st, sizeof(st));
   return true;
 }
@@ -1775,8 +1776,6 @@ cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8
   StaticState st;
   memcpy(&st, plan.opaque, sizeof(st));
   GLayer& L = st.plan.L;
-  uint8_t* const layer_at = mem + ((st.plan.w_bytes + 255) & ~(size_t)255);
-  uint16_t* const ranks = reinterpret_cast<uint16_t*>(layer_at + ((sizeof(GLayer) + 255) & ~(size_t)255));
   L.wt = mem;
   L.alpha = alpha_dev;
   GStepOf step_of;
@@ -1786,19 +1785,17 @@ cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8
       if (st.plan.taps.row[t][c] < 3) step_of.at[st.plan.taps.row[t][c]][st.plan.taps.col[t][c]] = (uint8_t)(2 * t + c);
   const long long n_bytes = ((long long)g.K * g.C * g.tau + 7) / 8;
   const dim3 blocks((unsigned)(st.plan.paired ? 1 : L.n_cb * L.cb_chunks), (unsigned)L.n_ct);
-  g_static_weights_kernel<<<blocks, G_ROWS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, reinterpret_cast<GLayer*>(layer_at),
-                                                           ranks, st.grid, g.tau, st.plan.paired, step_of);
+  g_static_weights_kernel<<<blocks, G_ROWS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, g.tau, st.plan.paired, step_of);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   *launched += 1;
   GParams p = st.ring;
-  p.layers = reinterpret_cast<const GLayer*>(layer_at);
-  p.ranks = ranks;
+  p.one = L;
   p.act[0] = l.act;
   p.out[0] = l.out;
   p.out_type[0] = (uint8_t)l.out_i32;
   p.status = status_dev;
-  // An ordinary launch, not a programmatic dependent of the kernel above: the set-up reads what that one writes.
+  // An ordinary launch, not a programmatic dependent of the kernel above: the weight producer does not wait for that one.
   static unsigned long long done = 0;
   e = allow_max_smem(tcg_conv_kernel<M_FP4, OUT_WORDS>, &done);
   if (e != cudaSuccess) return e;
