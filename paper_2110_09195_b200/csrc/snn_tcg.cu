@@ -540,14 +540,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         } else {
           uint32_t* const obase = out32 + (size_t)((uint32_t)(g_lane * K + co));
           // (a last slice of 16 columns is read as 32: the others belong to the next buffer or the scales and go nowhere)
-          uint32_t v[32];
-          __syncwarp();
-          tmem_ld32(d0 + (uint32_t)(32 * half), v);
 #pragma unroll 1
           for (int s = half; s < n_slices; s += 2) {   // the two warps of a lane quarter take the slices in turn
-            const bool last = s + 2 >= n_slices;
-            tmem_ld_wait();
-            if (last) release();
+            uint32_t v[32];
+            __syncwarp();   // the load is a warp-wide instruction
+            tmem_ld32(d0 + (uint32_t)(32 * s), v);
+            if (s + 2 >= n_slices) release();
             if (WORDS || out_kind != 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
               // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubled the code, and the
@@ -570,8 +568,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                                "r"(v[e + j]), "r"(mask & (1u << (e + j)))
                                : "memory");
               }
-              __syncwarp();   // the load is a warp-wide instruction
-              if (!last) tmem_ld32(d0 + (uint32_t)(32 * s + 64), v);
             } else {
               // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): bit of a channel =
               // fl(fl(alpha*S) + shift) >= 0 = sign bit clear (no sum is -0 or NaN: alpha and shift are finite and
@@ -596,8 +592,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                   part[c] = __funnelshift_l(y0, part[c], 1);
                 }
               }
-              __syncwarp();
-              if (!last) tmem_ld32(d0 + (uint32_t)(32 * s + 64), v);   // beside the transposition and the store
               uint32_t w = part[0] | (part[1] << 8) | (part[2] << 16) | (part[3] << 24);
               w = co < K ? ~w : 0u;   // bits of channels that do not exist are 0
               w = g_transpose32(w, lane);
