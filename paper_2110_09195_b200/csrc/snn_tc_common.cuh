@@ -1,5 +1,5 @@
 // Device and host helpers of the tensor-core kernel: PTX wrappers for mbarriers,
-// bulk copies and tcgen05, bit -> e2m1 expansion, exact division by run-time constants.
+// bulk copies and tcgen05, bit -> e2m1 expansion.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -12,26 +12,6 @@ namespace snn {
 namespace {
 
 constexpr uint32_t WAIT_LIMIT = 1u << 20;  // try_wait attempts before a wait gives up
-
-// Division by a run-time constant as multiply-high + shifts (round-up method,
-// exact for every 32-bit numerator).
-struct FastDiv {
-  uint32_t d, m, s;
-};
-FastDiv make_fastdiv(uint32_t d) {
-  FastDiv f;
-  f.d = d;
-  uint32_t s = 0;
-  while ((1ull << s) < d) ++s;
-  f.s = s;
-  f.m = d == 1 ? 0u : (uint32_t)((((1ull << s) - d) << 32) / d + 1);
-  return f;
-}
-__device__ __forceinline__ uint32_t fdiv(uint32_t q, const FastDiv& f) {
-  if (f.d == 1) return q;
-  const uint32_t t = __umulhi(f.m, q);
-  return (t + ((q - t) >> 1)) >> (f.s - 1);
-}
 
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -197,7 +177,6 @@ __device__ __forceinline__ uint4 expand_word_fp4(uint32_t bits, uint32_t sign, u
 // 32 x 32 -> 64-bit product in one instruction (element offsets of pixels: both factors are non-negative 32-bit)
 __device__ __forceinline__ size_t wide_mul(uint32_t a, uint32_t b) { return (size_t)a * (size_t)b; }
 
-static inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 static inline int sm_count() {
   static int sms = 0;

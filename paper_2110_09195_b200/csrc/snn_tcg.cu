@@ -65,93 +65,11 @@
 #include <cuda.h>   // tensor maps (types only; the encoder is looked up at run time)
 
 #include "snn_tc_common.cuh"
+#include "snn_tc_plan.h"
 
 namespace snn {
 
 namespace {
-
-// Operand modes of the kernel.  Binary activations run on 4-bit e2m1 operands (+1 / -1 / 0 are exact, the
-// block scales are all 1, and the fp32 accumulators hold the exact integer sums: |S| <= 9 * c_in < 2^24);
-// an MMA then covers 64 input channels in the time an 8-bit MMA covers 32.  fp16 activations run on fp16
-// operands.  Both accumulate in fp32.
-enum { M_F16 = 1, M_FP4 = 2 };
-constexpr int G_EW = 8;                       // epilogue warps = expander warps
-
-// Warps 13 and 17 do not expand: a warp's scheduler is warp % 4, and the MMA-issuing warp (1) then shares its
-// scheduler with two epilogue warps and the table warp (13, which has little to do) instead of two expander warps.
-constexpr int G_THREADS = 64 + 64 * G_EW + 64;
-constexpr int G_EXP_THREADS = 32 * G_EW;
-constexpr int G_XTEAMS = 2;                    // teams of expander warps (4-bit operands)
-constexpr int G_EXP_ITEMS = 4;                 // loads one expander thread has in flight together
-constexpr int G_ROWS = 128;                    // rows of the weight operand: lanes of an accumulator
-constexpr int G_MAX_CHUNKS = 8;                // 32-column slices of an accumulator (at most 256 columns)
-// What the epilogue needs to know of a tile, written by the table warp (see there), four tiles deep.
-struct GTile {
-  int l, mg, co, n_slices;             // problem (-1: no more tiles), position tile, first channel, 32-column slices
-  int K, kp_log, Np, out_kind;         // channels; logarithm of the rows per pixel; positions; 0 fp32, 1 int32, 2 packed signs
-  uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
-  uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
-  float alpha[G_ROWS], shift[G_ROWS];
-};
-constexpr int G_TILES = 4;
-constexpr int G_EPI_BYTES = G_TILES * (int)sizeof(GTile);
-constexpr int G_NS_MAX = 8;
-constexpr uint32_t G_TMEM_FP4 = 480;          // 4-bit mode: columns 480..511 hold the (unit) block scales
-constexpr uint32_t G_TMEM_F16 = 512;
-constexpr uint32_t G_SCALE_COL = 480;
-constexpr size_t kGTail = 512;
-constexpr size_t kGSmemBudget = 226 * 1024;
-constexpr uint32_t kGASlotMax = 44 * 1024;         // largest activation unit a problem may stage
-constexpr uint32_t kGASlotMaxTma = 60 * 1024;      // ... when it is fetched by TMA (fp16; whole rows of positions)
-constexpr int kGRowsMax = 1600;                    // ... and its most rows (the pixel tables hold one word per row)
-constexpr uint32_t kGBSlot = 32 * 1024, kGBSlotF16 = 16 * 1024;   // bytes of a weight-stage slot
-constexpr int kGTapsMax = 52;                      // 3 kernel rows x at most 17 columns of a group of 8 pixels
-
-// One problem of a launch, as the kernel reads it from shared memory.
-struct GLayer {
-  const uint8_t* wt;      // [channel tile][channel block][step][chunk][128][16 B], owned by the group
-  const float* alpha;
-  const float* shift;     // per-channel constant added to alpha*S before the sign is taken (packed-sign output)
-  int N, H, W, C, K, Cw, pad, Ho, Wo;
-  int rs, cm, cs;         // input pixel of position (i, j) in plane (pr, pc): row rs*i + pr - pad, column cm*j + cs*pc - pad
-  int G, lg;              // output pixels per position and its logarithm
-  int Hq, Wg;             // rows per image / positions per row of the flattened position space
-  FastDiv dWg, dHq, dCt, dRr;
-  int n_planes, cpl;      // planes of a unit, logarithm of the number of column planes
-  int Np, Rr;             // positions per tile; staged rows per plane = Np + largest tap shift
-  int cb_chunks, n_cb, kpt;
-  int tma;                // fp16: units are fetched by TMA, rows of 64 channels in the 128-byte swizzle
-  int n_pu, pu_end[4];    // units per channel block (fetched by TMA, each plane is a unit of its own) and the last step of each
-  int steps;              // taps of a tile, or pairs of taps (one activation word per pixel: a K = 64 step covers two taps)
-  int st_steps;           // steps per weight stage (the last stage of a channel block holds steps % st_steps, if not 0)
-  uint32_t step_bytes;    // weights of one step of one channel block = kpt * 2 * 128 * 16
-  int n_ct, total_tiles;  // channel tiles of 128
-  int first;              // this CTA's first tile, filled in by the kernel (GParams::ranks)
-  uint32_t Qtot;
-  // A chain (every member reads the packed signs its predecessor writes, all in one launch): a tile may be
-  // staged once the predecessor's tiles that hold its input pixels are complete, and says so itself when done.
-  const uint2* deps;          // [position tiles] first and last position tile of the predecessor this one reads (x > y: none)
-  const uint32_t* prev_done;  // the predecessor's completion counters, and the count that means "complete"
-  uint32_t prev_target;
-  uint32_t* done;             // [position tiles] epilogue warps that have written their part, over all its channel tiles
-  uint32_t tap[kGTapsMax];    // per step: start of its rows in the unit (16-byte units) | distance of its two chunks << 16
-};
-
-struct GParams {
-  const GLayer* layers;
-  const uint16_t* ranks;  // [n_layers][grid] CTA b takes a problem's tiles ranks[b], ranks[b] + grid, ...
-  int n_layers;
-  const void* act[SNN_GROUP_MAX];
-  void* out[SNN_GROUP_MAX];
-  int* status;
-  uint8_t out_type[SNN_GROUP_MAX];   // per member: 0 fp32 alpha*S, 1 int32 S, 2 packed signs of alpha*S + shift
-  uint32_t acc_cols;      // tensor-memory columns of one accumulator buffer
-  int n_acc;              // accumulator buffers (tile seq of a CTA uses buffer seq % n_acc)
-  int NA, NS;
-  uint32_t a_slot_bytes, b_slot_bytes;
-  uint32_t off_b, off_epi, off_pix, off_lay, off_tail;
-  GLayer one;             // n_layers == 1: the problem itself (layers and ranks are not read: its tiles go to the CTAs in order)
-};
 
 // Profiling aid (build with -DSNN_TRACE): every role's reporting lane adds up the cycles it spends in its
 // waits; the host prints the averages over the CTAs after each launch.  No effect on an ordinary build.
@@ -168,11 +86,10 @@ __device__ long long g_trace[256 * 16];
 #define TR_REPORT(role, total, w0, w1, w2) do { } while (0)
 #endif
 
-// input pixel of row q (a position, possibly past a tile's own) in plane pl, or -1: padding or past the batch
-__host__ __device__ __forceinline__ int g_pixel_of(const GLayer& L, uint32_t n, int i, int j, int pl) {
-  const int r = L.rs * i + (pl >> L.cpl) - L.pad, c = L.cm * j + L.cs * (pl & ((1 << L.cpl) - 1)) - L.pad;
-  if (r < 0 || r >= L.H || c < 0 || c >= L.W) return -1;
-  return ((int)n * L.H + r) * L.W + c;
+__device__ __forceinline__ uint32_t fdiv(uint32_t q, const FastDiv& f) {
+  if (f.d == 1) return q;
+  const uint32_t t = __umulhi(f.m, q);
+  return (t + ((q - t) >> 1)) >> (f.s - 1);
 }
 __device__ __forceinline__ int g_position_to_pixel(const GLayer& L, uint32_t q, int pl) {
   if (q >= L.Qtot) return -1;
@@ -210,12 +127,6 @@ __device__ __forceinline__ uint2 g_ld2(const uint32_t* p, bool fresh) {
 __device__ __forceinline__ uint4 g_ld4(const uint32_t* p, bool fresh) {
   return fresh ? __ldcg(reinterpret_cast<const uint4*>(p)) : __ldg(reinterpret_cast<const uint4*>(p));
 }
-// Words of a row that are loaded together: activations are 16-byte aligned, so a row can be read four (two) words
-// at a time where the words per pixel and per channel block are multiples of four (two).
-__host__ __device__ __forceinline__ int g_word_step(int Cw, int cb_chunks) {
-  return (Cw & 3) == 0 && (cb_chunks & 3) == 0 ? 4 : (Cw & 1) == 0 && (cb_chunks & 1) == 0 ? 2 : 1;
-}
-
 // Tensor maps of the fp16 activations, a kernel parameter of its own (the other variants have one unused entry).
 template <int MODE>
 struct GMaps {
@@ -1125,12 +1036,6 @@ MapEncoder g_map_encoder() {
   return f;
 }
 
-// Which tap each step of a layer applies, for the weight operand: per chunk of a step the kernel row and the column
-// s of the group's window (kernel column s - stride*g for pixel g), 255: none.  Steps of single taps name one tap twice.
-struct GTaps {
-  uint8_t row[kGTapsMax][2], col[kGTapsMax][2];
-};
-
 // Operand of the weights: wt[channel tile][channel block][step][chunk][128][16 B]; a chunk is 16 bytes along the
 // input channels (8 fp16 or 32 e2m1 values), cb_chunks chunks per block.  Row r of a tile is channel r % (128/G) of
 // pixel r / (128/G).  Channels that do not exist, and columns outside a pixel's window, are zeros, so whatever the
@@ -1174,324 +1079,6 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
   reinterpret_cast<uint4*>(wt)[i] = v;
 }
 
-inline int g_mode_for(int act_type) { return act_type == SNN_ACT_F16 ? M_F16 : M_FP4; }
-
-// A planned layer and the planner's estimate of one tile, in SM cycles.
-struct GPlan {
-  GLayer L;
-  GTaps taps;
-  int paired = 0;
-  size_t w_bytes = 0, unit_bytes = 0;
-  double mma = 0, weights = 0, expand = 0, drain = 0;
-  double through() const {   // a tile among others: the slowest role
-    double t = mma;
-    if (weights > t) t = weights;
-    if (expand > t) t = expand;
-    if (drain > t) t = drain;
-    return t + 300.0;
-  }
-  double alone() const { return expand + (mma > weights ? mma : weights) + drain + 1500.0; }   // a tile by itself
-};
-
-// The plan of one layer with tiles of Np positions of 2^lg pixels; false where that does not fit.
-bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, GPlan* P) {
-  GLayer& o = P->L;
-  o.wt = nullptr; o.alpha = o.shift = nullptr; o.deps = nullptr; o.prev_done = nullptr; o.prev_target = 0; o.done = nullptr;
-  o.first = 0;
-  const int cpc = mode == M_F16 ? 8 : 32;
-  const int S = g.stride, G = 1 << lg;
-  const bool one = g.ksize == 1;
-  o.N = g.N; o.H = g.H; o.W = g.W; o.C = g.C; o.K = g.K; o.Cw = g.Cw;
-  o.pad = g.pad; o.Ho = g.Ho; o.Wo = g.Wo; o.G = G; o.lg = lg; o.Np = Np;
-  if (lg && (mode != M_FP4 || g.K > G_ROWS >> lg)) return false;
-  o.rs = S;
-  o.cs = one ? S : 1;
-  o.cm = S * G;
-  int row_planes = 1, col_planes = G;
-  if (one) {
-    // 1x1 layer: the positions are (groups of) the output pixels themselves, no halo
-    o.Hq = g.Ho;
-    o.Wg = (g.Wo + G - 1) / G;
-  } else {
-    // one zero column per image row and one zero row per image are shared by neighbours; stride 2 splits the input
-    // into its row and column parity planes, in each of which the taps are plain shifts
-    row_planes = S;
-    col_planes = S * G;
-    o.Hq = S == 1 ? g.H + g.pad : g.Ho + 1;
-    o.Wg = ((S == 1 ? g.W + g.pad : g.Wo + 1) + G - 1) / G;
-  }
-  o.n_planes = row_planes * col_planes;
-  o.cpl = 0;
-  while ((1 << o.cpl) < col_planes) ++o.cpl;
-  const long long Q = (long long)g.N * o.Hq * o.Wg;
-  const int span = one ? S * (G - 1) + 1 : S * (G - 1) + 3;   // columns of a group's window, in input pixels
-  const int halo = one ? 0 : (2 / S) * o.Wg + (span - 1) / col_planes;
-  if (Q + 1024 + halo >= (1ll << 31)) return false;
-  o.Qtot = (uint32_t)Q;
-  o.Rr = Np + halo;
-  // fp16 units are fetched by TMA where the rows of the tensor are multiples of 16 bytes and a row of positions fits a box
-  o.tma = tma && mode == M_F16 && (g.C & 7) == 0 && o.Wg * S <= 256;
-  const int tma_rows = (2 * o.Wg + o.Rr - 2) / o.Wg;   // rows of positions a tile can touch
-  if (mode == M_F16 && !o.tma) o.Rr |= 1;   // odd: the chunks of a row are copied together, into different banks
-  if (!o.tma && (long long)o.n_planes * o.Rr > kGRowsMax) return false;
-  P->paired = mode == M_FP4 && g.Cw == 1;
-  int d = 0;
-  if (o.tma) {
-    // 64 channels (fewer where there are no more); every plane is a unit of its own
-    P->unit_bytes = (size_t)tma_rows * o.Wg * 128;
-    if (P->unit_bytes > kGASlotMaxTma) return false;
-    o.n_cb = (g.C + 63) / 64;
-    d = o.n_cb > 1 ? 8 : round_up(g.C, 16) / 8;
-    o.cb_chunks = d;
-    o.kpt = d / 2;
-    o.n_pu = o.n_planes;
-  } else {
-    // channel block: the largest of 8/6/4/2 chunks that divides the channels and whose unit fits a slot; one chunk where
-    // there is one activation word per pixel: a K = 64 step then covers two taps, one per chunk
-    const int raw = P->paired ? 1 : round_up(g.C, 2 * cpc) / cpc;  // 16-byte chunks along the channels, even
-    for (int c = P->paired ? 1 : 8; c >= 1; c -= 2) {
-      if (raw % c) continue;
-      if ((size_t)o.n_planes * c * o.Rr * 16 <= kGASlotMax) { d = c; break; }
-    }
-    if (!d) return false;
-    o.cb_chunks = d;
-    o.n_cb = raw / d;
-    o.kpt = P->paired ? 1 : d / 2;
-    o.n_pu = 1;
-    P->unit_bytes = (size_t)o.n_planes * d * o.Rr * 16;
-  }
-  const int taps = one ? G : 3 * span;
-  o.steps = P->paired ? (taps + 1) / 2 : taps;
-  if (o.steps >= kGTapsMax) return false;
-  const uint32_t reach = o.tma ? 8u * (uint32_t)halo : (uint32_t)(o.n_planes * o.Rr);   // largest start of a tap, and chunk distance
-  if (reach > 0xffffu || (!o.tma && reach >= (1u << 14))) return false;                 // (the leading-offset field has 14 bits)
-  o.n_ct = lg ? 1 : (g.K + G_ROWS - 1) / G_ROWS;
-  const long long tiles = (Q + Np - 1) / Np * o.n_ct;
-  if (tiles > 0x7fffffffLL || (Q + Np - 1) / Np * o.Rr >= (1ll << 31)) return false;
-  o.total_tiles = (int)tiles;
-  // weight stage: as many whole steps of a channel block as fit a slot
-  o.step_bytes = (uint32_t)(o.kpt * 2 * G_ROWS * 16);
-  o.st_steps = (int)((mode == M_F16 ? kGBSlotF16 : kGBSlot) / o.step_bytes);
-  if (o.st_steps > o.steps) o.st_steps = o.steps;
-  P->w_bytes = (size_t)o.n_ct * o.n_cb * o.steps * o.step_bytes;
-  // One MMA reads 32 + Np/4 shared-memory lines and takes at least Np/2 cycles (measured).  The other figures are the
-  // rates the roles reach in the traces: bulk copies of weights 64 bytes per cycle, a 16-byte chunk of activations
-  // in 0.6 cycles (0.4 copied) plus the latency of the loads, stores 16 bytes per cycle.
-  const double mmas = (double)o.n_cb * o.steps * o.kpt;
-  const double lines = mmas * (32 + Np / 4) + (double)o.n_cb * (o.steps * o.step_bytes + (double)o.n_pu * P->unit_bytes) / 128.0;
-  P->mma = std::max(mmas * (Np / 2), 1.1 * lines);
-  P->weights = (double)o.n_cb * o.steps * o.step_bytes / 64.0;
-  P->expand = o.tma ? o.n_cb * o.n_pu * (P->unit_bytes / 40.0) + 1000.0 : o.n_cb * ((double)o.n_planes * o.Rr * d * (mode == M_F16 ? 3.0 : 0.6) + 500.0);
-  const int k_tile = g.K < G_ROWS ? g.K : G_ROWS;
-  P->drain = kind == TCG_WORDS ? (double)Np * G * k_tile * 4 / 16.0 : Np * 5.0;
-  return true;
-}
-
-// The rest of a chosen plan: division constants, and where each step's rows start in the unit.
-void g_finish_plan(const Geom& g, GPlan* P) {
-  GLayer& o = P->L;
-  o.dWg = make_fastdiv((uint32_t)o.Wg);
-  o.dHq = make_fastdiv((uint32_t)o.Hq);
-  o.dCt = make_fastdiv((uint32_t)o.n_ct);
-  o.dRr = make_fastdiv((uint32_t)o.Rr);
-  const int S = g.stride, col_planes = 1 << o.cpl, span = S * (o.G - 1) + 3;
-  // taps in ascending order of where their rows start in the unit
-  struct Tap { int plane; uint32_t at; uint8_t row, col; } taps[64];
-  int n = 0;
-  if (g.ksize == 1) {
-    for (int q = 0; q < o.G; ++q) taps[n++] = {q, 0, 0, (uint8_t)(S * q)};
-  } else {
-    for (int ky = 0; ky < 3; ++ky)
-      for (int s = 0; s < span; ++s)
-        taps[n++] = {(ky % S) * col_planes + s % col_planes, (uint32_t)((ky / S) * o.Wg + s / col_planes), (uint8_t)ky, (uint8_t)s};
-  }
-  for (int t = 0; t < n; ++t) taps[t].at = o.tma ? taps[t].at * 8 : taps[t].at + (uint32_t)(taps[t].plane * o.Rr);
-  std::sort(taps, taps + n, [](const Tap& a, const Tap& b) { return a.plane != b.plane ? a.plane < b.plane : a.at < b.at; });
-  for (int t = 0; t < o.steps; ++t) {
-    const Tap& a = taps[P->paired ? 2 * t : t];
-    const bool second = P->paired && 2 * t + 1 < n;
-    const Tap& b = second ? taps[2 * t + 1] : a;
-    const uint32_t dist = P->paired ? b.at - a.at : o.tma ? 1u : (uint32_t)(o.n_planes * o.Rr);
-    o.tap[t] = a.at | (dist << 16);
-    P->taps.row[t][0] = a.row; P->taps.col[t][0] = a.col;
-    P->taps.row[t][1] = P->paired && !second ? 255 : b.row;
-    P->taps.col[t][1] = b.col;
-  }
-  for (int u = 0; u < 4; ++u) o.pu_end[u] = o.steps;
-  if (o.n_pu > 1)
-    for (int u = 0, t = 0; u < o.n_pu; ++u) {
-      while (t < n && taps[t].plane == u) ++t;
-      o.pu_end[u] = t;
-    }
-}
-
-// Does the tensor-core path take this layer?  The bound is that of a unit of 128 positions with its halo (row pitch of
-// the padded map) in a 40.5 KB slot, two of which fit beside the weight ring; shapes beyond it go to the other paths.
-// The tiles themselves are planned by g_plan_layer, which needs less.
-bool g_path_takes(const Geom& g, int mode) {
-  constexpr size_t slot_max = 40 * 1024 + 512, b_slot = 32 * 1024, epi = 40 * 1024, budget = 226 * 1024;
-  if (g.N < 1 || g.C > (1 << 20)) return false;            // 9 * c_in stays far below 2^24: exact fp32 sums
-  if ((long long)g.N * g.H * g.W >= (1ll << 31) || (long long)g.N * g.Ho * g.Wo >= (1ll << 31)) return false;
-  if ((long long)g.N * g.Ho * g.Wo * g.K >= 0xffffffffLL) return false;   // output element offsets are 32-bit
-  const int cpc = mode == M_F16 ? 8 : 32, raw = round_up(g.C, 2 * cpc) / cpc;
-  const bool one = g.ksize == 1;
-  const int Hq = one ? g.Ho : g.stride == 1 ? g.H + g.pad : g.Ho + 1;
-  const int Wq = one ? g.Wo : g.stride == 1 ? g.W + g.pad : g.Wo + 1;
-  const int planes = one || g.stride == 1 ? 1 : 4;
-  const int halo = one ? 0 : g.stride == 1 ? 2 * Wq + 2 : Wq + 1;
-  const long long Q = (long long)g.N * Hq * Wq;
-  if (Q + 1024 + halo >= (1ll << 31)) return false;
-  int d = 0;
-  for (int c = 8; c >= 2 && !d; c -= 2)
-    if (raw % c == 0 && (size_t)planes * c * (128 + halo) * 16 <= slot_max) d = c;
-  if (!d) return false;
-  for (int n_acc = 2; n_acc <= (mode == M_FP4 ? 3 : 2); ++n_acc) {
-    const int cols = mode == M_F16 ? 256 : n_acc == 3 ? 160 : 240;
-    const int nt = mode == M_FP4 ? (g.K <= cols ? round_up(g.K, 16) : 128)
-                                 : (g.K <= 256 ? round_up(g.K, 16) : (round_up(g.K, 256) - g.K < 64 ? 256 : 128));
-    const long long mtiles = (Q + 127) / 128;
-    int mt = 1;
-    for (int m = 4; m >= 2 && mt == 1; --m)
-      if ((size_t)planes * d * (128 * m + halo) * 16 <= slot_max && m * nt <= cols) mt = m;
-    while (mt > 1 && mtiles < mt) --mt;
-    const int rows = 128 * mt + halo;
-    const long long groups = (mtiles + mt - 1) / mt;
-    if ((uint32_t)rows * 16 >= (1u << 18)) return false;
-    if (groups * ((g.K + nt - 1) / nt) > 0x7fffffffLL || groups * rows >= (1ll << 31)) return false;
-    const size_t unit = (((size_t)planes * d * rows * 16) + 127) & ~(size_t)127;
-    const size_t pix = (((size_t)planes * rows * 4) + 127) & ~(size_t)127;
-    if (2 * unit + epi + 2 * pix + 256 + kGTail + 3 * b_slot > budget) return false;
-  }
-  return true;
-}
-
-// Tile sizes the planner chooses from (positions; multiples of 16).
-constexpr int kNpTable[] = {256, 240, 208, 192, 160, 144, 128, 112, 96, 80, 64, 48, 32, 16};
-
-// A tile size under consideration: what has to be planned, and the estimates the choice is made by.
-struct GChoice {
-  int lg = 0, Np = 0, tiles = 0;
-  bool tma = false;
-  double through = 0, alone = 0;
-};
-
-// Best choice for one layer and tiles of at most `cap` positions: the group size 2^lg with the least time over all its tiles.
-bool g_best_group(const Geom& g, int mode, int kind, int cap, bool tma, GChoice* out) {
-  bool found = false;
-  double best = 0;
-  GPlan P;
-  for (int lg = 0; lg <= 3; ++lg) {
-    if (lg && (mode != M_FP4 || g.K > G_ROWS >> lg)) break;
-    for (int Np : kNpTable) {
-      if (Np > cap) continue;
-      if (!g_plan_layer(g, mode, kind, lg, Np, tma, &P) && !(tma && g_plan_layer(g, mode, kind, lg, Np, false, &P))) continue;
-      const double t = P.L.total_tiles * P.through();
-      if (!found || t < best) {
-        best = t;
-        *out = {lg, Np, P.L.total_tiles, P.L.tma != 0, P.through(), P.alone()};
-        found = true;
-      }
-      break;   // the largest that fits
-    }
-  }
-  return found;
-}
-
-// The ring geometry of a launch of these problems and where its parts lie in shared memory; false where it does not fit.
-bool g_ring(const GPlan* plan, int count, int mode, GParams* p, size_t* smem) {
-  const uint32_t tmem = mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16;
-  size_t a_slot = 0, pix_bytes = 0;
-  int widest = 16;
-  for (int i = 0; i < count; ++i) {
-    const GLayer& o = plan[i].L;
-    a_slot = std::max(a_slot, plan[i].unit_bytes);
-    if (mode == M_F16 && !o.tma) pix_bytes = std::max(pix_bytes, (size_t)o.n_planes * o.Rr * 4);
-    widest = std::max(widest, o.Np);
-  }
-  // accumulator buffers: as many as fit, up to four
-  int n_acc = (int)tmem / widest;
-  if (n_acc > 4) n_acc = 4;
-  a_slot = (a_slot + 1023) & ~(size_t)1023;   // (the swizzle of the TMA units repeats every 1024 bytes)
-  const uint32_t b_slot = mode == M_F16 ? kGBSlotF16 : kGBSlot;
-  pix_bytes = (pix_bytes + 127) & ~(size_t)127;
-  const size_t lay_bytes = ((size_t)count * sizeof(GLayer) + 127) & ~(size_t)127;
-  const size_t fixed = (size_t)G_EPI_BYTES + pix_bytes + lay_bytes + kGTail;
-  // Ring depths: four activation slots if they fit beside four weight slots, else two (with the 4-bit expanders a
-  // multiple of the number of teams) or three; the weights take what is left.
-  static_assert(G_XTEAMS == 1 || G_XTEAMS == 2, "the ring depths below are multiples of the team count");
-  int na = 4, ns = 0;
-  for (; na >= 2; --na) {
-    if (mode == M_FP4 && na % G_XTEAMS) continue;
-    const int ns_min = mode == M_F16 ? 4 : na > 2 ? 4 : 3;
-    if ((size_t)na * a_slot + fixed + ns_min * (size_t)b_slot > kGSmemBudget) continue;
-    ns = (int)((kGSmemBudget - fixed - (size_t)na * a_slot) / b_slot);
-    break;
-  }
-  if (na < 2 || ns < 3) return false;
-  if (ns > G_NS_MAX) ns = G_NS_MAX;
-  p->n_layers = count;
-  p->NA = na;
-  p->NS = ns;
-  p->acc_cols = (tmem / (uint32_t)n_acc) & ~15u;
-  p->n_acc = n_acc;
-  p->a_slot_bytes = (uint32_t)a_slot;
-  p->b_slot_bytes = b_slot;
-  p->off_b = (uint32_t)((size_t)na * a_slot);
-  p->off_epi = p->off_b + (uint32_t)ns * b_slot;
-  p->off_pix = p->off_epi + G_EPI_BYTES;
-  p->off_lay = p->off_pix + (uint32_t)pix_bytes;
-  p->off_tail = p->off_lay + (uint32_t)lay_bytes;
-  *smem = (size_t)p->off_tail + kGTail;
-  return *smem <= (size_t)kMaxDynSmem && *smem < (1u << 18);
-}
-
-// Tiles of independent problems: one size limit for all of them, by the estimated time of the launch.
-bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma, int sms, GPlan* plan) {
-  GChoice trial[SNN_GROUP_MAX], chosen[SNN_GROUP_MAX];
-  double best = -1;
-  for (int cap : kNpTable) {
-    if (cap > (int)(mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16) / 2) continue;
-    bool ok = true;
-    for (int i = 0; i < count && ok; ++i) ok = g_best_group(gs[i], mode, kind, cap, tma, &trial[i]);
-    if (!ok) continue;
-    // the machine's share of all tiles (whole tiles where there is one problem), and the last tile's way through the roles
-    double sum = 0, last = 0, slowest = 0;
-    for (int i = 0; i < count; ++i) {
-      const GChoice& c = trial[i];
-      sum += count == 1 ? (double)((c.tiles + sms - 1) / sms) * sms * c.through : c.tiles * c.through;
-      last = std::max(last, c.alone - c.through);
-      slowest = std::max(slowest, c.through);
-    }
-    const double t = std::max(sum / sms, slowest) + last + (count > 1 ? slowest / 2 : 0);
-    if (best < 0 || t < best) {
-      best = t;
-      std::copy(trial, trial + count, chosen);
-    }
-  }
-  if (best < 0) return false;
-  for (int i = 0; i < count; ++i) g_plan_layer(gs[i], mode, kind, chosen[i].lg, chosen[i].Np, chosen[i].tma, &plan[i]);
-  return true;
-}
-
-// Which CTAs take a problem's odd tiles.  Every CTA gets floor(tiles / grid) tiles of a problem
-// and the first (tiles % grid) CTAs in the problem's rank order get one more; the rank order is
-// by the time the CTAs have been given so far, least first, so that the CTAs end close
-// together although a tile of one problem may take six times as long as a tile of another.
-void g_assign(const std::vector<GPlan>& P, int grid, std::vector<uint16_t>* ranks) {
-  std::vector<double> busy(grid, 0.0);
-  std::vector<int> order(grid);
-  for (size_t i = 0; i < P.size(); ++i) {
-    const double cost = P[i].through();
-    for (int b = 0; b < grid; ++b) order[b] = b;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return busy[a] < busy[b]; });
-    const int base = P[i].L.total_tiles / grid, rem = P[i].L.total_tiles % grid;
-    for (int r = 0; r < grid; ++r) {
-      (*ranks)[i * grid + order[r]] = (uint16_t)r;
-      busy[order[r]] += cost * (base + (r < rem ? 1 : 0));
-    }
-  }
-}
-
 }  // namespace
 
 cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int act_type, int kind, cudaStream_t s,
@@ -1504,32 +1091,14 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   for (int i = 0; i < count; ++i)
     if (!g_path_takes(gs[i], mode)) return cudaErrorInvalidConfiguration;
   const int sms = sm_count();
-  const int cap_max = (int)G_TMEM_FP4 / 2;   // (a chain has binary activations)
   const bool tma = mode == M_F16 && g_map_encoder() != nullptr;
   // Tile sizes.  A chain's members run one after the other as far as their inputs go, so each takes the size that makes
   // its own tiles end first; the members of a group share the machine, and one size limit for all of them is chosen by
   // the time of the busiest CTA.
   std::vector<GPlan> plan(count);
-  if (chain) {
-    for (int i = 0; i < count; ++i) {
-      double best = -1;
-      int best_lg = 0, best_np = 0;
-      GPlan P;
-      for (int Np : kNpTable) {
-        if (Np > cap_max) continue;
-        for (int lg = 0; lg <= 3; ++lg) {
-          if (!g_plan_layer(gs[i], mode, kind, lg, Np, false, &P)) continue;
-          const int waves = (P.L.total_tiles + sms - 1) / sms;
-          const double t = P.alone() + (waves - 1) * P.through();
-          if (best < 0 || t < best) { best = t; best_lg = lg; best_np = Np; }
-        }
-      }
-      if (best < 0) return cudaErrorInvalidConfiguration;
-      g_plan_layer(gs[i], mode, kind, best_lg, best_np, false, &plan[i]);
-    }
-  } else if (!g_plan_independent(gs, count, mode, kind, tma, sms, plan.data())) {
-    return cudaErrorInvalidConfiguration;
-  }
+  for (int i = 0; i < count && chain; ++i)
+    if (!g_plan_by_end(gs[i], mode, kind, sms, &plan[i])) return cudaErrorInvalidConfiguration;
+  if (!chain && !g_plan_independent(gs, count, mode, kind, tma, sms, plan.data())) return cudaErrorInvalidConfiguration;
   for (int i = 0; i < count; ++i) g_finish_plan(gs[i], &plan[i]);
   GParams ring{};
   size_t smem = 0;

@@ -1,0 +1,81 @@
+// The planner of the tensor-core kernel for tests/test_plan.py: host code, no GPU.
+#include <cstring>
+
+#include "snn_tc_plan.h"
+
+using namespace snn;
+
+namespace {
+
+Geom geom(const int* v) {   // N, H, W, C, K, stride, pad, ksize
+  Geom g;
+  g.N = v[0]; g.H = v[1]; g.W = v[2]; g.C = v[3]; g.K = v[4]; g.stride = v[5]; g.pad = v[6]; g.ksize = v[7];
+  g.Cw = (g.C + 31) / 32;
+  g.Ho = (g.H + 2 * g.pad - g.ksize) / g.stride + 1;
+  g.Wo = (g.W + 2 * g.pad - g.ksize) / g.stride + 1;
+  g.tau = 5; g.T = 32;
+  return g;
+}
+
+// Everything the kernel's index arithmetic relies on.
+const char* wrong(const GPlan* plan, int count, int mode, const GParams& p, size_t smem) {
+  if (smem > (size_t)kMaxDynSmem) return "shared memory";
+  if (p.NA < 2 || p.NA > 4 || p.NS < 3 || p.NS > G_NS_MAX) return "ring depths";
+  if (mode == M_FP4 && p.NA % G_XTEAMS) return "activation slots are no multiple of the teams";
+  const uint32_t tmem = mode == M_FP4 ? G_TMEM_FP4 : G_TMEM_F16;
+  if (p.n_acc < 2 || p.n_acc > 4 || p.n_acc * p.acc_cols > tmem) return "accumulators";
+  for (int i = 0; i < count; ++i) {
+    const GLayer& o = plan[i].L;
+    if (o.Np < 16 || o.Np % 16 || (uint32_t)o.Np > p.acc_cols) return "tile width";
+    // slices of 32 columns are read whole
+    if ((p.n_acc - 1) * p.acc_cols + ((o.Np + 31) / 32) * 32 > 512 || (o.Np + 31) / 32 > G_MAX_CHUNKS) return "slices";
+    if (o.steps < 1 || o.steps >= kGTapsMax || o.st_steps < 1) return "steps";
+    if (o.st_steps * o.step_bytes > p.b_slot_bytes) return "weight stage";
+    if (plan[i].w_bytes != (size_t)o.n_ct * o.n_cb * o.steps * o.step_bytes) return "weight operand";
+    if (plan[i].unit_bytes > p.a_slot_bytes) return "activation unit";
+    const int units = o.tma ? o.n_pu : 1;
+    for (int t = 0; t < o.steps; ++t) {
+      const uint32_t at = o.tap[t] & 0xffffu, dist = o.tap[t] >> 16;
+      size_t end;   // in 16-byte units of the slot
+      if (o.tma)    // rows of 128 bytes; the first row of a tile is any of a row of positions
+        end = (size_t)8 * (o.Wg - 1) + at + (size_t)8 * o.Np;
+      else
+        end = (size_t)at + dist + (size_t)(o.kpt - 1) * 2 * o.n_planes * o.Rr + o.Np;
+      if (end * 16 > plan[i].unit_bytes) return "operand past the unit";
+    }
+    if (o.pu_end[units - 1] != o.steps) return "units";
+  }
+  return nullptr;
+}
+
+}  // namespace
+
+extern "C" {
+
+int plan_takes(const int* g, int f16) { return g_path_takes(geom(g), f16 ? M_F16 : M_FP4); }
+
+// out per problem: lg, Np, tma, tiles.  Returns what is wrong with the plan, or null.
+const char* plan_make(const int* gs, int count, int f16, int kind, int sms, int* out) {
+  const int mode = f16 ? M_F16 : M_FP4;
+  std::vector<Geom> g(count);
+  std::vector<GPlan> plan(count);
+  for (int i = 0; i < count; ++i) g[i] = geom(gs + 8 * i);
+  if (kind == TCG_CHAIN) {
+    for (int i = 0; i < count; ++i)
+      if (!g_plan_by_end(g[i], mode, kind, sms, &plan[i])) return "no plan";
+  } else if (!g_plan_independent(g.data(), count, mode, kind, f16 != 0, sms, plan.data())) {
+    return "no plan";
+  }
+  for (int i = 0; i < count; ++i) g_finish_plan(g[i], &plan[i]);
+  GParams ring{};
+  size_t smem = 0;
+  if (!g_ring(plan.data(), count, mode, &ring, &smem)) return "no ring";
+  for (int i = 0; i < count; ++i) {
+    const GLayer& o = plan[i].L;
+    const int v[4] = {o.lg, o.Np, o.tma, o.total_tiles};
+    memcpy(out + 4 * i, v, sizeof(v));
+  }
+  return wrong(plan.data(), count, mode, ring, smem);
+}
+
+}  // extern "C"
