@@ -46,7 +46,7 @@ constexpr int G_MAX_CHUNKS = 8;                // 32-column slices of an accumul
 // What the epilogue needs to know of a tile, written by the table warp (see there), four tiles deep.
 struct GTile {
   int l, mg, co, n_slices;             // problem (-1: no more tiles), position tile, first channel, 32-column slices
-  int K, kp_log, Np, out_kind;         // channels; logarithm of the rows per pixel; positions; 0 fp32, 1 int32, 2 packed signs
+  int K, kp_log, lg, out_kind;         // channels; GLayer::kp_log, lg; 0 fp32, 1 int32, 2 packed signs
   uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
   uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
   float alpha[G_ROWS], shift[G_ROWS];
@@ -82,6 +82,8 @@ struct GLayer {
   int n_pu, pu_end[4];    // units per channel block (fetched by TMA, each plane is a unit of its own) and the last step of each
   int steps;              // taps of a tile, or pairs of taps (one activation word per pixel: a K = 64 step covers two taps)
   int st_steps;           // steps per weight stage (the last stage of a channel block holds steps % st_steps, if not 0)
+  int kp_log;             // logarithm of the rows of the weight operand that hold the channels once: of each pixel of a group, or
+                          // - with single pixels - of each copy of the channels
   uint32_t step_bytes;    // weights of one step of one channel block = kpt * 2 * 128 * 16
   int n_ct, total_tiles;  // channel tiles of 128
   int first;              // this CTA's first tile, filled in by the kernel (GParams::ranks)
@@ -225,6 +227,10 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   const long long tiles = (Q + Np - 1) / Np * o.n_ct;
   if (tiles > 0x7fffffffLL || (Q + Np - 1) / Np * o.Rr >= (1ll << 31)) return false;
   o.total_tiles = (int)tiles;
+  // Single pixels of at most 64 channels: the other rows hold copies of the channels, so that warps of all lane quarters
+  // share a tile's columns.  A warp reads its own quarter's lanes only, and two of the eight would write the whole tile
+  // (fp16, 16 channels of 32x32 maps at batch 128: 13.8 us, with copies 10.0; the multiplications take 128 rows anyway).
+  o.kp_log = lg ? 7 - lg : g.K <= 32 ? 5 : g.K <= 64 ? 6 : 7;
   // weight stage: as many whole steps of a channel block as fit a slot
   o.step_bytes = (uint32_t)(o.kpt * 2 * G_ROWS * 16);
   o.st_steps = (int)((mode == M_F16 ? kGBSlotF16 : kGBSlot) / o.step_bytes);
@@ -319,6 +325,18 @@ bool g_path_takes(const Geom& g, int mode) {
     if (2 * unit + epi + 2 * pix + 256 + kGTail + 3 * b_slot > budget) return false;
   }
   return true;
+}
+
+// Epilogue warps that have something to write of a position tile (of all its channel tiles): of each 32 rows that hold a
+// channel those two that have a slice.
+int g_writing_warps(const GLayer& L) {
+  int warps = 0;
+  for (int at = 0; at < L.n_ct * G_ROWS; at += 32) {
+    const int r = at % G_ROWS, first = L.lg ? 0 : 2 * (r >> L.kp_log);
+    if (at - r + (r & ((1 << L.kp_log) - 1)) >= L.K) continue;
+    for (int half = 0; half < 2; ++half) warps += first + half < (L.Np + 31) / 32 ? 1 : 0;
+  }
+  return warps;
 }
 
 // Tile sizes the planner chooses from (positions; multiples of 16).

@@ -418,13 +418,15 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       }
       __syncwarp();
       const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
-      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y;
+      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, lg = h1.z;
       if (l < 0) break;   // no more tiles
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : h1.w;
       uint32_t* const out32 = reinterpret_cast<uint32_t*>(p.out[l]);  // int32 and fp32 outputs share the layout
-      // this lane's row of the weight operand: pixel g of a position's group, channel c of the channel tile
-      const int g_lane = row >> kp_log, c_lane = row & ((1 << kp_log) - 1);
-      const int g_warp = (rq * 32) >> kp_log, c_warp = (rq * 32) & ((1 << kp_log) - 1);   // of lane 0
+      // this lane's row of the weight operand: channel c of pixel g of a position's group, or of a copy of the channels
+      const int c_lane = row & ((1 << kp_log) - 1), c_warp = (rq * 32) & ((1 << kp_log) - 1);   // (_warp: of lane 0)
+      const int g_lane = lg ? row >> kp_log : 0, g_warp = lg ? (rq * 32) >> kp_log : 0;
+      // the warps of a lane quarter, and the copies, take the 32-column slices in turn
+      const int s_first = half + (lg ? 0 : 2 * ((rq * 32) >> kp_log)), s_step = lg ? 2 : 2 << (7 - kp_log);
       const int co = h0.z + c_lane, co_warp = h0.z + c_warp;
       const bool active = co_warp < K;   // does any of the warp's rows hold a channel?
       const float al = T->alpha[c_lane], sh = WORDS ? 0.f : T->shift[c_lane];
@@ -446,17 +448,17 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           __syncwarp();
           if (lane == 0) mbar_arrive(bar_accempty + 8 * acc_slot);
         };
-        if (!active || half >= n_slices) {
+        if (!active || s_first >= n_slices) {
           release();
         } else {
           uint32_t* const obase = out32 + (size_t)((uint32_t)(g_lane * K + co));
           // (a last slice of 16 columns is read as 32: the others belong to the next buffer or the scales and go nowhere)
 #pragma unroll 1
-          for (int s = half; s < n_slices; s += 2) {   // the two warps of a lane quarter take the slices in turn
+          for (int s = s_first; s < n_slices; s += s_step) {
             uint32_t v[32];
             __syncwarp();   // the load is a warp-wide instruction
             tmem_ld32(d0 + (uint32_t)(32 * s), v);
-            if (s + 2 >= n_slices) release();
+            if (s + s_step >= n_slices) release();
             if (WORDS || out_kind != 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
               // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubled the code, and the
@@ -519,7 +521,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         }
         if (CHAIN) {
           // chain: this warp's part of the tile is written; the successor may read it
-          if (active && half < n_slices) {
+          if (active && s_first < n_slices) {
             __syncwarp();
             if (lane == 0) {
               __threadfence();   // (cumulative: it covers what the other lanes wrote before the barrier)
@@ -574,7 +576,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         }
         if (lane == 0) {
           *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
-          *reinterpret_cast<int4*>(&T->K) = make_int4(K, 7 - lg, Np, out_kind);
+          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, lg, out_kind);
         }
 #pragma unroll 4
         for (int s = 0; s < n_slices; ++s) {
@@ -1037,13 +1039,13 @@ MapEncoder g_map_encoder() {
 }
 
 // Operand of the weights: wt[channel tile][channel block][step][chunk][128][16 B]; a chunk is 16 bytes along the
-// input channels (8 fp16 or 32 e2m1 values), cb_chunks chunks per block.  Row r of a tile is channel r % (128/G) of
-// pixel r / (128/G).  Channels that do not exist, and columns outside a pixel's window, are zeros, so whatever the
+// input channels (8 fp16 or 32 e2m1 values), cb_chunks chunks per block.  With p = 2^kp_log, row r of a tile is channel
+// r % p of pixel r / p or, with single pixels, of copy r / p.  Channels that do not exist, and columns outside a pixel's window, are zeros, so whatever the
 // activation operand holds there adds 0.
 template <int MODE>
 __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, uint8_t* __restrict__ wt, int C, int K,
                                         int Cw, long long total, int cb_chunks, int n_cb, int steps, int paired, int lg,
-                                        int win_step, int ksize, const GTaps taps) {
+                                        int kp_log, int win_step, int ksize, const GTaps taps) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= total) return;
   const int row = (int)(i & (G_ROWS - 1));
@@ -1054,8 +1056,7 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
   const int t = (int)(r % steps);
   r /= steps;
   const int cb = (int)(r % n_cb), tile = (int)(r / n_cb);
-  const int kp_log = 7 - lg;
-  const int g = row >> kp_log, co = tile * G_ROWS + (row & ((1 << kp_log) - 1));
+  const int g = lg ? row >> kp_log : 0, co = tile * G_ROWS + (row & ((1 << kp_log) - 1));
   const int which = paired ? c : 0;
   const int ky = taps.row[t][which], kx = (int)taps.col[t][which] - win_step * g;
   constexpr int cpc = MODE == M_F16 ? 8 : 32;
@@ -1201,15 +1202,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
       if (i > 0) {
         L.deps = deps_dev + deps_off[i];
         L.prev_done = Gd->done + done_off[i - 1];
-        // the epilogue warps that have something to write of a position tile: one per 32 rows that hold a
-        // channel and, from two slices on, two per lane quarter
-        const GLayer& P = plan[i - 1].L;
-        int quarters = (gs[i - 1].K + 31) / 32;
-        if (P.lg) {
-          quarters = 0;
-          for (int r = 0; r < G_ROWS; r += 32) quarters += (r & ((G_ROWS >> P.lg) - 1)) < gs[i - 1].K ? 1 : 0;
-        }
-        L.prev_target = (uint32_t)(quarters * (P.Np > 32 ? 2 : 1));
+        L.prev_target = (uint32_t)g_writing_warps(plan[i - 1].L);
       }
     }
     const long long total = (long long)plan[i].w_bytes / 16;
@@ -1217,12 +1210,12 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     const int win_step = gs[i].stride, ks = gs[i].ksize;
     if (mode == M_F16)
       g_expand_weights_kernel<M_F16><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
-                                                            total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, win_step,
-                                                            ks, plan[i].taps);
+                                                            total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
+                                                            win_step, ks, plan[i].taps);
     else
       g_expand_weights_kernel<M_FP4><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
-                                                            total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, win_step,
-                                                            ks, plan[i].taps);
+                                                            total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
+                                                            win_step, ks, plan[i].taps);
     e = cudaGetLastError();
     if (e == cudaSuccess) *launched += 1;
   }
@@ -1269,7 +1262,7 @@ __global__ void __launch_bounds__(128) g_static_weights_kernel(const uint8_t* __
                                                                const GLayer L, int tau, int paired,
                                                                const GStepOf step_of) {
   const int row = threadIdx.x, wd = blockIdx.x, ct = blockIdx.y;   // row of the operand, 32-channel word, channel tile
-  const int kp_log = 7 - L.lg, g = row >> kp_log, co = ct * G_ROWS + (row & ((1 << kp_log) - 1));
+  const int g = L.lg ? row >> L.kp_log : 0, co = ct * G_ROWS + (row & ((1 << L.kp_log) - 1));
   __shared__ uint16_t codes[512];
   for (int i = row; i < (1 << tau); i += 128) codes[i] = codebook[i];
   const int n_ch = co < L.K ? (L.C - 32 * wd < 32 ? L.C - 32 * wd : 32) : 0;   // channels of this word (none: all zeros)

@@ -54,6 +54,14 @@ extern "C" {
 
 int plan_takes(const int* g, int f16) { return g_path_takes(geom(g), f16 ? M_F16 : M_FP4); }
 
+// A plan of a given tile: the epilogue warps that write of a position tile, rows a copy or pixel of it has (0: cannot be planned).
+int plan_tile(const int* v, int f16, int kind, int lg, int Np, int* rows) {
+  GPlan plan;
+  if (!g_plan_layer(geom(v), f16 ? M_F16 : M_FP4, kind, lg, Np, f16 != 0, &plan)) return 0;
+  *rows = 1 << plan.L.kp_log;
+  return g_writing_warps(plan.L);
+}
+
 // out per problem: lg, Np, tma, tiles.  Returns what is wrong with the plan, or null.
 const char* plan_make(const int* gs, int count, int f16, int kind, int sms, int* out) {
   const int mode = f16 ? M_F16 : M_FP4;

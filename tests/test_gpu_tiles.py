@@ -115,6 +115,22 @@ def test_fp16_units(snn, oracle_mod, c_in, c_out, h, w, stride, pad, n):
     layer.destroy()
 
 
+@pytest.mark.parametrize("c_out", [1, 16, 17, 32, 33, 64, 65])
+@pytest.mark.parametrize("c_in,h,w,n,stride", [(16, 32, 32, 40, 1), (24, 9, 11, 3, 2), (20, 40, 28, 36, 1)])
+def test_fp16_few_channels(snn, oracle_mod, c_in, c_out, h, w, n, stride):
+    """Lanes that hold copies of the channels: tiles of one slice and of many, fetched and copied units."""
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, 1)
+    p = wl.draw_layer_params(shape, 5, 800 + c_out)
+    act = wl.draw_activation_f16(shape, n, 801 + c_in)
+    ref = oracle_mod.conv_f16(p.codebook, 5, p.idx_packed, p.alpha, c_in, c_out, stride, 1, act).astype(np.float64)
+    layer = snn.SnnConv(c_in, c_out, 5, p.codebook, p.idx_packed, p.alpha, stride, 1, snn.ACT_F16)
+    y = layer.forward(torch.from_numpy(act).cuda(), path=snn.PATH_DECODED_TC).cpu().numpy().astype(np.float64)
+    # 9 * c_in exact products summed in fp32: each addition rounds by at most 2^-24 of the sum of magnitudes
+    mag = p.alpha.astype(np.float64) * 9 * c_in * np.abs(act.astype(np.float64)).max()
+    assert (np.abs(y - ref) <= 9 * c_in * 2.0 ** -24 * mag).all()
+    layer.destroy()
+
+
 @pytest.mark.parametrize("stride,pad", [(1, 1), (2, 0)])
 @pytest.mark.parametrize("c_in,c_out,h,w,n,tau", [
     (1, 1, 3, 3, 1, 1), (16, 16, 9, 8, 2, 3), (31, 33, 6, 7, 2, 9), (64, 64, 5, 12, 2, 5), (70, 20, 8, 5, 3, 7), (129, 200, 4, 6, 2, 8),

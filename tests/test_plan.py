@@ -67,3 +67,33 @@ def test_every_group_of_such_shapes_can_be_planned(lib, f16):
         shapes = [s for s in (draw(rng) for _ in range(80)) if takes(lib, s, f16)][:rng.randint(2, 32)]
         for kind in (WORDS,) if f16 else (WORDS, SIGNS):
             make(lib, shapes, f16, kind)
+
+
+@pytest.mark.parametrize("c_out", [1, 8, 16, 17, 31, 32, 33, 48, 64, 65, 96, 128, 129, 160, 300])
+@pytest.mark.parametrize("lg", [0, 1, 2, 3])
+@pytest.mark.parametrize("np_", [16, 32, 48, 112, 160, 240])
+def test_the_warps_that_write_share_the_columns(lib, c_out, lg, np_):
+    """Every (channel, 32-column slice) is written by exactly one warp and lane; with few channels and single pixels by as many
+    warps as there are slices; and a chain's counters expect the warps that do write."""
+    rows = ctypes.c_int(0)
+    warps = lib.plan_tile(_array((4, 20, 20, 96, c_out, 1, 1, 3)), 0, WORDS, lg, np_, ctypes.byref(rows))
+    if not warps:
+        return   # no such tile
+    rows, slices = rows.value, (np_ + 31) // 32
+    written, writing = {}, 0
+    for co in range(0, c_out, 128):
+        for warp in range(8):   # the kernel's epilogue: lane quarter warp % 4, half warp // 4
+            first = 32 * (warp % 4)
+            copy = 0 if lg else first // rows
+            mine = range(warp // 4 + 2 * copy, slices, 2 if lg else 2 * (128 // rows))
+            if co + first % rows >= c_out or not mine:
+                continue
+            writing += 1
+            for row in range(first, first + 32):
+                pixel, channel = (row // rows if lg else 0), co + row % rows
+                for s in mine if channel < c_out else ():
+                    written[pixel, channel, s] = written.get((pixel, channel, s), 0) + 1
+    assert writing == warps
+    assert written == {(g, c, s): 1 for g in range(1 << lg) for c in range(c_out) for s in range(slices)}
+    if lg == 0 and c_out <= 32:
+        assert warps == min(8, slices)
