@@ -269,8 +269,10 @@ SNN_API snn_status_t snn_conv_stack_destroy(snn_conv_stack_t* s);
  * the copy engine (keep them alive and unchanged until the stream has passed them
  * unless they are pageable memory, which the runtime stages before returning).
  *
- * The first call on a device resolves the device address of the array
- * (cudaGetSymbolAddress); make that first call outside any stream capture.
+ * The first call on a device resolves the device address of the array and pins one
+ * page of the library's own host memory (cudaGetSymbolAddress, cudaHostRegister);
+ * make that first call outside any stream capture.  Until the page is pinned the
+ * layer runs on the slower popcount kernel; every call outside a capture tries again.
  * All calls on a device share the one array and it keeps the previous call's
  * contents: each call rewrites in full every region it reads, so results never
  * depend on an earlier call, but two calls whose GPU work overlaps (different

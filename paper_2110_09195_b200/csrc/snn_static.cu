@@ -8,6 +8,7 @@
 // kernel does not take is decoded to bit-planes and run by the XOR + popcount kernel.
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 
@@ -29,31 +30,40 @@ std::mutex g_setup_mu;
 unsigned char* g_scratch_dev[kMaxDevices] = {nullptr};
 
 // Where a tensor-core launch reports a bounded wait that gave up: one word per device in a page of the library image,
-// pinned and mapped at the first call (host memory; nothing is allocated on a device).
+// pinned and mapped at the first call (host memory; nothing is allocated on a device).  While that fails, calls take the
+// popcount kernel, which does not wait.
 struct alignas(4096) StatusPage {
   volatile int word[4096 / sizeof(int)];
 };
 StatusPage g_status;
-int g_status_state = 0;   // 0: not pinned yet, 1: pinned, 2: cannot be (the popcount kernel, which does not wait, is used)
+bool g_status_pinned = false;
 int* g_status_dev[kMaxDevices] = {nullptr};
 
-// Device addresses of the scratch and of the status word on the current device, resolved once per device.
-cudaError_t scratch_address(int device, unsigned char** out, int** status) {
+// Device addresses of the scratch and of the status word on the current device, resolved once per device.  What failed is
+// tried again by the next call; pinning only where no capture is under way, which it could invalidate.
+cudaError_t scratch_address(int device, cudaStream_t s, unsigned char** out, int** status) {
   std::lock_guard<std::mutex> lk(g_setup_mu);
   if (!g_scratch_dev[device]) {
     void* ptr = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_static_scratch);
     if (e != cudaSuccess) return e;
-    if (g_status_state == 0) {
-      g_status_state = cudaHostRegister(&g_status, sizeof(g_status), cudaHostRegisterMapped | cudaHostRegisterPortable) == cudaSuccess ? 1 : 2;
-      cudaGetLastError();
-    }
-    void* st = nullptr;
-    if (g_status_state == 1 && cudaHostGetDevicePointer(&st, const_cast<int*>(g_status.word), 0) == cudaSuccess)
-      g_status_dev[device] = static_cast<int*>(st) + device * 16;
-    else
-      cudaGetLastError();
     g_scratch_dev[device] = static_cast<unsigned char*>(ptr);
+  }
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  if (!g_status_dev[device] && cudaStreamIsCapturing(s, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone) {
+    void* st = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!g_status_pinned) {
+      e = cudaHostRegister(&g_status, sizeof(g_status), cudaHostRegisterMapped | cudaHostRegisterPortable);
+      g_status_pinned = e == cudaSuccess;
+    }
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(&st, const_cast<int*>(g_status.word), 0);
+    if (e == cudaSuccess) {
+      g_status_dev[device] = static_cast<int*>(st) + device * 16;
+    } else {
+      cudaGetLastError();
+      if (getenv("SNN_LOG")) fprintf(stderr, "[snnconv] no status page, the popcount kernel is used: %s\n", cudaGetErrorString(e));
+    }
   }
   *status = g_status_dev[device];
   *out = g_scratch_dev[device];
@@ -140,8 +150,8 @@ extern "C" SNN_API snn_status_t snn_conv_forward_static(const snn_conv_desc_t* d
   snn_status_t st = SNN_OK;
   unsigned char* base = nullptr;
   int* status_dev = nullptr;
-  cudaError_t e = scratch_address(d->device, &base, &status_dev);  // first call on a device resolves the symbol
   cudaStream_t s = (cudaStream_t)cuda_stream;
+  cudaError_t e = scratch_address(d->device, s, &base, &status_dev);
   int launched = 0;
   // The tensor-core kernel where it takes the shape (8 images of a 128-channel 28x28 layer: 19 us a call, by
   // popcounts 48): [codebook][scales][index stream][weight operand].
