@@ -227,10 +227,6 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   const long long tiles = (Q + Np - 1) / Np * o.n_ct;
   if (tiles > 0x7fffffffLL || (Q + Np - 1) / Np * o.Rr >= (1ll << 31)) return false;
   o.total_tiles = (int)tiles;
-  // Single pixels of at most 64 channels: the other rows hold copies of the channels, so that warps of all lane quarters
-  // share a tile's columns.  A warp reads its own quarter's lanes only, and two of the eight would write the whole tile
-  // (fp16, 16 channels of 32x32 maps at batch 128: 13.8 us, with copies 10.0; the multiplications take 128 rows anyway).
-  o.kp_log = lg ? 7 - lg : g.K <= 32 ? 5 : g.K <= 64 ? 6 : 7;
   // weight stage: as many whole steps of a channel block as fit a slot
   o.step_bytes = (uint32_t)(o.kpt * 2 * G_ROWS * 16);
   o.st_steps = (int)((mode == M_F16 ? kGBSlotF16 : kGBSlot) / o.step_bytes);
@@ -243,6 +239,13 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   const double lines = mmas * (32 + Np / 4) + (double)o.n_cb * (o.steps * o.step_bytes + (double)o.n_pu * P->unit_bytes) / 128.0;
   P->mma = std::max(mmas * (Np / 2), 1.1 * lines);
   P->weights = (double)o.n_cb * o.steps * o.step_bytes / 64.0;
+  // Single pixels of at most 64 channels: a warp reads its own quarter's lanes only, and two or four of the eight would write
+  // the whole tile, at 24 cycles a column.  Where that takes longer than the tile's MMAs, the other rows hold copies of the
+  // channels and warps of all lane quarters share the columns (fp16, 16 channels of 32x32 maps at batch 128: 13.8 us, with
+  // copies 9.7).  Elsewhere they stay zeros, which take less power (64 channels of 56x56: 3 % of the launch).
+  const int slices = (Np + 31) / 32;
+  const bool copies = lg == 0 && g.K <= 64 && P->mma < 24.0 * std::min(Np, 32 * ((slices + 1) / 2));
+  o.kp_log = lg ? 7 - lg : !copies ? 7 : g.K <= 32 ? 5 : 6;
   P->expand = o.tma ? o.n_cb * o.n_pu * (P->unit_bytes / 40.0) + 1000.0 : o.n_cb * ((double)o.n_planes * o.Rr * d * (mode == M_F16 ? 3.0 : 0.6) + 500.0);
   const int k_tile = g.K < G_ROWS ? g.K : G_ROWS;
   P->drain = kind == TCG_WORDS ? (double)Np * G * k_tile * 4 / 16.0 : Np * 5.0;

@@ -76,7 +76,7 @@ def test_the_warps_that_write_share_the_columns(lib, c_out, lg, np_):
     """Every (channel, 32-column slice) is written by exactly one warp and lane; with few channels and single pixels by as many
     warps as there are slices; and a chain's counters expect the warps that do write."""
     rows = ctypes.c_int(0)
-    warps = lib.plan_tile(_array((4, 20, 20, 96, c_out, 1, 1, 3)), 0, WORDS, lg, np_, ctypes.byref(rows))
+    warps = lib.plan_tile(_array((4, 20, 20, 32, c_out, 1, 1, 3)), 0, WORDS, lg, np_, ctypes.byref(rows))
     if not warps:
         return   # no such tile
     rows, slices = rows.value, (np_ + 31) // 32
@@ -97,3 +97,10 @@ def test_the_warps_that_write_share_the_columns(lib, c_out, lg, np_):
     assert written == {(g, c, s): 1 for g in range(1 << lg) for c in range(c_out) for s in range(slices)}
     if lg == 0 and c_out <= 32:
         assert warps == min(8, slices)
+
+
+@pytest.mark.parametrize("c_in,c_out,copies", [(16, 16, True), (16, 64, True), (32, 32, True), (64, 64, False), (512, 16, False), (512, 32, False)])
+def test_copies_only_where_the_stores_take_longer_than_the_mmas(lib, c_in, c_out, copies):
+    rows = ctypes.c_int(0)
+    assert lib.plan_tile(_array((64, 32, 32, c_in, c_out, 1, 1, 3)), 1, WORDS, 0, 256, ctypes.byref(rows))
+    assert (rows.value < 128) == copies
