@@ -149,6 +149,13 @@ struct GPlan {
     return t + 300.0;
   }
   double alone() const { return expand + (mma > weights ? mma : weights) + drain + 1500.0; }   // a tile by itself
+  // The end of a launch of this layer alone: staging and stores have the time they take with idle neighbours (below).
+  double mma_one = 0, stage_one = 0, drain_one = 0;
+  double end(int sms) const {
+    const int waves = (L.total_tiles + sms - 1) / sms;
+    const double work = std::max(mma_one, weights);
+    return stage_one + work + 0.7 * drain_one + 1500.0 + (waves - 1) * (std::max(work, std::max(stage_one, drain_one)) + 300.0);
+  }
 };
 
 // The plan of one layer with tiles of Np positions of 2^lg pixels; false where that does not fit.
@@ -249,6 +256,16 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   P->expand = o.tma ? o.n_cb * o.n_pu * (P->unit_bytes / 40.0) + 1000.0 : o.n_cb * ((double)o.n_planes * o.Rr * d * (mode == M_F16 ? 3.0 : 0.6) + 500.0);
   const int k_tile = g.K < G_ROWS ? g.K : G_ROWS;
   P->drain = kind == TCG_WORDS ? (double)Np * G * k_tile * 4 / 16.0 : Np * 5.0;
+  // In a launch of this layer alone little else waits for memory: what counts is how many loads one thread does in a row
+  // (200 cycles each; 0.2 a chunk where they are many), and the stores go to L2 at 32 bytes a cycle, 24 cycles a column and
+  // 250 a slice of signs for the warp that has the most of them.  Fitted to 12,000 plans: all widths and group sizes of 384
+  // layers of 16 to 512 channels, maps of 6 to 57, 1 to 128 images.
+  const int team = G_EXP_THREADS / G_XTEAMS, word_step = g_word_step(g.Cw, d);
+  const int loads = (o.Rr + team - 1) / team * o.n_planes * ((d + word_step - 1) / word_step);
+  const int sharing = lg ? 2 : 2 * (G_ROWS >> o.kp_log), most = (slices + sharing - 1) / sharing;
+  P->mma_one = mmas * std::max(Np / 2.0, 1.1 * (32 + Np / 4.0));
+  P->stage_one = mode == M_F16 ? P->expand : o.n_cb * std::max(0.2 * o.n_planes * o.Rr * d, 200.0 * loads);
+  P->drain_one = kind == TCG_WORDS ? std::max((double)Np * G * k_tile * 4 / 32.0, 24.0 * std::min(32 * most, Np)) : 250.0 * most;
   return true;
 }
 
@@ -438,6 +455,33 @@ bool g_ring(const GPlan* plan, int count, int mode, GParams* p, size_t* smem) {
   return *smem <= (size_t)kMaxDynSmem && *smem < (1u << 18);
 }
 
+// Another plan for a launch of one layer of few channels, with single pixels or pairs, where its tiles would end at least 15 %
+// earlier: the group size of the most throughput leaves most SMs idle when a small layer's work is packed into few heavy
+// tiles.  96 to 20 channels, 16 images of 14x14 at stride 2: 16 tiles 20.7 us, 64 tiles 8.2; 6.3 % over those 384 layers.
+// The 15 % are what the estimate errs by: without them one layer in thirty got slower, by up to a third.  Of the widths
+// only the narrowest that leaves no SM a second tile and the two above are looked at: the no-allocation entry point plans in
+// every call, and all of them took it another microsecond.
+void g_plan_alone(const Geom& g, int mode, int kind, int sms, GPlan* plan) {
+  constexpr int widths = sizeof(kNpTable) / sizeof(kNpTable[0]);
+  double best = 0.85 * plan->end(sms);
+  int best_lg = -1, best_np = 0;
+  GPlan P;
+  for (int lg = 0; lg <= std::min(plan->L.lg, 1); ++lg) {
+    // positions of the whole layer, as g_plan_layer counts them
+    const int rows = g.ksize == 1 ? g.Ho : g.stride == 1 ? g.H + g.pad : g.Ho + 1, cols = g.ksize == 1 ? g.Wo : g.stride == 1 ? g.W + g.pad : g.Wo + 1;
+    const long long Q = (long long)g.N * rows * ((cols + (1 << lg) - 1) >> lg);
+    int at = widths - 1;
+    while (at > 0 && Q > (long long)kNpTable[at] * sms) --at;
+    for (int w = std::max(at - 2, 0); w <= at; ++w) {
+      const int Np = kNpTable[w];
+      if (Np > (int)G_TMEM_FP4 / 2 || !g_plan_layer(g, mode, kind, lg, Np, false, &P)) continue;
+      const double t = P.end(sms);
+      if (t < best) { best = t; best_lg = lg; best_np = Np; }
+    }
+  }
+  if (best_lg >= 0) g_plan_layer(g, mode, kind, best_lg, best_np, false, plan);
+}
+
 // Tiles of independent problems: one size limit for all of them, by the estimated time of the launch.
 bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma, int sms, GPlan* plan) {
   GChoice trial[SNN_GROUP_MAX], chosen[SNN_GROUP_MAX];
@@ -463,6 +507,7 @@ bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma,
   }
   if (best < 0) return false;
   for (int i = 0; i < count; ++i) g_plan_layer(gs[i], mode, kind, chosen[i].lg, chosen[i].Np, chosen[i].tma, &plan[i]);
+  if (count == 1 && mode == M_FP4 && gs[0].K <= G_ROWS / 2) g_plan_alone(gs[0], mode, kind, sms, plan);
   return true;
 }
 

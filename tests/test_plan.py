@@ -69,6 +69,17 @@ def test_every_group_of_such_shapes_can_be_planned(lib, f16):
             make(lib, shapes, f16, kind)
 
 
+@pytest.mark.parametrize("shape,kind,tiles", [
+    # N, H, W, C, K, stride, pad, ksize: what packs each of these into fewer tiles takes 1.2 to 3 times as long
+    ((16, 14, 14, 96, 20, 2, 1, 3), WORDS, 32), ((4, 14, 14, 512, 16, 1, 1, 3), WORDS, 16), ((4, 46, 33, 93, 31, 2, 1, 3), WORDS, 50),
+    ((1, 30, 30, 96, 16, 1, 1, 3), WORDS, 20), ((4, 56, 56, 256, 16, 1, 1, 3), SIGNS, 100), ((21, 10, 43, 214, 24, 2, 1, 3), SIGNS, 31),
+    ((4, 56, 56, 96, 16, 1, 0, 1), SIGNS, 98),
+])
+def test_a_small_layer_of_few_channels_is_spread_over_the_machine(lib, shape, kind, tiles):
+    (lg, _, _, got), = make(lib, [shape], kind=kind)
+    assert lg <= 1 and got >= tiles   # (a tile of a group of pixels takes two to eight times the MMAs of one of pixels)
+
+
 @pytest.mark.parametrize("c_out", [1, 8, 16, 17, 31, 32, 33, 48, 64, 65, 96, 128, 129, 160, 300])
 @pytest.mark.parametrize("lg", [0, 1, 2, 3])
 @pytest.mark.parametrize("np_", [16, 32, 48, 112, 160, 240])
