@@ -115,6 +115,49 @@ def test_fp16_units(snn, oracle_mod, c_in, c_out, h, w, stride, pad, n):
     layer.destroy()
 
 
+def _whole_f16(shape, n, seed):
+    """fp16 activations of small whole numbers: every sum is exact in fp32, and one multiplication by the scale rounds."""
+    return np.random.default_rng(seed).integers(-8, 9, size=(n, shape.h, shape.w, shape.c_in)).astype(np.float16)
+
+
+# units that the threads copy (rows that are no multiple of 16 bytes, or longer than a box), more of them per tile than the
+# ring has slots: three in flight, slots reused behind them
+COPIED = [(260, 24, 14, 14, 1, 1, 40), (330, 40, 12, 20, 1, 0, 9), (256, 16, 5, 300, 1, 1, 6), (260, 40, 14, 14, 2, 1, 40), (1, 3, 40, 40, 1, 1, 30)]
+
+
+@pytest.mark.parametrize("c_in,c_out,h,w,stride,pad,n", COPIED)
+def test_fp16_copied_units(snn, oracle_mod, c_in, c_out, h, w, stride, pad, n):
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, pad)
+    p = wl.draw_layer_params(shape, 5, 900 + w)
+    act = _whole_f16(shape, n, 901 + c_in)
+    ref = oracle_mod.conv_f16(p.codebook, 5, p.idx_packed, p.alpha, c_in, c_out, stride, pad, act).astype(np.float64)
+    layer = snn.SnnConv(c_in, c_out, 5, p.codebook, p.idx_packed, p.alpha, stride, pad, snn.ACT_F16)
+    y = layer.forward(torch.from_numpy(act).cuda(), path=snn.PATH_DECODED_TC).cpu().numpy().astype(np.float64)
+    assert (np.abs(y - ref) <= 2.0 ** -23 * np.abs(ref)).all()
+    layer.destroy()
+
+
+def test_fp16_copied_and_fetched_members_in_one_launch(snn, oracle_mod):
+    """Members whose units are copied and members whose units are fetched by TMA take turns, with several tiles per CTA: the
+    copies in flight are finished before the next member's units, and the ring carries on."""
+    shapes = [(wl.LayerShape(260, 24, 14, 14, 1, 1), 40), (wl.LayerShape(72, 40, 20, 20, 1, 1), 90), (wl.LayerShape(330, 16, 12, 20, 1, 0), 30),
+              (wl.LayerShape(256, 32, 14, 14, 2, 1), 60), (wl.LayerShape(36, 130, 16, 16, 2, 1), 60), (wl.LayerShape(64, 64, 28, 28, 1, 1), 40)]
+    layers, acts, refs = [], [], []
+    for i, (s, n) in enumerate(shapes):
+        p = wl.draw_layer_params(s, 5, 950 + i)
+        act = _whole_f16(s, n, 960 + i)
+        refs.append(oracle_mod.conv_f16(p.codebook, 5, p.idx_packed, p.alpha, s.c_in, s.c_out, s.stride, s.pad, act).astype(np.float64))
+        layers.append(snn.SnnConv(s.c_in, s.c_out, 5, p.codebook, p.idx_packed, p.alpha, s.stride, s.pad, snn.ACT_F16))
+        acts.append(torch.from_numpy(act).cuda())
+    group = snn.SnnConvGroup(layers, [(n, s.h, s.w) for s, n in shapes])
+    for _ in range(2):
+        for out, ref in zip(group.forward(acts), refs):
+            assert (np.abs(out.cpu().numpy().astype(np.float64) - ref) <= 2.0 ** -23 * np.abs(ref)).all()
+    group.destroy()
+    for l in layers:
+        l.destroy()
+
+
 @pytest.mark.parametrize("c_out", [1, 16, 17, 32, 33, 64, 65])
 @pytest.mark.parametrize("c_in,h,w,n,stride", [(16, 32, 32, 40, 1), (24, 9, 11, 3, 2), (20, 40, 28, 36, 1)])
 def test_fp16_few_channels(snn, oracle_mod, c_in, c_out, h, w, n, stride):
