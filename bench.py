@@ -191,7 +191,7 @@ def _kernel_fingerprint():
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in ("snn_tcg.cu", "snn_tc_common.cuh"):
+    for f in ("snn_tcg.cu", "snn_tc_common.cuh", "snn_tc_plan.h"):
         with open(os.path.join(ROOT, "paper_2110_09195_b200", "csrc", f), "r") as fh:
             text = re.sub(r"//[^\n]*", "", fh.read())
         h.update("".join(text.split()).encode())

@@ -68,7 +68,6 @@ cudaError_t tcg_create(const LayerDev* const* layers, const Geom* geoms, int cou
 cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, int out_type, cudaStream_t s,
                         int* status_dev, int* launched);
 void tcg_destroy(GroupDev* G);
-int tcg_count(const GroupDev* G);
 // One launch from the stored form of a layer (index stream, codebook and scales in device memory), in memory of the
 // caller's: tcg_static_plan says how many bytes that takes (binary activations, fp32 / int32 outputs; false where the
 // tensor-core kernel cannot run the layer), tcg_static_forward writes the weight operand there and runs the layer.

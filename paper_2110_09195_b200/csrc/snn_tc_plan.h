@@ -239,9 +239,10 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   o.st_steps = (int)((mode == M_F16 ? kGBSlotF16 : kGBSlot) / o.step_bytes);
   if (o.st_steps > o.steps) o.st_steps = o.steps;
   P->w_bytes = (size_t)o.n_ct * o.n_cb * o.steps * o.step_bytes;
-  // One MMA reads 32 + Np/4 shared-memory lines and takes at least Np/2 cycles (measured).  The other figures are the
-  // rates the roles reach in the traces: bulk copies of weights 64 bytes per cycle, a 16-byte chunk of activations
-  // in 0.6 cycles (0.4 copied) plus the latency of the loads, stores 16 bytes per cycle.
+  // One MMA reads 32 + Np/4 shared-memory lines and takes at least Np/2 cycles (measured).  The other figures are set by
+  // hand after traces of single roles, for launches that keep every SM busy: bulk copies of weights 64 bytes a cycle, a
+  // 16-byte chunk of activations 0.6 cycles (3 where fp16 is copied by the threads) and 500 a block of channels, units
+  // fetched by TMA 40 bytes a cycle and 1000 for the first, stores 16 bytes a cycle, signs 5 cycles a position.
   const double mmas = (double)o.n_cb * o.steps * o.kpt;
   const double lines = mmas * (32 + Np / 4) + (double)o.n_cb * (o.steps * o.step_bytes + (double)o.n_pu * P->unit_bytes) / 128.0;
   P->mma = std::max(mmas * (Np / 2), 1.1 * lines);
@@ -310,6 +311,7 @@ void g_finish_plan(const Geom& g, GPlan* P) {
 // Does the tensor-core path take this layer?  The bound is that of a unit of 128 positions with its halo (row pitch of
 // the padded map) in a 40.5 KB slot, two of which fit beside the weight ring; shapes beyond it go to the other paths.
 // The tiles themselves are planned by g_plan_layer, which needs less.
+// (So it refuses some shapes that could be planned, 3x3 layers of 64 channels on maps wider than 600 among them.)
 bool g_path_takes(const Geom& g, int mode) {
   constexpr size_t slot_max = 40 * 1024 + 512, b_slot = 32 * 1024, epi = 40 * 1024, budget = 226 * 1024;
   if (g.N < 1 || g.C > (1 << 20)) return false;            // 9 * c_in stays far below 2^24: exact fp32 sums

@@ -18,18 +18,19 @@
 //   * the 32 lanes of an epilogue warp are 32 consecutive channels of one pixel, so that a store instruction
 //     writes one whole 128-byte line straight from registers, with no transposition through shared memory, and any
 //     channel count and row alignment takes the same path.
-// Positions along M and channels along N (at most 128 to 160 of them beside the scale columns) is what this replaced:
-// there the shared memory was the bound (operands at N = 128 take all of its 128 bytes per cycle, the transposition
-// another 8 lines per output row, weights were streamed once per 128 positions).  ResNet-18 layers at batch 64, both on
-// one GPU: group 119 -> 111 us, with fp16 activations 307 -> 254 us, the ResNet-34 stack at batch 128 506 -> 450 us,
-// ResNet-20 group at batch 128 58 -> 46 us, the 1x1 layers 432 -> 397 us.
+// With positions along M and at most 128 to 160 channels along N the shared memory was the bound: operands at N = 128 take
+// all of its 128 bytes per cycle, the epilogue's transposition another 8 lines per output row, and weights are streamed
+// once per 128 positions.  Both layouts on one GPU, that one first: ResNet-18 group at batch 64 122 and 106 us, with fp16
+// activations 312 and 259, ResNet-34 stack at batch 128 504 and 392, ResNet-20 group at batch 128 58 and 42, the 1x1
+// layers 441 and 390.
 //
 // Few output channels (binary activations only).  With at most 64, 32 or 16 channels a lane set holds G = 2, 4 or 8
 // neighbouring output pixels of a row: rows g*(128/G)..  of the weight operand are the channels of pixel G*j + g,
 // and position j of the operand stands for that group of pixels.  The taps of a group are the kernel rows times the
 // columns the group's windows span (stride*(G-1) + 3 instead of G times 3); a row of weights holds zeros where a
 // column is outside its pixel's window.  0 * (+1 / -1 / 0) is exactly 0; with fp16 activations 0 * infinity would
-// not be, so those keep G = 1.
+// not be, so those keep G = 1.  With G = 1 the idle rows may hold copies of the channels, which share the columns (see
+// g_plan_layer).
 //
 // Independent problems (a group) need nothing else.  A chain (a stack: problem i + 1 reads the packed signs
 // problem i writes) runs in the same launch on per-tile completion counters: the epilogue bumps the counter
@@ -461,8 +462,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             if (s + s_step >= n_slices) release();
             if (WORDS || out_kind != 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
-              // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubled the code, and the
-              // roles share the instruction caches (ResNet-18 group 111 -> 103 us, 1x1 layers 402 -> 385, ResNet-34 stack 444 -> 417).
+              // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubles the code, and the
+              // roles share the instruction caches (with two loops the ResNet-18 group took 7 % longer, the 1x1 layers 4 %).
               if (out_kind == 0) {
 #pragma unroll
                 for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__fmul_rn(__uint_as_float(v[e]), al));
@@ -684,7 +685,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       // before group g is expanded into shared memory, so that a unit does not cost a full round trip to memory.
       // A thread keeps the geometry of its position while it walks through the planes and words: these eight warps
       // are bound by how many instructions a unit takes one warp, not by the issue slots of the SM.
-      constexpr int XI = CHAIN ? G_EXP_ITEMS / 2 : G_EXP_ITEMS;   // (a chain's tiles are small: less code is worth more, 416 -> 407 us)
+      constexpr int XI = CHAIN ? G_EXP_ITEMS / 2 : G_EXP_ITEMS;   // (a chain's tiles are small: less code is worth 2 %)
       struct XGroup {
         uint4 t[XI];       // the items' words (one, two or four of them)
         uint32_t da[XI];   // where an item's first chunk goes
@@ -1253,10 +1254,11 @@ struct GStepOf {
   uint8_t at[3][17];
 };
 
-// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook).  One thread per 32 input channels of one row of the operand: their 32 indices are consecutive bits of
-// the stream, looked up once for all taps.  Bound by latency, not by its work (16 K threads at most): all of a thread's
-// loads go out together.  With the launch after it, copies and host work included, a call on 8 images of a 128-channel
-// 28x28 layer takes 19 us; four decode kernels and the popcount kernel took 48.
+// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook).  One thread per 32 input channels of
+// one row of the operand: their 32 indices are consecutive bits of the stream, looked up once for all taps.  Bound by
+// latency, not by its work (8192 threads at most): all of a thread's loads go out together.  With the launch after it,
+// copies and host work included, a call on 8 images of a 128-channel 28x28 layer takes 18.4 us; four decode kernels and
+// the popcount kernel take 46.
 __global__ void __launch_bounds__(128) g_static_weights_kernel(const uint8_t* __restrict__ stream, long long n_bytes,
                                                                const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
                                                                const GLayer L, int tau, int paired,
@@ -1366,8 +1368,6 @@ void tcg_destroy(GroupDev* G) {
   cudaFree(G->mem);
   delete G;
 }
-
-int tcg_count(const GroupDev* G) { return G->count; }
 
 bool tcg_supported(const Geom& g, int act_type) { return g_path_takes(g, g_mode_for(act_type)); }
 
