@@ -181,8 +181,8 @@ def run_reference(args):
 # the kernel's sources are the ones that were profiled: {kernel: (workload, batch, bytes, sha256 of sources)}
 _TRAFFIC = {
     # profiles/dram_traffic_resnet18_stack_n64_grouped.txt: mean of the two captured launches
-    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351645312,
-                                             "80cb07752f0febac30141a098d3da70cbee8f49414eaad1867e0df037338bf63"),
+    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351160832,
+                                             "d81498325bdffe3f7b64264f0ec0072f1a7915d3a28ade10a75d463469e0fadb"),
 }
 
 
