@@ -259,7 +259,7 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   P->drain = kind == TCG_WORDS ? (double)Np * G * k_tile * 4 / 16.0 : Np * 5.0;
   // In a launch of this layer alone little else waits for memory: what counts is how many loads one thread does in a row
   // (200 cycles each; 0.2 a chunk where they are many), and the stores go to L2 at 32 bytes a cycle, 24 cycles a column and
-  // 250 a slice of signs for the warp that has the most of them.  Fitted to 12,000 plans: all widths and group sizes of 384
+  // 250 a slice of signs for the warp that has the most of them.  Fitted to 7,500 plans: all widths and group sizes of 384
   // layers of 16 to 512 channels, maps of 6 to 57, 1 to 128 images.
   const int team = G_EXP_THREADS / G_XTEAMS, word_step = g_word_step(g.Cw, d);
   const int loads = (o.Rr + team - 1) / team * o.n_planes * ((d + word_step - 1) / word_step);
