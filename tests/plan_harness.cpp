@@ -62,7 +62,7 @@ int plan_tile(const int* v, int f16, int kind, int lg, int Np, int* rows) {
   return g_writing_warps(plan.L);
 }
 
-// out per problem: lg, Np, tma, tiles.  Returns what is wrong with the plan, or null.
+// out per problem: lg, Np, tma, tiles, channel blocks.  Returns what is wrong with the plan, or null.
 const char* plan_make(const int* gs, int count, int f16, int kind, int sms, int* out) {
   const int mode = f16 ? M_F16 : M_FP4;
   std::vector<Geom> g(count);
@@ -80,8 +80,8 @@ const char* plan_make(const int* gs, int count, int f16, int kind, int sms, int*
   if (!g_ring(plan.data(), count, mode, &ring, &smem)) return "no ring";
   for (int i = 0; i < count; ++i) {
     const GLayer& o = plan[i].L;
-    const int v[4] = {o.lg, o.Np, o.tma, o.total_tiles};
-    memcpy(out + 4 * i, v, sizeof(v));
+    const int v[5] = {o.lg, o.Np, o.tma, o.total_tiles, o.n_cb};
+    memcpy(out + 5 * i, v, sizeof(v));
   }
   return wrong(plan.data(), count, mode, ring, smem);
 }

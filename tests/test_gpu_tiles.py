@@ -57,6 +57,23 @@ def test_binary_tile_edges(snn, oracle_mod, c_in, c_out, h, w, n, stride, pad):
     layer.destroy()
 
 
+@pytest.mark.parametrize("c_in", [65, 96, 160, 214, 224])
+@pytest.mark.parametrize("c_out,h,w,n,stride,pad", [(20, 14, 14, 5, 2, 1), (130, 9, 40, 3, 2, 0), (48, 30, 31, 2, 1, 1), (16, 6, 70, 2, 1, 0)])
+def test_binary_split_blocks(snn, oracle_mod, c_in, c_out, h, w, n, stride, pad):
+    """Odd numbers of activation words: the one tile of a CTA as several units."""
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, pad)
+    p = wl.draw_layer_params(shape, 6, 340 + c_in)
+    packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 341 + w))
+    s_ref, _ = oracle_mod.conv_bin(p.codebook, 6, p.idx_packed, p.alpha, c_in, c_out, stride, pad, packed)
+    layer = snn.SnnConv(c_in, c_out, 6, p.codebook, p.idx_packed, p.alpha, stride, pad)
+    act = torch.from_numpy(packed.view(np.int32)).cuda()
+    assert (layer.forward(act, out_type=snn.OUT_I32).cpu().numpy() == s_ref).all()
+    out = torch.full(s_ref.shape, -7, dtype=torch.int32, device="cuda")
+    snn.forward_static(c_in, c_out, 6, p.codebook, p.idx_packed, p.alpha, act, out, stride, pad, snn.OUT_I32)
+    assert (out.cpu().numpy() == s_ref).all()
+    layer.destroy()
+
+
 def test_binary_tile_edges_in_one_launch(snn, oracle_mod):
     """Members of every group size in one launch: one ring geometry for all of them."""
     shapes = [(wl.LayerShape(16, 16, 32, 32, 1, 1), 9), (wl.LayerShape(40, 32, 9, 13, 2, 1), 2), (wl.LayerShape(64, 64, 20, 21, 1, 1), 6),

@@ -32,8 +32,8 @@ def takes(lib, shape, f16):
 
 
 def make(lib, shapes, f16=False, kind=WORDS):
-    """[(lg, Np, tma, tiles)] of the problems (N, H, W, C, K, stride, pad, ksize)."""
-    out = np.zeros((len(shapes), 4), np.int32)
+    """[(lg, Np, tma, tiles, channel blocks)] of the problems (N, H, W, C, K, stride, pad, ksize)."""
+    out = np.zeros((len(shapes), 5), np.int32)
     err = lib.plan_make(_array(shapes), len(shapes), int(f16), kind, SMS, out.ctypes.data_as(ctypes.POINTER(ctypes.c_int)))
     assert err is None, (err, shapes, f16, kind)
     return out.tolist()
@@ -76,8 +76,19 @@ def test_every_group_of_such_shapes_can_be_planned(lib, f16):
     ((4, 56, 56, 96, 16, 1, 0, 1), SIGNS, 98),
 ])
 def test_a_small_layer_of_few_channels_is_spread_over_the_machine(lib, shape, kind, tiles):
-    (lg, _, _, got), = make(lib, [shape], kind=kind)
+    (lg, _, _, got, _), = make(lib, [shape], kind=kind)
     assert lg <= 1 and got >= tiles   # (a tile of a group of pixels takes two to eight times the MMAs of one of pixels)
+
+
+@pytest.mark.parametrize("shape,blocks", [
+    # both teams of expanders stage the one tile of a CTA where words come one at a time ...
+    ((16, 14, 14, 96, 20, 2, 1, 3), 2), ((9, 43, 55, 83, 48, 2, 1, 3), 2), ((4, 14, 14, 160, 300, 2, 1, 3), 3), ((2, 14, 14, 214, 24, 2, 1, 3), 2),
+    # ... but not where loads are wider, or there are few of them
+    ((4, 14, 14, 128, 64, 2, 1, 3), 1), ((4, 14, 14, 96, 64, 1, 1, 3), 1),
+])
+def test_a_single_tile_is_staged_by_both_teams(lib, shape, blocks):
+    (_, _, _, _, got), = make(lib, [shape])
+    assert got == blocks
 
 
 @pytest.mark.parametrize("c_out", [1, 8, 16, 17, 31, 32, 33, 48, 64, 65, 96, 128, 129, 160, 300])
