@@ -181,8 +181,8 @@ def run_reference(args):
 # the kernel's sources are the ones that were profiled: {kernel: (workload, batch, bytes, sha256 of sources)}
 _TRAFFIC = {
     # profiles/dram_traffic_resnet18_stack_n64_grouped.txt: mean of the two captured launches
-    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351160832,
-                                             "d81498325bdffe3f7b64264f0ec0072f1a7915d3a28ade10a75d463469e0fadb"),
+    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351464832,
+                                             "2aacd569fd126091cadd713af9b2b9fc993619f64de18b93f30db2c2385ed133"),
 }
 
 
