@@ -51,9 +51,11 @@ __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok;
 }
-// Bounded wait for the phase with the given parity; false when the limit ran out.
+// Bounded wait for the phase with the given parity; false when the limit ran out.  (Not unrolled, and neither are the kernel's
+// other loops around waits: the roles share the instruction caches.)
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   if (mbar_test(bar, parity)) return true;
+#pragma unroll 1
   for (uint32_t it = 0; it < WAIT_LIMIT; ++it)
     if (mbar_try_hint(bar, parity, 1000u)) return true;
   return false;
@@ -62,6 +64,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
 // hardware may keep the thread parked per attempt; the attempt limit bounds the whole wait
 // (to a second or so) whatever the hardware makes of the hint.
 __device__ __forceinline__ bool mbar_wait_backoff(uint32_t bar, uint32_t parity, uint32_t ns) {
+#pragma unroll 1
   for (uint32_t it = 0; it < WAIT_LIMIT; ++it)
     if (mbar_try_hint(bar, parity, 20u * ns)) return true;
   return false;

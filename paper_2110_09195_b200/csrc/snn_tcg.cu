@@ -56,6 +56,11 @@
 //      warp 13       writes the epilogue's tables (where the columns of a tile go) ahead of it
 // The kernel is compiled per operand mode and per output kind (words, packed signs, chain), so that no variant
 // carries another one's code in its loops; the plan (tile shapes, accumulator buffers) is made per output kind.
+// The loops around the waits, tiles and problems are not unrolled (the compiler unrolls them four times, innermost and all
+// around): a variant is 62 KB of code then instead of 112, and five kinds of roles share an SM's instruction caches.  On one GPU,
+// as a graph, unrolled and not: 1x1 layers at batch 16 108.8 and 94.6 us (signs 79.8 and 71.0), ResNet-18 group at
+// batch 16 36.7 and 32.3, ResNet-34 stack at batch 128 390 and 362, one layer of 256 channels 9.8 and 9.3, 39 layers 4 %.
+// (Rolling up the expanders' two copies of the load issue as well takes another 12 KB out and made chains 6 % slower.)
 // Every wait is bounded; one that runs out raises a status word the host reads, and
 // the CTA still frees its tensor memory and returns.
 #include <algorithm>
@@ -240,6 +245,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     if (p.n_layers == 1) {
       // a launch of one problem is short: its description comes with the launch, not from memory
       const uint32_t* src = reinterpret_cast<const uint32_t*>(&p.one);
+#pragma unroll 1
       for (int i = tid; i < (int)(sizeof(GLayer) / 4); i += G_THREADS) dst[i] = src[i];
     } else {
       const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
@@ -280,6 +286,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       bool ok = true;
       long long tr_w0 = 0, tr_t0 = clock64();
       (void)tr_w0; (void)tr_t0;
+#pragma unroll 1
       for (int l = 0; l < p.n_layers && ok; ++l) {
         const GLayer& L = lay[l];
         const int n_cb = L.n_cb, n_ct = L.n_ct, total = L.total_tiles, steps = L.steps, st_steps = L.st_steps, n_pu = L.n_pu;
@@ -287,11 +294,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         const uint8_t* wt = L.wt;
         const size_t ct_bytes = (size_t)n_cb * (size_t)steps * step_bytes;   // one channel tile
         const FastDiv dCt = L.dCt;
+#pragma unroll 1
         for (int tile = L.first; tile < total && ok; tile += G) {
           if (*abort_flag) { ok = false; break; }
           const uint8_t* src = wt + (size_t)(tile - (int)fdiv((uint32_t)tile, dCt) * n_ct) * ct_bytes;
+#pragma unroll 1
           for (int u = 0, t = 0; u < n_cb * n_pu && ok; ++u) {
             const int t_last = L.pu_end[u & (n_pu - 1)];
+#pragma unroll 1
             for (t = t >= steps ? 0 : t; t < t_last; t += st_steps) {
               const uint32_t stage_bytes = (uint32_t)(t_last - t < st_steps ? t_last - t : st_steps) * step_bytes;
               if (b_issued >= NS && !TR_WAIT(tr_w0, mbar_wait_backoff(bar_bempty + 8 * b_slot, b_phase, 32))) { ok = false; break; }
@@ -311,6 +321,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       }
       TR_REPORT(0, clock64() - tr_t0, tr_w0, 0, 0);
       // never leave with copies in flight: wait (bounded) for the last load of every slot
+#pragma unroll 1
       for (int s = 0; s < NS; ++s) {
         long long last = -1;
         if (b_issued > s) last = s + (b_issued - 1 - s) / NS * NS;
@@ -333,6 +344,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       (void)tr_w0; (void)tr_w1; (void)tr_w2; (void)tr_t0;
       const uint32_t a_slot_units = p.a_slot_bytes >> 4, b_slot_units = p.b_slot_bytes >> 4;
       const uint32_t a_base = smem_u32(a_smem) >> 4, w_base = smem_u32(b_smem) >> 4, sf = tmem_base + G_SCALE_COL;
+#pragma unroll 1
       for (int l = 0; l < p.n_layers && ok; ++l) {
         const GLayer& L = lay[l];
         const int n_units = L.n_cb * L.n_pu, n_pu = L.n_pu, kpt = L.kpt, total = L.total_tiles;
@@ -347,6 +359,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         const uint32_t idesc =
             F16 ? ((1u << 4) | ((uint32_t)(L.Np >> 3) << 17) | ((128u >> 4) << 24))
                 : ((1u << 7) | (1u << 10) | ((uint32_t)(L.Np >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24));
+#pragma unroll 1
         for (int tile = L.first; tile < total && ok; tile += G, ++tiles_done) {
           if (tiles_done >= n_acc) {
             if (!TR_WAIT(tr_w0, mbar_wait(bar_accempty + 8 * acc_slot, acc_phase))) { ok = false; break; }
@@ -359,6 +372,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             const uint32_t Q0 = fdiv((uint32_t)tile, L.dCt) * (uint32_t)L.Np;
             row0 = 8u * (Q0 - fdiv(Q0, L.dWg) * (uint32_t)L.Wg);
           }
+#pragma unroll 1
           for (int u = 0, t = 0; u < n_units && ok; ++u) {
             if (!TR_WAIT(tr_w1, mbar_wait(bar_afull + 8 * a_slot, a_phase))) { ok = false; break; }
             tc_fence_after();
@@ -556,6 +570,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       }
       return okw != 0;
     };
+#pragma unroll 1
     for (int l = 0; l < p.n_layers && ok; ++l) {
       const GLayer& L = lay[l];
       const FastDiv dWg = L.dWg, dHq = L.dHq, dCt = L.dCt;
@@ -564,6 +579,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const int n_slices = (Np + 31) >> 5;
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
       const uint32_t scale = out_kind == 2 ? 1u : (uint32_t)K;
+#pragma unroll 1
       for (int tile = L.first; tile < total; tile += G, ++seq) {
         if (!take_slot()) { ok = false; break; }
         GTile* const T = reinterpret_cast<GTile*>(epi_smem) + (seq & 3u);
@@ -579,7 +595,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
           *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, lg, out_kind);
         }
-#pragma unroll 4
+#pragma unroll 1
         for (int s = 0; s < n_slices; ++s) {
           const int c = 32 * s + lane;
           const uint32_t q = (uint32_t)mg * (uint32_t)Np + (uint32_t)c;
@@ -587,6 +603,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           const int x = (int)(q - rg * (uint32_t)Wg) << lg, y = (int)(rg - n * (uint32_t)Hq);
           T->offset[c] = ((n * (uint32_t)Ho + (uint32_t)y) * (uint32_t)Wo + (uint32_t)x) * scale;
           const int rem = c < Np && q < Qtot && y < Ho ? Wo - x : 0;   // pixels from x to the end of the row
+#pragma unroll 1
           for (int g = 0; g < (1 << lg); ++g) {
             const uint32_t m = __ballot_sync(0xffffffffu, g < rem);
             if (lane == 0) T->mask[g * G_MAX_CHUNKS + s] = m;
@@ -671,10 +688,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       // Independent problems: all inputs exist when the launch starts and are small beside the L2 (1/29 of the
       // outputs; fp16 inputs are not: half of the outputs).  The CTAs pull them into L2 together, once, so that the
       // staging loads below see L2 latency instead of DRAM latency.
+#pragma unroll 1
       for (int l = 0; l < p.n_layers; ++l) {
         const GLayer& L = lay[l];
         const size_t bytes = (size_t)L.N * L.H * L.W * ((size_t)L.Cw * 4);
         const char* base = reinterpret_cast<const char*>(p.act[l]);
+#pragma unroll 1
         for (size_t off = ((size_t)blockIdx.x * G_EXP_THREADS + et) * 128; off < bytes; off += (size_t)G * G_EXP_THREADS * 128)
           asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
       }
@@ -867,6 +886,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     } else {
       int pending = 0, oldest = 0;   // units whose copies are still in flight, the slot of the oldest
       auto complete = [&](int left) {   // say that all of them but the `left` newest are written
+#pragma unroll 1
         while (pending > left) {
           if (pending == 3) asm volatile("cp.async.wait_group 2;" ::: "memory");
           else if (pending == 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
@@ -876,6 +896,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           --pending;
         }
       };
+#pragma unroll 1
       for (int l = 0; l < p.n_layers && !stop; ++l) {
         const GLayer& L = lay[l];
         const int Rr = L.Rr, n_cb = L.n_cb, cb_chunks = L.cb_chunks, all_rows = L.n_planes * Rr;
@@ -890,9 +911,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           const uint32_t row_bytes = (uint32_t)L.Wg * 128u, ew = (uint32_t)(et >> 5), Hq = (uint32_t)L.Hq;
           const FastDiv dHq = L.dHq, dWg = L.dWg;
           const int n_pu = L.n_pu, rs = L.rs, pad = L.pad, cpl = L.cpl, Np = L.Np;
+#pragma unroll 1
           for (int tile = L.first; tile < total && !stop; tile += G) {
             const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)Np;
             const uint32_t r_first = fdiv(Q0, dWg), r_last = fdiv(Q0 + (uint32_t)Rr - 1u, dWg);
+#pragma unroll 1
             for (int u = 0; u < n_cb * n_pu; ++u) {
               if (pending) complete(0);
               if (a_done >= NA && !wait_slot()) {
@@ -919,15 +942,18 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           continue;
         }
         oldest = pending ? oldest : a_slot;
+#pragma unroll 1
         for (int tile = L.first; tile < total && !stop; tile += G) {
           const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)L.Np;
           // Input pixel of every staged row, once per tile; a thread reads back only entries it wrote itself.
           // (plane, row) pairs form one index space f = plane*Rr + row, dealt to the threads at a stride of
           // the expander count.
+#pragma unroll 1
           for (int f = et; f < all_rows; f += G_EXP_THREADS) {
             const int pl = (int)fdiv((uint32_t)f, dRr);
             pix_tab[f] = g_position_to_pixel(L, Q0 + (uint32_t)(f - pl * Rr), pl);
           }
+#pragma unroll 1
           for (int cb = 0; cb < n_cb; ++cb) {
             // the next slot is not free yet: finish the units in flight first, the MMAs may be waiting for them
             if (pending && a_done >= NA &&
@@ -959,8 +985,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                 }
               }
             } else {
+#pragma unroll 1
               for (int f = et; f < all_rows; f += G_EXP_THREADS) {
                 const int px = pix_tab[f];
+#pragma unroll 1
                 for (int c0 = 0; c0 < cb_chunks; ++c0) {
                   const int ch = (cb * cb_chunks + c0) * 8;
                   uint32_t w[4] = {0, 0, 0, 0};
