@@ -12,18 +12,16 @@
 namespace snn {
 namespace {
 
-// Division by a run-time constant as multiply-high + shifts (round-up method,
-// exact for every 32-bit numerator).
+// Division of a numerator below 2^31 by a run-time constant d below 2^31: q / d = (2q * m) >> (32 + s) with 2^s >= d and
+// m = floor(2^(31 + s) / d) + 1.  m exceeds 2^(31 + s) / d by at most 1, so the quotient by at most q * 2^-(31 + s) < 2^-s <= 1 / d: exact.
 struct FastDiv {
-  uint32_t d, m, s;
+  uint32_t m, s;
 };
 FastDiv make_fastdiv(uint32_t d) {
   FastDiv f;
-  f.d = d;
-  uint32_t s = 0;
-  while ((1ull << s) < d) ++s;
-  f.s = s;
-  f.m = d == 1 ? 0u : (uint32_t)((((1ull << s) - d) << 32) / d + 1);
+  f.s = 0;
+  while ((1ull << f.s) < d) ++f.s;
+  f.m = (uint32_t)((1ull << (31 + f.s)) / d + 1);
   return f;
 }
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }

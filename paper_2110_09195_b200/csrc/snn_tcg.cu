@@ -93,9 +93,7 @@ __device__ long long g_trace[256 * 16];
 #endif
 
 __device__ __forceinline__ uint32_t fdiv(uint32_t q, const FastDiv& f) {
-  if (f.d == 1) return q;
-  const uint32_t t = __umulhi(f.m, q);
-  return (t + ((q - t) >> 1)) >> (f.s - 1);
+  return __umulhi(2u * q, f.m) >> f.s;
 }
 __device__ __forceinline__ int g_position_to_pixel(const GLayer& L, uint32_t q, int pl) {
   if (q >= L.Qtot) return -1;

@@ -54,6 +54,12 @@ extern "C" {
 
 int plan_takes(const int* g, int f16) { return g_path_takes(geom(g), f16 ? M_F16 : M_FP4); }
 
+// q / d as the kernel divides
+uint32_t plan_divide(uint32_t q, uint32_t d) {
+  const FastDiv f = make_fastdiv(d);
+  return (uint32_t)((uint64_t)(2u * q) * f.m >> 32) >> f.s;
+}
+
 // A plan of a given tile: the epilogue warps that write of a position tile, rows a copy or pixel of it has (0: cannot be planned).
 int plan_tile(const int* v, int f16, int kind, int lg, int Np, int* rows) {
   GPlan plan;

@@ -126,3 +126,13 @@ def test_copies_only_where_the_stores_take_longer_than_the_mmas(lib, c_in, c_out
     rows = ctypes.c_int(0)
     assert lib.plan_tile(_array((64, 32, 32, c_in, c_out, 1, 1, 3)), 1, WORDS, 0, 256, ctypes.byref(rows))
     assert (rows.value < 128) == copies
+
+
+def test_division_by_run_time_constants_is_exact_below_2_to_the_31(lib):
+    lib.plan_divide.restype = ctypes.c_uint32
+    rng = random.Random(9)
+    top = (1 << 31) - 1
+    for d in [*range(1, 130), *(1 << k for k in range(31)), *((1 << k) - 1 for k in range(2, 32)), *(rng.randint(1, top) for _ in range(200))]:
+        last = top // d * d   # the largest multiple: the quotient changes there
+        for q in (0, 1, d - 1, d, min(2 * d - 1, top), last - 1 if last else 0, last, top, *(rng.randint(0, top) for _ in range(20))):
+            assert lib.plan_divide(q, d) == q // d, (q, d)
