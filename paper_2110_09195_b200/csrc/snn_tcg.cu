@@ -147,13 +147,35 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
   constexpr uint64_t fixed = ((uint64_t)1 << 46) | ((uint64_t)8 << 32);   // descriptor version; 8-row groups 128 bytes apart
   constexpr uint64_t w_fixed = fixed | ((uint64_t)128 << 16);             // the weights' chunks are 128 rows apart
   const int st_steps = L.st_steps;
-  uint32_t tap = L.tap[t];
+  uint32_t tap = MODE == M_FP4 && KPT == 1 ? 0u : L.tap[t];
 #pragma unroll 1
   while (t < t_last) {
     // a weight stage holds whole steps: one wait, then nothing but MMAs until its last step
     if (!TR_WAIT(tr_b, mbar_wait(bar_bfull + 8 * b_slot, b_phase))) return false;
     tc_fence_after();
     uint32_t wa = w_base + (uint32_t)b_slot * b_slot_units;
+    if constexpr (MODE == M_FP4 && KPT == 1) {
+      // One MMA a step: those of a stage are straight-line code behind one branch, their taps read together.  In the loop
+      // below the read, the branch and the address arithmetic of a step run between two MMAs (one warp by itself, 9 MMAs of
+      // 64 positions: 1870 cycles, so 1080; 70 channels 45x37 at stride 2: 8.0 and 7.4 us).  With two or more MMAs a step, and
+      // with fp16 operands, the longer code costs the other roles more than this gains (fp16 group at batch 1 12 %).
+      constexpr int ST = (int)(kGBSlot / (KPT * 2 * G_ROWS * 16));   // most steps of a stage (g_plan_layer)
+      const int n = t_last - t < st_steps ? t_last - t : st_steps;
+      if (leader) {
+        uint32_t rows[ST];
+#pragma unroll
+        for (int i = 0; i < ST; ++i) rows[i] = i < n ? L.tap[t + i] + a_unit : 0u;   // (start and chunk distance of the low word)
+#pragma unroll
+        for (int i = 0; i < ST; ++i) {
+          if (i < n) mma_ss_fp4(d0, w_fixed | (uint64_t)(wa + (uint32_t)(i * 256)), a_fixed | (uint64_t)rows[i], idesc, i == 0 ? acc : 1u, sf, sf + 16);
+        }
+        tc_commit(bar_bempty + 8 * b_slot);
+      }
+      t += n;
+      acc = 1;
+      if (++b_slot == NS) { b_slot = 0; b_phase ^= 1u; }
+      continue;
+    }
     const int t_end = t + st_steps < t_last ? t + st_steps : t_last;
 #pragma unroll 1
     for (; t < t_end; ++t) {
