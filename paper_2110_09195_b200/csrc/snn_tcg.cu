@@ -249,53 +249,64 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   const int NS = p.NS, NA = p.NA;
   const int G = (int)gridDim.x;
 
-  if (tid < 40) {
-    uint32_t count = 1;
-    if ((tid >= 28 && tid < 32) || tid >= 36) count = G_EW;               // acc_empty, tab_empty: one arrival per epilogue warp of the tile
-    if (tid >= 16 && tid < 20) count = FP4 ? G_EW / G_XTEAMS : G_EW;    // a_full: one arrival per expander warp of the unit
-    mbar_init(smem_u32(bars + tid), count);
-  }
-  if (tid == 64) {
-    *abort_flag = 0;
-    *ready_tiles = 0;
-  }
-  int first = (int)blockIdx.x;
-  {
-    uint32_t* dst = reinterpret_cast<uint32_t*>(smem + p.off_lay);
-    if (p.n_layers == 1) {
-      // a launch of one problem is short: its description comes with the launch, not from memory
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(&p.one);
-#pragma unroll 1
-      for (int i = tid; i < (int)(sizeof(GLayer) / 4); i += G_THREADS) dst[i] = src[i];
-    } else {
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
-      const int words = p.n_layers * (int)(sizeof(GLayer) / 4);
-      for (int i = tid; i < words; i += G_THREADS) dst[i] = __ldg(src + i);
-      // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
-      if (tid < p.n_layers) first = (int)__ldg(p.ranks + (size_t)tid * G + blockIdx.x);
-    }
-  }
+  // Set-up.  Warp 2 allocates tensor memory while the others write the barriers and the problems' descriptions; only the MMA
+  // issuer and the epilogue warps wait for it (barrier 1).  The producer, the expanders and the table warp start as
+  // soon as the descriptions are there (barrier 2): 39 single layers 1.4 % faster, as a graph, than with both behind two barriers
+  // of all threads.
+  constexpr int SETUP_THREADS = G_THREADS - 32;
+  uint32_t tmem_base = 0;
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                  "r"(512)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  } else {
+    const int rank = warp > 2 ? tid - 32 : tid;
+    if (rank < 40) {
+      uint32_t count = 1;
+      if ((rank >= 28 && rank < 32) || rank >= 36) count = G_EW;               // acc_empty, tab_empty: one arrival per epilogue warp of the tile
+      if (rank >= 16 && rank < 20) count = FP4 ? G_EW / G_XTEAMS : G_EW;    // a_full: one arrival per expander warp of the unit
+      mbar_init(smem_u32(bars + rank), count);
+    }
+    if (rank == 64) {
+      *abort_flag = 0;
+      *ready_tiles = 0;
+    }
+    constexpr int at_first = (int)offsetof(GLayer, first) / 4;   // (this CTA's first tile is put in here)
+    uint32_t* dst = reinterpret_cast<uint32_t*>(smem + p.off_lay);
+    if (p.n_layers == 1) {
+      // a launch of one problem is short: its description comes with the launch, not from memory
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(&p.one);
+#pragma unroll 1
+      for (int i = rank; i < (int)(sizeof(GLayer) / 4); i += SETUP_THREADS) dst[i] = i == at_first ? blockIdx.x : src[i];
+    } else {
+      const uint32_t* src = reinterpret_cast<const uint32_t*>(p.layers);
+      const int words = p.n_layers * (int)(sizeof(GLayer) / 4);
+      for (int i = rank; i < words; i += SETUP_THREADS) dst[i] = __ldg(src + i);
+      // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
+      int first = 0;
+      if (rank < p.n_layers) first = (int)__ldg(p.ranks + (size_t)rank * G + blockIdx.x);
+      asm volatile("bar.sync 2, %0;" ::"n"(SETUP_THREADS) : "memory");
+      if (rank < p.n_layers) lay[rank].first = first;
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("bar.sync 2, %0;" ::"n"(SETUP_THREADS) : "memory");
   }
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
   grid_dep_launch();
-  if (tid < p.n_layers) lay[tid].first = first;
-  if (FP4) {
-    // unit block scales: every byte of the scale columns is the ue8m0 code of 1.0, in all 128 lanes
-    // (warps 2..5 cover the four lane quarters), whatever part of them an MMA reads
-    if (warp >= 2 && warp < 6) tmem_fill32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + G_SCALE_COL, 0x7f7f7f7fu);
+  if (warp >= 1 && warp < 2 + G_EW) {
     tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * (1 + G_EW)) : "memory");
+    tc_fence_after();
+    tmem_base = *tmem_slot;
+    if (FP4) {
+      // unit block scales: every byte of the scale columns is the ue8m0 code of 1.0, in all 128 lanes
+      // (warps 2..5 cover the four lane quarters), whatever part of them an MMA reads
+      if (warp >= 2 && warp < 6) tmem_fill32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + G_SCALE_COL, 0x7f7f7f7fu);
+      tc_fence_before();
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * (1 + G_EW)) : "memory");
+      tc_fence_after();
+    }
   }
-  __syncthreads();
-  if (FP4) tc_fence_after();
 
   if (warp == 0) {
     // ------------------------------------------------ weight producer (one lane)
