@@ -870,27 +870,18 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       seek_own();
       // completion side: this team's slots gx, gx + XG, ... of the ring
       a_slot = gx;
-      XGroup cur, nxt;
-      bool nvalid = false;
-      while (ivalid || nvalid) {
-        if (!nvalid) {
-          if (!check_ready(true)) {
-            if (lane == 0 && !*abort_flag) {
-              *abort_flag = 1;
-              raise_status(p.status, 5);
-            }
-            stop = true;
-            break;
-          }
-          issue(nxt);
+      XGroup cur = {}, nxt;
+      auto not_ready = [&]() {     // the wait for a chain's input ran out
+        if (lane == 0 && !*abort_flag) {
+          *abort_flag = 1;
+          raise_status(p.status, 5);
         }
-        cur = nxt;
-        // (a chain's next input may depend on the unit in hand: it is only looked at, never waited for, here)
-        nvalid = ivalid && check_ready(false);
-        if (nvalid) issue(nxt);
+        stop = true;
+      };
+      auto expand = [&]() {        // the group in hand into shared memory
         if ((cur.flags & 0x200u) && a_done >= NA / XG && !wait_slot()) {
           stop = true;
-          break;
+          return;
         }
 #pragma unroll
         for (int j = 0; j < XI; ++j) {
@@ -913,6 +904,36 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           ++a_done;
           a_slot += XG;
           if (a_slot >= NA) { a_slot -= NA; a_phase ^= 1u; }
+        }
+      };
+      if constexpr (CHAIN) {
+        bool nvalid = false;
+        while (ivalid || nvalid) {
+          if (!nvalid) {
+            if (!check_ready(true)) {
+              not_ready();
+              break;
+            }
+            issue(nxt);
+          }
+          cur = nxt;
+          // (the next input may depend on the unit in hand: it is only looked at, never waited for, here)
+          nvalid = ivalid && check_ready(false);
+          if (nvalid) issue(nxt);
+          expand();
+          if (stop) break;
+        }
+      } else {
+        // One copy of the load issue instead of two: 10 KB of code.  (In chains, whose tiles are small, two are 1 to 3 % faster.)
+        bool in_hand = false;   // is there a group to expand?
+#pragma unroll 1
+        for (;;) {
+          const bool more = ivalid;
+          if (more) issue(nxt);
+          if (in_hand) expand();
+          if (!more || stop) break;
+          cur = nxt;
+          in_hand = true;
         }
       }
     } else {
