@@ -99,6 +99,13 @@ __device__ __forceinline__ bool elect_one() {
   return elected != 0;
 }
 
+// Barrier ID among THREADS of the CTA's threads, whole warps (which come together first: the barrier counts warps).
+template <int ID, int THREADS>
+__device__ __forceinline__ void bar_sync_some() {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(THREADS) : "memory");
+}
+
 // Programmatic dependent launch: a kernel launched with the serialization attribute may start
 // while its predecessor in the stream still runs; grid_dep_wait() blocks until the predecessor has
 // completed and its writes are visible (a no-op for an ordinary launch), grid_dep_launch() lets the

@@ -286,16 +286,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
       int first = 0;
       if (rank < p.n_layers) first = (int)__ldg(p.ranks + (size_t)rank * G + blockIdx.x);
-      asm volatile("bar.sync 2, %0;" ::"n"(SETUP_THREADS) : "memory");
+      bar_sync_some<2, SETUP_THREADS>();
       if (rank < p.n_layers) lay[rank].first = first;
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("bar.sync 2, %0;" ::"n"(SETUP_THREADS) : "memory");
+    bar_sync_some<2, SETUP_THREADS>();
   }
   grid_dep_launch();
   if (warp >= 1 && warp < 2 + G_EW) {
     tc_fence_before();
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * (1 + G_EW)) : "memory");
+    bar_sync_some<1, 32 * (1 + G_EW)>();
     tc_fence_after();
     tmem_base = *tmem_slot;
     if (FP4) {
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       // (warps 2..5 cover the four lane quarters), whatever part of them an MMA reads
       if (warp >= 2 && warp < 6) tmem_fill32(tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + G_SCALE_COL, 0x7f7f7f7fu);
       tc_fence_before();
-      asm volatile("bar.sync 1, %0;" ::"n"(32 * (1 + G_EW)) : "memory");
+      bar_sync_some<1, 32 * (1 + G_EW)>();
       tc_fence_after();
     }
   }
