@@ -44,7 +44,7 @@ constexpr int G_MAX_CHUNKS = 8;                // 32-column slices of an accumul
 // What the epilogue needs to know of a tile, written by the table warp (see there), four tiles deep.
 struct GTile {
   int l, mg, co, n_slices;             // problem (-1: no more tiles), position tile, first channel, 32-column slices
-  int K, kp_log, lg, out_kind;         // channels; GLayer::kp_log, lg; 0 fp32, 1 int32, 2 packed signs
+  int K, kp_log, lg, out_kind;         // channels; GLayer::kp_log, lg; GParams::out_type
   uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
   uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
   float alpha[G_ROWS], shift[G_ROWS];
@@ -102,7 +102,8 @@ struct GParams {
   const void* act[SNN_GROUP_MAX];
   void* out[SNN_GROUP_MAX];
   int* status;
-  uint8_t out_type[SNN_GROUP_MAX];   // per member: 0 fp32 alpha*S, 1 int32 S, 2 packed signs of alpha*S + shift
+  uint32_t* launches;     // chain of words with tags: [grid] launches each CTA has been through; the next one's tag is one more
+  uint8_t out_type[SNN_GROUP_MAX];   // per member: 0 fp32 alpha*S, 1 int32 S, 2 packed signs of alpha*S + shift, 3 those with tags
   uint32_t acc_cols;      // tensor-memory columns of one accumulator buffer
   int n_acc;              // accumulator buffers (tile seq of a CTA uses buffer seq % n_acc)
   int NA, NS;
@@ -408,6 +409,13 @@ bool g_plan_by_end(const Geom& g, int mode, int kind, int sms, GPlan* plan) {
   }
   return best >= 0 && g_plan_layer(g, mode, kind, best_lg, best_np, false, plan);
 }
+
+// Do the packed signs between the members of a chain carry tags?  words: the most between two members.  A layer's signs then reach
+// the next layer's expanders 1.2 us sooner, but each word is twice as long and the expanders load two of them at a time
+// instead of four, which shows once a CTA has many tiles.  Measured on one B200 as graphs, counters and tags, us: ResNet-18 stack
+// batch 1 88 and 69, batch 8 95 and 82, 16 (100 k words) 100 and 99, 32 113 and 117, 64 134 and 145; ResNet-34 batch 1 169 and 132,
+// 16 191 and 188, 32 219 and 226; ResNet-20 batch 1 72 and 52, 64 99 and 88, 96 104 and 96, 128 (131 k words) 124 and 119.
+inline bool g_tagged(size_t words) { return words <= (size_t)1 << 17; }
 
 // The ring geometry of a launch of these problems and where its parts lie in shared memory; false where it does not fit.
 bool g_ring(const GPlan* plan, int count, int mode, GParams* p, size_t* smem) {

@@ -33,7 +33,10 @@
 // g_plan_layer).
 //
 // Independent problems (a group) need nothing else.  A chain (a stack: problem i + 1 reads the packed signs
-// problem i writes) runs in the same launch on per-tile completion counters: the epilogue bumps the counter
+// problem i writes) runs in the same launch.  Where few words lie between its members (g_tagged) every word carries the tag of
+// the launch that wrote it, and the expanders look at the words themselves until all they need are there: no fence, counter
+// or memset between a sign and its reader.  The tag is a count of launches kept per CTA in device memory, so that a
+// replayed graph counts too.  Other chains run on per-tile completion counters: the epilogue bumps the counter
 // of a position tile when its part is written, and the expanders of the successor wait (bounded) until the
 // tiles under a tile's input window are complete.  The launch is cooperative then, so that all CTAs are
 // resident while some of them wait.
@@ -131,6 +134,18 @@ __device__ __forceinline__ uint2 g_ld2(const uint32_t* p, bool fresh) {
 __device__ __forceinline__ uint4 g_ld4(const uint32_t* p, bool fresh) {
   return fresh ? __ldcg(reinterpret_cast<const uint4*>(p)) : __ldg(reinterpret_cast<const uint4*>(p));
 }
+// Words with tags, between the members of a chain: the word in the low half, the tag of the launch that wrote it in the high half,
+// stored and loaded 64 bits at once.  A word whose tag is this launch's is this launch's word, so that neither side
+// needs a fence or a counter.
+__device__ __forceinline__ void g_st_tagged(void* p, size_t i, uint32_t word, uint32_t tag) {
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(reinterpret_cast<uint64_t*>(p) + i), "l"((uint64_t)word | (uint64_t)tag << 32) : "memory");
+}
+__device__ __forceinline__ uint4 g_ld_tagged(const uint64_t* p, bool two) {   // a word and its tag, or two of each
+  uint64_t a, b = 0;
+  if (two) asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  else asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(a) : "l"(p) : "memory");
+  return make_uint4((uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32));
+}
 // Tensor maps of the fp16 activations, a kernel parameter of its own (the other variants have one unused entry).
 template <int MODE>
 struct GMaps {
@@ -215,13 +230,14 @@ __device__ __forceinline__ uint32_t g_transpose32(uint32_t x, int lane) {
 
 // OUTK: what the epilogue is compiled for.  0: fp32 or int32 words for every member; 1: packed signs for every
 // member; 2: a chain - packed signs between the members, any type for the last, and the dependency waits and
-// completion counters.  Keeping the variants apart keeps each one's registers and code to what it needs.
-enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2 };
+// completion counters; 3: a chain whose words carry tags instead.  Keeping the variants apart keeps each one's registers and code to what it needs.
+enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2, OUT_TAGGED = 3 };
 
 template <int MODE, int OUTK>
 __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_constant__ GParams p, const __grid_constant__ GMaps<MODE> maps) {
   constexpr bool F16 = MODE == M_F16;   // fp16 activations (copied, not expanded)
   constexpr bool FP4 = MODE == M_FP4;   // binary activations as e2m1 nibbles
+  constexpr bool TAGGED = OUTK == OUT_TAGGED;   // a chain without waits for whole tiles: every word is looked at until it is there
   constexpr bool CHAIN = OUTK == OUT_CHAIN;
   constexpr bool WORDS = OUTK == OUT_WORDS;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -293,6 +309,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     bar_sync_some<2, SETUP_THREADS>();
   }
   grid_dep_launch();
+  const uint32_t tag = TAGGED ? __ldcg(p.launches + blockIdx.x) + 1u : 0u;   // the same in all CTAs (counted up at the end)
   if (warp >= 1 && warp < 2 + G_EW) {
     tc_fence_before();
     bar_sync_some<1, 32 * (1 + G_EW)>();
@@ -505,7 +522,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             __syncwarp();   // the load is a warp-wide instruction
             tmem_ld32(d0 + (uint32_t)(32 * s), v);
             if (s + s_step >= n_slices) release();
-            if (WORDS || out_kind != 2) {
+            if (WORDS || out_kind < 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
               // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubles the code, and the
               // roles share the instruction caches (with two loops the ResNet-18 group took 7 % longer, the 1x1 layers 4 %).
@@ -557,7 +574,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
               const uint32_t px = T->offset[32 * s + lane], here = 1u << lane;
               const uint32_t Kw = (uint32_t)(K + 31) >> 5;
               if (kp_log >= 5) {
-                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) out32[wide_mul(px + (uint32_t)g_warp, Kw) + (uint32_t)(co_warp >> 5)] = w;
+                const size_t at = wide_mul(px + (uint32_t)g_warp, Kw) + (uint32_t)(co_warp >> 5);
+                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) {
+                  if (TAGGED && out_kind == 3) g_st_tagged(out32, at, w, tag);
+                  else out32[at] = w;
+                }
+              } else if (TAGGED && out_kind == 3) {
+                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) g_st_tagged(out32, px + (uint32_t)g_warp, w & 0xffffu, tag);
+                if (T->mask[(g_warp + 1) * G_MAX_CHUNKS + s] & here) g_st_tagged(out32, px + (uint32_t)g_warp + 1, w >> 16, tag);
               } else {   // 16 rows per pixel: one word each for two pixels
                 if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) out32[px + (uint32_t)g_warp] = w & 0xffffu;
                 if (T->mask[(g_warp + 1) * G_MAX_CHUNKS + s] & here) out32[px + (uint32_t)g_warp + 1] = w >> 16;
@@ -609,7 +633,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const uint32_t Qtot = L.Qtot;
       const int n_slices = (Np + 31) >> 5;
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
-      const uint32_t scale = out_kind == 2 ? 1u : (uint32_t)K;
+      const uint32_t scale = out_kind >= 2 ? 1u : (uint32_t)K;
 #pragma unroll 1
       for (int tile = L.first; tile < total; tile += G, ++seq) {
         if (!take_slot()) { ok = false; break; }
@@ -715,7 +739,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_afull + 8 * slot);
     };
-    if (FP4 && !CHAIN && (p.n_layers > 1 || lay[0].total_tiles > G)) {
+    if (FP4 && !CHAIN && !TAGGED && (p.n_layers > 1 || lay[0].total_tiles > G)) {
       // Independent problems: all inputs exist when the launch starts and are small beside the L2 (1/29 of the
       // outputs; fp16 inputs are not: half of the outputs).  The CTAs pull them into L2 together, once, so that the
       // staging loads below see L2 latency instead of DRAM latency.  (Not where every CTA has one tile: its loads go out now anyway,
@@ -736,13 +760,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       // before group g is expanded into shared memory, so that a unit does not cost a full round trip to memory.
       // A thread keeps the geometry of its position while it walks through the planes and words: these eight warps
       // are bound by how many instructions a unit takes one warp, not by the issue slots of the SM.
-      constexpr int XI = CHAIN ? G_EXP_ITEMS / 2 : G_EXP_ITEMS;   // (a chain's tiles are small: less code is worth 2 %)
+      constexpr int XI = CHAIN || TAGGED ? G_EXP_ITEMS / 2 : G_EXP_ITEMS;   // (a chain's tiles are small: less code is worth 2 %)
       struct XGroup {
         uint4 t[XI];       // the items' words (one, two or four of them)
         uint32_t da[XI];   // where an item's first chunk goes
         uint32_t cstride;  // bytes from one chunk to the next
         uint32_t flags;    // bit j: item j exists; bit 4 + j: its words exist (the pixel is inside the image); bits
-                           // 12..14: words per item; 9: first group of its unit; 10: last group of its unit
+                           // 12..14: words per item; 9: first group of its unit; 10: last group of its unit; 11: words with tags
+        const uint64_t* src[TAGGED ? XI : 1];   // words with tags: where they are, to be looked at again
       };
       // The expander warps form XG teams that take the units in turn (the ring has a multiple of XG slots, so a
       // slot always belongs to the same team): with few rows per unit a unit is a chain of latencies, and two
@@ -766,21 +791,35 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         ready = !CHAIN;
         ++tile_seq;
       };
+      auto read_layer = [&]() {
+        const GLayer& L = lay[il];
+        Rr = L.Rr; n_cb = L.n_cb; cbc = L.cb_chunks; Cw = L.Cw; planes = L.n_planes; cpl = L.cpl; H = L.H; W = L.W; cs = L.cs;
+        act = reinterpret_cast<const uint32_t*>(p.act[il]);
+        kstep = g_word_step(Cw, cbc);
+        if (TAGGED && il > 0 && kstep > 2) kstep = 2;
+        icb = 0;
+        ivalid = true;
+        enter_tile();
+      };
       auto enter_layer = [&]() {   // first layer from il on in which this CTA has a tile
-        for (; il < p.n_layers; ++il) {
-          const GLayer& L = lay[il];
-          itile = L.first;
-          itotal = L.total_tiles;
-          if (itile >= itotal) continue;
-          Rr = L.Rr; n_cb = L.n_cb; cbc = L.cb_chunks; Cw = L.Cw; planes = L.n_planes; cpl = L.cpl; H = L.H; W = L.W; cs = L.cs;
-          act = reinterpret_cast<const uint32_t*>(p.act[il]);
-          kstep = g_word_step(Cw, cbc);
-          icb = 0;
-          ivalid = true;
-          enter_tile();
-          return;
+        if constexpr (TAGGED) {
+          // (not the loop below: compiled for this variant, one of its copies went on to the next layer after it had found one)
+#pragma unroll 1
+          while (il < p.n_layers && (itile = lay[il].first) >= lay[il].total_tiles) ++il;
+          ivalid = il < p.n_layers;
+          if (!ivalid) return;
+          itotal = lay[il].total_tiles;
+          read_layer();
+        } else {
+          for (; il < p.n_layers; ++il) {
+            itile = lay[il].first;
+            itotal = lay[il].total_tiles;
+            if (itile >= itotal) continue;
+            read_layer();
+            return;
+          }
+          ivalid = false;
         }
-        ivalid = false;
       };
       auto next_unit = [&]() {     // the unit after (il, itile, icb) in the CTA's sequence
         ++iu;
@@ -814,13 +853,18 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         const GLayer& L = lay[il];
         const bool fresh = CHAIN && L.deps != nullptr;   // written by other CTAs of this launch: read from L2
         const uint32_t cstride = (uint32_t)(planes * Rr) * 16u;
-        uint32_t flags = ((uint32_t)kstep << 12) | ((pos0 | ipl | ik0) == 0 ? 0x200u : 0u);
+        const bool tagged = TAGGED && il > 0;   // (the first member's input is the caller's)
+        uint32_t flags = ((uint32_t)kstep << 12) | ((pos0 | ipl | ik0) == 0 ? 0x200u : 0u) | (tagged ? 0x800u : 0u);
+        // the items of a position are dealt to 2^tpl neighbouring threads, so that a small tile's are all looked at together
+        // instead of one look after another
+        const int items = cbc >> (kstep >> 1), tpl = !TAGGED ? 0 : items == 4 ? 2 : items == 2 ? 1 : 0;
+        const int own = TAGGED ? (etg & ((1 << tpl) - 1)) * kstep : 0;   // this thread's words of a position start there
         const uint32_t unit = smem_u32(a_smem) + (uint32_t)i_slot * p.a_slot_bytes;
         bool ended = false;
 #pragma unroll
         for (int j = 0; j < XI; ++j) {
           if (ended) break;
-          const int pos = pos0 + etg;
+          const int pos = pos0 + (TAGGED ? etg >> tpl : etg), ik = ik0 + own;
           if ((ipl | ik0) == 0) {
             const uint32_t q = Q0 + (uint32_t)pos;
             const uint32_t rg = fdiv(q, L.dWg), n = fdiv(rg, L.dHq);
@@ -829,15 +873,19 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             img_row = (int)n * H;
             inside = q < L.Qtot;
           }
-          const int r = row + (ipl >> cpl), c = col + cs * (ipl & ((1 << cpl) - 1)), word = icb * cbc + ik0;
+          const int r = row + (ipl >> cpl), c = col + cs * (ipl & ((1 << cpl) - 1)), word = icb * cbc + ik;
           const bool on = inside && pos < Rr && (uint32_t)r < (uint32_t)H && (uint32_t)c < (uint32_t)W && word < Cw;
-          g.da[j] = unit + (uint32_t)ik0 * cstride + (uint32_t)(ipl * Rr + pos) * 16u;
+          g.da[j] = unit + (uint32_t)ik * cstride + (uint32_t)(ipl * Rr + pos) * 16u;
           g.t[j] = make_uint4(0, 0, 0, 0);
           if (pos < Rr) flags |= 1u << j;
           if (on) {
             flags |= 0x10u << j;
-            const uint32_t* src = act + wide_mul((uint32_t)((img_row + r) * W + c), (uint32_t)Cw) + word;
-            if (kstep == 4) {
+            const size_t at = wide_mul((uint32_t)((img_row + r) * W + c), (uint32_t)Cw) + (size_t)word;
+            const uint32_t* src = act + at;
+            if (TAGGED && tagged) {
+              g.src[TAGGED ? j : 0] = reinterpret_cast<const uint64_t*>(act) + at;
+              g.t[j] = g_ld_tagged(g.src[TAGGED ? j : 0], kstep == 2);
+            } else if (kstep == 4) {
               g.t[j] = g_ld4(src, fresh);
             } else if (kstep == 2) {
               const uint2 v = g_ld2(src, fresh);
@@ -847,12 +895,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
               g.t[j].x = g_ld1(src, fresh);
             }
           }
-          ik0 += kstep;
+          ik0 += TAGGED ? kstep << tpl : kstep;
           if (ik0 >= cbc) {
             ik0 = 0;
             if (++ipl == planes) {
               ipl = 0;
-              pos0 += XT;
+              pos0 += TAGGED ? XT >> tpl : XT;
               ended = pos0 >= Rr;
             }
           }
@@ -906,6 +954,27 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           if (a_slot >= NA) { a_slot -= NA; a_phase ^= 1u; }
         }
       };
+      // words with tags: looks (bounded) until all of the group's are this launch's
+      auto settle = [&]() -> bool {
+        const bool two = (cur.flags & 0x6000u) != 0;
+#pragma unroll 1
+        for (uint32_t it = 0;; ++it) {
+          bool all = true;
+#pragma unroll
+          for (int j = 0; j < XI; ++j) {
+            if ((cur.flags & (0x10u << j)) && (cur.t[j].y != tag || (two && cur.t[j].w != tag))) {
+              all = false;
+              cur.t[j] = g_ld_tagged(cur.src[TAGGED ? j : 0], two);
+            }
+          }
+          if (__all_sync(0xffffffffu, all)) break;
+          if (it >= (1u << 21) || __any_sync(0xffffffffu, *abort_flag != 0)) return false;
+          if (it > 2) __nanosleep(20);
+        }
+#pragma unroll
+        for (int j = 0; j < XI; ++j) cur.t[j].y = cur.t[j].z;
+        return true;
+      };
       if constexpr (CHAIN) {
         bool nvalid = false;
         while (ivalid || nvalid) {
@@ -930,6 +999,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         for (;;) {
           const bool more = ivalid;
           if (more) issue(nxt);
+          if (TAGGED && in_hand && (cur.flags & 0x800u) && !settle()) {
+            not_ready();
+            break;
+          }
           if (in_hand) expand();
           if (!more || stop) break;
           cur = nxt;
@@ -1078,6 +1151,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   // ---------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
+  if (TAGGED && tid == 0) p.launches[blockIdx.x] = tag;
   if (warp == 2) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
   }
@@ -1091,6 +1165,7 @@ struct GroupDev {
   uint8_t* mem = nullptr;         // all device memory of the group; the pointers below lie in it
   uint8_t* chain_buf = nullptr;   // the packed signs between the members, one buffer per boundary
   size_t chain_off[SNN_GROUP_MAX] = {};
+  int tagged = 0;                 // a chain of words with tags (and without counters)
   uint32_t* done = nullptr;       // completion counters of all members' position tiles
   size_t done_words = 0;
   GLayer* layers_dev = nullptr;   // [count]
@@ -1202,6 +1277,9 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   std::vector<size_t> deps_off(count, 0), done_off(count, 0);
   size_t done_words = 0, chain_bytes = 0;
   size_t chain_off[SNN_GROUP_MAX] = {};
+  size_t words = 0;   // most words between two members
+  for (int i = 0; i + 1 < count && chain; ++i) words = std::max(words, (size_t)gs[i].N * gs[i].Ho * gs[i].Wo * ((gs[i].K + 31) / 32));
+  const bool tagged = chain && g_tagged(words);
   if (chain) {
     for (int i = 0; i < count; ++i) {
       if (i > 0 && (gs[i].C != gs[i - 1].K || gs[i].H != gs[i - 1].Ho || gs[i].W != gs[i - 1].Wo || gs[i].N != gs[0].N))
@@ -1209,12 +1287,12 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
       const GLayer& L = plan[i].L;
       const int mgroups = L.total_tiles / L.n_ct;
       done_off[i] = done_words;
-      done_words += (size_t)mgroups;
+      if (!tagged) done_words += (size_t)mgroups;
       if (i + 1 < count) {
         chain_off[i] = chain_bytes;
-        chain_bytes += (((size_t)gs[i].N * gs[i].Ho * gs[i].Wo * ((gs[i].K + 31) / 32) * 4) + 255) & ~(size_t)255;
+        chain_bytes += ((size_t)gs[i].N * gs[i].Ho * gs[i].Wo * ((gs[i].K + 31) / 32) * (tagged ? 8 : 4) + 255) & ~(size_t)255;
       }
-      if (i == 0) continue;
+      if (i == 0 || tagged) continue;
       // which position tiles of the predecessor hold the input pixels of each of this member's position tiles
       const GLayer& P = plan[i - 1].L;
       deps_off[i] = deps.size();
@@ -1261,7 +1339,8 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
   const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint16_t));
   const size_t blob_bytes = deps_at + up(deps.size() * sizeof(uint2)), blob_at = up(w_total), done_at = blob_at + blob_bytes;
-  const size_t chain_at = done_at + up(done_words * sizeof(uint32_t));
+  const size_t launches_at = done_at + up(done_words * sizeof(uint32_t));
+  const size_t chain_at = launches_at + (tagged ? up((size_t)grid * sizeof(uint32_t)) : 0);
   cudaError_t e = cudaMalloc(&Gd->mem, chain_at + chain_bytes);
   if (e == cudaSuccess) {
     Gd->layers_dev = reinterpret_cast<GLayer*>(Gd->mem + blob_at);
@@ -1270,6 +1349,9 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     Gd->chain_buf = Gd->mem + chain_at;
   }
   Gd->done_words = done_words;
+  Gd->tagged = tagged;
+  // no launch has written a word yet: tags start at 1
+  if (tagged && e == cudaSuccess) e = cudaMemsetAsync(Gd->mem + launches_at, 0, chain_at + chain_bytes - launches_at, s);
   for (int i = 0; i < count; ++i) Gd->chain_off[i] = chain_off[i];
   const uint2* const deps_dev = reinterpret_cast<const uint2*>(Gd->mem + blob_at + deps_at);
   std::vector<uint8_t> blob(blob_bytes);
@@ -1279,7 +1361,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     Gd->map[i] = {L.tma != 0, L.C, L.W, L.H, L.N, L.rs, L.Wg};
     L.alpha = Ls[i]->alpha;
     L.shift = Ls[i]->shift;
-    if (chain) {
+    if (chain && !tagged) {
       L.done = Gd->done + done_off[i];
       if (i > 0) {
         L.deps = deps_dev + deps_off[i];
@@ -1313,6 +1395,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->p = ring;
   Gd->p.layers = Gd->layers_dev;
   Gd->p.ranks = Gd->ranks;
+  if (tagged) Gd->p.launches = reinterpret_cast<uint32_t*>(Gd->mem + launches_at);
   Gd->p.one = plan[0].L;
   Gd->smem = smem;
   *out = Gd;
@@ -1462,9 +1545,9 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
     for (int i = 0; i < G->count; ++i) {
       p.act[i] = i == 0 ? act[0] : (const void*)(G->chain_buf + G->chain_off[i - 1]);
       p.out[i] = i + 1 == G->count ? out[0] : (void*)(G->chain_buf + G->chain_off[i]);
-      p.out_type[i] = (uint8_t)(i + 1 == G->count ? out_type : 2);
+      p.out_type[i] = (uint8_t)(i + 1 == G->count ? out_type : G->tagged ? 3 : 2);
     }
-    cudaError_t e0 = cudaMemsetAsync(G->done, 0, G->done_words * sizeof(uint32_t), s);
+    cudaError_t e0 = G->tagged ? cudaSuccess : cudaMemsetAsync(G->done, 0, G->done_words * sizeof(uint32_t), s);
     if (e0 != cudaSuccess) return e0;
     attr[0].id = cudaLaunchAttributeCooperative;   // the CTAs wait for one another: all must be resident
     attr[0].val.cooperative = 1;
@@ -1489,7 +1572,7 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
   cfg.dynamicSmemBytes = G->smem;
   cudaError_t e;
   GMaps<M_FP4> none{};
-  const int outk = G->chain ? OUT_CHAIN : (out_type == 2 ? OUT_SIGNS : OUT_WORDS);
+  const int outk = G->tagged ? OUT_TAGGED : G->chain ? OUT_CHAIN : (out_type == 2 ? OUT_SIGNS : OUT_WORDS);
   if (!G->chain && (outk == OUT_SIGNS) != (G->kind == TCG_SIGNS)) return cudaErrorInvalidValue;  // planned for the other kind
 #define G_LAUNCH(M, O, MAPS)                                                    \
   do {                                                                          \
@@ -1515,7 +1598,8 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
     else return cudaErrorInvalidValue;   // packed signs and chains need binary activations
   } else if (outk == OUT_WORDS) G_LAUNCH(M_FP4, OUT_WORDS, none);
   else if (outk == OUT_SIGNS) G_LAUNCH(M_FP4, OUT_SIGNS, none);
-  else G_LAUNCH(M_FP4, OUT_CHAIN, none);
+  else if (outk == OUT_CHAIN) G_LAUNCH(M_FP4, OUT_CHAIN, none);
+  else G_LAUNCH(M_FP4, OUT_TAGGED, none);
 #undef G_LAUNCH
   if (e != cudaSuccess) return e;
   *launched += 1;

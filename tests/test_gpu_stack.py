@@ -115,3 +115,42 @@ def test_stack_argument_errors(snn):
     st.destroy()
     for l in (la, lb, lf):
         l.destroy()
+
+
+@pytest.mark.parametrize("chans,hw,n", [
+    ((33, 64, 96, 128, 40), 9, 2),          # one and two words a pixel, blocks of two and four chunks
+    ((160, 192, 256, 288, 70), 8, 1),       # five to nine words: blocks of six and eight chunks, odd word counts
+    ((16, 16, 16), 32, 128),                # as many words between the members as may carry tags ...
+    ((16, 16, 16), 32, 129),                # ... and one image more
+])
+def test_stack_words_between_members(snn, oracle_mod, chans, hw, n):
+    """Chains whose words carry tags and the first that runs on counters; several launches of one stack, and its graph."""
+    shapes = [wl.LayerShape(a, b, hw, hw, 1, 1) for a, b in zip(chans, chans[1:])]
+    _check_chain(snn, oracle_mod, shapes, 6, n, 341, repeats=1 if n > 2 else 3)
+
+
+def test_stack_replayed_as_a_graph(snn, oracle_mod):
+    """A replay is a launch like any other to the tags: new inputs in the same buffer give new outputs every time."""
+    shapes = [wl.LayerShape(64, 64, 10, 10, 1, 1), wl.LayerShape(64, 128, 10, 10, 2, 1), wl.LayerShape(128, 96, 5, 5, 1, 1)]
+    layers, first, _, _ = _build_chain(snn, oracle_mod, shapes, 5, 2, 351)
+    stack = snn.SnnConvStack(layers, 2, 10, 10)
+    inputs = [torch.from_numpy(first.view(np.int32)).cuda()]
+    inputs += [torch.randint(-2 ** 31, 2 ** 31, inputs[0].shape, dtype=torch.int32, device="cuda") for _ in range(3)]
+    want = [stack.forward(x).clone() for x in inputs]
+    act, out = inputs[0].clone(), stack.alloc_out()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            stack.forward(act, out)
+            stack.forward(act, out)
+        for i in (1, 2, 3, 0, 2):
+            act.copy_(inputs[i])
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, want[i])
+    del graph
+    stack.destroy()
+    for l in layers:
+        l.destroy()
