@@ -328,6 +328,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   if (warp == 0) {
     // ------------------------------------------------ weight producer (one lane)
     if (lane == 0) {
+      if (p.after_weights) grid_dep_wait();
       int b_slot = 0;
       long long b_issued = 0;
       uint32_t b_phase = 1;  // parity of the previous use of a slot (valid from the second lap)
@@ -1421,12 +1422,13 @@ struct GStepOf {
 // The weight operand straight from the stored form (Sec. 4.4: index stream, codebook).  One thread per 32 input channels of
 // one row of the operand: their 32 indices are consecutive bits of the stream, looked up once for all taps.  Bound by
 // latency, not by its work (8192 threads at most): all of a thread's loads go out together.  With the launch after it,
-// copies and host work included, a call on 8 images of a 128-channel 28x28 layer takes 18.4 us; four decode kernels and
-// the popcount kernel take 46.
+// copies and host work included, a call on 8 images of a 128-channel 28x28 layer takes 18.5 us, waited for 31.7 (19.0 and 34.9 where the launch after it
+// is an ordinary one); four decode kernels and the popcount kernel take 46.
 __global__ void __launch_bounds__(128) g_static_weights_kernel(const uint8_t* __restrict__ stream, long long n_bytes,
                                                                const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
                                                                const GLayer L, int tau, int paired,
                                                                const GStepOf step_of) {
+  grid_dep_launch();   // the layer's launch may set itself up beside this one; its weight producer waits for this one to end
   const int row = threadIdx.x, wd = blockIdx.x, ct = blockIdx.y;   // row of the operand, 32-channel word, channel tile
   const int g = L.lg ? row >> L.kp_log : 0, co = ct * G_ROWS + (row & ((1 << L.kp_log) - 1));
   __shared__ uint16_t codes[512];
@@ -1517,12 +1519,23 @@ cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8
   p.out[0] = l.out;
   p.out_type[0] = (uint8_t)l.out_i32;
   p.status = status_dev;
-  // An ordinary launch, not a programmatic dependent of the kernel above: the weight producer does not wait for that one.
+  // A programmatic dependent of the kernel above: the weight producer waits for that one, and the expanders and the epilogue do
+  // as after any other.  (The scales are the copy's, which the kernel above has waited for.)
+  p.after_weights = 1;
   static unsigned long long done = 0;
   e = allow_max_smem(tcg_conv_kernel<M_FP4, OUT_WORDS>, &done);
   if (e != cudaSuccess) return e;
-  tcg_conv_kernel<M_FP4, OUT_WORDS><<<st.grid, G_THREADS, st.smem, l.stream>>>(p, GMaps<M_FP4>{});
-  e = cudaGetLastError();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.stream = l.stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.gridDim = dim3((unsigned)st.grid);
+  cfg.blockDim = dim3(G_THREADS);
+  cfg.dynamicSmemBytes = st.smem;
+  e = cudaLaunchKernelEx(&cfg, tcg_conv_kernel<M_FP4, OUT_WORDS>, p, GMaps<M_FP4>{});
   if (e == cudaSuccess) *launched += 1;
   return e;
 }
