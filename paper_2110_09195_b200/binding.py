@@ -8,6 +8,8 @@ if the shared library is missing or a call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import importlib
+import struct
 from pathlib import Path
 
 import numpy as np
@@ -20,6 +22,7 @@ _STATUS = {0: "OK", 1: "INVALID_ARG", 2: "UNSUPPORTED", 3: "CUDA", 4: "OOM", 5: 
 
 _LIB_PATH = Path(__file__).resolve().parent / "libsnnconv.so"
 _lib = None
+_fast = None   # the module of csrc/snn_fast.cpp
 
 # every symbol include/snn_conv.h declares
 EXPORTED_SYMBOLS = (
@@ -102,6 +105,19 @@ def load_library():
     lib.snn_microbench.argtypes = [i32, i32, ctypes.POINTER(ctypes.c_double)]
     _lib = lib
     return lib
+
+
+def _load_fast():
+    """The forward calls' checks in native code (csrc/snn_fast.cpp); built beside the library, and as necessary."""
+    global _fast
+    if _fast is None:
+        import torch  # noqa: F401  (its libraries are what the module is linked with)
+        lib = load_library()
+        module = importlib.import_module(__package__ + "._snn_fast")
+        module.bind(*(ctypes.cast(f, ctypes.c_void_p).value
+                      for f in (lib.snn_conv_forward, lib.snn_conv_group_forward, lib.snn_conv_stack_forward)))
+        _fast = module
+    return _fast
 
 
 def _check(status: int):
@@ -211,6 +227,10 @@ class SnnConv:
         self.c_in, self.c_out, self.tau = int(c_in), int(c_out), int(tau)
         self.stride, self.pad, self.act_type, self.device = int(stride), int(pad), int(act_type), int(device)
         self.ksize = int(ksize)
+        self._desc = struct.pack("=QQ8i", h.value, 0, self.device, self.act_type,
+                                 (self.c_in + 31) // 32 if self.act_type == ACT_BIN else self.c_in, self.c_out, self.ksize,
+                                 self.stride, self.pad, 0)
+        _load_fast()
 
     # -- helpers ------------------------------------------------------------
     def out_hw(self, h, w):
@@ -243,6 +263,12 @@ class SnnConv:
     def forward(self, act, out=None, out_type=OUT_F32, path=PATH_AUTO, stream=None):
         """snn_conv_forward: act / out are CUDA tensors; asynchronous on `stream`
         (default: torch's current stream)."""
+        if out is not None and stream is None:
+            st = _fast.layer_forward(self._desc, act, out, out_type, path)
+            if st == 0:
+                return out
+            if st > 0:
+                _check(st)
         if act.get_device() != self.device:
             raise SnnError(1, f"activations must live on cuda:{self.device}")
         self._check_act(act)
@@ -295,6 +321,7 @@ class SnnConv:
 
     def destroy(self):
         if getattr(self, "_h", None) is not None:
+            self._desc = None
             load_library().snn_conv_destroy(self._h)
             self._h = None
 
@@ -333,6 +360,8 @@ class SnnConvGroup:
         self._act_shapes = [(*s, (l.c_in + 31) // 32 if l.act_type == ACT_BIN else l.c_in) for l, s in zip(self.layers, self.shapes)]
         self._out_shapes = [(s[0], *l.out_hw(s[1], s[2]), l.c_out) for l, s in zip(self.layers, self.shapes)]
         self._sign_shapes = [(*o[:3], (o[3] + 31) // 32) for o in self._out_shapes]
+        self._desc = struct.pack("=Qii", g.value, self.device, self.layers[0].act_type) + b"".join(
+            struct.pack("=8i", *a, *o[1:], 0) for a, o in zip(self._act_shapes, self._out_shapes))
 
     def alloc_outs(self, out_type=OUT_F32):
         import torch
@@ -344,6 +373,12 @@ class SnnConvGroup:
     def forward(self, acts, outs=None, out_type=OUT_F32, stream=None):
         """snn_conv_group_forward: acts / outs are lists of CUDA tensors, one per member;
         asynchronous on `stream` (default: torch's current stream)."""
+        if outs is not None and stream is None:
+            st = _fast.group_forward(self._desc, acts, outs, out_type)
+            if st == 0:
+                return outs
+            if st > 0:
+                _check(st)
         import torch
         n = len(self.layers)
         if len(acts) != n:
@@ -370,6 +405,7 @@ class SnnConvGroup:
 
     def destroy(self):
         if getattr(self, "_g", None) is not None:
+            self._desc = None
             load_library().snn_conv_group_destroy(self._g)
             self._g = None
 
@@ -402,6 +438,8 @@ class SnnConvStack:
         for l in self.layers:
             ho, wo = l.out_hw(ho, wo)
         self.out_hw = (ho, wo)
+        self._desc = struct.pack("=Qii8i", st.value, self.device, ACT_BIN, self.n, self.h, self.w, (self.layers[0].c_in + 31) // 32,
+                                 ho, wo, self.layers[-1].c_out, 0)
 
     def alloc_out(self, out_type=OUT_F32):
         import torch
@@ -412,6 +450,12 @@ class SnnConvStack:
 
     def forward(self, act, out=None, out_type=OUT_F32, stream=None):
         """snn_conv_stack_forward: act is the first layer's input, out the last layer's output."""
+        if out is not None and stream is None:
+            st = _fast.stack_forward(self._desc, act, out, out_type)
+            if st == 0:
+                return out
+            if st > 0:
+                _check(st)
         import torch
         first = self.layers[0]
         if not act.is_cuda or act.device.index != self.device:
@@ -433,6 +477,7 @@ class SnnConvStack:
 
     def destroy(self):
         if getattr(self, "_s", None) is not None:
+            self._desc = None
             load_library().snn_conv_stack_destroy(self._s)
             self._s = None
 

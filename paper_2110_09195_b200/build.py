@@ -1,9 +1,11 @@
-"""Builds libsnnconv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libsnnconv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and _snn_fast (the binding's checks as a
+Python module in C++) with the host compiler."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 from pathlib import Path
 
@@ -11,6 +13,8 @@ PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 LIB = PKG / "libsnnconv.so"
+FAST = PKG / ("_snn_fast" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+FAST_SOURCE = CSRC / "snn_fast.cpp"
 SOURCES = ["snn_api.cu", "snn_decode.cu", "snn_popc.cu", "snn_reuse.cu", "snn_reuse_f16.cu", "snn_tcg.cu", "snn_microbench.cu", "snn_static.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -31,7 +35,30 @@ def _stale() -> bool:
     return any(d.stat().st_mtime > t for d in deps)
 
 
+def build_fast(force: bool = False, verbose: bool = False) -> Path:
+    """The module needs torch's headers and libraries (those of the torch that will call it)."""
+    deps = (FAST_SOURCE, INCLUDE / "snn_conv.h")
+    if not force and FAST.exists() and all(d.stat().st_mtime <= FAST.stat().st_mtime for d in deps):
+        return FAST
+    import torch
+    root = Path(torch.__file__).resolve().parent
+    tmp = FAST.with_name(f"_snn_fast.tmp{os.getpid()}.so")
+    cuda = Path(_nvcc()).parent.parent / "include"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-w",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f"-I{INCLUDE}", f"-I{root}/include",
+           f"-I{root}/include/torch/csrc/api/include", f"-I{sysconfig.get_paths()['include']}", f"-I{cuda}", str(FAST_SOURCE),
+           "-o", str(tmp), f"-L{root}/lib", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if verbose or r.returncode:
+        sys.stderr.write(r.stdout + r.stderr)
+    if r.returncode:
+        raise RuntimeError(f"{cmd[0]} failed on {FAST_SOURCE.name}")
+    os.replace(tmp, FAST)
+    return FAST
+
+
 def build(force: bool = False, verbose: bool = False) -> Path:
+    build_fast(force, verbose)
     if not force and not _stale():
         return LIB
     objdir = PKG / "_build"

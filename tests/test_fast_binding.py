@@ -1,0 +1,88 @@
+"""The native checks of the forward calls: what they do not take goes through binding.py's own, which raise as ever."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2110_09195_b200 as snn
+import workloads as wl
+from paper_2110_09195_b200 import binding
+
+
+def test_anything_unusual_is_left_to_the_python_checks():
+    fast = binding._load_fast()
+    x, y = torch.zeros((1, 4, 4, 1), dtype=torch.int32), torch.zeros((1, 4, 4, 16))
+    desc = bytes(48)
+    for args in ((desc, x, y, 0, 0), (desc[:40], x, y, 0, 0), (None, x, y, 0, 0), (desc, [x], y, 0, 0), (desc, x, y, 0),
+                 (desc, x, y, 7, 0), (desc, x, y, 0.0, 0), (desc, x, y, 0, None)):
+        assert fast.layer_forward(*args) == -1
+    for args in ((desc, [x], [y], 0), (desc, (x,), [y], 0), (desc[:16], [], [], 0), (desc, [x, x], [y, y], 0)):
+        assert fast.group_forward(*args) == -1
+    assert fast.stack_forward(desc, x, y, 0) == -1 and fast.stack_forward(desc, x, y, None) == -1
+
+
+def _layer(shape, seed=3, act_type=snn.ACT_BIN):
+    p = wl.draw_layer_params(shape, 5, seed)
+    return snn.SnnConv(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha, shape.stride, shape.pad, act_type)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("act_type", [snn.ACT_BIN, snn.ACT_F16])
+def test_both_ways_launch_the_same(act_type):
+    shape = wl.LayerShape(40, 72, 9, 7, 2, 1)
+    layer, other = _layer(shape, 3, act_type), _layer(shape, 4, act_type)
+    if act_type == snn.ACT_BIN:
+        x = torch.from_numpy(wl.pack_activation_bits(wl.draw_activation_bits(shape, 3, 1)).view(np.int32)).cuda()
+    else:
+        x = torch.randn((3, 9, 7, 40), dtype=torch.float16, device="cuda")
+    stream = torch.cuda.current_stream()
+    for out_type in (snn.OUT_F32, snn.OUT_I32, snn.OUT_BITS) if act_type == snn.ACT_BIN else (snn.OUT_F32,):
+        a, b = layer.alloc_out(3, 9, 7, out_type), layer.alloc_out(3, 9, 7, out_type)
+        layer.forward(x, out=a, out_type=out_type)
+        layer.forward(x, out=b, out_type=out_type, stream=stream)
+        assert torch.equal(a, b)
+        group = snn.SnnConvGroup([layer, other], [(3, 9, 7)] * 2)
+        outs, want = group.alloc_outs(out_type), group.alloc_outs(out_type)
+        group.forward([x, x], outs, out_type=out_type)
+        group.forward((x, x), tuple(want), out_type=out_type)   # (not lists: the Python checks)
+        assert all(torch.equal(p, q) for p, q in zip(outs, want)) and torch.equal(outs[0], a)
+
+
+@pytest.mark.gpu
+def test_wrong_tensors_are_refused():
+    shape = wl.LayerShape(40, 72, 9, 7, 1, 1)
+    layer = _layer(shape)
+    x = torch.zeros((2, 9, 7, 2), dtype=torch.int32, device="cuda")
+    out = layer.alloc_out(2, 9, 7)
+    wide = torch.zeros((2, 9, 7, 144), device="cuda")
+    for act, o in ((x.cpu(), out), (x.float(), out), (x[..., :1], out), (x.transpose(1, 2), out), (x, out.cpu()), (x, out.int()),
+                   (x, out[:1]), (x, wide[..., ::2]), (x[0], out)):
+        with pytest.raises(snn.SnnError):
+            layer.forward(act, out=o)
+        with pytest.raises(snn.SnnError):
+            snn.SnnConvGroup([layer], [(2, 9, 7)]).forward([act], [o])
+    with pytest.raises(snn.SnnError):
+        layer.forward(x, out=out, out_type=9)
+    shifted = torch.zeros(x.numel() + 1, dtype=torch.int32, device="cuda")[1:].view(x.shape)   # 4 bytes past a boundary of 16
+    with pytest.raises(snn.SnnError):
+        layer.forward(shifted, out=out)
+    assert layer.forward(x[:0], out=out[:0]).numel() == 0
+    layer.destroy()
+    with pytest.raises(snn.SnnError):
+        layer.forward(x, out=out)
+
+
+@pytest.mark.gpu
+def test_the_current_stream_is_used():
+    shape = wl.LayerShape(32, 32, 32, 32, 1, 1)
+    layer = _layer(shape)
+    x = torch.zeros((4, 32, 32, 1), dtype=torch.int32, device="cuda")
+    out = layer.alloc_out(4, 32, 32)
+    layer.forward(x, out=out)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):      # a launch on any other stream would break the capture
+        layer.forward(x, out=out)
+    want = out.clone()
+    out.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
