@@ -1435,63 +1435,72 @@ struct GStepOf {
   uint8_t at[3][17];
 };
 
-// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook).  One thread per 32 input channels of
-// one row of the operand: their 32 indices are consecutive bits of the stream, looked up once for all taps.  Bound by
-// latency, not by its work (8192 threads at most): all of a thread's loads go out together.  With the launch after it,
-// copies and host work included, a call on 8 images of a 128-channel 28x28 layer takes 18.5 us, waited for 31.7 (19.0 and 34.9 where the launch after it
-// is an ordinary one); four decode kernels and the popcount kernel take 46.
-__global__ void __launch_bounds__(128) g_static_weights_kernel(const uint8_t* __restrict__ stream, long long n_bytes,
-                                                               const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
-                                                               const GLayer L, int tau, int paired,
-                                                               const GStepOf step_of) {
+// The weight operand straight from the stored form (Sec. 4.4: index stream, codebook).  A warp takes 8 rows of the operand, one
+// after the other but with all their loads out together; a lane is an input channel of a 32-channel word.  The indices of a
+// row's word are consecutive bits of the stream, nine votes of the codes' bits are its nine taps, and lane t writes tap t.
+// Bound by latency: two loads, a look-up, nine votes and the launch around them.
+// With one thread per row and word, 64 byte loads and 33 KB of straight-line code a thread, 14 calls took 4 % longer waited for
+// (193->168 channels of 9x26: 36.8 us, now 33.8).  8 images of a 128-channel 28x28 layer, copies and host work included: 16.6 us a
+// call back to back, all of it the host's, 30.2 waited for; by four decode kernels and the popcount kernel 46.
+constexpr int G_SW_ROWS = 8, G_SW_WARPS = 4;
+__global__ void __launch_bounds__(32 * G_SW_WARPS) g_static_weights_kernel(const uint8_t* __restrict__ stream, int n_bytes,
+                                                                           const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
+                                                                           const __grid_constant__ GLayer L, int tau, int paired,
+                                                                           const __grid_constant__ GStepOf step_of) {
   grid_dep_launch();   // the layer's launch may set itself up beside this one; its weight producer waits for this one to end
-  const int row = threadIdx.x, wd = blockIdx.x, ct = blockIdx.y;   // row of the operand, 32-channel word, channel tile
-  const int g = L.lg ? row >> L.kp_log : 0, co = ct * G_ROWS + (row & ((1 << L.kp_log) - 1));
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wd = blockIdx.x, ct = blockIdx.y;                       // 32-channel word, channel tile
+  const int row0 = (blockIdx.z * G_SW_WARPS + warp) * G_SW_ROWS;    // (all of the warp's rows are of one pixel of a group)
+  const int g = L.lg ? row0 >> L.kp_log : 0, co0 = ct * G_ROWS + (row0 & ((1 << L.kp_log) - 1));
   __shared__ uint16_t codes[512];
-  for (int i = row; i < (1 << tau); i += 128) codes[i] = codebook[i];
-  const int n_ch = co < L.K ? (L.C - 32 * wd < 32 ? L.C - 32 * wd : 32) : 0;   // channels of this word (none: all zeros)
-  const uint32_t exists = n_ch <= 0 ? 0u : 0xffffffffu >> (32 - n_ch);
-  // all loads first: one round trip to memory instead of one per index
-  uint32_t index[32];
-  {
-    long long bit = ((long long)co * L.C + 32 * wd) * tau;
+  // all loads first: one round trip to memory instead of one per row
+  const int n_ch = L.C - 32 * wd < 32 ? L.C - 32 * wd : 32;   // channels of this word
+  uint32_t index[G_SW_ROWS];
 #pragma unroll
-    for (int b = 0; b < 32; ++b, bit += tau) {
-      const long long at = bit >> 3;   // an index spans at most two bytes (9 bits from any bit of a byte: 16 bits)
-      uint32_t v = 0;
-      if (b < n_ch) {
-        v = stream[at];
-        if (at + 1 < n_bytes) v |= (uint32_t)stream[at + 1] << 8;
-      }
-      index[b] = (v >> (bit & 7)) & ((1u << tau) - 1u);
+  for (int i = 0; i < G_SW_ROWS; ++i) {
+    index[i] = 0;
+    if (co0 + i < L.K && lane < n_ch) {
+      const int bit = ((co0 + i) * L.C + 32 * wd + lane) * tau;   // (at most 512 x 512 indices)
+      const int at = bit >> 3;   // an index spans at most two bytes (9 bits from any bit of a byte: 16 bits)
+      uint32_t v = stream[at];
+      if (at + 1 < n_bytes) v |= (uint32_t)stream[at + 1] << 8;
+      index[i] = (v >> (bit & 7)) & ((1u << tau) - 1u);
     }
   }
+  for (int i = threadIdx.x; i < (1 << tau); i += 32 * G_SW_WARPS) codes[i] = codebook[i];
   __syncthreads();
-  uint32_t plane[9];   // bit b of plane t: tap t of channel 32*wd + b is +1
-#pragma unroll
-  for (int t = 0; t < 9; ++t) plane[t] = 0;
-#pragma unroll
-  for (int b = 0; b < 32; ++b) {
-    const uint32_t code = codes[index[b]];
-#pragma unroll
-    for (int t = 0; t < 9; ++t) plane[t] |= ((code >> (8 - t)) & 1u) << b;
-  }
-  // nibbles in the expanders' order: channel 4n + k of the word in nibble n of word k
-  auto nibbles = [&](uint32_t bits, int k) {
-    const uint32_t e = ((exists >> k) & 0x11111111u) * 15u;
-    return ((~(bits << (3 - k)) & 0x88888888u) | 0x22222222u) & e;
-  };
   const int chunks = paired ? 2 : L.cb_chunks, cb = paired ? 0 : wd / L.cb_chunks, c0 = paired ? 0 : wd - cb * L.cb_chunks;
-  uint4* const base = reinterpret_cast<uint4*>(wt) + (size_t)(ct * L.n_cb + cb) * L.steps * chunks * G_ROWS + row;
-  if (L.G > 1 || paired) {   // columns outside this pixel's window, and a last step's missing tap
-    for (int t = 0; t < L.steps; ++t)
-      for (int c = 0; c < (paired ? 2 : 1); ++c) base[(size_t)(t * chunks + c0 + c) * G_ROWS] = make_uint4(0, 0, 0, 0);
+  uint4* const base = reinterpret_cast<uint4*>(wt) + (size_t)(ct * L.n_cb + cb) * L.steps * chunks * G_ROWS + row0;
+  if (L.G > 1 || paired) {   // columns outside the pixel's window, and a last step's missing tap
+    const int kinds = paired ? 2 : 1;
+#pragma unroll 1
+    for (int i = lane; i < L.steps * kinds * G_SW_ROWS; i += 32) {
+      const int place = i / G_SW_ROWS, t = paired ? place >> 1 : place, c = paired ? place & 1 : 0;
+      base[(size_t)(t * chunks + c0 + c) * G_ROWS + (i & (G_SW_ROWS - 1))] = make_uint4(0, 0, 0, 0);
+    }
+    __syncwarp();   // before the taps are written over some of them
   }
+  const int tap = lane < 9 ? lane : 0, at = step_of.at[tap / 3][tap % 3 + L.rs * g];
+  uint4* const dst = base + (size_t)((at >> 1) * chunks + c0 + (at & 1)) * G_ROWS;
+  const uint32_t channels = n_ch > 0 ? 0xffffffffu >> (32 - n_ch) : 0u;   // (a block's last words may hold none)
+#pragma unroll 2
+  for (int i = 0; i < G_SW_ROWS; ++i) {
+    uint32_t mine = index[0];
 #pragma unroll
-  for (int t = 0; t < 9; ++t) {
-    const int at = step_of.at[t / 3][t % 3 + L.rs * g];
-    base[(size_t)((at >> 1) * chunks + c0 + (at & 1)) * G_ROWS] =
-        make_uint4(nibbles(plane[t], 0), nibbles(plane[t], 1), nibbles(plane[t], 2), nibbles(plane[t], 3));
+    for (int j = 1; j < G_SW_ROWS; ++j) mine = i == j ? index[j] : mine;
+    const uint32_t code = codes[mine];
+    uint32_t plane = 0;   // bit b: this lane's tap of channel 32*wd + b is +1
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+      const uint32_t v = __ballot_sync(0xffffffffu, (code >> (8 - t)) & 1u);
+      plane = lane == t ? v : plane;
+    }
+    // nibbles in the expanders' order: channel 4n + k of the word in nibble n of word k; channels that do not exist are 0
+    const uint32_t exists = co0 + i < L.K ? channels : 0u;
+    uint32_t w[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) w[k] = ((~(plane << (3 - k)) & 0x88888888u) | 0x22222222u) & (((exists >> k) & 0x11111111u) * 15u);
+    if (lane < 9) dst[i] = make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -1523,9 +1532,9 @@ cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8
   for (int t = 0; t < L.steps; ++t)
     for (int c = 0; c < (st.plan.paired ? 2 : 1); ++c)
       if (st.plan.taps.row[t][c] < 3) step_of.at[st.plan.taps.row[t][c]][st.plan.taps.col[t][c]] = (uint8_t)(2 * t + c);
-  const long long n_bytes = ((long long)g.K * g.C * g.tau + 7) / 8;
-  const dim3 blocks((unsigned)(st.plan.paired ? 1 : L.n_cb * L.cb_chunks), (unsigned)L.n_ct);
-  g_static_weights_kernel<<<blocks, G_ROWS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, g.tau, st.plan.paired, step_of);
+  const int n_bytes = (int)(((long long)g.K * g.C * g.tau + 7) / 8);
+  const dim3 blocks((unsigned)(st.plan.paired ? 1 : L.n_cb * L.cb_chunks), (unsigned)L.n_ct, G_ROWS / (G_SW_ROWS * G_SW_WARPS));
+  g_static_weights_kernel<<<blocks, 32 * G_SW_WARPS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, g.tau, st.plan.paired, step_of);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   *launched += 1;

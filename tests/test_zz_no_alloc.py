@@ -122,3 +122,16 @@ def test_wrong_buffers_are_refused_on_the_host(snn):
     with pytest.raises(snn.SnnError):
         snn.forward_static(64, 48, 5, p.codebook, p.idx_packed, p.alpha, act, good, stride=2)       # out is stride-1 sized
     assert snn.kernel_launches() == before
+
+
+@pytest.mark.parametrize("c_in,c_out,h,w,stride,pad,tau,n", [
+    (1, 1, 5, 4, 1, 1, 1, 1),          # one channel of a word, one row of the operand
+    (31, 5, 9, 9, 2, 1, 9, 3),         # pairs of taps, groups of pixels, indices across byte borders
+    (32, 16, 32, 32, 1, 1, 5, 8),      # eight pixels a position: sixteen rows each
+    (33, 17, 12, 7, 1, 0, 7, 2),       # words without any channel in a block of two chunks
+    (65, 64, 14, 14, 2, 1, 6, 4),
+    (160, 127, 9, 26, 1, 1, 3, 2),     # blocks of six chunks
+    (200, 129, 6, 6, 1, 1, 8, 2),      # a second channel tile of one row
+])
+def test_operand_from_the_stored_form(snn, oracle_mod, c_in, c_out, h, w, stride, pad, tau, n):
+    _check_case(snn, oracle_mod, wl.LayerShape(c_in, c_out, h, w, stride, pad), tau, n, 17)
