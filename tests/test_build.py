@@ -1,0 +1,26 @@
+"""The build: the C library is built by itself, whatever becomes of the Python module beside it."""
+import sys
+
+import pytest
+
+from paper_2110_09195_b200 import build
+
+
+def test_the_library_is_built_without_torch(monkeypatch, tmp_path, capfd):
+    monkeypatch.setattr(build, "FAST", tmp_path / "_snn_fast.so")
+    monkeypatch.setitem(sys.modules, "torch", None)   # importing it raises
+    assert build.build() == build.LIB and build.LIB.exists()
+    assert "_snn_fast.so was not built" in capfd.readouterr().err
+    with pytest.raises(ImportError):
+        build.build_fast()
+
+
+def test_the_library_is_built_where_the_module_cannot_be(monkeypatch, tmp_path, capfd):
+    monkeypatch.setattr(build, "FAST", tmp_path / "_snn_fast.so")
+    for compiler in ("/bin/false", str(tmp_path / "no-such-compiler")):
+        monkeypatch.setenv("CXX", compiler)
+        assert build.build() == build.LIB and build.LIB.exists()
+        assert "_snn_fast.so was not built" in capfd.readouterr().err
+        with pytest.raises((RuntimeError, OSError)):
+            build.build_fast()
+    assert not build.FAST.exists()
