@@ -10,6 +10,8 @@ from __future__ import annotations
 import ctypes
 import importlib
 import struct
+import sys
+import warnings
 from pathlib import Path
 
 import numpy as np
@@ -22,7 +24,7 @@ _STATUS = {0: "OK", 1: "INVALID_ARG", 2: "UNSUPPORTED", 3: "CUDA", 4: "OOM", 5: 
 
 _LIB_PATH = Path(__file__).resolve().parent / "libsnnconv.so"
 _lib = None
-_fast = None   # the module of csrc/snn_fast.cpp
+_fast = None   # the module of csrc/snn_fast.cpp, or what stands in for it
 
 # every symbol include/snn_conv.h declares
 EXPORTED_SYMBOLS = (
@@ -107,15 +109,30 @@ def load_library():
     return lib
 
 
+class _PythonChecks:
+    """In the place of the native module where there is none: leaves every call to the checks in Python."""
+
+    @staticmethod
+    def layer_forward(*_):
+        return -1
+
+    group_forward = stack_forward = layer_forward
+
+
 def _load_fast():
-    """The forward calls' checks in native code (csrc/snn_fast.cpp); built beside the library, and as necessary."""
+    """The forward calls' checks in native code (csrc/snn_fast.cpp).  Without them the checks below do the same, more slowly."""
     global _fast
     if _fast is None:
-        import torch  # noqa: F401  (its libraries are what the module is linked with)
         lib = load_library()
-        module = importlib.import_module(__package__ + "._snn_fast")
-        module.bind(*(ctypes.cast(f, ctypes.c_void_p).value
-                      for f in (lib.snn_conv_forward, lib.snn_conv_group_forward, lib.snn_conv_stack_forward)))
+        try:
+            import torch  # noqa: F401  (its libraries are what the module is linked with)
+            module = importlib.import_module(__package__ + "._snn_fast")
+            module.bind(*(ctypes.cast(f, ctypes.c_void_p).value
+                          for f in (lib.snn_conv_forward, lib.snn_conv_group_forward, lib.snn_conv_stack_forward)))
+        except ImportError as e:
+            warnings.warn(f"the forward calls are checked in Python, which takes longer: {e} "
+                          "(python -m paper_2110_09195_b200.build builds _snn_fast)", RuntimeWarning, stacklevel=3)
+            module = _PythonChecks
         _fast = module
     return _fast
 
@@ -230,7 +247,8 @@ class SnnConv:
         self._desc = struct.pack("=QQ8i", h.value, 0, self.device, self.act_type,
                                  (self.c_in + 31) // 32 if self.act_type == ACT_BIN else self.c_in, self.c_out, self.ksize,
                                  self.stride, self.pad, 0)
-        _load_fast()
+        if sys.modules.get("torch"):   # (a program without torch has no tensors to pass)
+            _load_fast()
 
     # -- helpers ------------------------------------------------------------
     def out_hw(self, h, w):
@@ -264,7 +282,7 @@ class SnnConv:
         """snn_conv_forward: act / out are CUDA tensors; asynchronous on `stream`
         (default: torch's current stream)."""
         if out is not None and stream is None:
-            st = _fast.layer_forward(self._desc, act, out, out_type, path)
+            st = (_fast or _load_fast()).layer_forward(self._desc, act, out, out_type, path)
             if st == 0:
                 return out
             if st > 0:
@@ -374,7 +392,7 @@ class SnnConvGroup:
         """snn_conv_group_forward: acts / outs are lists of CUDA tensors, one per member;
         asynchronous on `stream` (default: torch's current stream)."""
         if outs is not None and stream is None:
-            st = _fast.group_forward(self._desc, acts, outs, out_type)
+            st = (_fast or _load_fast()).group_forward(self._desc, acts, outs, out_type)
             if st == 0:
                 return outs
             if st > 0:
@@ -451,7 +469,7 @@ class SnnConvStack:
     def forward(self, act, out=None, out_type=OUT_F32, stream=None):
         """snn_conv_stack_forward: act is the first layer's input, out the last layer's output."""
         if out is not None and stream is None:
-            st = _fast.stack_forward(self._desc, act, out, out_type)
+            st = (_fast or _load_fast()).stack_forward(self._desc, act, out, out_type)
             if st == 0:
                 return out
             if st > 0:

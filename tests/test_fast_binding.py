@@ -1,4 +1,6 @@
 """The native checks of the forward calls: what they do not take goes through binding.py's own, which raise as ever."""
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -20,9 +22,59 @@ def test_anything_unusual_is_left_to_the_python_checks():
     assert fast.stack_forward(desc, x, y, 0) == -1 and fast.stack_forward(desc, x, y, None) == -1
 
 
-def _layer(shape, seed=3, act_type=snn.ACT_BIN):
+class _Library:
+    """Stands in for the C library where there is no GPU: notes the calls, and every one of them succeeds."""
+
+    def __init__(self):
+        self.calls = []
+
+    def __getattr__(self, name):
+        def call(*args):
+            self.calls.append(name)
+            if name.endswith("_create"):
+                args[-1]._obj.value = 1   # the handle, passed by reference
+            return 0
+        return call
+
+
+@pytest.fixture
+def without_module(monkeypatch):
+    lib = _Library()
+    monkeypatch.setattr(binding, "_lib", lib)
+    monkeypatch.setattr(binding, "_fast", None)
+    monkeypatch.setattr(binding, "_raw_stream", lambda device, stream: 0)
+    monkeypatch.setitem(sys.modules, "paper_2110_09195_b200._snn_fast", None)   # importing it raises
+    monkeypatch.delattr("paper_2110_09195_b200._snn_fast", raising=False)
+    return lib
+
+
+def test_a_layer_needs_neither_torch_nor_the_module(without_module, monkeypatch):
+    monkeypatch.setitem(sys.modules, "torch", None)   # importing it raises
+    layer = _layer(wl.LayerShape(40, 72, 9, 7, 1, 1))
+    assert without_module.calls == ["snn_conv_create"] and binding._fast is None
+    layer.destroy()
+
+
+def test_without_the_module_the_python_checks_make_the_calls(without_module):
+    with pytest.warns(RuntimeWarning, match="checked in Python"):
+        layer = _layer(wl.LayerShape(40, 72, 9, 7, 1, 1), device=-1)   # (where torch says that CPU tensors live)
+    x, out = torch.zeros((2, 9, 7, 2), dtype=torch.int32), torch.zeros((2, 9, 7, 72))
+    assert layer.forward(x, out=out) is out
+    group = snn.SnnConvGroup([layer], [(2, 9, 7)])
+    outs = [out]
+    assert group.forward([x], outs) is outs
+    assert without_module.calls == ["snn_conv_create", "snn_conv_forward", "snn_conv_group_create", "snn_conv_group_forward"]
+    with pytest.raises(snn.SnnError):
+        layer.forward(x, out=out[:1])
+    with pytest.raises(snn.SnnError):
+        group.forward([x[:1]], outs)
+    group.destroy()
+    layer.destroy()
+
+
+def _layer(shape, seed=3, act_type=snn.ACT_BIN, device=0):
     p = wl.draw_layer_params(shape, 5, seed)
-    return snn.SnnConv(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha, shape.stride, shape.pad, act_type)
+    return snn.SnnConv(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha, shape.stride, shape.pad, act_type, device)
 
 
 @pytest.mark.gpu
