@@ -37,6 +37,15 @@ class _Library:
         return call
 
 
+class _Layer(snn.SnnConv):
+    def __del__(self):   # a handle of _Library must not reach the library, whenever it is collected
+        pass
+
+
+class _Group(snn.SnnConvGroup):
+    __del__ = _Layer.__del__
+
+
 @pytest.fixture
 def without_module(monkeypatch):
     lib = _Library()
@@ -50,17 +59,17 @@ def without_module(monkeypatch):
 
 def test_a_layer_needs_neither_torch_nor_the_module(without_module, monkeypatch):
     monkeypatch.setitem(sys.modules, "torch", None)   # importing it raises
-    layer = _layer(wl.LayerShape(40, 72, 9, 7, 1, 1))
+    layer = _layer(wl.LayerShape(40, 72, 9, 7, 1, 1), cls=_Layer)
     assert without_module.calls == ["snn_conv_create"] and binding._fast is None
     layer.destroy()
 
 
 def test_without_the_module_the_python_checks_make_the_calls(without_module):
     with pytest.warns(RuntimeWarning, match="checked in Python"):
-        layer = _layer(wl.LayerShape(40, 72, 9, 7, 1, 1), device=-1)   # (where torch says that CPU tensors live)
+        layer = _layer(wl.LayerShape(40, 72, 9, 7, 1, 1), device=-1, cls=_Layer)   # (where torch says that CPU tensors live)
     x, out = torch.zeros((2, 9, 7, 2), dtype=torch.int32), torch.zeros((2, 9, 7, 72))
     assert layer.forward(x, out=out) is out
-    group = snn.SnnConvGroup([layer], [(2, 9, 7)])
+    group = _Group([layer], [(2, 9, 7)])
     outs = [out]
     assert group.forward([x], outs) is outs
     assert without_module.calls == ["snn_conv_create", "snn_conv_forward", "snn_conv_group_create", "snn_conv_group_forward"]
@@ -72,9 +81,9 @@ def test_without_the_module_the_python_checks_make_the_calls(without_module):
     layer.destroy()
 
 
-def _layer(shape, seed=3, act_type=snn.ACT_BIN, device=0):
+def _layer(shape, seed=3, act_type=snn.ACT_BIN, device=0, cls=snn.SnnConv):
     p = wl.draw_layer_params(shape, 5, seed)
-    return snn.SnnConv(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha, shape.stride, shape.pad, act_type, device)
+    return cls(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha, shape.stride, shape.pad, act_type, device)
 
 
 @pytest.mark.gpu
