@@ -125,8 +125,10 @@ def _load_fast():
     if _fast is None:
         lib = load_library()
         try:
-            import torch  # noqa: F401  (its libraries are what the module is linked with)
+            import torch   # (its libraries are what the module is linked with)
             module = importlib.import_module(__package__ + "._snn_fast")
+            if module.TORCH_VERSION != torch.__version__:
+                raise ImportError(f"_snn_fast was built for torch {module.TORCH_VERSION}, not {torch.__version__}")
             module.bind(*(ctypes.cast(f, ctypes.c_void_p).value
                           for f in (lib.snn_conv_forward, lib.snn_conv_group_forward, lib.snn_conv_stack_forward)))
         except ImportError as e:

@@ -15,6 +15,7 @@ INCLUDE = PKG.parent / "include"
 LIB = PKG / "libsnnconv.so"
 FAST = PKG / ("_snn_fast" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 FAST_SOURCE = CSRC / "snn_fast.cpp"
+FAST_TORCH = PKG / "_build" / "_snn_fast.torch"   # the version of torch it was built for
 SOURCES = ["snn_api.cu", "snn_decode.cu", "snn_popc.cu", "snn_reuse.cu", "snn_reuse_f16.cu", "snn_tcg.cu", "snn_microbench.cu", "snn_static.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -36,15 +37,17 @@ def _stale() -> bool:
 
 
 def build_fast(force: bool = False, verbose: bool = False) -> Path:
-    """The module needs torch's headers and libraries (those of the torch that will call it)."""
-    deps = (FAST_SOURCE, INCLUDE / "snn_conv.h")
-    if not force and FAST.exists() and all(d.stat().st_mtime <= FAST.stat().st_mtime for d in deps):
-        return FAST
+    """The module reads torch's tensors by the layout in torch's headers: it is built for the torch that will call it."""
     import torch
+    deps = (FAST_SOURCE, INCLUDE / "snn_conv.h")
+    if (not force and FAST.exists() and all(d.stat().st_mtime <= FAST.stat().st_mtime for d in deps)
+            and FAST_TORCH.exists() and FAST_TORCH.read_text() == torch.__version__):
+        return FAST
     root = Path(torch.__file__).resolve().parent
     tmp = FAST.with_name(f"_snn_fast.tmp{os.getpid()}.so")
     cuda = Path(_nvcc()).parent.parent / "include"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-w",
+           f'-DSNN_TORCH_VERSION="{torch.__version__}"',
            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f"-I{INCLUDE}", f"-I{root}/include",
            f"-I{root}/include/torch/csrc/api/include", f"-I{sysconfig.get_paths()['include']}", f"-I{cuda}", str(FAST_SOURCE),
            "-o", str(tmp), f"-L{root}/lib", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
@@ -54,6 +57,8 @@ def build_fast(force: bool = False, verbose: bool = False) -> Path:
     if r.returncode:
         raise RuntimeError(f"{cmd[0]} failed on {FAST_SOURCE.name}")
     os.replace(tmp, FAST)
+    FAST_TORCH.parent.mkdir(exist_ok=True)
+    FAST_TORCH.write_text(torch.__version__)
     return FAST
 
 

@@ -182,4 +182,12 @@ PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_snn_fast", nullptr, -1, metho
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__snn_fast() { return PyModule_Create(&module_def); }
+// (the version of torch is asked for before any tensor is handed in: tensors are read by the layout of its headers)
+PyMODINIT_FUNC PyInit__snn_fast() {
+  PyObject* m = PyModule_Create(&module_def);
+  if (m && PyModule_AddStringConstant(m, "TORCH_VERSION", SNN_TORCH_VERSION) < 0) {
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}

@@ -1,7 +1,9 @@
 """The build: the C library is built by itself, whatever becomes of the Python module beside it."""
+import subprocess
 import sys
 
 import pytest
+import torch
 
 from paper_2110_09195_b200 import build
 
@@ -24,3 +26,15 @@ def test_the_library_is_built_where_the_module_cannot_be(monkeypatch, tmp_path, 
         with pytest.raises((RuntimeError, OSError)):
             build.build_fast()
     assert not build.FAST.exists()
+
+
+def test_the_module_is_built_anew_for_another_torch(monkeypatch):
+    build.build_fast()
+    commands = []
+    monkeypatch.setattr(subprocess, "run", lambda cmd, **_: commands.append(cmd) or subprocess.CompletedProcess(cmd, 1, "", ""))
+    build.build_fast()
+    assert not commands   # up to date
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.raises(RuntimeError):
+        build.build_fast()
+    assert len(commands) == 1 and any("0.0.1" in a for a in commands[0])

@@ -81,6 +81,15 @@ def test_without_the_module_the_python_checks_make_the_calls(without_module):
     layer.destroy()
 
 
+def test_a_module_built_for_another_torch_is_not_used(monkeypatch):
+    assert binding._load_fast().TORCH_VERSION == torch.__version__
+    monkeypatch.setattr(binding, "_fast", None)
+    monkeypatch.setattr(torch, "__version__", "0.0.1")
+    with pytest.warns(RuntimeWarning, match="not 0.0.1"):
+        assert binding._load_fast().layer_forward(bytes(48), None, None, 0, 0) == -1
+    assert binding._fast is binding._PythonChecks
+
+
 def _layer(shape, seed=3, act_type=snn.ACT_BIN, device=0, cls=snn.SnnConv):
     p = wl.draw_layer_params(shape, 5, seed)
     return cls(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha, shape.stride, shape.pad, act_type, device)
