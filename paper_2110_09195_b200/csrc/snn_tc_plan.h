@@ -95,6 +95,18 @@ struct GLayer {
   uint32_t tap[kGTapsMax];    // per step: start of its rows in the unit (16-byte units) | distance of its two chunks << 16
 };
 
+// The launches of a chain of words with tags, counted in one number in device memory: every CTA adds its share when it ends, the
+// shares of a launch make 2^32, and the upper half is what all CTAs of the next launch take their tag from.  (A count per CTA
+// would never come together again once launches that must not overlap did; this one is whole whenever all have ended.)
+struct GLaunches {
+  unsigned long long* count;
+  unsigned long long share, rest;   // each CTA's; what CTA 0 adds on top
+};
+inline GLaunches g_launches(unsigned long long* count, uint32_t ctas) {
+  const unsigned long long share = (1ull << 32) / ctas;
+  return {count, share, (1ull << 32) - share * ctas};
+}
+
 struct GParams {
   const GLayer* layers;
   const uint16_t* ranks;  // [n_layers][grid] CTA b takes a problem's tiles ranks[b], ranks[b] + grid, ...
@@ -102,7 +114,7 @@ struct GParams {
   const void* act[SNN_GROUP_MAX];
   void* out[SNN_GROUP_MAX];
   int* status;
-  uint32_t* launches;     // chain of words with tags: [grid] launches each CTA has been through; the next one's tag is one more
+  GLaunches launches;     // chain of words with tags
   uint8_t out_type[SNN_GROUP_MAX];   // per member: 0 fp32 alpha*S, 1 int32 S, 2 packed signs of alpha*S + shift, 3 those with tags
   uint32_t acc_cols;      // tensor-memory columns of one accumulator buffer
   int n_acc;              // accumulator buffers (tile seq of a CTA uses buffer seq % n_acc)

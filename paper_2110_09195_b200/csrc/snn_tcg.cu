@@ -35,7 +35,7 @@
 // Independent problems (a group) need nothing else.  A chain (a stack: problem i + 1 reads the packed signs
 // problem i writes) runs in the same launch.  Where few words lie between its members (g_tagged) every word carries the tag of
 // the launch that wrote it, and the expanders look at the words themselves until all they need are there: no fence, counter
-// or memset between a sign and its reader.  The tag is a count of launches kept per CTA in device memory, so that a
+// or memset between a sign and its reader.  The tag is a count of launches kept in device memory (GLaunches), so that a
 // replayed graph counts too.  Other chains run on per-tile completion counters: the epilogue bumps the counter
 // of a position tile when its part is written, and the expanders of the successor wait (bounded) until the
 // tiles under a tile's input window are complete.  The launch is cooperative then, so that all CTAs are
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     bar_sync_some<2, SETUP_THREADS>();
   }
   grid_dep_launch();
-  const uint32_t tag = TAGGED ? __ldcg(p.launches + blockIdx.x) + 1u : 0u;   // the same in all CTAs (counted up at the end)
+  const uint32_t tag = TAGGED ? (uint32_t)(__ldcg(p.launches.count) >> 32) + 1u : 0u;   // (complete only when all CTAs have ended)
   if (warp >= 1 && warp < 2 + G_EW) {
     tc_fence_before();
     bar_sync_some<1, 32 * (1 + G_EW)>();
@@ -1168,7 +1168,9 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   // ---------------------------------------------------------------- teardown
   tc_fence_before();
   __syncthreads();
-  if (TAGGED && tid == 0) p.launches[blockIdx.x] = tag;
+  if (TAGGED && tid == 0)
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p.launches.count), "l"(p.launches.share + (blockIdx.x == 0 ? p.launches.rest : 0ull))
+                 : "memory");
   if (warp == 2) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");
   }
@@ -1357,7 +1359,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint16_t));
   const size_t blob_bytes = deps_at + up(deps.size() * sizeof(uint2)), blob_at = up(w_total), done_at = blob_at + blob_bytes;
   const size_t launches_at = done_at + up(done_words * sizeof(uint32_t));
-  const size_t chain_at = launches_at + (tagged ? up((size_t)grid * sizeof(uint32_t)) : 0);
+  const size_t chain_at = launches_at + (tagged ? up(sizeof(unsigned long long)) : 0);
   cudaError_t e = cudaMalloc(&Gd->mem, chain_at + chain_bytes);
   if (e == cudaSuccess) {
     Gd->layers_dev = reinterpret_cast<GLayer*>(Gd->mem + blob_at);
@@ -1412,7 +1414,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->p = ring;
   Gd->p.layers = Gd->layers_dev;
   Gd->p.ranks = Gd->ranks;
-  if (tagged) Gd->p.launches = reinterpret_cast<uint32_t*>(Gd->mem + launches_at);
+  if (tagged) Gd->p.launches = g_launches(reinterpret_cast<unsigned long long*>(Gd->mem + launches_at), (uint32_t)grid);
   Gd->p.one = plan[0].L;
   Gd->smem = smem;
   *out = Gd;

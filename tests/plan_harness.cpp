@@ -60,6 +60,14 @@ uint32_t plan_divide(uint32_t q, uint32_t d) {
   return (uint32_t)((uint64_t)(2u * q) * f.m >> 32) >> f.s;
 }
 
+// The count of a chain's launches of `ctas` CTAs after those in `ended` (ranks, in this order) have ended.
+uint64_t plan_launches(uint32_t ctas, const uint32_t* ended, int n) {
+  unsigned long long count = 0;
+  const GLaunches l = g_launches(&count, ctas);
+  for (int i = 0; i < n; ++i) *l.count += l.share + (ended[i] == 0 ? l.rest : 0ull);   // as the kernel's tear-down does
+  return count;
+}
+
 // A plan of a given tile: the epilogue warps that write of a position tile, rows a copy or pixel of it has (0: cannot be planned).
 int plan_tile(const int* v, int f16, int kind, int lg, int Np, int* rows) {
   GPlan plan;

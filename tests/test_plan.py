@@ -136,3 +136,21 @@ def test_division_by_run_time_constants_is_exact_below_2_to_the_31(lib):
         last = top // d * d   # the largest multiple: the quotient changes there
         for q in (0, 1, d - 1, d, min(2 * d - 1, top), last - 1 if last else 0, last, top, *(rng.randint(0, top) for _ in range(20))):
             assert lib.plan_divide(q, d) == q // d, (q, d)
+
+
+@pytest.mark.parametrize("ctas", [1, 2, 3, 7, 64, 100, 147, 148, 160])
+def test_launches_of_a_chain_are_counted_whole(lib, ctas):
+    """The upper half of the count is the same for every CTA of a launch, and right again after launches that overlapped."""
+    lib.plan_launches.restype = ctypes.c_uint64
+    rng = random.Random(ctas)
+
+    def count(ended):
+        a = np.array(ended, np.uint32)
+        return lib.plan_launches(ctas, a.ctypes.data_as(ctypes.POINTER(ctypes.c_uint32)), len(a))
+
+    once, twice = list(range(ctas)), list(range(ctas)) * 2
+    for _ in range(20):
+        rng.shuffle(once)
+        rng.shuffle(twice)   # two launches whose CTAs end in any order
+        assert [count(once[:k]) >> 32 for k in range(ctas)] == [0] * ctas   # a CTA that starts late takes the same tag
+        assert count(once) == 1 << 32 and count(twice) == 2 << 32
