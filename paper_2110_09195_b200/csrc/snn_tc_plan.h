@@ -100,11 +100,11 @@ struct GLayer {
 // would never come together again once launches that must not overlap did; this one is whole whenever all have ended.)
 struct GLaunches {
   unsigned long long* count;
-  unsigned long long share, rest;   // each CTA's; what CTA 0 adds on top
+  unsigned long long share;   // each CTA's; CTA 0 adds what they leave of 2^32 on top
 };
-inline GLaunches g_launches(unsigned long long* count, uint32_t ctas) {
-  const unsigned long long share = (1ull << 32) / ctas;
-  return {count, share, (1ull << 32) - share * ctas};
+inline GLaunches g_launches(unsigned long long* count, uint32_t ctas) { return {count, (1ull << 32) / ctas}; }
+__host__ __device__ inline unsigned long long g_launch_share(const GLaunches& l, uint32_t cta, uint32_t ctas) {
+  return cta ? l.share : (1ull << 32) - l.share * (ctas - 1);
 }
 
 struct GParams {

@@ -1169,7 +1169,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   tc_fence_before();
   __syncthreads();
   if (TAGGED && tid == 0)
-    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p.launches.count), "l"(p.launches.share + (blockIdx.x == 0 ? p.launches.rest : 0ull))
+    asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(p.launches.count), "l"(g_launch_share(p.launches, blockIdx.x, gridDim.x))
                  : "memory");
   if (warp == 2) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512) : "memory");

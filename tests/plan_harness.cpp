@@ -64,7 +64,7 @@ uint32_t plan_divide(uint32_t q, uint32_t d) {
 uint64_t plan_launches(uint32_t ctas, const uint32_t* ended, int n) {
   unsigned long long count = 0;
   const GLaunches l = g_launches(&count, ctas);
-  for (int i = 0; i < n; ++i) *l.count += l.share + (ended[i] == 0 ? l.rest : 0ull);   // as the kernel's tear-down does
+  for (int i = 0; i < n; ++i) *l.count += g_launch_share(l, ended[i], ctas);   // as the kernel's tear-down does
   return count;
 }
 
