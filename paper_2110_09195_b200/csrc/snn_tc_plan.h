@@ -91,6 +91,7 @@ struct GLayer {
   const uint2* deps;          // [position tiles] first and last position tile of the predecessor this one reads (x > y: none)
   const uint32_t* prev_done;  // the predecessor's completion counters, and the count that means "complete"
   uint32_t prev_target;
+  int next;                   // the next problem in which this CTA has a tile, filled in as `first` is
   uint32_t* done;             // [position tiles] epilogue warps that have written their part, over all its channel tiles
   uint32_t tap[kGTapsMax];    // per step: start of its rows in the unit (16-byte units) | distance of its two chunks << 16
 };
@@ -109,7 +110,8 @@ __host__ __device__ inline unsigned long long g_launch_share(const GLaunches& l,
 
 struct GParams {
   const GLayer* layers;
-  const uint16_t* ranks;  // [n_layers][grid] CTA b takes a problem's tiles ranks[b], ranks[b] + grid, ...
+  const uint32_t* ranks;  // [n_layers][grid] CTA b takes a problem's tiles r, r + grid, ... (r: lower half of ranks[b]); upper half:
+                          // the next problem in which it has a tile (n_layers: none)
   int n_layers;
   const void* act[SNN_GROUP_MAX];
   void* out[SNN_GROUP_MAX];
@@ -177,6 +179,7 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   GLayer& o = P->L;
   o.wt = nullptr; o.alpha = o.shift = nullptr; o.deps = nullptr; o.prev_done = nullptr; o.prev_target = 0; o.done = nullptr;
   o.first = 0;
+  o.next = 1;   // (as it is in a launch of one problem)
   const int cpc = mode == M_F16 ? 8 : 32;
   const int S = g.stride, G = 1 << lg;
   const bool one = g.ksize == 1;
@@ -551,7 +554,7 @@ bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma,
 // and the first (tiles % grid) CTAs in the problem's rank order get one more; the rank order is
 // by the time the CTAs have been given so far, least first, so that the CTAs end close
 // together although a tile of one problem may take six times as long as a tile of another.
-void g_assign(const std::vector<GPlan>& P, int grid, std::vector<uint16_t>* ranks) {
+void g_assign(const std::vector<GPlan>& P, int grid, std::vector<uint32_t>* ranks) {
   std::vector<double> busy(grid, 0.0);
   std::vector<int> order(grid);
   for (size_t i = 0; i < P.size(); ++i) {
@@ -560,8 +563,17 @@ void g_assign(const std::vector<GPlan>& P, int grid, std::vector<uint16_t>* rank
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return busy[a] < busy[b]; });
     const int base = P[i].L.total_tiles / grid, rem = P[i].L.total_tiles % grid;
     for (int r = 0; r < grid; ++r) {
-      (*ranks)[i * grid + order[r]] = (uint16_t)r;
+      (*ranks)[i * grid + order[r]] = (uint32_t)r;
       busy[order[r]] += cost * (base + (r < rem ? 1 : 0));
+    }
+  }
+  for (int b = 0; b < grid; ++b) {
+    uint32_t next = (uint32_t)P.size();
+    for (size_t i = P.size(); i-- > 0;) {
+      uint32_t& at = (*ranks)[i * grid + b];
+      const bool has = at < (uint32_t)P[i].L.total_tiles;
+      at |= next << 16;
+      if (has) next = (uint32_t)i;
     }
   }
 }

@@ -316,10 +316,13 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const int words = p.n_layers * (int)(sizeof(GLayer) / 4);
       for (int i = rank; i < words; i += SETUP_THREADS) dst[i] = __ldg(src + i);
       // (loaded here for all problems: a global load at the start of a problem would queue behind the epilogue's stores)
-      int first = 0;
-      if (rank < p.n_layers) first = (int)__ldg(p.ranks + (size_t)rank * G + blockIdx.x);
+      uint32_t own = 0;
+      if (rank < p.n_layers) own = __ldg(p.ranks + (size_t)rank * G + blockIdx.x);
       bar_sync_some<2, SETUP_THREADS>();
-      if (rank < p.n_layers) lay[rank].first = first;
+      if (rank < p.n_layers) {
+        lay[rank].first = (int)(own & 0xffffu);
+        lay[rank].next = (int)(own >> 16);
+      }
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     bar_sync_some<2, SETUP_THREADS>();
@@ -808,35 +811,20 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         ready = !CHAIN;
         ++tile_seq;
       };
-      auto read_layer = [&]() {
+      // The CTA's first tile in layer il (n_layers: there is none).  Which layers it has tiles in comes from the host: a search
+      // for the next one in here was compiled wrongly for the variant with tags (nvcc 12.9.86: found in layer 1, it went on with the
+      // first tile of layer 2; not with the compiler's optimiser at -O1, whatever ptxas did, nor with a note taken in the loop).
+      auto enter_layer = [&]() {
+        ivalid = il < p.n_layers;
+        if (!ivalid) return;
         const GLayer& L = lay[il];
+        itile = L.first; itotal = L.total_tiles;
         Rr = L.Rr; n_cb = L.n_cb; cbc = L.cb_chunks; Cw = L.Cw; planes = L.n_planes; cpl = L.cpl; H = L.H; W = L.W; cs = L.cs;
         act = reinterpret_cast<const uint32_t*>(p.act[il]);
         kstep = g_word_step(Cw, cbc);
         if (TAGGED && il > 0 && kstep > 2) kstep = 2;
         icb = 0;
-        ivalid = true;
         enter_tile();
-      };
-      auto enter_layer = [&]() {   // first layer from il on in which this CTA has a tile
-        if constexpr (TAGGED) {
-          // (not the loop below: compiled for this variant, one of its copies went on to the next layer after it had found one)
-#pragma unroll 1
-          while (il < p.n_layers && (itile = lay[il].first) >= lay[il].total_tiles) ++il;
-          ivalid = il < p.n_layers;
-          if (!ivalid) return;
-          itotal = lay[il].total_tiles;
-          read_layer();
-        } else {
-          for (; il < p.n_layers; ++il) {
-            itile = lay[il].first;
-            itotal = lay[il].total_tiles;
-            if (itile >= itotal) continue;
-            read_layer();
-            return;
-          }
-          ivalid = false;
-        }
       };
       auto next_unit = [&]() {     // the unit after (il, itile, icb) in the CTA's sequence
         ++iu;
@@ -845,7 +833,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           icb = 0;
           itile += G;
           if (itile >= itotal) {
-            ++il;
+            il = lay[il].next;
             enter_layer();
           } else {
             enter_tile();
@@ -931,11 +919,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         g.cstride = cstride;
         g.flags = flags;
       };
+      if (lay[0].first >= lay[0].total_tiles) il = lay[0].next;
       enter_layer();
       seek_own();
       // completion side: this team's slots gx, gx + XG, ... of the ring
       a_slot = gx;
-      XGroup cur = {}, nxt;
+      XGroup cur, nxt = {};   // (a unit's last group leaves items unwritten, and all of them are copied)
       auto not_ready = [&]() {     // the wait for a chain's input ran out
         if (lane == 0 && !*abort_flag) {
           *abort_flag = 1;
@@ -1188,7 +1177,7 @@ struct GroupDev {
   uint32_t* done = nullptr;       // completion counters of all members' position tiles
   size_t done_words = 0;
   GLayer* layers_dev = nullptr;   // [count]
-  uint16_t* ranks = nullptr;      // [count][grid] tile assignment, see tcg_create
+  uint32_t* ranks = nullptr;      // [count][grid] tile assignment, see GParams
   GParams p{};                    // everything but the per-call pointers
   size_t smem = 0;
   int grid = 0;
@@ -1344,7 +1333,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
       }
     }
   }
-  std::vector<uint16_t> ranks((size_t)count * grid);
+  std::vector<uint32_t> ranks((size_t)count * grid);
   g_assign(plan, grid, &ranks);
   GroupDev* Gd = new GroupDev();
   Gd->count = count;
@@ -1356,14 +1345,14 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   // One allocation and one copy for everything the group owns: [weight operands][descriptions][ranks][dependencies]
   // [counters][packed signs between the members]; the middle three come from the host.
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
-  const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint16_t));
+  const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint32_t));
   const size_t blob_bytes = deps_at + up(deps.size() * sizeof(uint2)), blob_at = up(w_total), done_at = blob_at + blob_bytes;
   const size_t launches_at = done_at + up(done_words * sizeof(uint32_t));
   const size_t chain_at = launches_at + (tagged ? up(sizeof(unsigned long long)) : 0);
   cudaError_t e = cudaMalloc(&Gd->mem, chain_at + chain_bytes);
   if (e == cudaSuccess) {
     Gd->layers_dev = reinterpret_cast<GLayer*>(Gd->mem + blob_at);
-    Gd->ranks = reinterpret_cast<uint16_t*>(Gd->mem + blob_at + rank_at);
+    Gd->ranks = reinterpret_cast<uint32_t*>(Gd->mem + blob_at + rank_at);
     Gd->done = reinterpret_cast<uint32_t*>(Gd->mem + done_at);
     Gd->chain_buf = Gd->mem + chain_at;
   }
@@ -1403,7 +1392,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     if (e == cudaSuccess) *launched += 1;
   }
   for (int i = 0; i < count; ++i) memcpy(blob.data() + sizeof(GLayer) * (size_t)i, &plan[i].L, sizeof(GLayer));
-  memcpy(blob.data() + rank_at, ranks.data(), ranks.size() * sizeof(uint16_t));
+  memcpy(blob.data() + rank_at, ranks.data(), ranks.size() * sizeof(uint32_t));
   if (!deps.empty()) memcpy(blob.data() + deps_at, deps.data(), deps.size() * sizeof(uint2));
   if (e == cudaSuccess) e = cudaMemcpyAsync(Gd->mem + blob_at, blob.data(), blob_bytes, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // the host arrays live on this stack

@@ -68,6 +68,15 @@ uint64_t plan_launches(uint32_t ctas, const uint32_t* ended, int n) {
   return count;
 }
 
+// The tiles of problems of so many dealt to `grid` CTAs: ranks per problem and CTA as GParams has them.
+void plan_assign(const int* tiles, int count, int grid, uint32_t* ranks) {
+  std::vector<GPlan> plan(count);
+  for (int i = 0; i < count; ++i) plan[i].L.total_tiles = tiles[i];
+  std::vector<uint32_t> r((size_t)count * grid);
+  g_assign(plan, grid, &r);
+  std::copy(r.begin(), r.end(), ranks);
+}
+
 // A plan of a given tile: the epilogue warps that write of a position tile, rows a copy or pixel of it has (0: cannot be planned).
 int plan_tile(const int* v, int f16, int kind, int lg, int Np, int* rows) {
   GPlan plan;

@@ -87,6 +87,27 @@ def test_group_ragged_members(snn, oracle_mod):
     check_bin_group(snn, oracle_mod, members, 5, 21)
 
 
+def test_group_whose_ctas_pass_members_by(snn, oracle_mod):
+    """Members of one tile between and after members of many: most CTAs have no tile in four and in three members in a row."""
+    few, many = wl.LayerShape(16, 16, 6, 6, 1, 1), wl.LayerShape(64, 64, 56, 56, 1, 1)
+    members = [(many, 8), *[(few, 1)] * 4, (wl.LayerShape(64, 64, 28, 28, 1, 1), 8), *[(few, 1)] * 3]
+    check_bin_group(snn, oracle_mod, members, 5, 27)
+    layers, acts, want = [], [], []
+    for i, (shape, n) in enumerate(members):
+        p = wl.draw_layer_params(shape, 5, 27 + i)
+        packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 27 + i))
+        want.append(_pack_signs(oracle_mod.conv_bin(p.codebook, 5, p.idx_packed, p.alpha, shape.c_in, shape.c_out, 1, 1, packed)[1]))
+        layers.append(snn.SnnConv(shape.c_in, shape.c_out, 5, p.codebook, p.idx_packed, p.alpha))
+        acts.append(torch.from_numpy(packed.view(np.int32)).cuda())
+    group = snn.SnnConvGroup(layers, [(n, s.h, s.w) for s, n in members])
+    outs = group.forward(acts, out_type=snn.OUT_BITS)
+    for got, ref in zip(outs, want):
+        assert (got.cpu().numpy().view(np.uint32) == ref).all()
+    group.destroy()
+    for l in layers:
+        l.destroy()
+
+
 @pytest.mark.parametrize("net,cfg", [("resnet20", 1), ("resnet18", 2)])
 def test_group_stack_small_batch(snn, oracle_mod, net, cfg):
     """The whole stack as one group (all layers, in order), batch 2."""

@@ -154,3 +154,14 @@ def test_stack_replayed_as_a_graph(snn, oracle_mod):
     stack.destroy()
     for l in layers:
         l.destroy()
+
+
+@pytest.mark.parametrize("h,w,n", [(40, 50, 4), (100, 150, 5)])   # words with tags, and counters
+def test_stack_whose_ctas_pass_members_by(snn, oracle_mod, h, w, n):
+    """Members of a few tiles in a row, then one of more: most CTAs have no tile in several members, and some have one again."""
+    chans, strides = (64, 40, 16, 16, 16, 16, 16, 512, 24), (1, 2, 2, 2, 2, 1, 1, 1)
+    shapes = []
+    for a, b, s in zip(chans, chans[1:], strides):
+        shapes.append(wl.LayerShape(a, b, h, w, s, 1))
+        h, w = shapes[-1].h_out, shapes[-1].w_out
+    _check_chain(snn, oracle_mod, shapes, 5, n, 361, repeats=1)

@@ -154,3 +154,18 @@ def test_launches_of_a_chain_are_counted_whole(lib, ctas):
         rng.shuffle(twice)   # two launches whose CTAs end in any order
         assert [count(once[:k]) >> 32 for k in range(ctas)] == [0] * ctas   # a CTA that starts late takes the same tag
         assert count(once) == 1 << 32 and count(twice) == 2 << 32
+
+
+def test_every_cta_finds_its_next_tile(lib):
+    """Tiles are dealt once each, and a CTA is told the next problem in which it has one, whatever it passes by."""
+    rng = random.Random(12)
+    for tiles in [[1], [1, 1, 1], [148] * 3, [414, 1, 1, 1, 1, 109, 1, 1, 1], [267, 135, 106, 88, 28, 28, 112, 28],
+                  *([rng.choice((1, 2, 5, 30, 147, 148, 149, 400)) for _ in range(rng.randint(1, 32))] for _ in range(40))]:
+        grid = min(SMS, sum(tiles))
+        ranks = np.zeros((len(tiles), grid), np.uint32)
+        lib.plan_assign(_array(tiles), len(tiles), grid, ranks.ctypes.data_as(ctypes.POINTER(ctypes.c_uint32)))
+        assert (np.sort(ranks & 0xffff, axis=1) == np.arange(grid)).all()
+        has = (ranks & 0xffff) < np.array(tiles)[:, None]
+        for i in range(len(tiles)):
+            for b in range(grid):
+                assert ranks[i, b] >> 16 == next((k for k in range(i + 1, len(tiles)) if has[k, b]), len(tiles))
