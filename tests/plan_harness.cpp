@@ -60,6 +60,9 @@ uint32_t plan_divide(uint32_t q, uint32_t d) {
   return (uint32_t)((uint64_t)(2u * q) * f.m >> 32) >> f.s;
 }
 
+// Does a chain with at most so many words between two members run on words with tags?
+int plan_tagged(uint64_t words) { return g_tagged((size_t)words); }
+
 // The count of a chain's launches of `ctas` CTAs after those in `ended` (ranks, in this order) have ended.
 uint64_t plan_launches(uint32_t ctas, const uint32_t* ended, int n) {
   unsigned long long count = 0;

@@ -1,6 +1,8 @@
 """The dependent stack (snn_conv_stack_*: layers chained through their packed thresholded signs, one
-persistent launch with per-tile completion counters) against the same chain through the CPU oracle:
-every layer's signs are an integer decision, so the chain is compared bit for bit."""
+persistent launch) against the same chain through the CPU oracle: every layer's signs are an integer
+decision, so the chain is compared bit for bit.  Where at most 2^17 words lie between two members the
+words carry tags, else the members' tiles are counted: two variants of the kernel, and each of the
+shapes that need care runs on both (tests/test_plan.py checks which of them a chain gets)."""
 import numpy as np
 import pytest
 import torch
@@ -47,13 +49,16 @@ def _build_chain(snn, oracle_mod, shapes, tau, n, seed):
         alpha[::7] *= -1.0
         # thresholds of the size of the sums' spread keep the signs balanced through the chain
         shift = (rng.normal(0.0, 1.0, size=shape.c_out) * np.sqrt(9.0 * shape.c_in) * 0.5).astype(np.float32)
-        s_ref, y_ref = oracle_mod.conv_bin(p.codebook, tau, p.idx_packed, alpha, shape.c_in, shape.c_out, shape.stride,
-                                           shape.pad, x)
+        if shape.ksize == 1:
+            s_ref, y_ref = oracle_mod.conv1x1_bin(p.codebook, tau, p.idx_packed, alpha, shape.c_in, shape.c_out, shape.stride, x)
+        else:
+            s_ref, y_ref = oracle_mod.conv_bin(p.codebook, tau, p.idx_packed, alpha, shape.c_in, shape.c_out, shape.stride,
+                                               shape.pad, x)
         last = (s_ref, y_ref)
         x = _pack_signs(y_ref, shift)
         mids.append(x)
         layers.append(snn.SnnConv(shape.c_in, shape.c_out, tau, p.codebook, p.idx_packed, alpha, shape.stride,
-                                  shape.pad, snn.ACT_BIN, shift=shift))
+                                  shape.pad, snn.ACT_BIN, shift=shift, ksize=shape.ksize))
     return layers, first, mids, last
 
 
@@ -165,3 +170,32 @@ def test_stack_whose_ctas_pass_members_by(snn, oracle_mod, h, w, n):
         shapes.append(wl.LayerShape(a, b, h, w, s, 1))
         h, w = shapes[-1].h_out, shapes[-1].w_out
     _check_chain(snn, oracle_mod, shapes, 5, n, 361, repeats=1)
+
+
+def chain_shapes(chans, h, w, strides, pads, ksizes):
+    shapes = []
+    for a, b, s, p, k in zip(chans, chans[1:], strides, pads, ksizes):
+        shapes.append(wl.LayerShape(a, b, h, w, s, p, k))
+        h, w = shapes[-1].h_out, shapes[-1].w_out
+    return shapes
+
+
+# channels, map, strides, pads, kernel sizes, batch with tags, batch with counters
+CHAINS = [
+    # two and three words a pixel, a last word of few channels, no padding, channel tiles of 2 and 9 channels
+    ((33, 40, 70, 24, 130, 9), 13, 11, (1, 2, 1, 1, 2), (1, 1, 0, 1, 1), (3,) * 5, 458, 480),
+    # five, seven and nine words a pixel: one word a load, blocks of several chunks; an odd map without padding
+    ((160, 200, 257, 288, 70), 15, 9, (1, 1, 2, 1), (1, 0, 1, 1), (3,) * 4, 138, 175),
+    # groups of two, four and eight pixels a position, stride 2
+    ((20, 64, 17, 31, 16, 48), 37, 29, (1, 1, 2, 1, 2), (1, 1, 1, 0, 1), (3,) * 5, 61, 67),
+    # a bottleneck: 1x1, 3x3 at stride 2, 1x1
+    ((256, 72, 136, 512), 28, 28, (1, 2, 1), (0, 1, 0), (1, 3, 1), 55, 58),
+    # one member: nothing lies between members (tags whatever the batch)
+    ((40, 70), 13, 11, (2,), (1,), (3,), 5, None),
+]
+
+
+@pytest.mark.parametrize("chain,n", [(c, n) for c in CHAINS for n in c[6:] if n],
+                         ids=lambda v: "-".join(map(str, v[0])) if isinstance(v, tuple) else str(v))
+def test_stack_by_tags_and_by_counters(snn, oracle_mod, chain, n):
+    _check_chain(snn, oracle_mod, chain_shapes(*chain[:6]), 6, n, 371, repeats=1)

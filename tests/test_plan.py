@@ -169,3 +169,23 @@ def test_every_cta_finds_its_next_tile(lib):
         for i in range(len(tiles)):
             for b in range(grid):
                 assert ranks[i, b] >> 16 == next((k for k in range(i + 1, len(tiles)) if has[k, b]), len(tiles))
+
+
+def _words(shapes, n):
+    return max((n * s.h_out * s.w_out * ((s.c_out + 31) // 32) for s in shapes[:-1]), default=0)
+
+
+def test_which_chains_of_the_gpu_tests_carry_tags(lib):
+    """The stacks that are compared on the GPU stand on the sides of the rule that they are meant to."""
+    import test_gpu_stack as gpu
+    import workloads as wl
+    lib.plan_tagged.argtypes = [ctypes.c_uint64]
+    assert lib.plan_tagged(0) and lib.plan_tagged(1 << 17) and not lib.plan_tagged((1 << 17) + 1)
+    for chain in gpu.CHAINS:
+        shapes = gpu.chain_shapes(*chain[:6])
+        assert lib.plan_tagged(_words(shapes, chain[6])), chain
+        assert chain[7] is None or not lib.plan_tagged(_words(shapes, chain[7])), chain
+    pair = [wl.LayerShape(16, 16, 32, 32, 1, 1)] * 2
+    assert _words(pair, 128) == 1 << 17 and not lib.plan_tagged(_words(pair, 129))
+    for net, n, tags in (("resnet18", 2, True), ("resnet18", 64, False), ("resnet20", 4, True)):
+        assert bool(lib.plan_tagged(_words(wl.get_workload(net).layers, n))) == tags
