@@ -11,6 +11,7 @@ from paper_2110_09195_b200 import binding
 
 
 def test_anything_unusual_is_left_to_the_python_checks():
+    """Where there is no GPU: CPU tensors, and arguments of other kinds, do no harm."""
     fast = binding._load_fast()
     x, y = torch.zeros((1, 4, 4, 1), dtype=torch.int32), torch.zeros((1, 4, 4, 16))
     desc = bytes(48)
@@ -115,6 +116,50 @@ def test_both_ways_launch_the_same(act_type):
         group.forward([x, x], outs, out_type=out_type)
         group.forward((x, x), tuple(want), out_type=out_type)   # (not lists: the Python checks)
         assert all(torch.equal(p, q) for p, q in zip(outs, want)) and torch.equal(outs[0], a)
+
+
+@pytest.mark.gpu
+def test_the_usual_call_is_taken_and_any_other_left():
+    """The native checks make a valid call themselves; with one argument changed they launch nothing and leave it."""
+    fast = binding._load_fast()
+    layer = _layer(wl.LayerShape(40, 72, 9, 7, 2, 1))
+    group, stack = snn.SnnConvGroup([layer, layer], [(3, 9, 7)] * 2), snn.SnnConvStack([layer], 3, 9, 7)
+    x, y = torch.zeros((3, 9, 7, 2), dtype=torch.int32, device="cuda"), layer.alloc_out(3, 9, 7)
+    bits, sums = layer.alloc_out(3, 9, 7, snn.OUT_BITS), layer.alloc_out(3, 9, 7, snn.OUT_I32)
+    base = (layer._desc, x, y, snn.OUT_F32, snn.PATH_AUTO)
+    no_x = [x.cpu(), x.float(), x[:2], x[..., :1].contiguous(), x.transpose(1, 2), x[0], x.to_sparse(), None, [x]]
+    no_y = [y.cpu(), sums, y[:2], y[..., :71].contiguous(), y.transpose(1, 2), bits, None, [y]]
+
+    class Tensor(torch.Tensor):
+        pass
+    no_x.append(x.as_subclass(Tensor))
+
+    def launches(call, *args):
+        before = snn.kernel_launches()
+        return call(*args), snn.kernel_launches() - before
+
+    for good in (base, (layer._desc, x.view(torch.uint32), *base[2:]), (layer._desc, x, bits, snn.OUT_BITS, 0),
+                 (layer._desc, x, sums, snn.OUT_I32, 0), (layer._desc, torch.nn.Parameter(x, requires_grad=False), *base[2:])):
+        st, n = launches(fast.layer_forward, *good)
+        assert st == 0 and n >= 1
+    for i, values in enumerate(([layer._desc[:40], None, bytearray(layer._desc)], no_x, no_y, [snn.OUT_I32, snn.OUT_BITS, 7, -1, 0.0, True, None],
+                                [7, -1, None])):
+        for v in values:
+            assert launches(fast.layer_forward, *base[:i], v, *base[i + 1:]) == (-1, 0), (i, v)
+
+    base = (group._desc, [x, x], [y, y.clone()], snn.OUT_F32)
+    assert launches(fast.group_forward, *base) == (0, 1)
+    for i, values in enumerate(([group._desc[:-8], group._desc[:47], None], [[x], (x, x), [x, x, x], *([x, v] for v in no_x), *([v, x] for v in no_x)],
+                                [[y], (y, y), *([y, v] for v in no_y)], [snn.OUT_I32, 7, None])):
+        for v in values:
+            assert launches(fast.group_forward, *base[:i], v, *base[i + 1:]) == (-1, 0), (i, v)
+
+    base = (stack._desc, x, y, snn.OUT_F32)
+    assert launches(fast.stack_forward, *base) == (0, 1)
+    for i, values in enumerate(([stack._desc[:47], None], no_x, no_y, [snn.OUT_I32, 7, None])):
+        for v in values:
+            assert launches(fast.stack_forward, *base[:i], v, *base[i + 1:]) == (-1, 0), (i, v)
+    torch.cuda.synchronize()
 
 
 @pytest.mark.gpu
