@@ -218,22 +218,24 @@ SNN_API snn_status_t snn_conv_group_destroy(snn_conv_group_t* g);
  * shift standing for the batch normalisation / Hardtanh between two binary layers, Sec. 5):
  * member i writes them into a buffer the stack owns and member i + 1 reads them as its
  * binary input.  Shortcut additions are not part of the path.  Inside the launch a tile of
- * member i + 1 starts as soon as the tiles of member i that hold its input pixels are
- * complete (per-tile completion counters in device memory, every wait bounded); there is
- * no grid-wide step between layers.
+ * member i + 1 starts as soon as member i has written its input pixels (every wait bounded);
+ * there is no grid-wide step between layers.  How it knows: where at most 2^17 words lie between
+ * any two members, every word carries a tag that says which launch wrote it; in larger stacks
+ * the tiles of member i that hold the pixels are complete (per-tile completion counters).
  *
  * snn_conv_stack_create: `layers` are `count` (1..SNN_GROUP_MAX) handles with binary
  * activations on one device whose shapes follow from one another (c_in of member i + 1 =
  * c_out of member i, its input map = member i's output map); N, H, W fix the input of
  * member 0.  The handles must outlive the stack.  The stack owns the buffers between its
- * members, the counters and its tiled weight operands.  Errors: INVALID_ARG (null, count,
+ * members, the counters or the count of its launches, and its tiled weight operands.  Errors: INVALID_ARG (null, count,
  * fp16 activations, shapes that do not chain, mixed devices), UNSUPPORTED (a member the
  * tensor-core path cannot run), CUDA, OOM.
  *
  * snn_conv_stack_forward: act_dev is member 0's input (DEVICE, binary layout), out_dev the
  * last member's output (DEVICE) of type out_type (SNN_OUT_F32, SNN_OUT_I32 or SNN_OUT_BITS);
  * both 16-byte aligned, neither kept.  Asynchronous on cuda_stream; allocates nothing.  Calls
- * on one stack must not overlap on the GPU (they share the buffers and counters).  All CTAs
+ * on one stack must not overlap on the GPU (they share the buffers and counters; the results
+ * of calls that did are undefined, or TIMEOUT, those of later calls are not affected).  All CTAs
  * of the launch must be resident together, which the launch checks (CUDA error otherwise).
  * Errors: INVALID_ARG, TIMEOUT (an earlier launch gave up a bounded wait), CUDA.
  */

@@ -51,8 +51,8 @@ __device__ __forceinline__ uint32_t mbar_test(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok;
 }
-// Bounded wait for the phase with the given parity; false when the limit ran out.  (Not unrolled, and neither are the kernel's
-// other loops around waits: the roles share the instruction caches.)
+// Bounded wait for the phase with the given parity; false when the limit ran out.  (Not unrolled: the roles share the
+// instruction caches, and every wait of the kernel is a copy of this.)
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   if (mbar_test(bar, parity)) return true;
 #pragma unroll 1

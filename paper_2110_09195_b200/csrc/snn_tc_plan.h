@@ -429,8 +429,10 @@ bool g_plan_by_end(const Geom& g, int mode, int kind, int sms, GPlan* plan) {
 // Do the packed signs between the members of a chain carry tags?  words: the most between two members.  A layer's signs then reach
 // the next layer's expanders 1.2 us sooner, but each word is twice as long and the expanders load two of them at a time
 // instead of four, which shows once a CTA has many tiles.  Measured on one B200 as graphs, counters and tags, us: ResNet-18 stack
-// batch 1 88 and 69, batch 8 95 and 82, 16 (100 k words) 100 and 99, 32 113 and 117, 64 134 and 145; ResNet-34 batch 1 169 and 132,
-// 16 191 and 188, 32 219 and 226; ResNet-20 batch 1 72 and 52, 64 99 and 88, 96 104 and 96, 128 (131 k words) 124 and 119.
+// batch 1 85 and 67, batch 8 93 and 81, 16 (100 k words) 98.6 and 96.9, 32 112 and 115, 64 132 and 142; ResNet-34 batch 1 162 and
+// 129, 16 187 and 184, 32 215 and 222; ResNet-20 batch 1 68 and 50, 64 99 and 86, 96 103 and 94, 128 (131 k words) 123 and 118.
+// (One rule for all: 200 k words are too many for the networks of one to sixteen words a pixel, and 131 k still gain where every
+// pixel is one.  A stack of one layer has no word between members, and with tags no counters to clear.)
 inline bool g_tagged(size_t words) { return words <= (size_t)1 << 17; }
 
 // The ring geometry of a launch of these problems and where its parts lie in shared memory; false where it does not fit.

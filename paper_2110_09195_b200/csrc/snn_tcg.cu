@@ -57,13 +57,14 @@
 //      warps 10-19   expanders (but 13 and 17): packed bits -> e2m1 nibbles (or fp16 copied)
 //                    into the activation ring
 //      warp 13       writes the epilogue's tables (where the columns of a tile go) ahead of it
-// The kernel is compiled per operand mode and per output kind (words, packed signs, chain), so that no variant
-// carries another one's code in its loops; the plan (tile shapes, accumulator buffers) is made per output kind.
-// The loops around the waits, tiles and problems are not unrolled (the compiler unrolls them four times, innermost and all
-// around): a variant is 62 KB of code then instead of 112, and five kinds of roles share an SM's instruction caches.  On one GPU,
+//      warp 17       in a chain on counters: waits for the tiles that the CTA's next tile reads
+// The kernel is compiled per operand mode and per output kind (words, packed signs, chains on counters, chains of words
+// with tags), so that no variant carries another one's code in its loops; the plan (tile shapes, accumulator buffers) is made
+// per output kind, the same for both kinds of chains.
+// The loops around the waits, tiles and problems that all variants have are not unrolled (the compiler unrolls them four times,
+// innermost and all around): a variant is 62 KB of code then instead of 112, and five kinds of roles share an SM's instruction caches.  On one GPU,
 // as a graph, unrolled and not: 1x1 layers at batch 16 108.8 and 94.6 us (signs 79.8 and 71.0), ResNet-18 group at
 // batch 16 36.7 and 32.3, ResNet-34 stack at batch 128 390 and 362, one layer of 256 channels 9.8 and 9.3, 39 layers 4 %.
-// (Rolling up the expanders' two copies of the load issue as well takes another 12 KB out and made chains 6 % slower.)
 // Every wait is bounded; one that runs out raises a status word the host reads, and
 // the CTA still frees its tensor memory and returns.
 #include <algorithm>
@@ -246,7 +247,8 @@ __device__ __forceinline__ uint32_t g_transpose32(uint32_t x, int lane) {
 
 // OUTK: what the epilogue is compiled for.  0: fp32 or int32 words for every member; 1: packed signs for every
 // member; 2: a chain - packed signs between the members, any type for the last, and the dependency waits and
-// completion counters; 3: a chain whose words carry tags instead.  Keeping the variants apart keeps each one's registers and code to what it needs.
+// completion counters; 3: a chain whose words carry tags instead.  Keeping the variants apart keeps each one's registers and
+// code to what it needs.
 enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2, OUT_TAGGED = 3 };
 
 template <int MODE, int OUTK>
@@ -999,7 +1001,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           if (stop) break;
         }
       } else {
-        // One copy of the load issue instead of two: 10 KB of code.  (In chains, whose tiles are small, two are 1 to 3 % faster.)
+        // One copy of the load issue instead of two: 10 KB of code.  (In chains on counters, whose tiles are small, two are 1 to 3 %
+        // faster; chains of words with tags have not been timed with two.)
         bool in_hand = false;   // is there a group to expand?
 #pragma unroll 1
         for (;;) {
@@ -1169,12 +1172,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
 struct GroupDev {
   int count = 0, act_type = 0, mode = M_FP4;
   int kind = TCG_WORDS;           // what the tiles were planned for (word outputs, packed signs, chain)
-  int chain = 0;                  // 1: member i + 1 reads the packed signs member i writes (one launch, dependency counters)
+  int chain = 0;                  // 1: member i + 1 reads the packed signs member i writes (one launch, on counters or with tags)
   uint8_t* mem = nullptr;         // all device memory of the group; the pointers below lie in it
   uint8_t* chain_buf = nullptr;   // the packed signs between the members, one buffer per boundary
   size_t chain_off[SNN_GROUP_MAX] = {};
   int tagged = 0;                 // a chain of words with tags (and without counters)
-  uint32_t* done = nullptr;       // completion counters of all members' position tiles
+  uint32_t* done = nullptr;       // a chain on counters: those of all members' position tiles
   size_t done_words = 0;
   GLayer* layers_dev = nullptr;   // [count]
   uint32_t* ranks = nullptr;      // [count][grid] tile assignment, see GParams
@@ -1343,7 +1346,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->chain = chain;
   Gd->kind = kind;
   // One allocation and one copy for everything the group owns: [weight operands][descriptions][ranks][dependencies]
-  // [counters][packed signs between the members]; the middle three come from the host.
+  // [counters][count of launches][packed signs between the members]; the three from the descriptions on come from the host.
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
   const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint32_t));
   const size_t blob_bytes = deps_at + up(deps.size() * sizeof(uint2)), blob_at = up(w_total), done_at = blob_at + blob_bytes;
@@ -1432,7 +1435,7 @@ struct GStepOf {
 // Bound by latency: two loads, a look-up, nine votes and the launch around them.
 // With one thread per row and word, 64 byte loads and 33 KB of straight-line code a thread, 14 calls took 4 % longer waited for
 // (193->168 channels of 9x26: 36.8 us, now 33.8).  8 images of a 128-channel 28x28 layer, copies and host work included: 16.6 us a
-// call back to back, all of it the host's, 30.2 waited for; by four decode kernels and the popcount kernel 46.
+// call back to back, all of it the host's (18.6 on another machine's), 30.2 waited for; by four decode kernels and the popcount kernel 46.
 constexpr int G_SW_ROWS = 8, G_SW_WARPS = 4;
 __global__ void __launch_bounds__(32 * G_SW_WARPS) g_static_weights_kernel(const uint8_t* __restrict__ stream, int n_bytes,
                                                                            const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
