@@ -47,7 +47,7 @@ struct GTile {
   int K, kp_log, lg, out_kind;         // channels; GLayer::kp_log, lg; GParams::out_type
   uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
   uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
-  float alpha[G_ROWS], shift[G_ROWS];
+  float alpha[G_ROWS], threshold[G_ROWS];
 };
 constexpr int G_TILES = 4;
 constexpr int G_EPI_BYTES = G_TILES * (int)sizeof(GTile);
@@ -67,7 +67,7 @@ constexpr int kGTapsMax = 52;                      // 3 kernel rows x at most 17
 struct GLayer {
   const uint8_t* wt;      // [channel tile][channel block][step][chunk][128][16 B], owned by the group
   const float* alpha;
-  const float* shift;     // per-channel constant added to alpha*S before the sign is taken (packed-sign output)
+  const float* threshold; // packed-sign output: per channel, the sum its bit changes at (g_sign_threshold)
   int N, H, W, C, K, Cw, pad, Ho, Wo;
   int rs, cm, cs;         // input pixel of position (i, j) in plane (pr, pc): row rs*i + pr - pad, column cm*j + cs*pc - pad
   int G, lg;              // output pixels per position and its logarithm
@@ -177,7 +177,7 @@ struct GPlan {
 // where that does not fit.
 bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, GPlan* P, int max_chunks = 8) {
   GLayer& o = P->L;
-  o.wt = nullptr; o.alpha = o.shift = nullptr; o.deps = nullptr; o.prev_done = nullptr; o.prev_target = 0; o.done = nullptr;
+  o.wt = nullptr; o.alpha = o.threshold = nullptr; o.deps = nullptr; o.prev_done = nullptr; o.prev_target = 0; o.done = nullptr;
   o.first = 0;
   o.next = 1;   // (as it is in a launch of one problem)
   const int cpc = mode == M_F16 ? 8 : 32;

@@ -232,15 +232,26 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
   return true;
 }
 
-// Rows of a 32 x 32 bit matrix (lane r holds row r) to columns (lane c holds column c, bit r = row r).
-__device__ __forceinline__ uint32_t g_transpose32(uint32_t x, int lane) {
+// Two 32 x 32 bit matrices side by side (lane r holds row r of both): rows to columns (lane c holds column c, bit r = row r).  A
+// stage is a shuffle and two instructions (the two widest one): bytes by a lane's own permutation, bits by its own rotation and mask.
+__device__ __forceinline__ void g_transpose32(uint32_t& x, uint32_t& z, int lane) {
+  uint32_t* const m[2] = {&x, &z};
 #pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) {
-    const uint32_t m = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u : 0x55555555u;
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
-    x = (lane & s) ? ((x & ~m) | ((y >> s) & m)) : ((x & m) | ((y << s) & ~m));
+  for (int s = 16; s >= 8; s >>= 1) {
+    const uint32_t order = s == 16 ? ((lane & 16) ? 0x3276u : 0x5410u) : (lane & 8) ? 0x3715u : 0x6240u;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) *m[i] = __byte_perm(*m[i], __shfl_xor_sync(0xffffffffu, *m[i], s), order);
   }
-  return x;
+#pragma unroll
+  for (int s = 4; s >= 1; s >>= 1) {
+    const uint32_t low = s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u : 0x55555555u, own = (lane & s) ? ~low : low;
+    const uint32_t turn = (lane & s) ? 32 - s : s;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const uint32_t y = __shfl_xor_sync(0xffffffffu, *m[i], s);
+      *m[i] = (*m[i] & own) | (__funnelshift_l(y, y, turn) & ~own);
+    }
+  }
 }
 
 }  // namespace
@@ -514,7 +525,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const int s_first = half + (lg ? 0 : 2 * ((rq * 32) >> kp_log)), s_step = lg ? 2 : 2 << (7 - kp_log);
       const int co = h0.z + c_lane, co_warp = h0.z + c_warp;
       const bool active = co_warp < K;   // does any of the warp's rows hold a channel?
-      const float al = T->alpha[c_lane], sh = WORDS ? 0.f : T->shift[c_lane];
+      const float al = T->alpha[c_lane], minus_threshold = WORDS ? 0.f : -T->threshold[c_lane];
+      const uint32_t flip = al < 0.f ? 0u : 0xffffffffu;   // (the bit is set below the threshold, or - where the sign bit of the difference is clear - from there on)
       {
         if (lane == 0) okw = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_accfull + 8u * (seq & 3u), tile_phase, 100))) ? 1 : 0;
         okw = __shfl_sync(0xffffffffu, okw, 0);
@@ -537,6 +549,28 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           release();
         } else {
           uint32_t* const obase = out32 + (size_t)((uint32_t)(g_lane * K + co));
+          uint32_t first = 0;   // signs: the bits of the slice before, where that waits for this one
+          bool held = false;
+          // this lane's column of slice s: word w of the warp's channels (the table's offsets are those of a pixel's words)
+          auto store_signs = [&](int s, uint32_t w) {
+            const uint32_t here = 1u << lane, Kw = (uint32_t)(K + 31) >> 5;
+            const uint32_t at = T->offset[32 * s + lane] + (uint32_t)g_warp * Kw + (uint32_t)(co_warp >> 5);
+            if (kp_log >= 5) {
+              if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) {
+                if (TAGGED && out_kind == 3) g_st_tagged(out32, at, w, tag);
+                else out32[at] = w;
+              }
+            } else {   // 16 rows per pixel: one word each for two pixels
+              const bool one = T->mask[g_warp * G_MAX_CHUNKS + s] & here, two = T->mask[(g_warp + 1) * G_MAX_CHUNKS + s] & here;
+              if (TAGGED && out_kind == 3) {
+                if (one) g_st_tagged(out32, at, w & 0xffffu, tag);
+                if (two) g_st_tagged(out32, at + 1, w >> 16, tag);
+              } else {
+                if (one) out32[at] = w & 0xffffu;
+                if (two) out32[at + 1] = w >> 16;
+              }
+            }
+          };
           // (a last slice of 16 columns is read as 32: the others belong to the next buffer or the scales and go nowhere)
 #pragma unroll 1
           for (int s = s_first; s < n_slices; s += s_step) {
@@ -567,14 +601,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                                : "memory");
               }
             } else {
-              // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): bit of a channel =
-              // fl(fl(alpha*S) + shift) >= 0 = sign bit clear (no sum is -0 or NaN: alpha and shift are finite and
-              // shift is not -0).  Multiply and add as packed fp32 pairs (each half rounds as the scalar instruction
-              // does), a lane gathers the bits of its channel over the 32 columns, and the transposition gives
-              // lane j the word of column j.
-              unsigned long long a2, t2;
-              asm("mov.b64 %0, {%1, %1};" : "=l"(a2) : "f"(al));
-              asm("mov.b64 %0, {%1, %1};" : "=l"(t2) : "f"(sh));
+              // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): a sum is compared with the
+              // channel's threshold (g_sign_threshold; the difference of two integers is exact), a lane gathers the bits of its
+              // channel over the 32 columns, and a 32 x 32 bit transposition in the warp gives lane j the word of column j.
+              // Bound by latency: 204 cycles of a slice's 970 went into scaled and shifted bits, 303 into the transposition, 290 into
+              // the table and the store.  The transposition and the stores behind it are a chain, so two slices go through them
+              // together.  Group of the 1x1 layers at batch 16 68.9 and 64.8 us, ResNet-18 68.8 and 65.2, ResNet-34 stack at batch 128
+              // 360 and 349; one slice a warp (64 channels of 56x56, 4 images) 5.21 and 5.24.  (The vote on a comparison is a column's word
+              // without any transposition, but 32 votes and selections take longer: those groups 79 and 75 us.)
+              unsigned long long t2;
+              asm("mov.b64 %0, {%1, %1};" : "=l"(t2) : "f"(minus_threshold));
               uint32_t part[4] = {0, 0, 0, 0};   // four chains of eight bits: one of 32 waits for itself
 #pragma unroll
               for (int e = 6; e >= 0; e -= 2) {
@@ -582,7 +618,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                 for (int c = 0; c < 4; ++c) {
                   unsigned long long x;
                   asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "r"(v[8 * c + e]), "r"(v[8 * c + e + 1]));
-                  asm("mul.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(a2));
                   asm("add.rn.f32x2 %0, %0, %1;" : "+l"(x) : "l"(t2));
                   uint32_t y0, y1;
                   asm("mov.b64 {%0, %1}, %2;" : "=r"(y0), "=r"(y1) : "l"(x));
@@ -590,24 +625,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                   part[c] = __funnelshift_l(y0, part[c], 1);
                 }
               }
-              uint32_t w = part[0] | (part[1] << 8) | (part[2] << 16) | (part[3] << 24);
-              w = co < K ? ~w : 0u;   // bits of channels that do not exist are 0
-              w = g_transpose32(w, lane);
-              const uint32_t px = T->offset[32 * s + lane], here = 1u << lane;
-              const uint32_t Kw = (uint32_t)(K + 31) >> 5;
-              if (kp_log >= 5) {
-                const size_t at = wide_mul(px + (uint32_t)g_warp, Kw) + (uint32_t)(co_warp >> 5);
-                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) {
-                  if (TAGGED && out_kind == 3) g_st_tagged(out32, at, w, tag);
-                  else out32[at] = w;
-                }
-              } else if (TAGGED && out_kind == 3) {
-                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) g_st_tagged(out32, px + (uint32_t)g_warp, w & 0xffffu, tag);
-                if (T->mask[(g_warp + 1) * G_MAX_CHUNKS + s] & here) g_st_tagged(out32, px + (uint32_t)g_warp + 1, w >> 16, tag);
-              } else {   // 16 rows per pixel: one word each for two pixels
-                if (T->mask[g_warp * G_MAX_CHUNKS + s] & here) out32[px + (uint32_t)g_warp] = w & 0xffffu;
-                if (T->mask[(g_warp + 1) * G_MAX_CHUNKS + s] & here) out32[px + (uint32_t)g_warp + 1] = w >> 16;
+              uint32_t w = (part[0] | (part[1] << 8) | (part[2] << 16) | (part[3] << 24)) ^ flip;
+              if (!held && s + s_step < n_slices) {
+                first = w;
+                held = true;
+                continue;
               }
+              g_transpose32(w, first, lane);
+              store_signs(s, w);
+              if (held) store_signs(s - s_step, first);
+              held = false;
             }
           }
         }
@@ -655,18 +682,18 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const uint32_t Qtot = L.Qtot;
       const int n_slices = (Np + 31) >> 5;
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
-      const uint32_t scale = out_kind >= 2 ? 1u : (uint32_t)K;
+      const uint32_t scale = out_kind >= 2 ? (uint32_t)(K + 31) >> 5 : (uint32_t)K;   // words of a pixel
 #pragma unroll 1
       for (int tile = L.first; tile < total; tile += G, ++seq) {
         if (!take_slot()) { ok = false; break; }
         GTile* const T = reinterpret_cast<GTile*>(epi_smem) + (seq & 3u);
         const int mg = (int)fdiv((uint32_t)tile, dCt), co = (tile - mg * n_ct) * G_ROWS;
-        float al[4], sh[4];
+        float al[4], th[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int c = co + 32 * i + lane;
           al[i] = c < K ? __ldg(L.alpha + c) : 0.f;
-          sh[i] = !WORDS && c < K ? __ldg(L.shift + c) : 0.f;
+          th[i] = !WORDS && c < K ? __ldg(L.threshold + c) : __int_as_float(0x7f800000);   // (no sum reaches infinity: bits of channels that do not exist are 0)
         }
         if (lane == 0) {
           *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
@@ -689,7 +716,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           T->alpha[32 * i + lane] = al[i];
-          if (!WORDS) T->shift[32 * i + lane] = __fadd_rn(sh[i], 0.f);   // -0 becomes +0: then no sum with it is -0
+          if (!WORDS) T->threshold[32 * i + lane] = th[i];
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tabfull + 8u * (seq & 3u));
@@ -1206,6 +1233,20 @@ MapEncoder g_map_encoder() {
   return f;
 }
 
+// The packed-sign bit of a channel is fl(fl(alpha*S) + shift) >= 0 for an integer sum S of -most..most: two roundings of a function that
+// never falls (alpha >= 0) or never rises (alpha < 0) along S, so the bit changes once, and comparing S with where it does is
+// the same decision.  Returns the least S whose bit is set (alpha < 0: clear), most + 1 where there is none.
+__device__ float g_sign_threshold(float alpha, float shift, int most) {
+  int lo = -most, hi = most + 1;
+  while (lo < hi) {
+    const int mid = lo + (hi - lo) / 2;   // (rounds towards lo: lo + hi may be negative)
+    const bool bit = __fadd_rn(__fmul_rn(alpha, (float)mid), __fadd_rn(shift, 0.f)) >= 0.f;   // (a shift of -0 is +0: no sum is -0)
+    if (bit == (alpha < 0.f)) lo = mid + 1;
+    else hi = mid;
+  }
+  return (float)lo;
+}
+
 // Operand of the weights: wt[channel tile][channel block][step][chunk][128][16 B]; a chunk is 16 bytes along the
 // input channels (8 fp16 or 32 e2m1 values), cb_chunks chunks per block.  With p = 2^kp_log, row r of a tile is channel
 // r % p of pixel r / p or, with single pixels, of copy r / p.  Channels that do not exist, and columns outside a pixel's window, are zeros, so whatever the
@@ -1213,9 +1254,11 @@ MapEncoder g_map_encoder() {
 template <int MODE>
 __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, uint8_t* __restrict__ wt, int C, int K,
                                         int Cw, long long total, int cb_chunks, int n_cb, int steps, int paired, int lg,
-                                        int kp_log, int win_step, int ksize, const GTaps taps) {
+                                        int kp_log, int win_step, int ksize, const GTaps taps, const float* __restrict__ alpha,
+                                        const float* __restrict__ shift, float* __restrict__ threshold) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= total) return;
+  if (threshold && i < K) threshold[i] = g_sign_threshold(alpha[i], shift[i], ksize * ksize * C);   // (there are more chunks than channels)
   const int row = (int)(i & (G_ROWS - 1));
   long long r = i / G_ROWS;
   const int chunks = paired ? 2 : cb_chunks;
@@ -1273,8 +1316,11 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   size_t smem = 0;
   if (!g_ring(plan.data(), count, mode, &ring, &smem)) return cudaErrorInvalidConfiguration;
   size_t w_off[SNN_GROUP_MAX], w_total = 0;
+  size_t threshold_off[SNN_GROUP_MAX], threshold_words = 0;
   long long tiles = 0, most = 0;
   for (int i = 0; i < count; ++i) {
+    threshold_off[i] = threshold_words;
+    if (kind != TCG_WORDS) threshold_words += (size_t)gs[i].K;
     w_off[i] = w_total;
     w_total += (plan[i].w_bytes + 255) & ~(size_t)255;
     tiles += plan[i].L.total_tiles;
@@ -1346,12 +1392,13 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->chain = chain;
   Gd->kind = kind;
   // One allocation and one copy for everything the group owns: [weight operands][descriptions][ranks][dependencies]
-  // [counters][count of launches][packed signs between the members]; the three from the descriptions on come from the host.
+  // [counters][count of launches][thresholds of the signs][packed signs between the members]; the three from the descriptions on come from the host.
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
   const size_t rank_at = up(sizeof(GLayer) * (size_t)count), deps_at = rank_at + up(ranks.size() * sizeof(uint32_t));
   const size_t blob_bytes = deps_at + up(deps.size() * sizeof(uint2)), blob_at = up(w_total), done_at = blob_at + blob_bytes;
   const size_t launches_at = done_at + up(done_words * sizeof(uint32_t));
-  const size_t chain_at = launches_at + (tagged ? up(sizeof(unsigned long long)) : 0);
+  const size_t threshold_at = launches_at + (tagged ? up(sizeof(unsigned long long)) : 0);
+  const size_t chain_at = threshold_at + up(threshold_words * sizeof(float));
   cudaError_t e = cudaMalloc(&Gd->mem, chain_at + chain_bytes);
   if (e == cudaSuccess) {
     Gd->layers_dev = reinterpret_cast<GLayer*>(Gd->mem + blob_at);
@@ -1362,7 +1409,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->done_words = done_words;
   Gd->tagged = tagged;
   // no launch has written a word yet: tags start at 1
-  if (tagged && e == cudaSuccess) e = cudaMemsetAsync(Gd->mem + launches_at, 0, chain_at + chain_bytes - launches_at, s);
+  if (tagged && e == cudaSuccess) e = cudaMemsetAsync(Gd->mem + launches_at, 0, chain_at + chain_bytes - launches_at, s);   // (thresholds are written later)
   for (int i = 0; i < count; ++i) Gd->chain_off[i] = chain_off[i];
   const uint2* const deps_dev = reinterpret_cast<const uint2*>(Gd->mem + blob_at + deps_at);
   std::vector<uint8_t> blob(blob_bytes);
@@ -1371,7 +1418,8 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     L.wt = Gd->mem + w_off[i];
     Gd->map[i] = {L.tma != 0, L.C, L.W, L.H, L.N, L.rs, L.Wg};
     L.alpha = Ls[i]->alpha;
-    L.shift = Ls[i]->shift;
+    float* const thresholds = kind == TCG_WORDS ? nullptr : reinterpret_cast<float*>(Gd->mem + threshold_at) + threshold_off[i];
+    L.threshold = thresholds;
     if (chain && !tagged) {
       L.done = Gd->done + done_off[i];
       if (i > 0) {
@@ -1386,11 +1434,11 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
     if (mode == M_F16)
       g_expand_weights_kernel<M_F16><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
                                                             total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
-                                                            win_step, ks, plan[i].taps);
+                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds);
     else
       g_expand_weights_kernel<M_FP4><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
                                                             total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
-                                                            win_step, ks, plan[i].taps);
+                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds);
     e = cudaGetLastError();
     if (e == cudaSuccess) *launched += 1;
   }

@@ -237,3 +237,29 @@ def test_stored_form_under_capture(snn, oracle_mod):
     graph.replay()
     torch.cuda.synchronize()
     assert (out.cpu().numpy() == refs[1]).all()
+
+
+@pytest.mark.parametrize("c_in,c_out,h,w,n", [(40, 48, 5, 6, 1), (64, 70, 9, 29, 4), (33, 16, 20, 21, 3), (128, 256, 14, 14, 12)])
+def test_signs_where_scaled_sums_round_or_cancel(snn, oracle_mod, c_in, c_out, h, w, n):
+    """The kernel compares a sum with the integer at which fl(fl(alpha*S) + shift) changes its sign: scales of zero, subnormal and
+    overflowing products, shifts that cancel a product exactly or miss it by a rounding, and shifts beyond every sum; tiles
+    of one slice of 32 positions, of several, and of an odd number."""
+    shape = wl.LayerShape(c_in, c_out, h, w, 1, 1)
+    p = wl.draw_layer_params(shape, 6, 500 + c_in)
+    packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 501 + w))
+    rng = np.random.default_rng(c_out)
+    f32 = np.float32
+    scales = np.array([1.0, -1.0, 0.0, -0.0, 1e-45, -1e-45, 1.2e-38, 3e38, -3e38, 0.1, -0.1, 0.3333333, 1.0000001], f32)
+    alpha = scales[rng.integers(0, len(scales), c_out)]
+    near = rng.integers(-30, 31, c_out).astype(f32)
+    with np.errstate(over="ignore"):
+        shift = np.clip(-(alpha * near), f32(-3.3e38), f32(3.3e38))
+        kind = rng.integers(0, 6, c_out)
+        shift = np.where(kind == 1, np.nextafter(shift, f32(-1)), np.where(kind == 2, np.nextafter(shift, f32(1)), shift))
+        shift = np.where(kind == 3, f32(-0.0), np.where(kind == 4, f32(1e30), np.where(kind == 5, f32(-1e30), shift))).astype(f32)
+        s_ref, _ = oracle_mod.conv_bin(p.codebook, 6, p.idx_packed, p.alpha, c_in, c_out, 1, 1, packed)
+        want = _signs((s_ref.astype(f32) * alpha) + shift)
+    layer = snn.SnnConv(c_in, c_out, 6, p.codebook, p.idx_packed, alpha, 1, 1, snn.ACT_BIN, shift=shift)
+    got = layer.forward(torch.from_numpy(packed.view(np.int32)).cuda(), out_type=snn.OUT_BITS).cpu().numpy().view(np.uint32)
+    assert (got == want).all()
+    layer.destroy()
