@@ -56,7 +56,8 @@
 //                    threshold -> 32 x 32 bit transposition in the warp -> packed sign words
 //      warps 10-19   expanders (but 13 and 17): packed bits -> e2m1 nibbles (or fp16 copied)
 //                    into the activation ring
-//      warp 13       writes the epilogue's tables (where the columns of a tile go) ahead of it
+//      warp 13       writes the epilogue's tables (where the columns of a tile go) ahead of it, and in a chain on counters says
+//                    which tiles have been written
 //      warp 17       in a chain on counters: waits for the tiles that the CTA's next tile reads
 // The kernel is compiled per operand mode and per output kind (words, packed signs, chains on counters, chains of words
 // with tags), so that no variant carries another one's code in its loops; the plan (tile shapes, accumulator buffers) is made
@@ -516,7 +517,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
       const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, lg = h1.z;
       if (l < 0) break;   // no more tiles
-      const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : h1.w;
+      const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : h1.w & 3;
       uint32_t* const out32 = reinterpret_cast<uint32_t*>(p.out[l]);  // int32 and fp32 outputs share the layout
       // this lane's row of the weight operand: channel c of pixel g of a position's group, or of a copy of the channels
       const int c_lane = row & ((1 << kp_log) - 1), c_warp = (rq * 32) & ((1 << kp_log) - 1);   // (_warp: of lane 0)
@@ -638,14 +639,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             }
           }
         }
-        if (CHAIN) {
-          // chain: this warp's part of the tile is written; the successor may read it
-          if (active && s_first < n_slices) {
-            __syncwarp();
-            if (lane == 0) {
-              __threadfence();   // (cumulative: it covers what the other lanes wrote before the barrier)
-              asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(lay[l].done + h0.y) : "memory");
-            }
+        if (CHAIN && (h1.w & 4) && active && s_first < n_slices) {
+          // one of the CTA's last tiles in this member of a chain: this warp's part is written, the successor may read it
+          __syncwarp();
+          if (lane == 0) {
+            __threadfence();   // (cumulative: it covers what the other lanes wrote before the barrier)
+            asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(lay[l].done + h0.y) : "memory");
           }
         }
       }
@@ -663,7 +662,34 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     // until those have drained).
     bool ok = true;
     uint32_t seq = 0;
+    // Chains on counters: the oldest tile whose counter has not been advanced.  The fence between a tile's signs and its counter waits
+    // for the stores to arrive, 1200 cycles: done by every epilogue warp for its part it was a fifth of their time in the shallow layers
+    // of large batches.  Here it is done once a tile, beside them (their arrivals and the fence are cumulative: it covers what they
+    // wrote).  That is some 300 cycles later, so the last two of a CTA's tiles in a member, and members with fewer than three tiles a
+    // CTA, whose successors wait for just those, are left to the epilogue warps.  ResNet-34 stack at batch 128 344 and 330 us, ResNet-18 at 96
+    // 156.4 and 151.8; without the line at three tiles ResNet-34 at 64 250 and 255, with it at four ResNet-34 at 128 338.
+    uint32_t unsaid = 0;
+    auto say_written = [&]() {
+      const GTile* const T = reinterpret_cast<const GTile*>(epi_smem) + (unsaid & 3u);
+      if (T->l + 1 < p.n_layers && !(T->out_kind & 4)) {
+        // the epilogue warps that had something to write (see there): lane w stands for warp 2 + w
+        const int first_row = ((lane + 2) & 3) * 32, first_slice = (lane >> 2) + (T->lg ? 0 : 2 * (first_row >> T->kp_log));
+        const uint32_t wrote = __ballot_sync(0xffffffffu, lane < G_EW && T->co + (first_row & ((1 << T->kp_log) - 1)) < T->K && first_slice < T->n_slices);
+        if (lane == 0) {
+          __threadfence();
+          asm volatile("red.relaxed.gpu.global.add.u32 [%0], %1;" ::"l"(lay[T->l].done + T->mg), "r"((uint32_t)__popc(wrote)) : "memory");
+        }
+        __syncwarp();
+      }
+      ++unsaid;
+    };
     auto take_slot = [&]() -> bool {
+      if (CHAIN) {   // what has been written meanwhile is said first
+        while (unsaid < seq && seq - unsaid < G_TILES &&
+               __shfl_sync(0xffffffffu, lane == 0 ? (int)mbar_test(bar_tabempty + 8u * (unsaid & 3u), (unsaid >> 2) & 1u) : 0, 0))
+          say_written();
+        if (seq - unsaid < G_TILES) return true;
+      }
       if (seq < G_TILES) return true;
       int okw = 1;
       if (lane == 0) okw = (!*abort_flag && mbar_wait_backoff(bar_tabempty + 8u * (seq & 3u), ((seq >> 2) & 1u) ^ 1u, 100)) ? 1 : 0;
@@ -672,6 +698,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         *abort_flag = 1;
         raise_status(p.status, 7);
       }
+      if (CHAIN && okw) say_written();
       return okw != 0;
     };
 #pragma unroll 1
@@ -683,6 +710,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const int n_slices = (Np + 31) >> 5;
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
       const uint32_t scale = out_kind >= 2 ? (uint32_t)(K + 31) >> 5 : (uint32_t)K;   // words of a pixel
+      const bool few = total < 3 * G;
 #pragma unroll 1
       for (int tile = L.first; tile < total; tile += G, ++seq) {
         if (!take_slot()) { ok = false; break; }
@@ -697,7 +725,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         }
         if (lane == 0) {
           *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
-          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, lg, out_kind);
+          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, lg, out_kind | (CHAIN && (few || tile + 2 * G >= total) ? 4 : 0));
         }
 #pragma unroll 1
         for (int s = 0; s < n_slices; ++s) {
@@ -728,6 +756,12 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         mbar_arrive(bar_tabfull + 8u * (seq & 3u));
       }
       __syncwarp();
+      if (CHAIN) {   // the last tiles
+        for (const uint32_t tiles = seq; ok && unsaid < tiles;) {
+          seq = unsaid + G_TILES;
+          ok = take_slot();
+        }
+      }
     }
   } else if (CHAIN && warp == 17) {
     // ------------------------------------------------ dependency warp (chains)
