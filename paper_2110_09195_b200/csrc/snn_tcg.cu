@@ -295,6 +295,21 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   const int NS = p.NS, NA = p.NA;
   const int G = (int)gridDim.x;
 
+  // Whole-warp wait of a role whose warps wait one lane each: a phase that is over already costs one look and a vote.  False: the wait ran
+  // out, or the CTA is giving up.
+  auto wait_phase = [&](uint32_t bar, uint32_t parity, uint32_t ns, int code) -> bool {
+    if (__any_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    int okw = 1;
+    if (lane == 0) {
+      okw = (!*abort_flag && mbar_wait_backoff(bar, parity, ns)) ? 1 : 0;
+      if (!okw && !*abort_flag) {
+        *abort_flag = 1;
+        raise_status(p.status, code);
+      }
+    }
+    return __shfl_sync(0xffffffffu, okw, 0) != 0;
+  };
+
   // Set-up.  Warp 2 allocates tensor memory while the others write the barriers and the problems' descriptions; only the MMA
   // issuer and the epilogue warps wait for it (barrier 1).  The producer, the expanders and the table warp start as
   // soon as the descriptions are there (barrier 2): 39 single layers 1.4 % faster, as a graph, than with both behind two barriers
@@ -503,17 +518,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     for (;;) {
       const GTile* const T = reinterpret_cast<const GTile*>(epi_smem) + (seq & 3u);
       const uint32_t tile_phase = (seq >> 2) & 1u;   // (acc_full and the tables are indexed and flip alike)
-      int okw = 1;
-      if (lane == 0) okw = (!*abort_flag && mbar_wait_backoff(bar_tabfull + 8u * (seq & 3u), tile_phase, 100)) ? 1 : 0;
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (!okw) {
-        if (lane == 0 && !*abort_flag) {
-          *abort_flag = 1;
-          raise_status(p.status, 6);
-        }
-        break;
-      }
-      __syncwarp();
+      if (!wait_phase(bar_tabfull + 8u * (seq & 3u), tile_phase, 100, 6)) break;
       const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
       const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, lg = h1.z;
       if (l < 0) break;   // no more tiles
@@ -529,15 +534,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const float al = T->alpha[c_lane], minus_threshold = WORDS ? 0.f : -T->threshold[c_lane];
       const uint32_t flip = al < 0.f ? 0u : 0xffffffffu;   // (the bit is set below the threshold, or - where the sign bit of the difference is clear - from there on)
       {
-        if (lane == 0) okw = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_accfull + 8u * (seq & 3u), tile_phase, 100))) ? 1 : 0;
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (!okw) {
-          if (lane == 0 && !*abort_flag) {
-            *abort_flag = 1;
-            raise_status(p.status, 4);
-          }
-          break;
-        }
+        if (!TR_WAIT(tr_w0, wait_phase(bar_accfull + 8u * (seq & 3u), tile_phase, 100, 4))) break;
         tc_fence_after();
         const uint32_t d0 = tmem_base + (uint32_t)acc_slot * p.acc_cols + ((uint32_t)(rq * 32) << 16);
         // this warp has read its part of the accumulator buffer: hand it back to the MMA issuer
@@ -685,21 +682,14 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     };
     auto take_slot = [&]() -> bool {
       if (CHAIN) {   // what has been written meanwhile is said first
-        while (unsaid < seq && seq - unsaid < G_TILES &&
-               __shfl_sync(0xffffffffu, lane == 0 ? (int)mbar_test(bar_tabempty + 8u * (unsaid & 3u), (unsaid >> 2) & 1u) : 0, 0))
+        while (unsaid < seq && seq - unsaid < G_TILES && __any_sync(0xffffffffu, mbar_test(bar_tabempty + 8u * (unsaid & 3u), (unsaid >> 2) & 1u)))
           say_written();
         if (seq - unsaid < G_TILES) return true;
       }
       if (seq < G_TILES) return true;
-      int okw = 1;
-      if (lane == 0) okw = (!*abort_flag && mbar_wait_backoff(bar_tabempty + 8u * (seq & 3u), ((seq >> 2) & 1u) ^ 1u, 100)) ? 1 : 0;
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (!okw && lane == 0 && !*abort_flag) {
-        *abort_flag = 1;
-        raise_status(p.status, 7);
-      }
-      if (CHAIN && okw) say_written();
-      return okw != 0;
+      if (!wait_phase(bar_tabempty + 8u * (seq & 3u), ((seq >> 2) & 1u) ^ 1u, 100, 7)) return false;
+      if (CHAIN) say_written();
+      return true;
     };
 #pragma unroll 1
     for (int l = 0; l < p.n_layers && ok; ++l) {
@@ -805,17 +795,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     bool stop = false;
     long long tr_w0 = 0, tr_t0 = clock64();
     (void)tr_w0; (void)tr_t0; (void)a_done;
-    // one lane per warp waits until the MMAs have read what slot a_slot held
-    auto wait_slot = [&]() -> bool {
-      int okf = 1;
-      if (lane == 0) okf = (!*abort_flag && TR_WAIT(tr_w0, mbar_wait_backoff(bar_aempty + 8 * a_slot, a_phase, 64))) ? 1 : 0;
-      okf = __shfl_sync(0xffffffffu, okf, 0);
-      if (!okf && lane == 0 && !*abort_flag) {
-        *abort_flag = 1;
-        raise_status(p.status, 1);
-      }
-      return okf != 0;
-    };
+    // until the MMAs have read what slot a_slot held
+    auto wait_slot = [&]() -> bool { return TR_WAIT(tr_w0, wait_phase(bar_aempty + 8 * a_slot, a_phase, 64, 1)); };
     // this warp's part of a unit is written: make it visible to the tensor core and say so
     auto unit_done = [&](int slot) {
       fence_proxy_async();  // generic-proxy writes -> visible to the tensor core's reads
