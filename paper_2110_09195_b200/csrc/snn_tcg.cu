@@ -1213,6 +1213,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
 // ------------------------------------------------------------------ host side
 struct GroupDev {
   int count = 0, act_type = 0, mode = M_FP4;
+  int order[SNN_GROUP_MAX] = {};  // which of the caller's problems each one is
   int kind = TCG_WORDS;           // what the tiles were planned for (word outputs, packed signs, chain)
   int chain = 0;                  // 1: member i + 1 reads the packed signs member i writes (one launch, on counters or with tags)
   uint8_t* mem = nullptr;         // all device memory of the group; the pointers below lie in it
@@ -1308,10 +1309,14 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
 
 }  // namespace
 
-cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int act_type, int kind, cudaStream_t s,
+cudaError_t tcg_create(const LayerDev* const* layers, const Geom* geoms, int count, int act_type, int kind, cudaStream_t s,
                        GroupDev** out, int* launched) {
   *out = nullptr;
   if (count < 1 || count > SNN_GROUP_MAX) return cudaErrorInvalidConfiguration;
+  const LayerDev* Ls[SNN_GROUP_MAX];   // in the order in which the CTAs walk through them
+  Geom gs[SNN_GROUP_MAX];
+  int order[SNN_GROUP_MAX];
+  for (int i = 0; i < count; ++i) { Ls[i] = layers[i]; gs[i] = geoms[i]; order[i] = i; }
   if (kind != TCG_WORDS && act_type != SNN_ACT_BIN) return cudaErrorInvalidConfiguration;
   const int chain = kind == TCG_CHAIN;
   const int mode = g_mode_for(act_type);
@@ -1326,6 +1331,11 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   for (int i = 0; i < count && chain; ++i)
     if (!g_plan_by_end(gs[i], mode, kind, sms, &plan[i])) return cudaErrorInvalidConfiguration;
   if (!chain && !g_plan_independent(gs, count, mode, kind, tma, sms, plan.data())) return cudaErrorInvalidConfiguration;
+  if (!chain) {
+    g_order(plan.data(), count, order);
+    const std::vector<GPlan> given(plan);
+    for (int i = 0; i < count; ++i) { plan[i] = given[order[i]]; Ls[i] = layers[order[i]]; gs[i] = geoms[order[i]]; }
+  }
   for (int i = 0; i < count; ++i) g_finish_plan(gs[i], &plan[i]);
   GParams ring{};
   size_t smem = 0;
@@ -1405,6 +1415,7 @@ cudaError_t tcg_create(const LayerDev* const* Ls, const Geom* gs, int count, int
   Gd->mode = mode;
   Gd->grid = grid;
   Gd->chain = chain;
+  std::copy(order, order + count, Gd->order);
   Gd->kind = kind;
   // One allocation and one copy for everything the group owns: [weight operands][descriptions][ranks][dependencies]
   // [counters][count of launches][thresholds of the signs][packed signs between the members]; the three from the descriptions on come from the host.
@@ -1648,8 +1659,8 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
     attr[0].val.cooperative = 1;
   } else {
     for (int i = 0; i < G->count; ++i) {
-      p.act[i] = act[i];
-      p.out[i] = out[i];
+      p.act[i] = act[G->order[i]];
+      p.out[i] = out[G->order[i]];
       p.out_type[i] = (uint8_t)out_type;
     }
     // Launched as a programmatic dependent of its predecessor in the stream: set-up overlaps that
@@ -1684,7 +1695,7 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
       const cuuint64_t dim[4] = {(cuuint64_t)m.C, (cuuint64_t)m.W, (cuuint64_t)m.H, (cuuint64_t)m.N};
       const cuuint64_t pitch[3] = {(cuuint64_t)m.C * 2, (cuuint64_t)m.W * m.C * 2, (cuuint64_t)m.H * m.W * m.C * 2};
       const cuuint32_t box[4] = {64, (cuuint32_t)((m.box - 1) * m.stride + 1), 1, 1}, step[4] = {1, (cuuint32_t)m.stride, 1, 1};
-      if (g_map_encoder()(&maps.m[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(act[i]), dim, pitch, box, step,
+      if (g_map_encoder()(&maps.m[i], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(act[G->order[i]]), dim, pitch, box, step,
                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;

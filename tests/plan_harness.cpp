@@ -112,4 +112,16 @@ const char* plan_make(const int* gs, int count, int f16, int kind, int sms, int*
   return wrong(plan.data(), count, mode, ring, smem);
 }
 
+
+// the order in which a group's problems are walked through, and the MMA cycles of a tile of each problem given
+int plan_order(const int* gs, int count, int f16, int sms, int* order, double* cycles) {
+  std::vector<Geom> g(count);
+  std::vector<GPlan> plan(count);
+  for (int i = 0; i < count; ++i) g[i] = geom(gs + 8 * i);
+  if (!g_plan_independent(g.data(), count, f16 ? M_F16 : M_FP4, TCG_WORDS, f16 != 0, sms, plan.data())) return 0;
+  g_order(plan.data(), count, order);
+  for (int i = 0; i < count; ++i) cycles[i] = plan[i].mma;
+  return 1;
+}
+
 }  // extern "C"

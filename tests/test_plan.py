@@ -189,3 +189,19 @@ def test_which_chains_of_the_gpu_tests_carry_tags(lib):
     assert _words(pair, 128) == 1 << 17 and not lib.plan_tagged(_words(pair, 129))
     for net, n, tags in (("resnet18", 2, True), ("resnet18", 64, False), ("resnet20", 4, True)):
         assert bool(lib.plan_tagged(_words(wl.get_workload(net).layers, n))) == tags
+
+
+@pytest.mark.parametrize("f16", [False, True])
+def test_heavy_problems_of_a_group_come_first(lib, f16):
+    """The order is a permutation by the tiles' MMAs, and keeps the order given among problems whose tiles are small or alike."""
+    rng = random.Random(11)
+    for _ in range(60):
+        shapes = [s for s in (draw(rng) for _ in range(rng.randint(1, 32))) if takes(lib, s, f16)]
+        if not shapes:
+            continue
+        shapes += shapes[:32 - len(shapes)]
+        order, cycles = (ctypes.c_int * 32)(), (ctypes.c_double * 32)()
+        assert lib.plan_order(_array(shapes), len(shapes), int(f16), SMS, order, cycles)
+        order = order[:len(shapes)]
+        assert sorted(order) == list(range(len(shapes)))
+        assert order == sorted(order, key=lambda i: (-max(cycles[i], 1200.0), i))
