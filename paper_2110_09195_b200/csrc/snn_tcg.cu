@@ -580,9 +580,11 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
               // Scaled (or converted) first, stored by one loop for both: a store loop for each kind doubles the code, and the
               // roles share the instruction caches (with two loops the ResNet-18 group took 7 % longer, the 1x1 layers 4 %).
+              // (Pairs are multiplied together, each half rounded as by itself: ResNet-20 group at batch 128 36.6 and 35.9 us, ResNet-18 94.0 and 92.6.)
               if (out_kind == 0) {
 #pragma unroll
-                for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__fmul_rn(__uint_as_float(v[e]), al));
+                for (int e = 0; e < 32; e += 2)
+                  asm("{\n\t.reg .b64 x, a;\n\tmov.b64 x, {%0, %1};\n\tmov.b64 a, {%2, %2};\n\tmul.rn.f32x2 x, x, a;\n\tmov.b64 {%0, %1}, x;\n\t}" : "+r"(v[e]), "+r"(v[e + 1]) : "f"(al));
               } else {
 #pragma unroll
                 for (int e = 0; e < 32; ++e) v[e] = (uint32_t)__float2int_rn(__uint_as_float(v[e]));   // integer sums: exact
