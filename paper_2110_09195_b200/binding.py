@@ -116,7 +116,7 @@ class _PythonChecks:
     def layer_forward(*_):
         return -1
 
-    group_forward = stack_forward = layer_forward
+    group_forward = stack_forward = static_forward = layer_forward
 
 
 def _load_fast():
@@ -131,6 +131,7 @@ def _load_fast():
                 raise ImportError(f"_snn_fast was built for torch {module.TORCH_VERSION}, not {torch.__version__}")
             module.bind(*(ctypes.cast(f, ctypes.c_void_p).value
                           for f in (lib.snn_conv_forward, lib.snn_conv_group_forward, lib.snn_conv_stack_forward)))
+            module.bind_static(ctypes.cast(lib.snn_conv_forward_static, ctypes.c_void_p).value, np.ndarray)
         except ImportError as e:
             warnings.warn(f"the forward calls are checked in Python, which takes longer: {e} "
                           "(python -m paper_2110_09195_b200.build builds _snn_fast)", RuntimeWarning, stacklevel=3)
@@ -168,6 +169,11 @@ def forward_static(c_in, c_out, tau, codebook, idx_packed, alpha, act, out, stri
     `act` and `out` are CUDA tensors the caller already owns.  Binary activations
     only, at most 512 channels in and out.  Calls share one fixed scratch array
     per GPU, so do not let two of them overlap on the device."""
+    if stream is None:
+        status = _load_fast().static_forward(c_in, c_out, tau, codebook, idx_packed, alpha, act, out, stride, pad, out_type, device)
+        if status >= 0:
+            _check(status)
+            return out
     import torch
     cb = np.ascontiguousarray(codebook, dtype=np.uint16)
     ip = np.ascontiguousarray(idx_packed, dtype=np.uint8)

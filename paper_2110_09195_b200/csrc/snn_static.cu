@@ -6,6 +6,7 @@
 // part of the library image.  Each call copies the layer description into that
 // array, writes the tensor-core kernel's weight operand there and runs that kernel on it; a shape the tensor-core
 // kernel does not take is decoded to bit-planes and run by the XOR + popcount kernel.
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -68,6 +69,32 @@ cudaError_t scratch_address(int device, cudaStream_t s, unsigned char** out, int
   *status = g_status_dev[device];
   *out = g_scratch_dev[device];
   return cudaSuccess;
+}
+
+// Plans of recent shapes (host memory): planning tries a dozen tile widths, half a microsecond of a call.
+struct Planned {
+  int N = 0, H, W, C, K, stride, pad;
+  bool taken;
+  TcgStatic plan;
+};
+constexpr int kPlans = 16;
+std::mutex g_plans_mu;
+Planned g_plans[kPlans];
+int g_next_plan = 0;
+
+bool planned(const Geom& g, TcgStatic* out) {
+  std::lock_guard<std::mutex> lk(g_plans_mu);
+  for (const Planned& p : g_plans)
+    if (p.N == g.N && p.H == g.H && p.W == g.W && p.C == g.C && p.K == g.K && p.stride == g.stride && p.pad == g.pad) {
+      if (p.taken) memcpy(out, &p.plan, sizeof(*out));
+      return p.taken;
+    }
+  Planned& p = g_plans[g_next_plan];
+  g_next_plan = (g_next_plan + 1) % kPlans;
+  p.taken = tcg_static_plan(g, &p.plan);
+  p.N = g.N; p.H = g.H; p.W = g.W; p.C = g.C; p.K = g.K; p.stride = g.stride; p.pad = g.pad;
+  if (p.taken) memcpy(out, &p.plan, sizeof(*out));
+  return p.taken;
 }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -135,10 +162,14 @@ extern "C" SNN_API snn_status_t snn_conv_forward_static(const snn_conv_desc_t* d
     return api_fail(SNN_ERR_UNSUPPORTED, "layer needs %zu bytes of scratch, the fixed array holds %zu", off,
                     kStaticScratchBytes);
 
-  int ndev = 0;
-  if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) {
-    cudaGetLastError();
-    return api_fail(SNN_ERR_CUDA, "no CUDA device available (this library has no CPU path)");
+  static std::atomic<int> devices{0};   // (asked for until there is one)
+  int ndev = devices.load(std::memory_order_relaxed);
+  if (ndev < 1) {
+    if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) {
+      cudaGetLastError();
+      return api_fail(SNN_ERR_CUDA, "no CUDA device available (this library has no CPU path)");
+    }
+    devices.store(ndev, std::memory_order_relaxed);
   }
   if (d->device < 0 || d->device >= ndev || d->device >= kMaxDevices)
     return api_fail(SNN_ERR_INVALID_ARG, "device %d of %d", d->device, ndev);
@@ -158,7 +189,7 @@ extern "C" SNN_API snn_status_t snn_conv_forward_static(const snn_conv_desc_t* d
   const size_t t_alpha = 1024, t_stream = t_alpha + align256((size_t)g.K * 4), t_mem = align256(t_stream + stream_bytes);
   TcgStatic plan;
   g.ksize = 3;
-  if (e == cudaSuccess && status_dev && tcg_static_plan(g, &plan) && t_mem + plan.bytes <= kStaticScratchBytes) {
+  if (e == cudaSuccess && status_dev && planned(g, &plan) && t_mem + plan.bytes <= kStaticScratchBytes) {
     volatile int* const status = &g_status.word[d->device * 16];
     if (*status) {
       const int code = *status;

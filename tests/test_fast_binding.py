@@ -201,3 +201,48 @@ def test_the_current_stream_is_used():
     graph.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, want)
+
+
+def _static_arguments(c_in=40, c_out=24, n=2, h=9, w=7, tau=4, seed=5, device="cuda"):
+    shape = wl.LayerShape(c_in, c_out, h, w, 1, 1)
+    p = wl.draw_layer_params(shape, tau, seed)
+    x = torch.from_numpy(wl.pack_activation_bits(wl.draw_activation_bits(shape, n, seed)).view(np.int32)).to(device)
+    return [c_in, c_out, tau, np.asarray(p.codebook, np.uint16), np.asarray(p.idx_packed, np.uint8), np.asarray(p.alpha, np.float32), x,
+            torch.empty((n, h, w, c_out), dtype=torch.float32, device=device), 1, 1, snn.OUT_F32, 0]
+
+
+def _with(args, i, v):
+    return [*args[:i], v, *args[i + 1:]]
+
+
+# arguments the library would read wrongly, each in the place of a good one
+_NOT_PLAIN = [(0, 40.0), (0, 513), (1, 25), (2, 5), (2, True), (3, [1] * 16), (3, np.zeros(16, np.int16)), (3, np.zeros(32, np.uint16)[::2]),
+              (3, np.zeros(15, np.uint16)), (4, bytes(480)), (4, np.zeros(479, np.uint8)), (5, np.zeros(24)), (5, np.zeros(24, ">f4")), (5, torch.zeros(24)),
+              (6, None), (7, None), (8, 3), (9, 2), (10, 2), (11, -1), (11, 1)]
+
+
+def test_the_arrays_of_the_no_allocation_call_are_numpys_own():
+    fast = binding._load_fast()
+    args = _static_arguments(device="cpu")
+    assert fast.static_forward(*args) == -1 and fast.static_forward(*args[:-1]) == -1
+    for i, v in _NOT_PLAIN:
+        assert fast.static_forward(*_with(args, i, v)) == -1
+
+
+@pytest.mark.gpu
+def test_the_no_allocation_call_both_ways():
+    args = _static_arguments()
+    fast = binding._load_fast()
+    first = snn.forward_static(*args).clone()
+    lists = _with(_with(_with(args, 3, args[3].tolist()), 5, args[5].astype(np.float64)), 7, torch.zeros_like(first))   # converted in Python
+    assert fast.static_forward(*lists) == -1 and torch.equal(snn.forward_static(*lists), first)
+    layer = snn.SnnConv(*args[:6])
+    assert torch.equal(layer.forward(args[6]), first)
+    for i, v in _NOT_PLAIN:
+        assert fast.static_forward(*_with(args, i, v)) == -1
+    for i, v in ((1, 25), (2, 5), (3, args[3][:-1]), (4, args[4][:-1]), (7, first[:1]), (8, 3)):
+        with pytest.raises(snn.SnnError):
+            snn.forward_static(*_with(args, i, v))
+    with pytest.raises(snn.SnnError):   # refused by the library: said as ever
+        snn.forward_static(*_with(args, 5, np.full(24, np.nan, np.float32)))
+    layer.destroy()
