@@ -69,10 +69,22 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
                         int* status_dev, int* launched);
 void tcg_destroy(GroupDev* G);
 // One launch from the stored form of a layer (index stream, codebook and scales in device memory), in memory of the
-// caller's: tcg_static_plan says how many bytes that takes (binary activations, fp32 / int32 outputs; false where the
+// caller's (with TcgStatic::stored it goes there with the launch, the scales to alpha_dev): tcg_static_plan says how many bytes that takes (binary activations, fp32 / int32 outputs; false where the
 // tensor-core kernel cannot run the layer), tcg_static_forward writes the weight operand there and runs the layer.
+// A layer's stored form in host memory, for a launch that takes it along as a kernel parameter (at most kTcgStoredMax bytes of
+// tcg_stored_bytes); codebook null: it is in device memory, where the arguments of tcg_static_forward point.
+struct TcgStored {
+  const uint16_t* codebook = nullptr;
+  const float* alpha = nullptr;
+  const uint8_t* stream = nullptr;
+};
+constexpr size_t kTcgStoredMax = 32000;
+inline size_t tcg_stored_bytes(const Geom& g) {
+  return 1024 + (size_t)g.K * 4 + ((size_t)g.K * g.C * g.tau + 7) / 8;   // [codebook][scales][index stream]
+}
 struct TcgStatic {
   size_t bytes;
+  TcgStored stored;
   alignas(16) unsigned char opaque[3072];
 };
 bool tcg_static_plan(const Geom& g, TcgStatic* out);

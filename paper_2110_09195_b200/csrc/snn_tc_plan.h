@@ -123,7 +123,7 @@ struct GParams {
   int NA, NS;
   uint32_t a_slot_bytes, b_slot_bytes;
   uint32_t off_b, off_epi, off_pix, off_lay, off_tail;
-  int after_weights;      // the launch before this one in the stream writes the weights: wait for it before they are read
+  int after_weights;      // the launch before this one in the stream writes the weights (2: and the scales): wait for it before they are read
   GLayer one;             // n_layers == 1: the problem itself (layers and ranks are not read: its tiles go to the CTAs in order)
 };
 

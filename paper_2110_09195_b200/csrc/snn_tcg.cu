@@ -659,6 +659,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     // of them exist, the scales and thresholds.  Done by the epilogue warps themselves, each for itself, this took a
     // fifth of their time (the geometry is a chain of divisions, and a global load behind a warp's own stores waits
     // until those have drained).
+    if (p.after_weights > 1) grid_dep_wait();
     bool ok = true;
     uint32_t seq = 0;
     // Chains on counters: the oldest tile whose counter has not been advanced.  The fence between a tile's signs and its counter waits
@@ -1510,14 +1511,31 @@ struct GStepOf {
 // row's word are consecutive bits of the stream, nine votes of the codes' bits are its nine taps, and lane t writes tap t.
 // Bound by latency: two loads, a look-up, nine votes and the launch around them.
 // With one thread per row and word, 64 byte loads and 33 KB of straight-line code a thread, 14 calls took 4 % longer waited for
-// (193->168 channels of 9x26: 36.8 us, now 33.8).  8 images of a 128-channel 28x28 layer, copies and host work included: 16.6 us a
-// call back to back, all of it the host's (18.6 on another machine's), 30.2 waited for; by four decode kernels and the popcount kernel 46.
+// (193->168 channels of 9x26: 36.8 us, now 33.8).  The stored form comes as a parameter where it fits one, read through its generic
+// address: 8 images of a 128-channel 28x28 layer 9.8 us a call back to back, copied to the device before the launch 14.4, by four
+// decode kernels and the popcount kernel 46.
 constexpr int G_SW_ROWS = 8, G_SW_WARPS = 4;
-__global__ void __launch_bounds__(32 * G_SW_WARPS) g_static_weights_kernel(const uint8_t* __restrict__ stream, int n_bytes,
-                                                                           const uint16_t* __restrict__ codebook, uint8_t* __restrict__ wt,
+template <int BYTES>
+struct alignas(16) GStored {
+  uint8_t b[BYTES];   // [codebook][scales][index stream]
+};
+template <int BYTES>   // of the stored form that come as a parameter; 16: it is in memory
+__global__ void __launch_bounds__(32 * G_SW_WARPS) g_static_weights_kernel(const uint8_t* stream, int n_bytes, const uint16_t* codebook, uint8_t* __restrict__ wt,
                                                                            const __grid_constant__ GLayer L, int tau, int paired,
-                                                                           const __grid_constant__ GStepOf step_of) {
+                                                                           const __grid_constant__ GStepOf step_of, float* alpha,
+                                                                           const __grid_constant__ GStored<BYTES> stored) {
   grid_dep_launch();   // the layer's launch may set itself up beside this one; its weight producer waits for this one to end
+  if (BYTES > 16) {
+    // (read through its generic address: as a parameter, addresses that differ by lane are served one after the other, 62 us a call)
+    const uint8_t* p;
+    asm volatile("mov.b64 %0, %1;" : "=l"(p) : "l"(stored.b));
+    codebook = reinterpret_cast<const uint16_t*>(p);
+    stream = p + 1024 + (size_t)L.K * 4;
+    if ((blockIdx.x | blockIdx.y | blockIdx.z) == 0) {
+      grid_dep_wait();   // the call before may still read them
+      for (int i = threadIdx.x; i < L.K; i += 32 * G_SW_WARPS) alpha[i] = reinterpret_cast<const float*>(p + 1024)[i];
+    }
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wd = blockIdx.x, ct = blockIdx.y;                       // 32-channel word, channel tile
   const int row0 = (blockIdx.z * G_SW_WARPS + warp) * G_SW_ROWS;    // (all of the warp's rows are of one pixel of a group)
@@ -1541,6 +1559,7 @@ __global__ void __launch_bounds__(32 * G_SW_WARPS) g_static_weights_kernel(const
   __syncthreads();
   const int chunks = paired ? 2 : L.cb_chunks, cb = paired ? 0 : wd / L.cb_chunks, c0 = paired ? 0 : wd - cb * L.cb_chunks;
   uint4* const base = reinterpret_cast<uint4*>(wt) + (size_t)(ct * L.n_cb + cb) * L.steps * chunks * G_ROWS + row0;
+  grid_dep_wait();   // the call before may still read its operand
   if (L.G > 1 || paired) {   // columns outside the pixel's window, and a last step's missing tap
     const int kinds = paired ? 2 : 1;
 #pragma unroll 1
@@ -1604,8 +1623,37 @@ cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8
       if (st.plan.taps.row[t][c] < 3) step_of.at[st.plan.taps.row[t][c]][st.plan.taps.col[t][c]] = (uint8_t)(2 * t + c);
   const int n_bytes = (int)(((long long)g.K * g.C * g.tau + 7) / 8);
   const dim3 blocks((unsigned)(st.plan.paired ? 1 : L.n_cb * L.cb_chunks), (unsigned)L.n_ct, G_ROWS / (G_SW_ROWS * G_SW_WARPS));
-  g_static_weights_kernel<<<blocks, 32 * G_SW_WARPS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, g.tau, st.plan.paired, step_of);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (!plan.stored.codebook) {
+    g_static_weights_kernel<16><<<blocks, 32 * G_SW_WARPS, 0, l.stream>>>(stream_dev, n_bytes, codebook_dev, mem, L, g.tau, st.plan.paired, step_of, nullptr,
+                                                                          GStored<16>{});
+    e = cudaGetLastError();
+  } else {
+    // Parameters are copied whole: three sizes.  A programmatic dependent of the call before: it reads the stored form beside that one's
+    // last tiles, and waits for its end before it writes.
+    const size_t bytes = tcg_stored_bytes(g);
+    GStored<(int)kTcgStoredMax> stored;
+    memcpy(stored.b, plan.stored.codebook, sizeof(uint16_t) << g.tau);
+    memcpy(stored.b + 1024, plan.stored.alpha, (size_t)g.K * 4);
+    memcpy(stored.b + 1024 + (size_t)g.K * 4, plan.stored.stream, (size_t)n_bytes);
+    float* alpha = const_cast<float*>(alpha_dev);
+    int n = n_bytes, tau = g.tau, paired = st.plan.paired;
+    const uint8_t* none = nullptr;
+    const uint16_t* no_codes = nullptr;
+    void* args[] = {&none, &n, &no_codes, &mem, &L, &tau, &paired, &step_of, &alpha, &stored};
+    cudaLaunchAttribute pdl[1];
+    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t wcfg{};
+    wcfg.stream = l.stream;
+    wcfg.attrs = pdl;
+    wcfg.numAttrs = 1;
+    wcfg.gridDim = blocks;
+    wcfg.blockDim = dim3(32 * G_SW_WARPS);
+    const void* const kernel = bytes <= 3072 ? (const void*)g_static_weights_kernel<3072> : bytes <= 12288 ? (const void*)g_static_weights_kernel<12288>
+                                                                                                         : (const void*)g_static_weights_kernel<(int)kTcgStoredMax>;
+    e = cudaLaunchKernelExC(&wcfg, kernel, args);
+  }
   if (e != cudaSuccess) return e;
   *launched += 1;
   GParams p = st.ring;
@@ -1615,8 +1663,8 @@ cudaError_t tcg_static_forward(const TcgStatic& plan, const Geom& g, const uint8
   p.out_type[0] = (uint8_t)l.out_i32;
   p.status = status_dev;
   // A programmatic dependent of the kernel above: the weight producer waits for that one, and the expanders and the epilogue do
-  // as after any other.  (The scales are the copy's, which the kernel above has waited for.)
-  p.after_weights = 1;
+  // as after any other.
+  p.after_weights = plan.stored.codebook ? 2 : 1;
   static unsigned long long done = 0;
   e = allow_max_smem(tcg_conv_kernel<M_FP4, OUT_WORDS>, &done);
   if (e != cudaSuccess) return e;

@@ -135,3 +135,23 @@ def test_wrong_buffers_are_refused_on_the_host(snn):
 ])
 def test_operand_from_the_stored_form(snn, oracle_mod, c_in, c_out, h, w, stride, pad, tau, n):
     _check_case(snn, oracle_mod, wl.LayerShape(c_in, c_out, h, w, stride, pad), tau, n, 17)
+
+
+@pytest.mark.parametrize("c_in,c_out,tau", [(32, 64, 7), (33, 64, 7), (96, 128, 7), (97, 128, 7), (272, 128, 7), (273, 128, 7), (17, 500, 9), (1, 1, 1)])
+def test_stored_forms_around_the_sizes_that_go_with_the_launch(snn, oracle_mod, c_in, c_out, tau):
+    """3072, 12288 and 32000 bytes and a little more: parameters of three sizes, and beyond them a copy.  Calls follow one another
+    without a wait, each with another layer's arrays, which are overwritten as soon as the call returns."""
+    shape = wl.LayerShape(c_in, c_out, 6, 9, 1, 1)
+    calls = []
+    for seed in range(4):
+        p = wl.draw_layer_params(shape, tau, 70 + seed)
+        packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, 2, 90 + seed))
+        ref = oracle_mod.conv_bin(p.codebook, tau, p.idx_packed, p.alpha, c_in, c_out, 1, 1, packed)[1]
+        calls.append((p, torch.from_numpy(packed.view(np.int32)).cuda(), torch.empty((2, 6, 9, c_out), device="cuda"), ref))
+    book, stream, alpha = (np.array(a) for a in (calls[0][0].codebook, calls[0][0].idx_packed, calls[0][0].alpha))
+    for p, act, out, _ in calls:
+        book[:], stream[:], alpha[:] = p.codebook, p.idx_packed, p.alpha
+        snn.forward_static(c_in, c_out, tau, book, stream, alpha, act, out)
+        book[:], stream[:], alpha[:] = 0, 0, 0
+    for _, _, out, ref in calls:
+        assert (out.cpu().numpy() == ref).all()
