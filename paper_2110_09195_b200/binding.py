@@ -132,7 +132,7 @@ def _load_fast():
             module.bind(*(ctypes.cast(f, ctypes.c_void_p).value
                           for f in (lib.snn_conv_forward, lib.snn_conv_group_forward, lib.snn_conv_stack_forward)))
             module.bind_static(ctypes.cast(lib.snn_conv_forward_static, ctypes.c_void_p).value, np.ndarray)
-        except ImportError as e:
+        except (ImportError, AttributeError) as e:   # (AttributeError: a module built from older source)
             warnings.warn(f"the forward calls are checked in Python, which takes longer: {e} "
                           "(python -m paper_2110_09195_b200.build builds _snn_fast)", RuntimeWarning, stacklevel=3)
             module = _PythonChecks

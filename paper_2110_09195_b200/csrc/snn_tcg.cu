@@ -166,6 +166,7 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
   constexpr uint64_t fixed = ((uint64_t)1 << 46) | ((uint64_t)8 << 32);   // descriptor version; 8-row groups 128 bytes apart
   constexpr uint64_t w_fixed = fixed | ((uint64_t)128 << 16);             // the weights' chunks are 128 rows apart
   const int st_steps = L.st_steps;
+  const uint32_t pair = MODE == M_F16 ? (uint32_t)L.pair : 0u;
   uint32_t tap = MODE == M_FP4 && KPT == 1 ? 0u : L.tap[t];
 #pragma unroll 1
   while (t < t_last) {
@@ -217,13 +218,14 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
       const uint32_t cur = tap;
       if (t + 1 < t_last) tap = L.tap[t + 1];
       const uint64_t bd = a_fixed | ((uint64_t)(cur >> 16) << 16) | (uint64_t)(a_unit + (cur & 0xffffu));
+      const uint32_t rows = MODE == M_F16 ? idesc - ((pair >> t & 2u) << 25) : idesc;   // (M >> 4 from bit 24 on: 64 rows instead of 128)
       const uint64_t wd = w_fixed | (uint64_t)wa;
       if (leader) {
 #pragma unroll
         for (int k = 0; k < KPT; ++k) {
           const uint32_t accum = k == 0 ? acc : 1u;
           if (MODE == M_FP4) mma_ss_fp4(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum, sf, sf + 16);
-          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum);
+          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), rows, accum);
         }
       }
       acc = 1;
@@ -468,7 +470,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           uint32_t acc = 0;  // 0 only for the first MMA of the tile
           uint32_t row0 = 0;   // a unit fetched by TMA starts at the beginning of a row of positions
           if (swz) {
-            const uint32_t Q0 = fdiv((uint32_t)tile, L.dCt) * (uint32_t)L.Np;
+            const uint32_t Q0 = fdiv((uint32_t)tile, L.dCt) * (uint32_t)(L.Np - (L.pair & 1));
             row0 = 8u * (Q0 - fdiv(Q0, L.dWg) * (uint32_t)L.Wg);
           }
 #pragma unroll 1
@@ -522,15 +524,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const uint32_t tile_phase = (seq >> 2) & 1u;   // (acc_full and the tables are indexed and flip alike)
       if (!wait_phase(bar_tabfull + 8u * (seq & 3u), tile_phase, 100, 6)) break;
       const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
-      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, lg = h1.z;
+      const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, lg = F16 ? 0 : h1.z;
+      const bool pair = F16 && h1.z;   // (see g_pairs)
       if (l < 0) break;   // no more tiles
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : h1.w & 3;
       uint32_t* const out32 = reinterpret_cast<uint32_t*>(p.out[l]);  // int32 and fp32 outputs share the layout
       // this lane's row of the weight operand: channel c of pixel g of a position's group, or of a copy of the channels
-      const int c_lane = row & ((1 << kp_log) - 1), c_warp = (rq * 32) & ((1 << kp_log) - 1);   // (_warp: of lane 0)
+      const int c_lane = pair ? 16 * rq + (lane & 15) : row & ((1 << kp_log) - 1), c_warp = pair ? 16 * rq : (rq * 32) & ((1 << kp_log) - 1);   // (_warp: of lane 0)
       const int g_lane = lg ? row >> kp_log : 0, g_warp = lg ? (rq * 32) >> kp_log : 0;
       // the warps of a lane quarter, and the copies, take the 32-column slices in turn
-      const int s_first = half + (lg ? 0 : 2 * ((rq * 32) >> kp_log)), s_step = lg ? 2 : 2 << (7 - kp_log);
+      const int s_first = half + (lg || pair ? 0 : 2 * ((rq * 32) >> kp_log)), s_step = lg || pair ? 2 : 2 << (7 - kp_log);
       const int co = h0.z + c_lane, co_warp = h0.z + c_warp;
       const bool active = co_warp < K;   // does any of the warp's rows hold a channel?
       const float al = T->alpha[c_lane], minus_threshold = WORDS ? 0.f : -T->threshold[c_lane];
@@ -577,6 +580,28 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             uint32_t v[32];
             __syncwarp();   // the load is a warp-wide instruction
             tmem_ld32(d0 + (uint32_t)(32 * s), v);
+            if (F16 && pair) {
+              // Lanes 0..15 hold a channel's sums over two columns of the kernel, lanes 16..31 those over the other, which belong to the
+              // position before: the lower lanes put even positions together and the upper ones odd positions, a shuffle for
+              // both.  A store writes 16 channels of two positions.
+              uint32_t next = 0;
+              const int after = 32 * s + 32;   // the upper lanes need the first column of the next slice
+              if (after < lay[l].Np) next = tmem_ld1(d0 + (uint32_t)after);
+              if (s + s_step >= n_slices) release();
+              const bool upper = lane >= 16;
+              const uint32_t mask = co < K ? T->mask[s] >> (lane >> 4) : 0u;
+              const uint32_t* const at = &T->offset[32 * s + (lane >> 4)];
+#pragma unroll
+              for (int e = 0; e < 32; e += 2) {
+                const float other = __uint_as_float(__shfl_xor_sync(0xffffffffu, v[e + 1], 16));
+                const float mine = __uint_as_float(upper ? (e + 2 < 32 ? v[e + 2] : next) : v[e]);
+                const uint32_t y = __float_as_uint(__fmul_rn(__fadd_rn(mine, other), al));
+                asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(obase + at[e]), "r"(y),
+                             "r"(mask & (1u << e))
+                             : "memory");
+              }
+              continue;
+            }
             if (s + s_step >= n_slices) release();
             if (WORDS || out_kind < 2) {
               const uint32_t mask = co < K ? T->mask[g_lane * G_MAX_CHUNKS + s] : 0u;
@@ -702,6 +727,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const FastDiv dWg = L.dWg, dHq = L.dHq, dCt = L.dCt;
       const int Np = L.Np, K = L.K, Wg = L.Wg, Hq = L.Hq, Ho = L.Ho, Wo = L.Wo, lg = L.lg, n_ct = L.n_ct, total = L.total_tiles;
       const uint32_t Qtot = L.Qtot;
+      const int own = Np - (F16 ? L.pair & 1 : 0);   // positions of a tile
       const int n_slices = (Np + 31) >> 5;
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
       const uint32_t scale = out_kind >= 2 ? (uint32_t)(K + 31) >> 5 : (uint32_t)K;   // words of a pixel
@@ -720,16 +746,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         }
         if (lane == 0) {
           *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
-          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, lg, out_kind | (CHAIN && (few || tile + 2 * G >= total) ? 4 : 0));
+          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, F16 ? L.pair & 1 : lg, out_kind | (CHAIN && (few || tile + 2 * G >= total) ? 4 : 0));
         }
 #pragma unroll 1
         for (int s = 0; s < n_slices; ++s) {
           const int c = 32 * s + lane;
-          const uint32_t q = (uint32_t)mg * (uint32_t)Np + (uint32_t)c;
+          const uint32_t q = (uint32_t)mg * (uint32_t)own + (uint32_t)c;
           const uint32_t rg = fdiv(q, dWg), n = fdiv(rg, dHq);
           const int x = (int)(q - rg * (uint32_t)Wg) << lg, y = (int)(rg - n * (uint32_t)Hq);
           T->offset[c] = ((n * (uint32_t)Ho + (uint32_t)y) * (uint32_t)Wo + (uint32_t)x) * scale;
-          const int rem = c < Np && q < Qtot && y < Ho ? Wo - x : 0;   // pixels from x to the end of the row
+          const int rem = c < own && q < Qtot && y < Ho ? Wo - x : 0;   // pixels from x to the end of the row
 #pragma unroll 1
           for (int g = 0; g < (1 << lg); ++g) {
             const uint32_t m = __ballot_sync(0xffffffffu, g < rem);
@@ -1092,10 +1118,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           // above and below the image and channels past the last are out of the tensor's bounds and read as zeros.
           const uint32_t row_bytes = (uint32_t)L.Wg * 128u, ew = (uint32_t)(et >> 5), Hq = (uint32_t)L.Hq;
           const FastDiv dHq = L.dHq, dWg = L.dWg;
-          const int n_pu = L.n_pu, rs = L.rs, pad = L.pad, cpl = L.cpl, Np = L.Np;
+          const int n_pu = L.n_pu, rs = L.rs, pad = L.pad, cpl = L.cpl, own = L.Np - (L.pair & 1);
 #pragma unroll 1
           for (int tile = L.first; tile < total && !stop; tile += G) {
-            const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)Np;
+            const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)own;
             const uint32_t r_first = fdiv(Q0, dWg), r_last = fdiv(Q0 + (uint32_t)Rr - 1u, dWg);
 #pragma unroll 1
             for (int u = 0; u < n_cb * n_pu; ++u) {
@@ -1276,7 +1302,7 @@ template <int MODE>
 __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, uint8_t* __restrict__ wt, int C, int K,
                                         int Cw, long long total, int cb_chunks, int n_cb, int steps, int paired, int lg,
                                         int kp_log, int win_step, int ksize, const GTaps taps, const float* __restrict__ alpha,
-                                        const float* __restrict__ shift, float* __restrict__ threshold) {
+                                        const float* __restrict__ shift, float* __restrict__ threshold, int pair) {
   long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= total) return;
   if (threshold && i < K) threshold[i] = g_sign_threshold(alpha[i], shift[i], ksize * ksize * C);   // (there are more chunks than channels)
@@ -1288,9 +1314,19 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
   const int t = (int)(r % steps);
   r /= steps;
   const int cb = (int)(r % n_cb), tile = (int)(r / n_cb);
-  const int g = lg ? row >> kp_log : 0, co = tile * G_ROWS + (row & ((1 << kp_log) - 1));
+  const int g = lg ? row >> kp_log : 0;
+  int co = tile * G_ROWS + (row & ((1 << kp_log) - 1));
   const int which = paired ? c : 0;
-  const int ky = taps.row[t][which], kx = (int)taps.col[t][which] - win_step * g;
+  const int ky = taps.row[t][which];
+  int kx = (int)taps.col[t][which] - win_step * g;
+  if (pair) {   // (see g_pairs)
+    if (kx == 0) {
+      co = (row >> 5) * 16 + (row & 15);
+      kx = (row & 16) ? win_step : 0;
+    } else {
+      co = row < 64 ? row : K;
+    }
+  }
   constexpr int cpc = MODE == M_F16 ? 8 : 32;
   uint4 v = make_uint4(0, 0, 0, 0);
   if (co < K && ky < ksize && kx >= 0 && kx < ksize) {
@@ -1465,11 +1501,11 @@ cudaError_t tcg_create(const LayerDev* const* layers, const Geom* geoms, int cou
     if (mode == M_F16)
       g_expand_weights_kernel<M_F16><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
                                                             total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
-                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds);
+                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds, L.pair & 1);
     else
       g_expand_weights_kernel<M_FP4><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
                                                             total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
-                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds);
+                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds, L.pair & 1);
     e = cudaGetLastError();
     if (e == cudaSuccess) *launched += 1;
   }

@@ -263,3 +263,29 @@ def test_signs_where_scaled_sums_round_or_cancel(snn, oracle_mod, c_in, c_out, h
     got = layer.forward(torch.from_numpy(packed.view(np.int32)).cuda(), out_type=snn.OUT_BITS).cpu().numpy().view(np.uint32)
     assert (got == want).all()
     layer.destroy()
+
+
+@pytest.mark.parametrize("stride,pad", [(1, 1), (1, 0), (2, 1), (2, 0)])
+@pytest.mark.parametrize("c_in,c_out,h,w,n", [(8, 33, 5, 5, 1), (64, 64, 15, 15, 3), (72, 48, 9, 31, 2), (128, 40, 20, 57, 4), (16, 64, 30, 30, 12)])
+def test_fp16_layers_of_33_to_64_channels(snn, oracle_mod, c_in, c_out, h, w, n, stride, pad):
+    """Two kernel columns in the rows of the weight operand: sums put together over two columns of the accumulator, tiles that overlap by
+    one position, one and several slices and channel blocks; an infinity reaches the outputs whose windows hold it and no others."""
+    shape = wl.LayerShape(c_in, c_out, h, w, stride, pad)
+    p = wl.draw_layer_params(shape, 6, 700 + c_in + c_out)
+    rng = np.random.default_rng(31)
+    x = rng.standard_normal((n, h, w, c_in)).astype(np.float16)
+    layer = snn.SnnConv(c_in, c_out, 6, p.codebook, p.idx_packed, p.alpha, stride, pad, snn.ACT_F16)
+    assert layer.path_supported(snn.PATH_DECODED_TC, n, h, w)
+    for k in range(2):
+        if k:
+            x[rng.random(x.shape) < 0.4 / (9 * c_in)] = np.inf
+            x[rng.random(x.shape) < 0.2 / (9 * c_in)] = -np.inf
+        with np.errstate(invalid="ignore"):
+            want = oracle_mod.conv_f16(p.codebook, 6, p.idx_packed, p.alpha, c_in, c_out, stride, pad, x)
+        got = layer.forward(torch.from_numpy(x).cuda(), path=snn.PATH_DECODED_TC).cpu().numpy()
+        finite = np.isfinite(want)
+        assert finite.all() or k
+        assert (np.isnan(got) == np.isnan(want)).all() and (got[np.isinf(want)] == want[np.isinf(want)]).all()
+        # exact products, fp32 sums of 9*c_in terms: 2^-24 a step of the sum at most, on terms of size one
+        assert (np.abs(got[finite] - want[finite]) <= 2.0 ** -24 * 9 * c_in * 1.5 * 4 * np.sqrt(9 * c_in)).all()
+    layer.destroy()
