@@ -97,6 +97,13 @@ __device__ long long g_trace[256 * 16];
 #define TR_REPORT(role, total, w0, w1, w2) do { } while (0)
 #endif
 
+// A value that is the same in all lanes, in a form that the compiler knows to be: tensor-core instructions take their operands from the
+// registers of a warp, and what it cannot know to be uniform is moved there one operand at a time before each of them.  The MMA issuer's loops
+// were bound by that (98 cycles an MMA whatever its width; the tensor core takes 40 to 64): with its values, and the warp's
+// number that the roles branch on, known to be uniform, and MMAs under a predicate instead of a branch, one layer of 256 channels
+// 8.95 and 8.31 us, 512 channels of 7x7 at batch 8 7.33 and 6.74, ResNet-18 stack on one image 64.1 and 60.5 (the predicates alone 8.32,
+// 6.74, 61.2; taps and the answers of waits made uniform, too: nothing, or less).
+__device__ __forceinline__ int uni(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 __device__ __forceinline__ uint32_t fdiv(uint32_t q, const FastDiv& f) {
   return __umulhi(2u * q, f.m) >> f.s;
 }
@@ -165,7 +172,7 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
                                               long long& tr_b) {
   constexpr uint64_t fixed = ((uint64_t)1 << 46) | ((uint64_t)8 << 32);   // descriptor version; 8-row groups 128 bytes apart
   constexpr uint64_t w_fixed = fixed | ((uint64_t)128 << 16);             // the weights' chunks are 128 rows apart
-  const int st_steps = L.st_steps;
+  const int st_steps = uni(L.st_steps);
   const uint32_t pair = MODE == M_F16 ? (uint32_t)L.pair : 0u;
   uint32_t tap = MODE == M_FP4 && KPT == 1 ? 0u : L.tap[t];
 #pragma unroll 1
@@ -181,15 +188,15 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
       // with fp16 operands, the longer code costs the other roles more than this gains (fp16 group at batch 1 12 %).
       constexpr int ST = (int)(kGBSlot / (KPT * 2 * G_ROWS * 16));   // most steps of a stage (g_plan_layer)
       const int n = t_last - t < st_steps ? t_last - t : st_steps;
-      if (leader) {
+      {
         uint32_t rows[ST];
 #pragma unroll
         for (int i = 0; i < ST; ++i) rows[i] = i < n ? L.tap[t + i] + a_unit : 0u;   // (start and chunk distance of the low word)
 #pragma unroll
         for (int i = 0; i < ST; ++i) {
-          if (i < n) mma_ss_fp4(d0, w_fixed | (uint64_t)(wa + (uint32_t)(i * 256)), a_fixed | (uint64_t)rows[i], idesc, i == 0 ? acc : 1u, sf, sf + 16);
+          if (i < n) mma_ss_fp4(d0, w_fixed | (uint64_t)(wa + (uint32_t)(i * 256)), a_fixed | (uint64_t)rows[i], idesc, i == 0 ? acc : 1u, sf, sf + 16, leader);
         }
-        tc_commit(bar_bempty + 8 * b_slot);
+        if (leader) tc_commit(bar_bempty + 8 * b_slot);
       }
       t += n;
       acc = 1;
@@ -203,10 +210,10 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
 #pragma unroll 1
       for (; t + 1 < t_end; t += 2) {
         const uint32_t one = L.tap[t] + a_unit, two = L.tap[t + 1] + a_unit;
-        if (leader) {
+        {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
-            mma_ss_fp4(d0, w_fixed | (uint64_t)(wa + (uint32_t)(k * 256)), a_fixed | (uint64_t)((k < 2 ? one : two) + (uint32_t)(k & 1) * k_step), idesc, k == 0 ? acc : 1u, sf, sf + 16);
+            mma_ss_fp4(d0, w_fixed | (uint64_t)(wa + (uint32_t)(k * 256)), a_fixed | (uint64_t)((k < 2 ? one : two) + (uint32_t)(k & 1) * k_step), idesc, k == 0 ? acc : 1u, sf, sf + 16, leader);
         }
         acc = 1;
         wa += 4 * 256;
@@ -220,12 +227,12 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last
       const uint64_t bd = a_fixed | ((uint64_t)(cur >> 16) << 16) | (uint64_t)(a_unit + (cur & 0xffffu));
       const uint32_t rows = MODE == M_F16 ? idesc - ((pair >> t & 2u) << 25) : idesc;   // (M >> 4 from bit 24 on: 64 rows instead of 128)
       const uint64_t wd = w_fixed | (uint64_t)wa;
-      if (leader) {
+      {
 #pragma unroll
         for (int k = 0; k < KPT; ++k) {
           const uint32_t accum = k == 0 ? acc : 1u;
-          if (MODE == M_FP4) mma_ss_fp4(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum, sf, sf + 16);
-          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), rows, accum);
+          if (MODE == M_FP4) mma_ss_fp4(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum, sf, sf + 16, leader);
+          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), rows, accum, leader);
         }
       }
       acc = 1;
@@ -295,7 +302,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   uint32_t* ready_tiles = tmem_slot + 2;   // chain: tiles of this CTA whose input has been written
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uni(tid >> 5), lane = tid & 31;
   const int NS = p.NS, NA = p.NA;
   const int G = (int)gridDim.x;
 
@@ -433,7 +440,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     // The whole warp walks the loops and waits together, so that every address and descriptor
-    // is a warp-uniform value; one elected lane issues the MMAs and the commits.
+    // is a warp-uniform value; the MMAs and the commits are predicated on one elected lane.
     {
       const bool leader = elect_one();
       bool ok = true;
@@ -448,20 +455,21 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
 #pragma unroll 1
       for (int l = 0; l < p.n_layers && ok; ++l) {
         const GLayer& L = lay[l];
-        const int n_units = L.n_cb * L.n_pu, n_pu = L.n_pu, kpt = L.kpt, total = L.total_tiles;
+        const int n_pu = uni(L.n_pu), n_units = uni(L.n_cb) * n_pu, kpt = uni(L.kpt), total = uni(L.total_tiles), tile0 = uni(L.first);
         // activation operand: rows of 16 bytes, 8-row groups 128 bytes apart, a K step two chunks on; or rows of 128 bytes
         // in the 128-byte swizzle, 8-row groups 1024 bytes apart, a K step 32 bytes on.  (The swizzle permutes address
         // bits, so a tap's start may be any row.)
-        const bool swz = F16 && L.tma;
+        const bool swz = F16 && uni(L.tma);
         const uint64_t a_fixed = ((uint64_t)1 << 46) | (swz ? ((uint64_t)2 << 61) | ((uint64_t)64 << 32) : (uint64_t)8 << 32);
-        const uint32_t k_step = swz ? 2u : 2u * (uint32_t)(L.n_planes * L.Rr);
+        const uint32_t k_step = swz ? 2u : 2u * (uint32_t)uni(L.n_planes * L.Rr);
+        const uint32_t Np = (uint32_t)uni(L.Np);
         // instruction descriptor: D format, A/B formats, K-major both, N>>3, M>>4
         // (4-bit mode: A/B format e2m1, scale format ue8m0, scale ids 0)
         const uint32_t idesc =
-            F16 ? ((1u << 4) | ((uint32_t)(L.Np >> 3) << 17) | ((128u >> 4) << 24))
-                : ((1u << 7) | (1u << 10) | ((uint32_t)(L.Np >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24));
+            F16 ? ((1u << 4) | ((Np >> 3) << 17) | ((128u >> 4) << 24))
+                : ((1u << 7) | (1u << 10) | ((Np >> 3) << 17) | (1u << 23) | ((128u >> 4) << 24));
 #pragma unroll 1
-        for (int tile = L.first; tile < total && ok; tile += G, ++tiles_done) {
+        for (int tile = tile0; tile < total && ok; tile += G, ++tiles_done) {
           if (tiles_done >= n_acc) {
             if (!TR_WAIT(tr_w0, mbar_wait(bar_accempty + 8 * acc_slot, acc_phase))) { ok = false; break; }
             tc_fence_after();
@@ -478,7 +486,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             if (!TR_WAIT(tr_w1, mbar_wait(bar_afull + 8 * a_slot, a_phase))) { ok = false; break; }
             tc_fence_after();
             const uint32_t a_unit = a_base + (uint32_t)a_slot * a_slot_units + row0;
-            const int pu = u & (n_pu - 1), t_last = L.pu_end[pu];
+            const int pu = u & (n_pu - 1), t_last = uni(L.pu_end[pu]);
             if (pu == 0) t = 0;
 #define G_ISSUE(KP)                                                                                                  \
   ok = g_issue_block<MODE, KP>(L, t, t_last, a_fixed, k_step, a_unit, w_base, b_slot_units, d0, idesc, acc, NS, bar_bfull, bar_bempty, b_slot, \
