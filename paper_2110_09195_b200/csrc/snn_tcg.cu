@@ -876,7 +876,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       // slot always belongs to the same team): with few rows per unit a unit is a chain of latencies, and two
       // chains in flight are what doubles the rate.
       constexpr int XG = G_XTEAMS, XT = G_EXP_THREADS / XG;
-      const int gx = et / XT, etg = et % XT;
+      // (from the warp's number, which is known to be uniform: single layers 1 % faster; chains with tags are as much slower)
+      const int gx = TAGGED ? et / XT : (warp - 10 - (warp > 13) - (warp > 17)) / (XT / 32), etg = et % XT;
       // issue side: the unit (il, itile, icb) with sequence number iu, and the next item to load in it
       int il = 0, itile = 0, itotal = 0, icb = 0, i_slot = 0, iu = 0;
       int pos0 = 0, ipl = 0, ik0 = 0;                 // first position of the thread's row of positions, plane, word
