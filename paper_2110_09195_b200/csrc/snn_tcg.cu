@@ -1044,7 +1044,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           if (a_slot >= NA) { a_slot -= NA; a_phase ^= 1u; }
         }
       };
-      // words with tags: looks (bounded) until all of the group's are this launch's
+      // words with tags: looks (bounded) until all of the group's are this launch's, without a pause between the looks (with 20 ns from the
+      // third on, ResNet-20 stacks 2 to 3.5 % slower, the others 1 to 1.5 %)
       auto settle = [&]() -> bool {
         const bool two = (cur.flags & 0x6000u) != 0;
 #pragma unroll 1
@@ -1059,7 +1060,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           }
           if (__all_sync(0xffffffffu, all)) break;
           if (it >= (1u << 21) || __any_sync(0xffffffffu, *abort_flag != 0)) return false;
-          if (it > 2) __nanosleep(20);
         }
 #pragma unroll
         for (int j = 0; j < XI; ++j) cur.t[j].y = cur.t[j].z;
