@@ -826,7 +826,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     // ------------------------------------------------ expanders (warps 10-12, 14-16, 18, 19)
     // Fill activation unit (problem, tile, channel block) of the ring: for every plane, row and
     // 32-channel word, bits -> one 16-byte chunk of nibbles (fp16: 8-channel chunks are copied).
-    grid_dep_wait();  // the activations may come from the previous kernel in the stream
+    if (F16) grid_dep_wait();  // the activations may come from the previous kernel in the stream (bits: below)
     const int et = (warp - 10 - (warp > 13) - (warp > 17)) * 32 + lane;  // rank among the expander threads
     int a_slot = 0;
     long long a_done = 0;
@@ -842,21 +842,6 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_afull + 8 * slot);
     };
-    if (FP4 && !CHAIN && !TAGGED && (p.n_layers > 1 || lay[0].total_tiles > G)) {
-      // Independent problems: all inputs exist when the launch starts and are small beside the L2 (1/29 of the
-      // outputs; fp16 inputs are not: half of the outputs).  The CTAs pull them into L2 together, once, so that the
-      // staging loads below see L2 latency instead of DRAM latency.  (Not where every CTA has one tile: its loads go out now anyway,
-      // 0.3 us earlier without this; 14 single layers 1 %.)
-#pragma unroll 1
-      for (int l = 0; l < p.n_layers; ++l) {
-        const GLayer& L = lay[l];
-        const size_t bytes = (size_t)L.N * L.H * L.W * ((size_t)L.Cw * 4);
-        const char* base = reinterpret_cast<const char*>(p.act[l]);
-#pragma unroll 1
-        for (size_t off = ((size_t)blockIdx.x * G_EXP_THREADS + et) * 128; off < bytes; off += (size_t)G * G_EXP_THREADS * 128)
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
-      }
-    }
     if constexpr (FP4) {
       // A two-stage software pipeline per thread: a "group" is up to four items of one unit - an item is the words of
       // one position in one plane that one load brings - and the loads of group g + 1 are issued (into registers)
@@ -938,6 +923,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         }
         return ready;
       };
+      // where position pos of the unit (il, itile) reads
+      auto locate = [&](int pos) {
+        const GLayer& L = lay[il];
+        const uint32_t q = Q0 + (uint32_t)pos;
+        const uint32_t rg = fdiv(q, L.dWg), n = fdiv(rg, L.dHq);
+        row = L.rs * (int)(rg - n * (uint32_t)L.Hq) - L.pad;
+        col = L.cm * (int)(q - rg * (uint32_t)L.Wg) - L.pad;
+        img_row = (int)n * H;
+        inside = q < L.Qtot;
+      };
       auto issue = [&](XGroup& g) {   // loads of the group at the issue position; moves the position on
         const GLayer& L = lay[il];
         const bool fresh = CHAIN && L.deps != nullptr;   // written by other CTAs of this launch: read from L2
@@ -954,14 +949,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         for (int j = 0; j < XI; ++j) {
           if (ended) break;
           const int pos = pos0 + (TAGGED ? etg >> tpl : etg), ik = ik0 + own;
-          if ((ipl | ik0) == 0) {
-            const uint32_t q = Q0 + (uint32_t)pos;
-            const uint32_t rg = fdiv(q, L.dWg), n = fdiv(rg, L.dHq);
-            row = L.rs * (int)(rg - n * (uint32_t)L.Hq) - L.pad;
-            col = L.cm * (int)(q - rg * (uint32_t)L.Wg) - L.pad;
-            img_row = (int)n * H;
-            inside = q < L.Qtot;
-          }
+          if (TAGGED && (ipl | ik0) == 0) locate(pos);
           const int r = row + (ipl >> cpl), c = col + cs * (ipl & ((1 << cpl) - 1)), word = icb * cbc + ik;
           const bool on = inside && pos < Rr && (uint32_t)r < (uint32_t)H && (uint32_t)c < (uint32_t)W && word < Cw;
           g.da[j] = unit + (uint32_t)ik * cstride + (uint32_t)(ipl * Rr + pos) * 16u;
@@ -991,6 +979,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
               ipl = 0;
               pos0 += TAGGED ? XT >> tpl : XT;
               ended = pos0 >= Rr;
+              if (!TAGGED && !ended) locate(pos0 + etg);
             }
           }
         }
@@ -999,6 +988,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           flags |= 0x400u;
           next_unit();
           seek_own();
+          if (!TAGGED && ivalid) locate(etg);
         }
         g.cstride = cstride;
         g.flags = flags;
@@ -1006,6 +996,26 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       if (lay[0].first >= lay[0].total_tiles) il = lay[0].next;
       enter_layer();
       seek_own();
+      if (!TAGGED && ivalid) locate(etg);
+      // The activations may come from the previous kernel in the stream.  (What does not read them stands before the wait, and a unit's first
+      // position is located when the unit before it has been issued: smallest layer 4.24 and 4.04 us, 256 channels 8.28 and 8.05, ragged layer 6.89 and
+      // 6.67.  In chains of words with tags the latter costs 1 to 3 % on one image.)
+      grid_dep_wait();
+      if (!CHAIN && !TAGGED && (p.n_layers > 1 || lay[0].total_tiles > G)) {
+        // Independent problems: all inputs exist when the launch starts and are small beside the L2 (1/29 of the
+        // outputs; fp16 inputs are not: half of the outputs).  The CTAs pull them into L2 together, once, so that the
+        // staging loads below see L2 latency instead of DRAM latency.  (Not where every CTA has one tile: its loads go out now anyway,
+        // 0.3 us earlier without this; 14 single layers 1 %.)
+#pragma unroll 1
+        for (int l = 0; l < p.n_layers; ++l) {
+          const GLayer& L = lay[l];
+          const size_t bytes = (size_t)L.N * L.H * L.W * ((size_t)L.Cw * 4);
+          const char* base = reinterpret_cast<const char*>(p.act[l]);
+#pragma unroll 1
+          for (size_t off = ((size_t)blockIdx.x * G_EXP_THREADS + et) * 128; off < bytes; off += (size_t)G * G_EXP_THREADS * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(base + off));
+        }
+      }
       // completion side: this team's slots gx, gx + XG, ... of the ring
       a_slot = gx;
       XGroup cur, nxt = {};   // (a unit's last group leaves items unwritten, and all of them are copied)
