@@ -44,7 +44,8 @@ constexpr int G_MAX_CHUNKS = 8;                // 32-column slices of an accumul
 // What the epilogue needs to know of a tile, written by the table warp (see there), four tiles deep.
 struct GTile {
   int l, mg, co, n_slices;             // problem (-1: no more tiles), position tile, first channel, 32-column slices
-  int K, kp_log, lg, out_kind;         // channels; GLayer::kp_log, lg; GParams::out_type
+  int K, kp_log, lg, out_kind;         // channels; GLayer::kp_log, lg (fp16: whether the rows hold pairs, GLayer::pair); GParams::out_type,
+                                       // + 4: the epilogue advances the tile's counter itself, + 8: the CTA's last tile
   uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
   uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
   float alpha[G_ROWS], threshold[G_ROWS];
