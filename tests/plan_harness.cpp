@@ -124,4 +124,12 @@ int plan_order(const int* gs, int count, int f16, int sms, int* order, double* c
   return 1;
 }
 
+// does a group's order differ from the one given?
+int plan_reorders(const int* gs, int count, int f16, int sms) {
+  std::vector<Geom> g(count);
+  std::vector<GPlan> plan(count);
+  for (int i = 0; i < count; ++i) g[i] = geom(gs + 8 * i);
+  return g_plan_independent(g.data(), count, f16 ? M_F16 : M_FP4, TCG_WORDS, f16 != 0, sms, plan.data()) && g_reorders(plan.data(), count);
+}
+
 }  // extern "C"
