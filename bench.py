@@ -181,8 +181,8 @@ def run_reference(args):
 # the kernel's sources are the ones that were profiled: {kernel: (workload, batch, bytes, sha256 of sources)}
 _TRAFFIC = {
     # profiles/dram_traffic_resnet18_stack_n64_grouped.txt: mean of the two captured launches
-    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351272320,
-                                             "2c91d818c0f84dfa3942668375260fe290d763a79931863956beecf907ab2ee6"),
+    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351403776,
+                                             "b25bfb339fa1c1bed04e62dd174992f6f71d370bfcd5e802fb057fafbcf6df70"),
 }
 
 
