@@ -447,10 +447,10 @@ bool g_plan_by_end(const Geom& g, int mode, int kind, int sms, GPlan* plan) {
 
 // Do the packed signs between the members of a chain carry tags?  words: the most between two members.  A layer's signs then reach
 // the next layer's expanders 1.2 us sooner, but each word is twice as long and the expanders load two of them at a time
-// instead of four, which shows once a CTA has many tiles.  Measured on one B200 as graphs, counters and tags, us: ResNet-18 stack
-// batch 1 85 and 67, batch 8 93 and 81, 16 (100 k words) 98.6 and 96.9, 32 112 and 115, 64 132 and 142; ResNet-34 batch 1 162 and
-// 129, 16 187 and 184, 32 215 and 222; ResNet-20 batch 1 68 and 50, 64 99 and 86, 96 103 and 94, 128 (131 k words) 123 and 118.
-// (One rule for all: 200 k words are too many for the networks of one to sixteen words a pixel, and 131 k still gain where every
+// instead of four, which shows once a CTA has many tiles.  Measured on one B200, counters and tags, us: ResNet-20 stack at batch 96
+// (98 k words) 103 and 90, 128 (131 k) 123 and 112; ResNet-34 16 (100 k) 180 and 177, 24 (150 k) 190 and 195; ResNet-18 24 102.0 and
+// 104.6, 32 (200 k) 108.7 and 111.4; on one image, when both kinds took longer, ResNet-18 85 and 67, ResNet-34 162 and 129, ResNet-20 68 and 50.
+// (One rule for all: 150 k words are too many for the networks of two to sixteen words a pixel, and 131 k still gain where every
 // pixel is one.  A stack of one layer has no word between members, and with tags no counters to clear.)
 inline bool g_tagged(size_t words) { return words <= (size_t)1 << 17; }
 
