@@ -181,8 +181,8 @@ def run_reference(args):
 # the kernel's sources are the ones that were profiled: {kernel: (workload, batch, bytes, sha256 of sources)}
 _TRAFFIC = {
     # profiles/dram_traffic_resnet18_stack_n64_grouped.txt: mean of the two captured launches
-    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 351403776,
-                                             "b25bfb339fa1c1bed04e62dd174992f6f71d370bfcd5e802fb057fafbcf6df70"),
+    "tcg_conv_kernel (grouped decoded_tc)": ("resnet18", 64, 350840448,
+                                             "2e025f3b5e9b582e959f3a0c8dc3c7a16330b8766838f6430dcf07fa34772ef6"),
 }
 
 
