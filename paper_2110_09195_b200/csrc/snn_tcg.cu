@@ -166,13 +166,12 @@ struct GMaps {
 // The MMAs of one activation unit of one tile: steps t..t_last x KPT.  The body of a step is straight-line code.
 // Weight stages are waited for and released as the step counter crosses their boundaries.
 template <int MODE, int KPT>
-__device__ __forceinline__ bool g_issue_block(const GLayer& L, int t, int t_last, uint64_t a_fixed, uint32_t k_step, uint32_t a_unit, uint32_t w_base, uint32_t b_slot_units,
+__device__ __forceinline__ bool g_issue_block(const GLayer& L, int st_steps, int t, int t_last, uint64_t a_fixed, uint32_t k_step, uint32_t a_unit, uint32_t w_base, uint32_t b_slot_units,
                                               uint32_t d0, uint32_t idesc, uint32_t& acc, int NS, uint32_t bar_bfull,
                                               uint32_t bar_bempty, int& b_slot, uint32_t& b_phase, bool leader, uint32_t sf,
                                               long long& tr_b) {
   constexpr uint64_t fixed = ((uint64_t)1 << 46) | ((uint64_t)8 << 32);   // descriptor version; 8-row groups 128 bytes apart
   constexpr uint64_t w_fixed = fixed | ((uint64_t)128 << 16);             // the weights' chunks are 128 rows apart
-  const int st_steps = uni(L.st_steps);
   const uint32_t pair = MODE == M_F16 ? (uint32_t)L.pair : 0u;
   uint32_t tap = MODE == M_FP4 && KPT == 1 ? 0u : L.tap[t];
 #pragma unroll 1
@@ -309,7 +308,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   // Whole-warp wait of a role whose warps wait one lane each: a phase that is over already costs one look and a vote.  False: the wait ran
   // out, or the CTA is giving up.
   auto wait_phase = [&](uint32_t bar, uint32_t parity, uint32_t ns, int code) -> bool {
-    if (__any_sync(0xffffffffu, mbar_test(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_test(bar, parity))) return true;   // (every lane has seen it for itself)
     int okw = 1;
     if (lane == 0) {
       okw = (!*abort_flag && mbar_wait_backoff(bar, parity, ns)) ? 1 : 0;
@@ -440,7 +439,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   } else if (warp == 1) {
     // ------------------------------------------------ MMA issuer
     // The whole warp walks the loops and waits together, so that every address and descriptor
-    // is a warp-uniform value; the MMAs and the commits are predicated on one elected lane.
+    // is a warp-uniform value; the MMAs and the commits are predicated on one elected lane.  Where a wait runs out in one
+    // lane it leaves the problem, and all lanes stop where they come together behind it (no shuffle stands inside).
     {
       const bool leader = elect_one();
       bool ok = true;
@@ -455,7 +455,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
 #pragma unroll 1
       for (int l = 0; l < p.n_layers && ok; ++l) {
         const GLayer& L = lay[l];
-        const int n_pu = uni(L.n_pu), n_units = uni(L.n_cb) * n_pu, kpt = uni(L.kpt), total = uni(L.total_tiles), tile0 = uni(L.first);
+        const int n_pu = uni(L.n_pu), n_units = uni(L.n_cb) * n_pu, kpt = uni(L.kpt), total = uni(L.total_tiles), tile0 = uni(L.first), st_steps = uni(L.st_steps);
+        const int end[4] = {uni(L.pu_end[0]), FP4 ? 0 : uni(L.pu_end[1]), FP4 ? 0 : uni(L.pu_end[2]), FP4 ? 0 : uni(L.pu_end[3])};
         // activation operand: rows of 16 bytes, 8-row groups 128 bytes apart, a K step two chunks on; or rows of 128 bytes
         // in the 128-byte swizzle, 8-row groups 1024 bytes apart, a K step 32 bytes on.  (The swizzle permutes address
         // bits, so a tap's start may be any row.)
@@ -486,10 +487,10 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             if (!TR_WAIT(tr_w1, mbar_wait(bar_afull + 8 * a_slot, a_phase))) { ok = false; break; }
             tc_fence_after();
             const uint32_t a_unit = a_base + (uint32_t)a_slot * a_slot_units + row0;
-            const int pu = u & (n_pu - 1), t_last = uni(L.pu_end[pu]);
+            const int pu = u & (n_pu - 1), t_last = FP4 || pu == 0 ? end[0] : pu == 1 ? end[1] : pu == 2 ? end[2] : end[3];
             if (pu == 0) t = 0;
 #define G_ISSUE(KP)                                                                                                  \
-  ok = g_issue_block<MODE, KP>(L, t, t_last, a_fixed, k_step, a_unit, w_base, b_slot_units, d0, idesc, acc, NS, bar_bfull, bar_bempty, b_slot, \
+  ok = g_issue_block<MODE, KP>(L, st_steps, t, t_last, a_fixed, k_step, a_unit, w_base, b_slot_units, d0, idesc, acc, NS, bar_bfull, bar_bempty, b_slot, \
                                b_phase, leader, sf, tr_w2)
             if (kpt == 4) G_ISSUE(4);
             else if (kpt == 2) G_ISSUE(2);
@@ -506,6 +507,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           full_slot = (full_slot + 1) & 3;
           if (++acc_slot == n_acc) { acc_slot = 0; acc_phase ^= 1u; }
         }
+        ok = __all_sync(0xffffffffu, ok);
       }
       if (!ok && leader && !*abort_flag) {
         *abort_flag = 1;
@@ -531,6 +533,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const GTile* const T = reinterpret_cast<const GTile*>(epi_smem) + (seq & 3u);
       const uint32_t tile_phase = (seq >> 2) & 1u;   // (acc_full and the tables are indexed and flip alike)
       if (!wait_phase(bar_tabfull + 8u * (seq & 3u), tile_phase, 100, 6)) break;
+      __syncwarp();   // the table that lane 0 may have waited for is the others', too
       const int4 h0 = *reinterpret_cast<const int4*>(&T->l), h1 = *reinterpret_cast<const int4*>(&T->K);
       const int l = h0.x, n_slices = h0.w, K = h1.x, kp_log = h1.y, lg = F16 ? 0 : h1.z;
       const bool pair = F16 && h1.z;   // (see g_pairs)
@@ -723,7 +726,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
     };
     auto take_slot = [&]() -> bool {
       if (CHAIN) {   // what has been written meanwhile is said first
-        while (unsaid < seq && seq - unsaid < G_TILES && __any_sync(0xffffffffu, mbar_test(bar_tabempty + 8u * (unsaid & 3u), (unsaid >> 2) & 1u)))
+        while (unsaid < seq && seq - unsaid < G_TILES && __all_sync(0xffffffffu, mbar_test(bar_tabempty + 8u * (unsaid & 3u), (unsaid >> 2) & 1u)))
           say_written();
         if (seq - unsaid < G_TILES) return true;
       }
