@@ -577,19 +577,17 @@ bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma,
 // 2000 on the ResNet-18 group on one image and the 1x1 layers lose what they gain).  us, in the order given and so: ResNet-18
 // group on one image 11.5 and 10.3, at batch 3 14.7 and 12.5, 8 21.6 and 18.4; ResNet-34 at 4 23.1 and
 // 20.6; with fp16 activations ResNet-18 at 2 36.3 and 24.7, 16 75 and 69, ResNet-20 at 16 13.8 and 12.2; signs of the 1x1 layers at 16
-// 60.4 and 57.6; signs of ResNet-20 at 64 18.9 and 19.3.  Not where the outputs are more than 256 MB, twice what the L2 holds, and the MMAs
-// more than a fifth of the stores' time: networks then begin with the layers that write the most, and end with outputs that
-// stay in the L2 (ResNet-18 group at batch 64, MMAs two fifths, into a flushed L2 88.5 and 94.9 us, back to back, at the power limit,
-// the same).  1x1 layers at 64, whose MMAs are a tenth, 387 and 381.
+// 60.4 and 57.6; signs of ResNet-20 at 64 18.9 and 19.3.  Not where the outputs are more than 256 MB, twice what the L2 holds: networks
+// then begin with the layers that write the most, and end with outputs that stay in the L2 (ResNet-18 group at batch 64 into a
+// flushed L2 88.5 and 94.9 us, back to back, at the power limit, the same; 1x1 layers at 64 back to back 387 and 381 on one GPU,
+// 375 and 392 on another).
 inline bool g_reorders(const GPlan* plan, int count) {
-  double bytes = 0, mma = 0, drain = 0;
+  double bytes = 0;
   for (int i = 0; i < count; ++i) {
     const GLayer& o = plan[i].L;
     bytes += (double)o.N * o.Ho * o.Wo * o.K * 4.0;
-    mma += o.total_tiles * plan[i].mma;
-    drain += o.total_tiles * plan[i].drain;
   }
-  return bytes <= 256e6 || mma < 0.2 * drain;
+  return bytes <= 256e6;
 }
 inline void g_order(const GPlan* plan, int count, int* order) {
   for (int i = 0; i < count; ++i) order[i] = i;

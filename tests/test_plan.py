@@ -208,8 +208,8 @@ def test_heavy_problems_of_a_group_come_first(lib, f16):
 
 
 @pytest.mark.parametrize("net,n,f16,reorders", [("resnet18", 64, False, False), ("resnet18", 32, False, True), ("resnet34", 64, False, False),
-                                                ("resnet18", 64, True, False), ("resnet50_1x1", 64, False, True), ("resnet20", 128, False, True)])
-def test_large_groups_whose_mmas_take_a_share_keep_their_order(lib, net, n, f16, reorders):
+                                                ("resnet18", 64, True, False), ("resnet50_1x1", 64, False, False), ("resnet50_1x1", 8, False, True), ("resnet20", 128, False, True)])
+def test_groups_of_large_outputs_keep_their_order(lib, net, n, f16, reorders):
     import workloads as wl
     shapes = [(n, s.h, s.w, s.c_in, s.c_out, s.stride, s.pad, s.ksize) for s in getattr(wl, net + "_layers")()]
     assert bool(lib.plan_reorders(_array(shapes), len(shapes), int(f16), SMS)) == reorders
