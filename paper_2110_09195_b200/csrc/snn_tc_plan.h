@@ -87,8 +87,8 @@ struct GLayer {
   int n_ct, total_tiles;  // channel tiles of 128
   int first;              // this CTA's first tile, filled in by the kernel (GParams::ranks)
   uint32_t Qtot;
-  int pair;               // fp16, 33 to 64 channels: the rows of the weight operand hold two columns of the kernel (see g_pairs); a tile's last
-                          // position is not its own then (bit 0; bit 1 + t: step t is an instruction of 64 rows)
+  int pair;               // fp16, 33 to 64 output channels: the rows of the weight operand hold two columns of the kernel (see g_pairs); a tile's last
+                          // position is not its own then
   // A chain (every member reads the packed signs its predecessor writes, all in one launch): a tile may be
   // staged once the predecessor's tiles that hold its input pixels are complete, and says so itself when done.
   const uint2* deps;          // [position tiles] first and last position tile of the predecessor this one reads (x > y: none)
@@ -176,15 +176,27 @@ struct GPlan {
   }
 };
 
-// Two columns of a 3x3 kernel in the rows of the weight operand (fp16 units fetched by TMA, 33 to 64 channels).  With single pixels half of the
-// 128 rows would be idle, and groups of pixels need zeros where a column is outside a pixel's window, which times an infinity
-// are no zeros.  Rows 32*q + 0..15 are channels 16*q.. with kernel column 0, rows 32*q + 16..31 the same channels with the next column of the
-// same parity plane (1, at stride 2 2): both are multiplied with the same positions, so the second column's sum of a position
-// stands one column of the accumulator on, and the epilogue puts the two together.  The third column (2, at stride 2 1) is an instruction
-// of 64 rows, whose accumulator is the first 16 lanes of every quarter: 6 instructions in the time of 128 rows each instead of 9,
-// and no product that is not part of a sum.  (An instruction of 64 rows takes as long as one of 128.)  All eight epilogue warps have channels
-// then, too.  fp16 ResNet-18 group at batch 64 247 and 232 us, 8 41.1 and 38.6; 64 channels of 56x56, 8 images 6.77 and 6.13.
-inline bool g_pairs(const Geom& g, bool tma) { return tma && g.ksize == 3 && g.K > 32 && g.K <= 64; }
+// Two columns of a 3x3 kernel in the rows of the weight operand (fp16 units fetched by TMA, 33 to 64 output channels, stride 1).  With single pixels
+// half of the 128 rows would be idle, and groups of pixels need zeros where a column is outside a pixel's window, which times an infinity
+// are no zeros.  Rows 32*q + 0..15 are channels 16*q.. with one column of the kernel, rows 32*q + 16..31 the same channels with the next one:
+// both are multiplied with the same positions, so the upper rows' sum of a position stands one column of the accumulator on, and the
+// epilogue puts the two together.  Of a kernel row's two steps the first has columns 0 and 1, the second columns 1 and 2: the middle
+// column is there twice, with weights of one half (products and sums of halves are as exact as those of ones), so that no row needs a
+// zero, an infinity reaches the outputs whose windows hold it and no others, and all instructions that add into an accumulator
+// have one shape - those of two shapes would not be ordered among one another.  6 steps instead of 9; all eight epilogue
+// warps have channels, too.  us without pairs and with: fp16 ResNet-18 group at batch 64 253 and 243, 8 40.2 and 38.0; 64 channels of 56x56,
+// 8 images 6.7 and 6.1; 32 to 64 channels of 28x28 4.5 and 4.2; 16 to 64 4.3 and 4.2, 24 to 64 of 56x56 14.4 and 14.3.  Error against 64
+// bits: 64 channels 5.9e-8 and 5.2e-8, 512 5.1e-7 and 3.5e-7, 32 3.4e-8 and 3.2e-8, 16 1.85e-8 and 1.96e-8: not below 32 channels, where there is next to
+// nothing to gain.  (At stride 2 the middle column is in a plane of its own, where the next position's window does not reach.)
+inline bool g_pairs(const Geom& g, bool tma) { return tma && g.ksize == 3 && g.stride == 1 && g.C >= 32 && g.K > 32 && g.K <= 64; }
+// Row r of the weight operand in a step whose lower rows hold kernel column `col` (0 or 1).
+struct GPairRow {
+  int channel, column, halves;   // (weight: so many halves)
+};
+__host__ __device__ inline GPairRow g_pair_row(int r, int col) {
+  const int column = col + (r >> 4 & 1);
+  return {(r >> 5) * 16 + (r & 15), column, column == 1 ? 1 : 2};
+}
 
 // The plan of one layer with tiles of Np positions of 2^lg pixels and blocks of at most max_chunks 16-byte chunks of channels; false
 // where that does not fit.
@@ -262,7 +274,7 @@ bool g_plan_layer(const Geom& g, int mode, int kind, int lg, int Np, bool tma, G
   const uint32_t reach = o.tma ? 8u * (uint32_t)halo : (uint32_t)(o.n_planes * o.Rr);   // largest start of a tap, and chunk distance
   if (reach > 0xffffu || (!o.tma && reach >= (1u << 14))) return false;                 // (the leading-offset field has 14 bits)
   o.n_ct = lg ? 1 : (g.K + G_ROWS - 1) / G_ROWS;
-  const int own = Np - (o.pair & 1);   // positions a tile gives the sums of
+  const int own = Np - o.pair;   // positions a tile gives the sums of
   const long long tiles = (Q + own - 1) / own * o.n_ct;
   if (tiles > 0x7fffffffLL || (Q + own - 1) / own * o.Rr >= (1ll << 31)) return false;
   o.total_tiles = (int)tiles;
@@ -313,9 +325,9 @@ void g_finish_plan(const Geom& g, GPlan* P) {
   // taps in ascending order of where their rows start in the unit
   struct Tap { int plane; uint32_t at; uint8_t row, col; } taps[64];
   int n = 0;
-  if (o.pair) {   // of a kernel row, columns 0 and the next in its plane, then the third
+  if (o.pair) {   // of a kernel row, columns 0 and 1, then 1 and 2
     for (int ky = 0; ky < 3; ++ky)
-      for (int s = 0; s <= 3 - S; s += 3 - S) taps[n++] = {(ky % S) * col_planes + s % col_planes, (uint32_t)((ky / S) * o.Wg + s / col_planes), (uint8_t)ky, (uint8_t)s};
+      for (int s = 0; s < 2; ++s) taps[n++] = {0, (uint32_t)(ky * o.Wg + s), (uint8_t)ky, (uint8_t)s};
   } else if (g.ksize == 1) {
     for (int q = 0; q < o.G; ++q) taps[n++] = {q, 0, 0, (uint8_t)(S * q)};
   } else {
@@ -331,7 +343,6 @@ void g_finish_plan(const Geom& g, GPlan* P) {
     const Tap& b = second ? taps[2 * t + 1] : a;
     const uint32_t dist = P->paired ? b.at - a.at : o.tma ? 1u : (uint32_t)(o.n_planes * o.Rr);
     o.tap[t] = a.at | (dist << 16);
-    if (o.pair && a.col) o.pair |= 2 << t;
     P->taps.row[t][0] = a.row; P->taps.col[t][0] = a.col;
     P->taps.row[t][1] = P->paired && !second ? 255 : b.row;
     P->taps.col[t][1] = b.col;

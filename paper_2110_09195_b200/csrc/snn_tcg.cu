@@ -172,7 +172,6 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int st_steps, int
                                               long long& tr_b) {
   constexpr uint64_t fixed = ((uint64_t)1 << 46) | ((uint64_t)8 << 32);   // descriptor version; 8-row groups 128 bytes apart
   constexpr uint64_t w_fixed = fixed | ((uint64_t)128 << 16);             // the weights' chunks are 128 rows apart
-  const uint32_t pair = MODE == M_F16 ? (uint32_t)L.pair : 0u;
   uint32_t tap = MODE == M_FP4 && KPT == 1 ? 0u : L.tap[t];
 #pragma unroll 1
   while (t < t_last) {
@@ -224,14 +223,13 @@ __device__ __forceinline__ bool g_issue_block(const GLayer& L, int st_steps, int
       const uint32_t cur = tap;
       if (t + 1 < t_last) tap = L.tap[t + 1];
       const uint64_t bd = a_fixed | ((uint64_t)(cur >> 16) << 16) | (uint64_t)(a_unit + (cur & 0xffffu));
-      const uint32_t rows = MODE == M_F16 ? idesc - ((pair >> t & 2u) << 25) : idesc;   // (M >> 4 from bit 24 on: 64 rows instead of 128)
       const uint64_t wd = w_fixed | (uint64_t)wa;
       {
 #pragma unroll
         for (int k = 0; k < KPT; ++k) {
           const uint32_t accum = k == 0 ? acc : 1u;
           if (MODE == M_FP4) mma_ss_fp4(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum, sf, sf + 16, leader);
-          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), rows, accum, leader);
+          else mma_ss_f16(d0, wd + (uint64_t)(k * 256), bd + (uint64_t)((uint32_t)k * k_step), idesc, accum, leader);
         }
       }
       acc = 1;
@@ -479,7 +477,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           uint32_t acc = 0;  // 0 only for the first MMA of the tile
           uint32_t row0 = 0;   // a unit fetched by TMA starts at the beginning of a row of positions
           if (swz) {
-            const uint32_t Q0 = fdiv((uint32_t)tile, L.dCt) * (uint32_t)(L.Np - (L.pair & 1));
+            const uint32_t Q0 = fdiv((uint32_t)tile, L.dCt) * (uint32_t)(L.Np - L.pair);
             row0 = 8u * (Q0 - fdiv(Q0, L.dWg) * (uint32_t)L.Wg);
           }
 #pragma unroll 1
@@ -592,8 +590,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
             __syncwarp();   // the load is a warp-wide instruction
             tmem_ld32(d0 + (uint32_t)(32 * s), v);
             if (F16 && pair) {
-              // Lanes 0..15 hold a channel's sums over two columns of the kernel, lanes 16..31 those over the other, which belong to the
-              // position before: the lower lanes put even positions together and the upper ones odd positions, a shuffle for
+              // Lanes 0..15 hold a channel's sums over one and a half columns of the kernel, lanes 16..31 those over the others, which belong to
+              // the position before: the lower lanes put even positions together and the upper ones odd positions, a shuffle for
               // both.  A store writes 16 channels of two positions.
               uint32_t next = 0;
               const int after = 32 * s + 32;   // the upper lanes need the first column of the next slice
@@ -741,7 +739,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const FastDiv dWg = L.dWg, dHq = L.dHq, dCt = L.dCt;
       const int Np = L.Np, K = L.K, Wg = L.Wg, Hq = L.Hq, Ho = L.Ho, Wo = L.Wo, lg = L.lg, n_ct = L.n_ct, total = L.total_tiles;
       const uint32_t Qtot = L.Qtot;
-      const int own = Np - (F16 ? L.pair & 1 : 0);   // positions of a tile
+      const int own = Np - (F16 ? L.pair : 0);   // positions of a tile
       const int n_slices = (Np + 31) >> 5;
       const int out_kind = WORDS ? (int)p.out_type[0] : OUTK == OUT_SIGNS ? 2 : (int)p.out_type[l];
       const uint32_t scale = out_kind >= 2 ? (uint32_t)(K + 31) >> 5 : (uint32_t)K;   // words of a pixel
@@ -760,7 +758,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
         }
         if (lane == 0) {
           *reinterpret_cast<int4*>(&T->l) = make_int4(l, mg, co, n_slices);
-          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, F16 ? L.pair & 1 : lg, out_kind | (CHAIN && (few || tile + 2 * G >= total) ? 4 : 0) |
+          *reinterpret_cast<int4*>(&T->K) = make_int4(K, L.kp_log, F16 ? L.pair : lg, out_kind | (CHAIN && (few || tile + 2 * G >= total) ? 4 : 0) |
                                                                  (!CHAIN && !TAGGED && tile + G >= total && L.next >= p.n_layers ? 8 : 0));
         }
 #pragma unroll 1
@@ -1146,7 +1144,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
           // above and below the image and channels past the last are out of the tensor's bounds and read as zeros.
           const uint32_t row_bytes = (uint32_t)L.Wg * 128u, ew = (uint32_t)(et >> 5), Hq = (uint32_t)L.Hq;
           const FastDiv dHq = L.dHq, dWg = L.dWg;
-          const int n_pu = L.n_pu, rs = L.rs, pad = L.pad, cpl = L.cpl, own = L.Np - (L.pair & 1);
+          const int n_pu = L.n_pu, rs = L.rs, pad = L.pad, cpl = L.cpl, own = L.Np - L.pair;
 #pragma unroll 1
           for (int tile = L.first; tile < total && !stop; tile += G) {
             const uint32_t Q0 = fdiv((uint32_t)tile, dCt) * (uint32_t)own;
@@ -1355,13 +1353,12 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
   const int which = paired ? c : 0;
   const int ky = taps.row[t][which];
   int kx = (int)taps.col[t][which] - win_step * g;
-  if (pair) {   // (see g_pairs)
-    if (kx == 0) {
-      co = (row >> 5) * 16 + (row & 15);
-      kx = (row & 16) ? win_step : 0;
-    } else {
-      co = row < 64 ? row : K;
-    }
+  uint32_t value = 0x3c00u;   // fp16 1.0
+  if (MODE == M_F16 && pair) {   // (see g_pairs)
+    const GPairRow at = g_pair_row(row, kx);
+    co = at.channel;
+    kx = at.column;
+    if (at.halves == 1) value = 0x3800u;   // 0.5
   }
   constexpr int cpc = MODE == M_F16 ? 8 : 32;
   uint4 v = make_uint4(0, 0, 0, 0);
@@ -1373,7 +1370,7 @@ __global__ void g_expand_weights_kernel(const uint32_t* __restrict__ wplanes, ui
     if (MODE == M_F16) {
 #pragma unroll
       for (int e = 0; e < 8; ++e)
-        if (ch0 + e < C) w[e >> 1] |= (((bits >> e) & 1u) ? 0x3c00u : 0xbc00u) << (16 * (e & 1));  // +1.0 / -1.0
+        if (ch0 + e < C) w[e >> 1] |= (((bits >> e) & 1u) ? value : value | 0x8000u) << (16 * (e & 1));  // + / -
     } else {
 #pragma unroll
       for (int e = 0; e < 32; ++e)
@@ -1537,11 +1534,11 @@ cudaError_t tcg_create(const LayerDev* const* layers, const Geom* geoms, int cou
     if (mode == M_F16)
       g_expand_weights_kernel<M_F16><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
                                                             total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
-                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds, L.pair & 1);
+                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds, L.pair);
     else
       g_expand_weights_kernel<M_FP4><<<blocks, 256, 0, s>>>(Ls[i]->wplanes, Gd->mem + w_off[i], gs[i].C, gs[i].K, gs[i].Cw,
                                                             total, L.cb_chunks, L.n_cb, L.steps, plan[i].paired, L.lg, L.kp_log,
-                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds, L.pair & 1);
+                                                            win_step, ks, plan[i].taps, Ls[i]->alpha, Ls[i]->shift, thresholds, L.pair);
     e = cudaGetLastError();
     if (e == cudaSuccess) *launched += 1;
   }

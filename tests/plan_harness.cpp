@@ -44,6 +44,8 @@ const char* wrong(const GPlan* plan, int count, int mode, const GParams& p, size
       if (end * 16 > plan[i].unit_bytes) return "operand past the unit";
     }
     if (o.pu_end[units - 1] != o.steps) return "units";
+    // a tile's instructions add into one accumulator, and only those of one shape do so in the order in which they are issued
+    if (o.pair != 0 && o.pair != 1) return "instructions of two shapes on one accumulator";
   }
   return nullptr;
 }
@@ -112,6 +114,31 @@ const char* plan_make(const int* gs, int count, int f16, int kind, int sms, int*
   return wrong(plan.data(), count, mode, ring, smem);
 }
 
+// The products that make output position 0 of a pair layer, from what the kernel is told: rows[i] = {channel, kernel row, kernel column, position
+// that is read, halves} of every row and step whose sum the epilogue adds to it, steps in ascending order.  Returns how many, 0: no pairs.
+int plan_pair_products(const int* v, int* rows) {
+  const Geom g = geom(v);
+  GPlan P;
+  if (!g_plan_independent(&g, 1, M_F16, TCG_WORDS, true, 148, &P) || !P.L.pair) return 0;
+  g_finish_plan(g, &P);
+  int n = 0;
+  for (int t = 0; t < P.L.steps; ++t)
+    for (int r = 0; r < G_ROWS; ++r) {
+      const GPairRow at = g_pair_row(r, P.taps.col[t][0]);
+      // (the sums of the upper lanes, 16 to 31 of each 32, are taken from the accumulator column after)
+      const int out[5] = {at.channel, P.taps.row[t][0], at.column, (int)((P.L.tap[t] & 0xffffu) / 8) + (r >> 4 & 1), at.halves};
+      memcpy(rows + 5 * n++, out, sizeof(out));
+    }
+  return n;
+}
+
+// positions of the layer, positions whose sums a tile gives, positions it multiplies, tiles of positions
+void plan_pair_tiles(const int* v, int* out) {
+  const Geom g = geom(v);
+  GPlan P;
+  g_plan_independent(&g, 1, M_F16, TCG_WORDS, true, 148, &P);
+  out[0] = (int)P.L.Qtot; out[1] = P.L.Np - P.L.pair; out[2] = P.L.Np; out[3] = P.L.total_tiles / P.L.n_ct; out[4] = P.L.Wg;
+}
 
 // the order in which a group's problems are walked through, and the MMA cycles of a tile of each problem given
 int plan_order(const int* gs, int count, int f16, int sms, int* order, double* cycles) {

@@ -289,3 +289,17 @@ def test_fp16_layers_of_33_to_64_channels(snn, oracle_mod, c_in, c_out, h, w, n,
         # exact products, fp32 sums of 9*c_in terms: 2^-24 a step of the sum at most, on terms of size one
         assert (np.abs(got[finite] - want[finite]) <= 2.0 ** -24 * 9 * c_in * 1.5 * 4 * np.sqrt(9 * c_in)).all()
     layer.destroy()
+
+
+@pytest.mark.parametrize("unit", [2.0 ** -24, 1024.0])
+@pytest.mark.parametrize("c_in,c_out,h,w,n", [(32, 33, 5, 5, 1), (64, 64, 13, 31, 3), (72, 48, 20, 57, 2)])
+def test_fp16_halves_of_kernel_columns_are_exact(snn, oracle_mod, c_in, c_out, h, w, n, unit):
+    """Activations of whole units, from the smallest fp16 number to near the largest: half a unit is exact, and so is every sum (below 2^24 halves)."""
+    shape = wl.LayerShape(c_in, c_out, h, w, 1, 1)
+    p = wl.draw_layer_params(shape, 6, 800 + c_in)
+    x = (np.random.default_rng(32).integers(-63, 64, (n, h, w, c_in)) * unit).astype(np.float16)
+    want = oracle_mod.conv_f16(p.codebook, 6, p.idx_packed, np.ones(c_out, np.float32), c_in, c_out, 1, 1, x)
+    layer = snn.SnnConv(c_in, c_out, 6, p.codebook, p.idx_packed, np.ones(c_out, np.float32), 1, 1, snn.ACT_F16)
+    got = layer.forward(torch.from_numpy(x).cuda(), path=snn.PATH_DECODED_TC).cpu().numpy()
+    assert (got == want).all()
+    layer.destroy()

@@ -213,3 +213,29 @@ def test_groups_of_large_outputs_keep_their_order(lib, net, n, f16, reorders):
     import workloads as wl
     shapes = [(n, s.h, s.w, s.c_in, s.c_out, s.stride, s.pad, s.ksize) for s in getattr(wl, net + "_layers")()]
     assert bool(lib.plan_reorders(_array(shapes), len(shapes), int(f16), SMS)) == reorders
+
+
+@pytest.mark.parametrize("c_in", [32, 64, 72, 512])
+@pytest.mark.parametrize("c_out", [33, 48, 64])
+@pytest.mark.parametrize("n,h,w,pad", [(1, 5, 5, 1), (3, 15, 15, 0), (2, 9, 31, 1), (8, 56, 56, 1)])
+def test_pairs_of_kernel_columns_make_every_product_once(lib, c_in, c_out, n, h, w, pad):
+    """Rows and steps of the weight operand, as the kernel lays them out and the epilogue adds them up: each (channel, kernel row, kernel
+    column) of an output has the weight one in all, on its own position; a tile's position more is the next tile's first."""
+    rows = np.zeros((6 * 128, 5), np.int32)
+    shape = _array((n, h, w, c_in, c_out, 1, pad, 3))
+    assert lib.plan_pair_products(shape, rows.ctypes.data_as(ctypes.POINTER(ctypes.c_int))) == len(rows)
+    tiles = (ctypes.c_int * 5)()
+    lib.plan_pair_tiles(shape, tiles)
+    positions, own, multiplied, count, pitch = tiles
+    halves = {}
+    for channel, ky, kx, at, weight in rows.tolist():
+        assert at == ky * pitch + kx
+        halves[channel, ky, kx] = halves.get((channel, ky, kx), 0) + weight
+    assert halves == {(c, ky, kx): 2 for c in range(64) for ky in range(3) for kx in range(3)}
+    assert own == multiplied - 1 and (count - 1) * own < positions <= count * own
+
+
+@pytest.mark.parametrize("c_in,c_out,stride,ksize", [(64, 32, 1, 3), (64, 65, 1, 3), (64, 64, 2, 3), (64, 64, 1, 1), (36, 64, 1, 3), (24, 64, 1, 3)])
+def test_other_layers_hold_no_pairs(lib, c_in, c_out, stride, ksize):
+    rows = np.zeros((6 * 128, 5), np.int32)
+    assert not lib.plan_pair_products(_array((2, 20, 20, c_in, c_out, stride, 0, ksize)), rows.ctypes.data_as(ctypes.POINTER(ctypes.c_int)))
