@@ -155,3 +155,27 @@ def test_stored_forms_around_the_sizes_that_go_with_the_launch(snn, oracle_mod, 
         book[:], stream[:], alpha[:] = 0, 0, 0
     for _, _, out, ref in calls:
         assert (out.cpu().numpy() == ref).all()
+
+
+@pytest.mark.parametrize("n,h,w", [(2, 6, 9), (8, 28, 28)])
+def test_calls_behind_the_kernel_that_writes_their_activations(snn, oracle_mod, n, h, w):
+    """A layer's launch writes the activations right before each call, no wait between; calls whose stored form goes with the launch (64
+    outputs) and calls whose arrays are copied (500, tau 9) in turn, each with scales of its own; few tiles, and one on every SM."""
+    first = wl.LayerShape(48, 64, h, w, 1, 1)
+    p = wl.draw_layer_params(first, 6, 300)
+    producer = snn.SnnConv(48, 64, 6, p.codebook, p.idx_packed, p.alpha, 1, 1)
+    act = torch.empty((n, h, w, 2), dtype=torch.int32, device="cuda")
+    calls = []
+    for k, (c_out, tau) in enumerate([(64, 7), (500, 9), (64, 7), (64, 7), (500, 9), (64, 7)]):
+        packed = wl.pack_activation_bits(wl.draw_activation_bits(first, n, 310 + k))
+        sums = oracle_mod.conv_bin(p.codebook, 6, p.idx_packed, p.alpha, 48, 64, 1, 1, packed)[0]
+        q = wl.draw_layer_params(wl.LayerShape(64, c_out, h, w, 1, 1), tau, 320 + k)
+        ref = oracle_mod.conv_bin(q.codebook, tau, q.idx_packed, q.alpha, 64, c_out, 1, 1, wl.pack_activation_bits(sums >= 0))[1]
+        calls.append((torch.from_numpy(packed.view(np.int32)).cuda(), q, c_out, torch.empty((n, h, w, c_out), device="cuda"), ref))
+    torch.cuda.synchronize()
+    for x, q, c_out, out, _ in calls:
+        producer.forward(x, out=act, out_type=snn.OUT_BITS)
+        snn.forward_static(64, c_out, q.tau, q.codebook, q.idx_packed, q.alpha, act, out)
+    for *_, out, ref in calls:
+        assert (out.cpu().numpy() == ref).all()
+    producer.destroy()
