@@ -582,27 +582,45 @@ bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma,
   return true;
 }
 
-// The order in which the CTAs walk through independent problems: those with the most MMAs a tile first, so that the tiles that even out
-// the CTAs' ends are small ones, and the heaviest are not all that is left when the others are done.  Tiles of less than 1200 cycles take as long as their
-// other roles and stay in the order given (by the MMAs alone the ResNet-20 group at batch 4 to 24 is 1 to 3 % slower, and from
-// 2000 on the ResNet-18 group on one image and the 1x1 layers lose what they gain).  us, in the order given and so: ResNet-18
-// group on one image 11.5 and 10.3, at batch 3 14.7 and 12.5, 8 21.6 and 18.4; ResNet-34 at 4 23.1 and
-// 20.6; with fp16 activations ResNet-18 at 2 36.3 and 24.7, 16 75 and 69, ResNet-20 at 16 13.8 and 12.2; signs of the 1x1 layers at 16
-// 60.4 and 57.6; signs of ResNet-20 at 64 18.9 and 19.3.  Not where the outputs are more than 256 MB, twice what the L2 holds: networks
-// then begin with the layers that write the most, and end with outputs that stay in the L2 (ResNet-18 group at batch 64 into a
-// flushed L2 88.5 and 94.9 us, back to back, at the power limit, the same; 1x1 layers at 64 back to back 387 and 381 on one GPU,
-// 375 and 392 on another).
-inline bool g_reorders(const GPlan* plan, int count) {
-  double bytes = 0;
+// The order in which the CTAs walk through independent problems.
+//
+// HEAVY_FIRST: those with the most MMAs a tile first, so that the tiles that even out the CTAs' ends are small ones, and the heaviest are not all that is
+// left when the others are done.  Tiles of less than 1200 cycles take as long as their other roles and stay in the order given (by the MMAs alone the
+// ResNet-20 group at batch 4 to 24 is 1 to 3 % slower).  us, in the order given and so: ResNet-18 group on one image 11.5 and 10.3, at batch 3 14.7
+// and 12.5, 8 21.6 and 18.4; ResNet-34 at 4 23.1 and 20.6; with fp16 activations ResNet-18 at 2 36.3 and 24.7, 16 75 and 69, ResNet-20 at 16
+// 13.8 and 12.2; signs of the 1x1 layers at 16 60.4 and 57.6; signs of ResNet-20 at 64 18.9 and 19.3.
+//
+// GIVEN: where the outputs are more than 256 MB, twice what the L2 holds: networks begin with the layers that write the most, and end with
+// outputs that stay in the L2 (ResNet-18 group at batch 64 into a flushed L2 88.5 and 94.9 us, back to back the same).
+//
+// IN_TURN: where the MMAs of all problems take less than a fifth of the time of their stores (1x1 layers: 0.10 to 0.15, one image 0.22; 3x3 networks from
+// 0.35 on), the one bound most by its stores, then the one bound least, and so on, so that the memory is neither idle nor asked for more
+// than it takes for long.  1x1 layers, us back to back in the order given, heavy first and in turn: batch 2 21.9, 21.5 and 20.6; 4 30.2, 29.1, 28.0; 8 53.8,
+// 56.3, 53.8; 12 81.6, 76.1, 72.8; 20 117.9, 115.2, 114.9; 24 139.2, 138.1, 141.7; 40 232, 229, 227; 64 391, 386, 370 (on a GPU that holds 1.7 GHz at its
+// power limit).  One image 15.8, 15.2, 15.5; ResNet-18 at 16 30.2, 29.1, 31.6, 64 95.9, 95.9, 97.3; ResNet-20 at 128 35.5, 34.8, 35.5.
+enum GOrder { ORDER_GIVEN, ORDER_HEAVY_FIRST, ORDER_IN_TURN };
+inline GOrder g_order_kind(const GPlan* plan, int count, int kind) {
+  if (kind == TCG_SIGNS) return ORDER_HEAVY_FIRST;
+  double bytes = 0, mma = 0, drain = 0;
   for (int i = 0; i < count; ++i) {
     const GLayer& o = plan[i].L;
     bytes += (double)o.N * o.Ho * o.Wo * o.K * 4.0;
+    mma += o.total_tiles * plan[i].mma;
+    drain += o.total_tiles * plan[i].drain;
   }
-  return bytes <= 256e6;
+  return mma < 0.2 * drain ? ORDER_IN_TURN : bytes <= 256e6 ? ORDER_HEAVY_FIRST : ORDER_GIVEN;
 }
-inline void g_order(const GPlan* plan, int count, int* order) {
+inline void g_order(const GPlan* plan, int count, GOrder by, int* order) {
   for (int i = 0; i < count; ++i) order[i] = i;
-  std::stable_sort(order, order + count, [&](int a, int b) { return std::max(plan[a].mma, 1200.0) > std::max(plan[b].mma, 1200.0); });
+  if (by == ORDER_HEAVY_FIRST) {
+    std::stable_sort(order, order + count, [&](int a, int b) { return std::max(plan[a].mma, 1200.0) > std::max(plan[b].mma, 1200.0); });
+  } else if (by == ORDER_IN_TURN) {
+    std::vector<int> bound(order, order + count);
+    std::vector<double> by_stores(count);
+    for (int i = 0; i < count; ++i) by_stores[i] = plan[i].drain / plan[i].mma;
+    std::stable_sort(bound.begin(), bound.end(), [&](int a, int b) { return by_stores[a] > by_stores[b]; });
+    for (int i = 0; i < count; ++i) order[i] = i & 1 ? bound[count - 1 - i / 2] : bound[i / 2];
+  }
 }
 
 // Which CTAs take a problem's odd tiles.  Every CTA gets floor(tiles / grid) tiles of a problem

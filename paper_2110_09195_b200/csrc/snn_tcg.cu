@@ -1409,8 +1409,8 @@ cudaError_t tcg_create(const LayerDev* const* layers, const Geom* geoms, int cou
   for (int i = 0; i < count && chain; ++i)
     if (!g_plan_by_end(gs[i], mode, kind, sms, &plan[i])) return cudaErrorInvalidConfiguration;
   if (!chain && !g_plan_independent(gs, count, mode, kind, tma, sms, plan.data())) return cudaErrorInvalidConfiguration;
-  if (!chain && (kind == TCG_SIGNS || g_reorders(plan.data(), count))) {
-    g_order(plan.data(), count, order);
+  if (!chain) {
+    g_order(plan.data(), count, g_order_kind(plan.data(), count, kind), order);
     const std::vector<GPlan> given(plan);
     for (int i = 0; i < count; ++i) { plan[i] = given[order[i]]; Ls[i] = layers[order[i]]; gs[i] = geoms[order[i]]; }
   }

@@ -140,23 +140,17 @@ void plan_pair_tiles(const int* v, int* out) {
   out[0] = (int)P.L.Qtot; out[1] = P.L.Np - P.L.pair; out[2] = P.L.Np; out[3] = P.L.total_tiles / P.L.n_ct; out[4] = P.L.Wg;
 }
 
-// the order in which a group's problems are walked through, and the MMA cycles of a tile of each problem given
-int plan_order(const int* gs, int count, int f16, int sms, int* order, double* cycles) {
+// the order in which a group's problems are walked through (by: a GOrder, -1: the one of the rule), and the cycles a tile of each problem given takes for
+// its MMAs and its stores.  Returns the GOrder, -1: cannot be planned.
+int plan_order(const int* gs, int count, int f16, int kind, int sms, int by, int* order, double* mma, double* drain) {
   std::vector<Geom> g(count);
   std::vector<GPlan> plan(count);
   for (int i = 0; i < count; ++i) g[i] = geom(gs + 8 * i);
-  if (!g_plan_independent(g.data(), count, f16 ? M_F16 : M_FP4, TCG_WORDS, f16 != 0, sms, plan.data())) return 0;
-  g_order(plan.data(), count, order);
-  for (int i = 0; i < count; ++i) cycles[i] = plan[i].mma;
-  return 1;
-}
-
-// does a group's order differ from the one given?
-int plan_reorders(const int* gs, int count, int f16, int sms) {
-  std::vector<Geom> g(count);
-  std::vector<GPlan> plan(count);
-  for (int i = 0; i < count; ++i) g[i] = geom(gs + 8 * i);
-  return g_plan_independent(g.data(), count, f16 ? M_F16 : M_FP4, TCG_WORDS, f16 != 0, sms, plan.data()) && g_reorders(plan.data(), count);
+  if (!g_plan_independent(g.data(), count, f16 ? M_F16 : M_FP4, kind, f16 != 0, sms, plan.data())) return -1;
+  if (by < 0) by = g_order_kind(plan.data(), count, kind);
+  g_order(plan.data(), count, (GOrder)by, order);
+  for (int i = 0; i < count; ++i) { mma[i] = plan[i].mma; drain[i] = plan[i].drain; }
+  return by;
 }
 
 }  // extern "C"

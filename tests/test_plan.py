@@ -191,6 +191,17 @@ def test_which_chains_of_the_gpu_tests_carry_tags(lib):
         assert bool(lib.plan_tagged(_words(wl.get_workload(net).layers, n))) == tags
 
 
+GIVEN, HEAVY_FIRST, IN_TURN = 0, 1, 2
+
+
+def group_order(lib, shapes, f16=False, kind=WORDS, by=-1):
+    """(which order, the problems in it, cycles of a tile's MMAs, cycles of its stores)"""
+    order, mma, drain = (ctypes.c_int * 32)(), (ctypes.c_double * 32)(), (ctypes.c_double * 32)()
+    by = lib.plan_order(_array(shapes), len(shapes), int(f16), kind, SMS, by, order, mma, drain)
+    assert by >= 0
+    return by, order[:len(shapes)], mma[:len(shapes)], drain[:len(shapes)]
+
+
 @pytest.mark.parametrize("f16", [False, True])
 def test_heavy_problems_of_a_group_come_first(lib, f16):
     """The order is a permutation by the tiles' MMAs, and keeps the order given among problems whose tiles are small or alike."""
@@ -200,19 +211,35 @@ def test_heavy_problems_of_a_group_come_first(lib, f16):
         if not shapes:
             continue
         shapes += shapes[:32 - len(shapes)]
-        order, cycles = (ctypes.c_int * 32)(), (ctypes.c_double * 32)()
-        assert lib.plan_order(_array(shapes), len(shapes), int(f16), SMS, order, cycles)
-        order = order[:len(shapes)]
+        _, order, cycles, _ = group_order(lib, shapes, f16, by=HEAVY_FIRST)
         assert sorted(order) == list(range(len(shapes)))
         assert order == sorted(order, key=lambda i: (-max(cycles[i], 1200.0), i))
 
 
-@pytest.mark.parametrize("net,n,f16,reorders", [("resnet18", 64, False, False), ("resnet18", 32, False, True), ("resnet34", 64, False, False),
-                                                ("resnet18", 64, True, False), ("resnet50_1x1", 64, False, False), ("resnet50_1x1", 8, False, True), ("resnet20", 128, False, True)])
-def test_groups_of_large_outputs_keep_their_order(lib, net, n, f16, reorders):
+def test_problems_bound_by_their_stores_come_in_turn_with_the_others(lib):
+    rng = random.Random(12)
+    for count in (1, 2, 3, 7, 32):
+        shapes = []
+        while len(shapes) < count:
+            shapes += [s for s in (draw(rng),) if takes(lib, s, False)]
+        _, order, mma, drain = group_order(lib, shapes, by=IN_TURN)
+        assert sorted(order) == list(range(count))
+        bound = [drain[i] / mma[i] for i in order]
+        most, least = bound[::2], bound[1::2]
+        assert most == sorted(most, reverse=True) and least == sorted(least) and (not least or min(most) >= max(least))
+
+
+@pytest.mark.parametrize("net,n,f16,kind,by", [
+    ("resnet18", 64, False, WORDS, GIVEN), ("resnet18", 32, False, WORDS, HEAVY_FIRST), ("resnet34", 64, False, WORDS, GIVEN),
+    ("resnet18", 64, True, WORDS, GIVEN), ("resnet20", 128, False, WORDS, HEAVY_FIRST),
+    # stores take most of the time: large groups and small ones, but one image, fp16 activations and packed signs
+    ("resnet50_1x1", 64, False, WORDS, IN_TURN), ("resnet50_1x1", 8, False, WORDS, IN_TURN), ("resnet50_1x1", 1, False, WORDS, HEAVY_FIRST),
+    ("resnet50_1x1", 64, True, WORDS, GIVEN), ("resnet50_1x1", 64, False, SIGNS, HEAVY_FIRST)])
+def test_the_order_of_the_networks_groups(lib, net, n, f16, kind, by):
     import workloads as wl
     shapes = [(n, s.h, s.w, s.c_in, s.c_out, s.stride, s.pad, s.ksize) for s in getattr(wl, net + "_layers")()]
-    assert bool(lib.plan_reorders(_array(shapes), len(shapes), int(f16), SMS)) == reorders
+    got, order, *_ = group_order(lib, shapes, f16, kind)
+    assert got == by and (by != GIVEN or order == sorted(order))
 
 
 @pytest.mark.parametrize("c_in", [32, 64, 72, 512])
