@@ -599,8 +599,10 @@ bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma,
 // 56.3, 53.8; 12 81.6, 76.1, 72.8; 20 117.9, 115.2, 114.9; 24 139.2, 138.1, 141.7; 40 232, 229, 227; 64 391, 386, 370 (on a GPU that holds 1.7 GHz at its
 // power limit).  One image 15.8, 15.2, 15.5; ResNet-18 at 16 30.2, 29.1, 31.6, 64 95.9, 95.9, 97.3; ResNet-20 at 128 35.5, 34.8, 35.5.
 enum GOrder { ORDER_GIVEN, ORDER_HEAVY_FIRST, ORDER_IN_TURN };
-inline GOrder g_order_kind(const GPlan* plan, int count, int kind) {
-  if (kind == TCG_SIGNS) return ORDER_HEAVY_FIRST;
+struct GStores {
+  bool large, bound;   // word outputs of more than twice the L2; MMAs of less than a fifth of the stores' time
+};
+inline GStores g_stores(const GPlan* plan, int count) {
   double bytes = 0, mma = 0, drain = 0;
   for (int i = 0; i < count; ++i) {
     const GLayer& o = plan[i].L;
@@ -608,7 +610,21 @@ inline GOrder g_order_kind(const GPlan* plan, int count, int kind) {
     mma += o.total_tiles * plan[i].mma;
     drain += o.total_tiles * plan[i].drain;
   }
-  return mma < 0.2 * drain ? ORDER_IN_TURN : bytes <= 256e6 ? ORDER_HEAVY_FIRST : ORDER_GIVEN;
+  return {bytes > 256e6, mma < 0.2 * drain};
+}
+inline GOrder g_order_kind(const GPlan* plan, int count, int kind) {
+  if (kind == TCG_SIGNS) return ORDER_HEAVY_FIRST;
+  const GStores stores = g_stores(plan, count);
+  return stores.bound ? ORDER_IN_TURN : stores.large ? ORDER_GIVEN : ORDER_HEAVY_FIRST;
+}
+// Do the words that a launch writes leave the L2 before what else is there?  Where they are more than it holds and most of the launch's time: the sooner
+// they go to memory, the better the memory takes them (64 to 256 channels of 56x56, 64 images: 37.5 and 35.9 us), and the inputs stay.  1x1 layers,
+// us: batch 10 (297 MB) 61.9 and 59.5, 12 72.5 and 70.5, 24 140.8 and 136.0, 32 189.7 and 181.2, 44 268.9 and 258.6, 64 367 and 356.  Below the line there
+// is nothing in it (batch 8 51.7 and 51.0, 6 39.7 and 40.0, 3 26.5 and 26.3) and a kernel that reads the outputs finds them in the L2; nor is
+// there where the MMAs take a share of the time (ResNet-18 at 64 95.6 and 95.3, into a flushed L2 the same).
+inline bool g_streams(const GPlan* plan, int count, int kind) {
+  const GStores stores = g_stores(plan, count);
+  return kind == TCG_WORDS && stores.bound && stores.large;
 }
 inline void g_order(const GPlan* plan, int count, GOrder by, int* order) {
   for (int i = 0; i < count; ++i) order[i] = i;

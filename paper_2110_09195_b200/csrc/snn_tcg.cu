@@ -59,7 +59,7 @@
 //      warp 13       writes the epilogue's tables (where the columns of a tile go) ahead of it, and in a chain on counters says
 //                    which tiles have been written
 //      warp 17       in a chain on counters: waits for the tiles that the CTA's next tile reads
-// The kernel is compiled per operand mode and per output kind (words, packed signs, chains on counters, chains of words
+// The kernel is compiled per operand mode and per output kind (words, words that leave the L2 first, packed signs, chains on counters, chains of words
 // with tags), so that no variant carries another one's code in its loops; the plan (tile shapes, accumulator buffers) is made
 // per output kind, the same for both kinds of chains.
 // The loops around the waits, tiles and problems that all variants have are not unrolled (the compiler unrolls them four times,
@@ -270,9 +270,9 @@ __device__ __forceinline__ void g_transpose32(uint32_t& x, uint32_t& z, int lane
 
 // OUTK: what the epilogue is compiled for.  0: fp32 or int32 words for every member; 1: packed signs for every
 // member; 2: a chain - packed signs between the members, any type for the last, and the dependency waits and
-// completion counters; 3: a chain whose words carry tags instead.  Keeping the variants apart keeps each one's registers and
-// code to what it needs.
-enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2, OUT_TAGGED = 3 };
+// completion counters; 3: a chain whose words carry tags instead; 4: words that leave the L2 first (g_streams).  Keeping the variants apart keeps each one's
+// registers and code to what it needs (a cache policy in a register for both kinds of words took all others 0.2 to 1 %).
+enum { OUT_WORDS = 0, OUT_SIGNS = 1, OUT_CHAIN = 2, OUT_TAGGED = 3, OUT_STREAM = 4 };
 
 template <int MODE, int OUTK>
 __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_constant__ GParams p, const __grid_constant__ GMaps<MODE> maps) {
@@ -280,7 +280,8 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
   constexpr bool FP4 = MODE == M_FP4;   // binary activations as e2m1 nibbles
   constexpr bool TAGGED = OUTK == OUT_TAGGED;   // a chain without waits for whole tiles: every word is looked at until it is there
   constexpr bool CHAIN = OUTK == OUT_CHAIN;
-  constexpr bool WORDS = OUTK == OUT_WORDS;
+  constexpr bool STREAM = OUTK == OUT_STREAM;
+  constexpr bool WORDS = OUTK == OUT_WORDS || STREAM;
   constexpr bool LATE = !CHAIN && !TAGGED;      // see g_ld
   extern __shared__ __align__(1024) uint8_t smem[];
   // carve-up: [NA activation slots][NS weight slots][epilogue tables][pixel tables][problem table][barriers, flags]
@@ -635,10 +636,16 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
                 const uint4 o4 = *reinterpret_cast<const uint4*>(&T->offset[32 * s + e]);
                 const uint32_t o[4] = {o4.x, o4.y, o4.z, o4.w};
 #pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(obase + o[j]),
-                               "r"(v[e + j]), "r"(mask & (1u << (e + j)))
-                               : "memory");
+                for (int j = 0; j < 4; ++j) {
+                  if (STREAM)
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.cs.b32 [%0], %1;\n\t}" ::"l"(obase + o[j]),
+                                 "r"(v[e + j]), "r"(mask & (1u << (e + j)))
+                                 : "memory");
+                  else
+                    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(obase + o[j]),
+                                 "r"(v[e + j]), "r"(mask & (1u << (e + j)))
+                                 : "memory");
+                }
               }
             } else {
               // Packed signs of the scaled output (Algorithm 1: the next layer consumes sign(a)): a sum is compared with the
@@ -1284,6 +1291,7 @@ struct GroupDev {
   int count = 0, act_type = 0, mode = M_FP4;
   int order[SNN_GROUP_MAX] = {};  // which of the caller's problems each one is
   int kind = TCG_WORDS;           // what the tiles were planned for (word outputs, packed signs, chain)
+  bool stream = false;            // word outputs leave the L2 first (g_streams)
   int chain = 0;                  // 1: member i + 1 reads the packed signs member i writes (one launch, on counters or with tags)
   uint8_t* mem = nullptr;         // all device memory of the group; the pointers below lie in it
   uint8_t* chain_buf = nullptr;   // the packed signs between the members, one buffer per boundary
@@ -1495,6 +1503,7 @@ cudaError_t tcg_create(const LayerDev* const* layers, const Geom* geoms, int cou
   Gd->chain = chain;
   std::copy(order, order + count, Gd->order);
   Gd->kind = kind;
+  Gd->stream = mode == M_FP4 && g_streams(plan.data(), count, kind);
   // One allocation and one copy for everything the group owns: [weight operands][descriptions][ranks][dependencies]
   // [counters][count of launches][thresholds of the signs][packed signs between the members]; the three from the descriptions on come from the host.
   auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
@@ -1803,7 +1812,7 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
   cfg.dynamicSmemBytes = G->smem;
   cudaError_t e;
   GMaps<M_FP4> none{};
-  const int outk = G->tagged ? OUT_TAGGED : G->chain ? OUT_CHAIN : (out_type == 2 ? OUT_SIGNS : OUT_WORDS);
+  const int outk = G->tagged ? OUT_TAGGED : G->chain ? OUT_CHAIN : (out_type == 2 ? OUT_SIGNS : G->stream ? OUT_STREAM : OUT_WORDS);
   if (!G->chain && (outk == OUT_SIGNS) != (G->kind == TCG_SIGNS)) return cudaErrorInvalidValue;  // planned for the other kind
 #define G_LAUNCH(M, O, MAPS)                                                    \
   do {                                                                          \
@@ -1828,6 +1837,7 @@ cudaError_t tcg_forward(GroupDev* G, const void* const* act, void* const* out, i
     if (outk == OUT_WORDS) G_LAUNCH(M_F16, OUT_WORDS, maps);
     else return cudaErrorInvalidValue;   // packed signs and chains need binary activations
   } else if (outk == OUT_WORDS) G_LAUNCH(M_FP4, OUT_WORDS, none);
+  else if (outk == OUT_STREAM) G_LAUNCH(M_FP4, OUT_STREAM, none);
   else if (outk == OUT_SIGNS) G_LAUNCH(M_FP4, OUT_SIGNS, none);
   else if (outk == OUT_CHAIN) G_LAUNCH(M_FP4, OUT_CHAIN, none);
   else G_LAUNCH(M_FP4, OUT_TAGGED, none);

@@ -153,4 +153,12 @@ int plan_order(const int* gs, int count, int f16, int kind, int sms, int by, int
   return by;
 }
 
+// do a group's word outputs leave the L2 first?
+int plan_streams(const int* gs, int count, int f16, int kind, int sms) {
+  std::vector<Geom> g(count);
+  std::vector<GPlan> plan(count);
+  for (int i = 0; i < count; ++i) g[i] = geom(gs + 8 * i);
+  return g_plan_independent(g.data(), count, f16 ? M_F16 : M_FP4, kind, f16 != 0, sms, plan.data()) ? g_streams(plan.data(), count, kind) : -1;
+}
+
 }  // extern "C"

@@ -68,6 +68,30 @@ def test_1x1_fp16(snn, oracle_mod):
         layer.destroy()
 
 
+# word outputs of 278 MB and few MMAs: they leave the L2 first (tests/test_plan.py asks the planner)
+STREAMED = [(64, 250, 56, 57, 1, 22), (64, 250, 56, 57, 1, 22), (2048, 33, 7, 7, 1, 3), (72, 250, 113, 113, 2, 22), (40, 333, 29, 57, 1, 31)]
+
+
+def test_1x1_group_of_large_outputs(snn, oracle_mod):
+    layers, acts, refs = [], [], []
+    for i, (c_in, c_out, h, w, stride, n) in enumerate(STREAMED):
+        shape = wl.LayerShape(c_in, c_out, h, w, stride, 0, 1)
+        p = wl.draw_layer_params(shape, 5, 490 + i)
+        packed = wl.pack_activation_bits(wl.draw_activation_bits(shape, n, 490 + i))
+        refs.append(oracle_mod.conv1x1_bin(p.codebook, 5, p.idx_packed, p.alpha, c_in, c_out, stride, packed))
+        layers.append(_layer(snn, shape, p, snn.ACT_BIN))
+        acts.append(torch.from_numpy(packed.view(np.int32)).cuda())
+    group = snn.SnnConvGroup(layers, [(n, h, w) for _, _, h, w, _, n in STREAMED])
+    for which, out_type in enumerate((snn.OUT_I32, snn.OUT_F32)):
+        outs = group.alloc_outs(out_type)
+        group.forward(acts, outs, out_type=out_type)
+        for out, ref in zip(outs, refs):
+            assert (out.cpu().numpy() == ref[which]).all()
+    group.destroy()
+    for l in layers:
+        l.destroy()
+
+
 def _pack_signs(y, shift):
     y = (y.astype(np.float32) + shift.astype(np.float32)[None, None, None, :]).astype(np.float32)
     bits = y >= 0

@@ -242,6 +242,20 @@ def test_the_order_of_the_networks_groups(lib, net, n, f16, kind, by):
     assert got == by and (by != GIVEN or order == sorted(order))
 
 
+@pytest.mark.parametrize("net,n,kind,streams", [("resnet50_1x1", 64, WORDS, True), ("resnet50_1x1", 9, WORDS, True), ("resnet50_1x1", 8, WORDS, False),
+                                                ("resnet50_1x1", 64, SIGNS, False), ("resnet18", 64, WORDS, False), ("resnet34", 64, WORDS, False)])
+def test_which_outputs_leave_the_l2_first(lib, net, n, kind, streams):
+    """More than twice what it holds, where the stores take most of the time."""
+    import workloads as wl
+    shapes = [(n, s.h, s.w, s.c_in, s.c_out, s.stride, s.pad, s.ksize) for s in getattr(wl, net + "_layers")()]
+    assert lib.plan_streams(_array(shapes), len(shapes), 0, kind, SMS) == streams
+
+
+def test_the_large_group_of_the_gpu_tests_leaves_the_l2_first(lib):
+    shapes = [(22, 56, 57, 64, 250, 1, 0, 1)] * 2 + [(3, 7, 7, 2048, 33, 1, 0, 1), (22, 113, 113, 72, 250, 2, 0, 1), (31, 29, 57, 40, 333, 1, 0, 1)]
+    assert lib.plan_streams(_array(shapes), len(shapes), 0, WORDS, SMS) == 1
+
+
 @pytest.mark.parametrize("c_in", [32, 64, 72, 512])
 @pytest.mark.parametrize("c_out", [33, 48, 64])
 @pytest.mark.parametrize("n,h,w,pad", [(1, 5, 5, 1), (3, 15, 15, 0), (2, 9, 31, 1), (8, 56, 56, 1)])
