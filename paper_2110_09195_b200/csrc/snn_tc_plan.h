@@ -48,7 +48,7 @@ struct GTile {
                                        // + 4: the epilogue advances the tile's counter itself, + 8: the CTA's last tile
   uint32_t offset[G_MAX_CHUNKS * 32];  // per column: first output pixel, times K for word outputs
   uint32_t mask[G_MAX_CHUNKS * 8];     // [pixel of the group][slice]: which columns' pixel exists
-  float alpha[G_ROWS], threshold[G_ROWS];
+  float alpha[G_ROWS], minus_threshold[G_ROWS];
 };
 constexpr int G_TILES = 4;
 constexpr int G_EPI_BYTES = G_TILES * (int)sizeof(GTile);
@@ -136,6 +136,10 @@ __host__ __device__ __forceinline__ int g_pixel_of(const GLayer& L, uint32_t n, 
   if (r < 0 || r >= L.H || c < 0 || c >= L.W) return -1;
   return ((int)n * L.H + r) * L.W + c;
 }
+
+// What the sign epilogue adds to a sum: minus the threshold it is compared with.  A threshold of 0 gives +0, so that a sum of 0 is at it whichever sign
+// the tensor core gives a zero.
+__host__ __device__ inline float g_minus_threshold(float threshold) { return 0.f - threshold; }
 
 // Words of a row that are loaded together: activations are 16-byte aligned, so a row can be read four (two) words
 // at a time where the words per pixel and per channel block are multiples of four (two).

@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
       const int s_first = half + (lg || pair ? 0 : 2 * ((rq * 32) >> kp_log)), s_step = lg || pair ? 2 : 2 << (7 - kp_log);
       const int co = h0.z + c_lane, co_warp = h0.z + c_warp;
       const bool active = co_warp < K;   // does any of the warp's rows hold a channel?
-      const float al = T->alpha[c_lane], minus_threshold = WORDS ? 0.f : -T->threshold[c_lane];
+      const float al = T->alpha[c_lane], minus_threshold = WORDS ? 0.f : T->minus_threshold[c_lane];
       const uint32_t flip = al < 0.f ? 0u : 0xffffffffu;   // (the bit is set below the threshold, or - where the sign bit of the difference is clear - from there on)
       {
         if (!TR_WAIT(tr_w0, wait_phase(bar_accfull + 8u * (seq & 3u), tile_phase, 100, 4))) break;
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(G_THREADS, 1) tcg_conv_kernel(const __grid_con
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           T->alpha[32 * i + lane] = al[i];
-          if (!WORDS) T->threshold[32 * i + lane] = th[i];
+          if (!WORDS) T->minus_threshold[32 * i + lane] = g_minus_threshold(th[i]);
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_tabfull + 8u * (seq & 3u));

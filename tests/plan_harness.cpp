@@ -62,6 +62,14 @@ uint32_t plan_divide(uint32_t q, uint32_t d) {
   return (uint32_t)((uint64_t)(2u * q) * f.m >> 32) >> f.s;
 }
 
+// The packed bit of a sum as the epilogue takes it
+int plan_sign(float sum, float threshold, int negative_scale) {
+  const float x = sum + g_minus_threshold(threshold);
+  uint32_t bits;
+  memcpy(&bits, &x, 4);
+  return (int)(bits >> 31) ^ (negative_scale ? 0 : 1);
+}
+
 // Does a chain with at most so many words between two members run on words with tags?
 int plan_tagged(uint64_t words) { return g_tagged((size_t)words); }
 

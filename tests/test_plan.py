@@ -280,3 +280,11 @@ def test_pairs_of_kernel_columns_make_every_product_once(lib, c_in, c_out, n, h,
 def test_other_layers_hold_no_pairs(lib, c_in, c_out, stride, ksize):
     rows = np.zeros((6 * 128, 5), np.int32)
     assert not lib.plan_pair_products(_array((2, 20, 20, c_in, c_out, stride, 0, ksize)), rows.ctypes.data_as(ctypes.POINTER(ctypes.c_int)))
+
+
+@pytest.mark.parametrize("threshold", [0.0, 1.0, -1.0, 4608.0, float("inf")])
+@pytest.mark.parametrize("value", [0.0, -0.0, 1.0, -1.0, 2.0, 4608.0, -4608.0])
+def test_a_sum_at_its_threshold_has_the_bit_whatever_its_zero(lib, value, threshold):
+    lib.plan_sign.argtypes = [ctypes.c_float, ctypes.c_float, ctypes.c_int]
+    assert lib.plan_sign(value, threshold, 0) == (value >= threshold)
+    assert lib.plan_sign(value, threshold, 1) == (value < threshold)
