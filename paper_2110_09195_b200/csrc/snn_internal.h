@@ -113,4 +113,17 @@ inline cudaError_t allow_max_smem(Kernel kernel, unsigned long long* done_mask) 
   return e;
 }
 
+// SMs of the current device, asked for once per device.
+inline int sm_count() {
+  static int known[64] = {0};
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  int* const slot = dev >= 0 && dev < 64 ? known + dev : nullptr;
+  if (slot) sms = __atomic_load_n(slot, __ATOMIC_RELAXED);
+  if (sms) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) return 148;
+  if (slot) __atomic_store_n(slot, sms, __ATOMIC_RELAXED);
+  return sms;
+}
+
 }  // namespace snn

@@ -3,9 +3,9 @@
 // Everything the ordinary path keeps in buffers it allocates at create time
 // (the copied index stream, unpacked indices, codebook, scales, decoded weight
 // bit-planes, border corrections) lives here in ONE fixed device array that is
-// part of the library image.  Each call copies the layer description into that
-// array, writes the tensor-core kernel's weight operand there and runs that kernel on it; a shape the tensor-core
-// kernel does not take is decoded to bit-planes and run by the XOR + popcount kernel.
+// part of the library image.  Each call writes the tensor-core kernel's weight operand there and runs that kernel on it; a layer of more than 32,000
+// bytes, or one whose arrays are not pageable, is copied into the array first.  A shape the tensor-core kernel does not take is copied there, decoded
+// to bit-planes and run by the XOR + popcount kernel.
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -71,9 +71,9 @@ cudaError_t scratch_address(int device, cudaStream_t s, unsigned char** out, int
   return cudaSuccess;
 }
 
-// Plans of recent shapes (host memory): planning tries a dozen tile widths, half a microsecond of a call.
+// Plans of recent shapes on a device (host memory): planning tries a dozen tile widths, half a microsecond of a call.
 struct Planned {
-  int N = 0, H, W, C, K, stride, pad;
+  int N = 0, H, W, C, K, stride, pad, device;
   bool taken;
   TcgStatic plan;
 };
@@ -82,17 +82,17 @@ std::mutex g_plans_mu;
 Planned g_plans[kPlans];
 int g_next_plan = 0;
 
-bool planned(const Geom& g, TcgStatic* out) {
+bool planned(const Geom& g, int device, TcgStatic* out) {   // (the device is the current one)
   std::lock_guard<std::mutex> lk(g_plans_mu);
   for (const Planned& p : g_plans)
-    if (p.N == g.N && p.H == g.H && p.W == g.W && p.C == g.C && p.K == g.K && p.stride == g.stride && p.pad == g.pad) {
+    if (p.N == g.N && p.H == g.H && p.W == g.W && p.C == g.C && p.K == g.K && p.stride == g.stride && p.pad == g.pad && p.device == device) {
       if (p.taken) *out = p.plan;
       return p.taken;
     }
   Planned& p = g_plans[g_next_plan];
   g_next_plan = (g_next_plan + 1) % kPlans;
   p.taken = tcg_static_plan(g, &p.plan);
-  p.N = g.N; p.H = g.H; p.W = g.W; p.C = g.C; p.K = g.K; p.stride = g.stride; p.pad = g.pad;
+  p.N = g.N; p.H = g.H; p.W = g.W; p.C = g.C; p.K = g.K; p.stride = g.stride; p.pad = g.pad; p.device = device;
   if (p.taken) *out = p.plan;
   return p.taken;
 }
@@ -189,7 +189,7 @@ extern "C" SNN_API snn_status_t snn_conv_forward_static(const snn_conv_desc_t* d
   const size_t t_alpha = 1024, t_stream = t_alpha + align256((size_t)g.K * 4), t_mem = align256(t_stream + stream_bytes);
   TcgStatic plan;   // (its `stored` is null)
   g.ksize = 3;
-  if (e == cudaSuccess && status_dev && planned(g, &plan) && t_mem + plan.bytes <= kStaticScratchBytes) {
+  if (e == cudaSuccess && status_dev && planned(g, d->device, &plan) && t_mem + plan.bytes <= kStaticScratchBytes) {
     volatile int* const status = &g_status.word[d->device * 16];
     if (*status) {
       const int code = *status;

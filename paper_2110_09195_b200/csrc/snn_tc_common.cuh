@@ -195,16 +195,5 @@ __device__ __forceinline__ uint4 expand_word_fp4(uint32_t bits, uint32_t sign, u
 // 32 x 32 -> 64-bit product in one instruction (element offsets of pixels: both factors are non-negative 32-bit)
 __device__ __forceinline__ size_t wide_mul(uint32_t a, uint32_t b) { return (size_t)a * (size_t)b; }
 
-
-static inline int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 148;
-  }
-  return sms;
-}
-
 }  // namespace
 }  // namespace snn

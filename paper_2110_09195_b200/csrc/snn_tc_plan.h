@@ -521,8 +521,8 @@ bool g_ring(const GPlan* plan, int count, int mode, GParams* p, size_t* smem) {
 // earlier: the group size of the most throughput leaves most SMs idle when a small layer's work is packed into few heavy
 // tiles.  96 to 20 channels, 16 images of 14x14 at stride 2: 16 tiles 20.7 us, 64 tiles 8.2; 6.3 % over those 384 layers.
 // The 15 % are what the estimate errs by: without them one layer in thirty got slower, by up to a third.  Of the widths
-// only the narrowest that leaves no SM a second tile and the two above are looked at: the no-allocation entry point plans in
-// every call, and all of them took it another microsecond.
+// only the narrowest that leaves no SM a second tile and the two above are looked at: all of them take another microsecond, which the
+// no-allocation entry point pays at the first call of each shape.
 void g_plan_alone(const Geom& g, int mode, int kind, int sms, GPlan* plan) {
   constexpr int widths = sizeof(kNpTable) / sizeof(kNpTable[0]);
   double best = 0.85 * plan->end(sms);

@@ -1,5 +1,5 @@
 """The no-allocation entry point's host code on a fake CUDA runtime: a status page that cannot be pinned at one call is tried
-again by the next (never under capture), and a wait that gave up is reported once."""
+again by the next (never under capture), a wait that gave up is reported once, and plans are a device's own."""
 import ctypes
 import subprocess
 from pathlib import Path
@@ -18,11 +18,23 @@ def call(tmp_path):
                     "-I/usr/local/cuda/include", "-o", str(so), str(ROOT / "tests/static_harness.cpp")], check=True)
     lib = ctypes.CDLL(str(so))
 
-    def one(register_fails=-1, capturing=0):
+    def one(register_fails=-1, capturing=0, device=0):
         out = (ctypes.c_int * 3)()
-        return lib.static_call(register_fails, capturing, out), *out
-    one.report = lib.static_report
+        return lib.static_call(register_fails, capturing, out, device), *out
+
+    def planned():
+        out = (ctypes.c_int * 3)()
+        lib.static_planned(out)
+        return tuple(out)
+    one.report, one.planned = lib.static_report, planned
     return one
+
+
+def test_each_device_has_plans_for_its_own_sms(call):
+    """SMs planned for, plans made, questions asked: a plan is kept for the shape on that device, and so is the number of SMs."""
+    for device, want in ((0, (148, 1, 1)), (0, (148, 1, 1)), (1, (132, 2, 2)), (0, (148, 2, 2)), (1, (132, 2, 2))):
+        assert call(device=device)[0] == SNN_OK
+        assert call.planned() == want
 
 
 def test_pinning_that_failed_is_tried_again(call):
