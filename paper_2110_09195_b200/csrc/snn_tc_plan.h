@@ -188,7 +188,7 @@ struct GPlan {
 // column is there twice, with weights of one half (products and sums of halves are as exact as those of ones), so that no row needs a
 // zero, an infinity reaches the outputs whose windows hold it and no others, and all instructions that add into an accumulator
 // have one shape - those of two shapes would not be ordered among one another.  6 steps instead of 9; all eight epilogue
-// warps have channels, too.  us without pairs and with: fp16 ResNet-18 group at batch 64 253 and 243, 8 40.2 and 38.0; 64 channels of 56x56,
+// warps have channels, too.  us without pairs and with: fp16 ResNet-18 group at batch 64 248 and 232, 8 38.1 and 36.2; 64 channels of 56x56,
 // 8 images 6.7 and 6.1; 32 to 64 channels of 28x28 4.5 and 4.2; 16 to 64 4.3 and 4.2, 24 to 64 of 56x56 14.4 and 14.3.  Error against 64
 // bits: 64 channels 5.9e-8 and 5.2e-8, 512 5.1e-7 and 3.5e-7, 32 3.4e-8 and 3.2e-8, 16 1.85e-8 and 1.96e-8: not below 32 channels, where there is next to
 // nothing to gain.  (At stride 2 the middle column is in a plane of its own, where the next position's window does not reach.)
@@ -463,8 +463,8 @@ bool g_plan_by_end(const Geom& g, int mode, int kind, int sms, GPlan* plan) {
 // Do the packed signs between the members of a chain carry tags?  words: the most between two members.  A layer's signs then reach
 // the next layer's expanders 1.2 us sooner, but each word is twice as long and the expanders load two of them at a time
 // instead of four, which shows once a CTA has many tiles.  Measured on one B200, counters and tags, us: ResNet-20 stack at batch 96
-// (98 k words) 103 and 90, 128 (131 k) 123 and 112; ResNet-34 16 (100 k) 180 and 177, 24 (150 k) 190 and 195; ResNet-18 24 102.0 and
-// 104.6, 32 (200 k) 108.7 and 111.4; on one image, when both kinds took longer, ResNet-18 85 and 67, ResNet-34 162 and 129, ResNet-20 68 and 50.
+// (98 k words) 94.6 and 79.9, 128 (131 k) 111.7 and 102.4; ResNet-18 16 (100 k) 87.8 and 87.1, 24 (150 k) 93.2 and 97.7, 32 (200 k) 99.6 and 108.0;
+// ResNet-34 16 162.9 and 164.6, 24 171.9 and 184.2; on one image ResNet-18 72.3 and 51.3, ResNet-34 139.0 and 96.4, ResNet-20 57.4 and 37.6.
 // (One rule for all: 150 k words are too many for the networks of two to sixteen words a pixel, and 131 k still gain where every
 // pixel is one.  A stack of one layer has no word between members, and with tags no counters to clear.)
 inline bool g_tagged(size_t words) { return words <= (size_t)1 << 17; }
@@ -590,18 +590,18 @@ bool g_plan_independent(const Geom* gs, int count, int mode, int kind, bool tma,
 //
 // HEAVY_FIRST: those with the most MMAs a tile first, so that the tiles that even out the CTAs' ends are small ones, and the heaviest are not all that is
 // left when the others are done.  Tiles of less than 1200 cycles take as long as their other roles and stay in the order given (by the MMAs alone the
-// ResNet-20 group at batch 4 to 24 is 1 to 3 % slower).  us, in the order given and so: ResNet-18 group on one image 11.5 and 10.3, at batch 3 14.7
-// and 12.5, 8 21.6 and 18.4; ResNet-34 at 4 23.1 and 20.6; with fp16 activations ResNet-18 at 2 36.3 and 24.7, 16 75 and 69, ResNet-20 at 16
-// 13.8 and 12.2; signs of the 1x1 layers at 16 60.4 and 57.6; signs of ResNet-20 at 64 18.9 and 19.3.
+// ResNet-20 group at batch 4 to 24 is 1 to 3 % slower).  us, in the order given and so: ResNet-18 group on one image 10.5 and 9.2, at batch 3 13.6
+// and 11.7, 8 20.2 and 17.2, 16 29.2 and 28.3; ResNet-34 at 4 22.0 and 19.8; with fp16 activations ResNet-18 at 2 32.6 and 23.8, 16 70.6 and 63.2,
+// ResNet-20 at 16 12.7 and 11.5; signs of the 1x1 layers at 16 56.0 and 54.0; signs of ResNet-20 at 64 17.4 and 17.8.
 //
 // GIVEN: where the outputs are more than 256 MB, twice what the L2 holds: networks begin with the layers that write the most, and end with
-// outputs that stay in the L2 (ResNet-18 group at batch 64 into a flushed L2 88.5 and 94.9 us, back to back the same).
+// outputs that stay in the L2 (ResNet-18 group at batch 64 into a flushed L2, heavy first 94.9 us and so 88.5, later 96.2 and 90.1; back to back the same).
 //
 // IN_TURN: where the MMAs of all problems take less than a fifth of the time of their stores (1x1 layers: 0.10 to 0.15, one image 0.22; 3x3 networks from
 // 0.35 on), the one bound most by its stores, then the one bound least, and so on, so that the memory is neither idle nor asked for more
-// than it takes for long.  1x1 layers, us back to back in the order given, heavy first and in turn: batch 2 21.9, 21.5 and 20.6; 4 30.2, 29.1, 28.0; 8 53.8,
-// 56.3, 53.8; 12 81.6, 76.1, 72.8; 20 117.9, 115.2, 114.9; 24 139.2, 138.1, 141.7; 40 232, 229, 227; 64 391, 386, 370 (on a GPU that holds 1.7 GHz at its
-// power limit).  One image 15.8, 15.2, 15.5; ResNet-18 at 16 30.2, 29.1, 31.6, 64 95.9, 95.9, 97.3; ResNet-20 at 128 35.5, 34.8, 35.5.
+// than it takes for long.  1x1 layers, us back to back in the order given, heavy first and in turn (from batch 9 on with stores that leave the L2 first, below):
+// batch 2 20.3, 20.5 and 19.3; 4 29.3, 29.0, 27.7; 8 50.9, 52.8, 50.4; 12 75.7, 71.9, 68.4; 24 130.4, 131.7, 132.7; 40 220, 220, 217; 64 385, 380, 367.
+// One image 15.1, 14.9, 15.4; ResNet-18 at 16 29.2, 28.3, 31.2, 64 92.3, 91.7, 93.3; ResNet-20 at 128 33.3, 33.1, 33.4.
 enum GOrder { ORDER_GIVEN, ORDER_HEAVY_FIRST, ORDER_IN_TURN };
 struct GStores {
   bool large, bound;   // word outputs of more than twice the L2; MMAs of less than a fifth of the stores' time
@@ -623,7 +623,7 @@ inline GOrder g_order_kind(const GPlan* plan, int count, int kind) {
 }
 // Do the words that a launch writes leave the L2 before what else is there?  Where they are more than it holds and most of the launch's time: the sooner
 // they go to memory, the better the memory takes them (64 to 256 channels of 56x56, 64 images: 37.5 and 35.9 us), and the inputs stay.  1x1 layers,
-// us: batch 10 (297 MB) 61.9 and 59.5, 12 72.5 and 70.5, 24 140.8 and 136.0, 32 189.7 and 181.2, 44 268.9 and 258.6, 64 367 and 356.  Below the line there
+// us: batch 10 (297 MB) 62.9 and 58.7, 12 73.3 and 67.9, 24 141.9 and 132.5, 32 192.4 and 181.2, 44 269.6 and 259.3, 64 376.5 and 363.6.  Below the line there
 // is nothing in it (batch 8 51.7 and 51.0, 6 39.7 and 40.0, 3 26.5 and 26.3) and a kernel that reads the outputs finds them in the L2; nor is
 // there where the MMAs take a share of the time (ResNet-18 at 64 95.6 and 95.3, into a flushed L2 the same).
 inline bool g_streams(const GPlan* plan, int count, int kind) {
